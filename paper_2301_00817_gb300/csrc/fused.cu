@@ -1,6 +1,6 @@
 // fused.cu -- launchers of the FP32-mixed form: the fused stage kernel
-// (fused_kernel.cuh; the jet-grid instantiations in fused_jet12.cu and
-// fused_jet28.cu), the once-per-step viscosity/CFL pass (k_prestep, and
+// (fused_kernel.cuh; the jet-grid instantiations in fused_jet4.cu,
+// fused_jet12.cu and fused_jet28.cu), the once-per-step viscosity/CFL pass (k_prestep, and
 // its four-node form k_prestep4 here) and the split and join of the
 // float-pair state.  Built with approximate FP32 division and
 // square root.
@@ -311,18 +311,21 @@ void launch_stage_fused(int mode, const Grid& g, const les_params& p, const Fuse
   P.dtl = io.dtl;
   const Consts<float> K = fused_consts<float>(p);
   const bool local = P.dtl != nullptr;
-  // The jet grids (xi and eta bounded, zeta periodic, shifted 16-byte
-  // staging) get instantiations with these fixed at compile time, which fold
-  // the face, wrap and one-sided-difference tests: PM = 12, and PM = 28 when
-  // the tiles also cover eta and zeta exactly (every thread owns a column).
+  // The jet grids (xi and eta bounded, zeta periodic) get instantiations with
+  // these fixed at compile time, which fold the face, wrap and one-sided-
+  // difference tests: PM = 28 when the rows take the shifted 16-byte staging
+  // and the tiles cover eta and zeta exactly (every thread owns a column),
+  // PM = 12 with that staging alone, PM = 4 for the other row lengths.
   // Other grids read them at run time (PM = -1).
-  const bool jet = !g.per[0] && !g.per[1] && g.per[2] && G.vec16;
+  const bool jet = !g.per[0] && !g.per[1] && g.per[2];
   const bool full = g.n[1] % FTJ == 0 && g.n[2] % FTK == 0;
-  const int pm = jet ? (full ? 28 : 12) : -1;
+  const int pm = !jet ? -1 : (!G.vec16 ? 4 : (full ? 28 : 12));
   if (pm == 28)
     launch_stage_jet28(mode, local, p.axis != 0, dyn, G, K, P, io.sc, alpha, L);
   else if (pm == 12)
     launch_stage_jet12(mode, local, p.axis != 0, dyn, G, K, P, io.sc, alpha, L);
+  else if (pm == 4)
+    launch_stage_jet4(mode, local, p.axis != 0, dyn, G, K, P, io.sc, alpha, L);
   else if (dyn)  // (not with an axis: rejected at creation)
     launch_stage_dispatch<false, true, -1>(mode, local, G, K, P, io.sc, alpha, L);
   else if (p.axis)

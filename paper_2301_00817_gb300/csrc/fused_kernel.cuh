@@ -1,6 +1,6 @@
 // fused_kernel.cuh -- one kernel per Runge-Kutta stage (residual + update
 // fused), its helpers and launch templates; fused.cu holds the launchers,
-// fused_jet12.cu and fused_jet28.cu the jet-grid instantiations.
+// fused_jet4.cu, fused_jet12.cu and fused_jet28.cu the jet-grid instantiations.
 //
 // A CTA owns a TJ x TK = 16 x 32 tile of (eta, zeta) columns and marches along
 // xi over a chunk of axial planes.  Per plane it stages the conserved state
@@ -578,8 +578,78 @@ __global__ void __launch_bounds__(FNT, 1)
   const int o1 = (ty + 1) * SK + tx + 2;  // own node, 1-node-halo planes
 
   // ---- stage plane x (state: 2-node halo; metrics, mu/kappa: 1-node halo)
+  // Rows that cannot go as 16-byte pieces (nk % 4 != 0, an open zeta, nk <
+  // FTK): a warp copies a row, one 4-byte cp.async per lane, so a request
+  // covers 128 contiguous bytes; the halo columns of all rows follow, spread
+  // over the threads.  (One thread per row, 36 copies in series and none of
+  // them coalesced, had made such a grid's stage four times the time per
+  // point of an aligned one: 242 us on 131 x 75 x 83.)  The lane's wrapped
+  // columns and the warp's rows do not change from plane to plane.
+  const int jr_q = vec_ok ? 0 : wrap_fast(j0 + ty - 2, nj, per1);
+  const int jr_m = vec_ok ? 0 : wrap_fast(j0 + ty - 1, nj, per1);
+  const int kr = vec_ok ? 0 : wrap_fast(k0 + tx, nk, per2);
+  auto put = [&](float* dst, const float* src, int ig, int jg, int kg, float benign) {
+    if (ig >= 0 && jg >= 0 && kg >= 0)
+      cp_async4(dst, src + ((ig * nj + jg) * nk + kg));
+    else
+      *dst = benign;
+  };
+  auto stage_rows = [&](int slot, int ig) {
+    float* dq = sQ + slot * 5 * PL2;
+    float* dm = sM + slot * 10 * PL1;
+    float* dk = sK + slot * NKF * PL1;
+    // tile rows -2 .. FTJ - 3 (state) and -1 .. FTJ - 2 (metrics, mu/kappa)
+    const int c2 = ty * SK + colk(tx);
+#pragma unroll
+    for (int f = 0; f < 5; ++f)
+      put(dq + f * PL2 + c2, P.qin[0] + (long long)f * G.N, ig, jr_q, kr,
+          (f == 0 || f == 4) ? 1.f : 0.f);
+#pragma unroll
+    for (int f = 0; f < 10; ++f)
+      put(dm + f * PL1 + c2, P.m[0] + (long long)f * G.N, ig, jr_m, kr, 1.f);
+#pragma unroll
+    for (int f = 0; f < NKF; ++f)
+      put(dk + f * PL1 + c2, P.mk[0] + (long long)f * G.N, ig, jr_m, kr, 0.f);
+    // the rows left: four of each state field, two of each other one
+    constexpr int XQ = 4 * 5, XM = 2 * 10, XK = 2 * NKF;
+    for (int r = ty; r < XQ + XM + XK; r += FTJ) {
+      if (r < XQ) {
+        const int f = r >> 2, jj = FTJ - 2 + (r & 3);
+        put(dq + f * PL2 + (jj + 2) * SK + colk(tx), P.qin[0] + (long long)f * G.N, ig,
+            wrap_fast(j0 + jj, nj, per1), kr, (f == 0 || f == 4) ? 1.f : 0.f);
+      } else {
+        const bool met = r < XQ + XM;
+        const int u = met ? r - XQ : r - XQ - XM, f = u >> 1, jj = FTJ - 1 + (u & 1);
+        put((met ? dm : dk) + f * PL1 + (jj + 1) * SK + colk(tx),
+            (met ? P.m[0] : P.mk[0]) + (long long)f * G.N, ig, wrap_fast(j0 + jj, nj, per1), kr,
+            met ? 1.f : 0.f);
+      }
+    }
+    // halo columns: -2, -1, FTK, FTK + 1 of the state rows, -1 and FTK of the others
+    constexpr int HQ = 5 * R2 * 4, HM = 10 * R1 * 2, HK = NKF * R1 * 2;
+    for (int e = tid; e < HQ + HM + HK; e += FNT) {
+      if (e < HQ) {
+        const int h = e & 3, row = e >> 2, f = row / R2, jj = row - f * R2 - 2;
+        const int kk = h < 2 ? h - 2 : FTK + h - 2;
+        put(dq + f * PL2 + (jj + 2) * SK + colk(kk), P.qin[0] + (long long)f * G.N, ig,
+            wrap_fast(j0 + jj, nj, per1), wrap_fast(k0 + kk, nk, per2),
+            (f == 0 || f == 4) ? 1.f : 0.f);
+      } else {
+        const bool met = e < HQ + HM;
+        const int u = met ? e - HQ : e - HQ - HM;
+        const int row = u >> 1, f = row / R1, jj = row - f * R1 - 1, kk = (u & 1) ? FTK : -1;
+        put((met ? dm : dk) + f * PL1 + (jj + 1) * SK + colk(kk),
+            (met ? P.m[0] : P.mk[0]) + (long long)f * G.N, ig, wrap_fast(j0 + jj, nj, per1),
+            wrap_fast(k0 + kk, nk, per2), met ? 1.f : 0.f);
+      }
+    }
+  };
   auto stage_plane = [&](int slot, int x) {
     const int ig = wrap_fast(x, ni, per0);
+    if (!vec_ok) {
+      stage_rows(slot, ig);
+      return;
+    }
     constexpr int JQ = 5 * R2, JM = 10 * R1, JK = NKF * R1;
     // one row per thread, taken by the highest-numbered threads: the lowest
     // ones derive a second node record in the same phase
@@ -587,28 +657,25 @@ __global__ void __launch_bounds__(FNT, 1)
     if (tid < 0) return;
     const float* src;
     float* dst;
-    int jj, halo;
+    int jj;
     float benign;
     if (tid < JQ) {
       const int f = tid / R2;
       jj = tid - f * R2 - 2;
       src = P.qin[0] + (long long)f * G.N;
       dst = sQ + (slot * 5 + f) * PL2 + (jj + 2) * SK;
-      halo = 2;
       benign = (f == 0 || f == 4) ? 1.f : 0.f;
     } else if (tid < JQ + JM) {
       const int u = tid - JQ, f = u / R1;
       jj = u - f * R1 - 1;
       src = P.m[0] + (long long)f * G.N;
       dst = sM + (slot * 10 + f) * PL1 + (jj + 1) * SK;
-      halo = 1;
       benign = 1.f;
     } else {
       const int u = tid - JQ - JM, f = u / R1;
       jj = u - f * R1 - 1;
       src = P.mk[0] + (long long)f * G.N;
       dst = sK + (slot * NKF + f) * PL1 + (jj + 1) * SK;
-      halo = 1;
       benign = 0.f;
     }
     const int jg = wrap_fast(j0 + jj, nj, per1);
@@ -617,12 +684,12 @@ __global__ void __launch_bounds__(FNT, 1)
       return;
     }
     const float* row = src + (ig * nj + jg) * nk;
-    if (vec_ok && kt + SK <= nk) {
+    if (kt + SK <= nk) {
       // the row's global columns kt .. kt + SK - 1, inside the row
       const float* rk = row + kt;
 #pragma unroll
       for (int v = 0; v < SK / 4; ++v) cp_async16(dst + 4 * v, rk + 4 * v);
-    } else if (vec_ok) {
+    } else {
       // the last tile: columns kt .. kt + SK - 1 wrapped at nk (a multiple
       // of 4, so no 16-byte piece straddles the wrap; kt + SK < 2 nk because
       // nk >= FTK)
@@ -630,14 +697,6 @@ __global__ void __launch_bounds__(FNT, 1)
       for (int v = 0; v < SK / 4; ++v) {
         const int kg = (kt + 4 * v < nk) ? kt + 4 * v : kt + 4 * v - nk;
         cp_async16(dst + 4 * v, row + kg);
-      }
-    } else {
-      for (int kk = -halo; kk < FTK + halo; ++kk) {
-        const int kg = wrap_fast(k0 + kk, nk, per2);
-        if (kg >= 0)
-          cp_async4(dst + colk(kk), row + kg);
-        else
-          dst[colk(kk)] = benign;
       }
     }
   };
@@ -1255,8 +1314,11 @@ static void launch_stage_dispatch(int mode, bool local, const FusedGeom& G, cons
     launch_stage_t<FMODE_LAST, true, AXIS, DYN, PM>(G, K, P, sc, alpha, L);
 }
 
-// The jet-grid instantiations (PM = 12 and 28), each compiled in a
+// The jet-grid instantiations (PM = 4, 12 and 28), each compiled in a
 // translation unit of its own so the build compiles them in parallel.
+void launch_stage_jet4(int mode, bool local, bool axis, bool dyn, const FusedGeom& G,
+                       const Consts<float>& K, const FusedPtrs& P, const DevScalars* sc,
+                       double alpha, const Launch& L);
 void launch_stage_jet12(int mode, bool local, bool axis, bool dyn, const FusedGeom& G,
                         const Consts<float>& K, const FusedPtrs& P, const DevScalars* sc,
                         double alpha, const Launch& L);
