@@ -451,9 +451,10 @@ __global__ void k_adj_sensor_terms(Grid g, const double* __restrict__ node,
         if (d == 0) sensor_triple<0>(g, n, c[0], xm, xc, xp);
         else if (d == 1) sensor_triple<1>(g, n, c[1], xm, xc, xp);
         else sensor_triple<2>(g, n, c[2], xm, xc, xp);
-        const double s = P[xp] - 2.0 * P[xc] + P[xm];
-        const double den = P[xp] + 2.0 * P[xc] + P[xm];
-        // nu = |s| / den
+        // nu = |s| / den, rounded as sensor3 does (the sign of s decides the
+        // branch where the pressure is uniform to rounding)
+        const double pm = P[xm] + P[xp];
+        const double s = pm - 2.0 * P[xc], den = pm + 2.0 * P[xc];
         const double iden = 1.0 / den;
         const double ls = ln * sgn_abs(s) * iden;
         const double lden = -ln * fabs(s) * iden * iden;
@@ -950,11 +951,11 @@ void launch_rhs_jvp(const Grid& g, const les_params& p, const Dual* Q, const dou
   const Consts<Dual> K = make_consts<Dual>(p);
   const int nb = nb_for(g.N);
   k_node<Dual, Dual, double, false><<<nb, 256, 0, L.s>>>(g, K, Q, M, nullptr, node, nullptr, nullptr);
-  k_flux<0, Dual, Dual, double><<<nb, 256, 0, L.s>>>(g, K, Q, M, node, mk, flux);
-  k_flux<1, Dual, Dual, double><<<nb, 256, 0, L.s>>>(g, K, Q, M, node, mk, flux + 5 * g.N);
-  k_flux<2, Dual, Dual, double><<<nb, 256, 0, L.s>>>(g, K, Q, M, node, mk, flux + 10 * g.N);
+  const FluxPlan f = flux_plan(g);
+  k_flux3<Dual, Dual, double><<<f.b2 + f.b0 + f.b1, kFluxThreads, 0, L.s>>>(
+      g, K, FluxIO<Dual, Dual, double>{Q, M, node, mk, flux}, f.b2, f.b0, f.len, f.len);
   k_update<Dual, double, Dual, 0><<<nb, 256, 0, L.s>>>(g, flux, nullptr, M, nullptr, 0.0, R);
-  *L.counter += 5;
+  *L.counter += 3;
 }
 
 void launch_pack_dual(long long count, const double* v, const double* d, Dual* out, const Launch& L) {

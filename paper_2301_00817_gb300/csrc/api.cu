@@ -267,8 +267,7 @@ void residual64(les_ctx* c, const lesjet::StageIO64& io, bool with_mu, bool with
     lesjet::launch_mu64(c->g, c->p, io, L);
   }
   ProfScope ps(c, PK_FLUX, L.s);
-  lesjet::launch_sensor64(c->g, io, L);
-  for (int d = 0; d < 3; ++d) lesjet::launch_flux64(c->g, c->p, io, d, L);
+  lesjet::launch_flux64(c->g, c->p, io, L);
 }
 
 // ---- mixed form: float pair (hi, lo) state in the workspace
@@ -756,8 +755,7 @@ int les_step_stage(les_ctx* c, int l, double* Q, les_stream_t stream) {
     if (l == 1) {
       // node quantities and viscosity of Q^n come from les_step_begin
       ProfScope ps(c, PK_FLUX, s);
-      lesjet::launch_sensor64(c->g, io, L);
-      for (int d = 0; d < 3; ++d) lesjet::launch_flux64(c->g, c->p, io, d, L);
+      lesjet::launch_flux64(c->g, c->p, io, L);
     } else {
       residual64(c, io, !c->p.freeze_visc, false, 0, L);
     }
@@ -1147,8 +1145,7 @@ void adj_forward(les_ctx* c, void* aw, const AdjLayout& Ly, double* const S[6], 
     io.Qin = S[l - 1];
     io.node = node_of(l);
     if (l > 1) lesjet::launch_node64(g, c->p, io, false, L);
-    lesjet::launch_sensor64(g, io, L);
-    for (int d = 0; d < 3; ++d) lesjet::launch_flux64(g, c->p, io, d, L);
+    lesjet::launch_flux64(g, c->p, io, L);
     lesjet::launch_update64(g, io, S[0], kAlpha[l - 1], 1, S[l], L);
   }
 }

@@ -38,6 +38,12 @@ __host__ __device__ inline Dual operator/(const Dual& a, const Dual& b) {
   const double q = a.v / b.v;
   return Dual(q, (a.d - q * b.d) / b.v);
 }
+__device__ __forceinline__ Dual dev_fma(const Dual& a, const Dual& b, const Dual& c) {
+  return Dual(fma(a.v, b.v, c.v), a.d * b.v + a.v * b.d + c.d);
+}
+__device__ __forceinline__ Dual dev_mul(const Dual& a, const Dual& b) {
+  return Dual(__dmul_rn(a.v, b.v), a.d * b.v + a.v * b.d);
+}
 __host__ __device__ inline Dual operator+(const Dual& a, double b) { return Dual(a.v + b, a.d); }
 __host__ __device__ inline Dual operator+(double a, const Dual& b) { return Dual(a + b.v, b.d); }
 __host__ __device__ inline Dual operator-(const Dual& a, double b) { return Dual(a.v - b, a.d); }

@@ -137,9 +137,31 @@ __device__ __forceinline__ float dev_sqrt<float>(float x) { return sqrtf(x); }
 
 template <typename T>
 __device__ __forceinline__ T dev_abs(T x) { return x < T(0) ? -x : x; }
+template <>
+__device__ __forceinline__ double dev_abs<double>(double x) { return fabs(x); }  // no FP64 compare
 
+// a > b ? a : b
 template <typename T>
 __device__ __forceinline__ T dev_max(T a, T b) { return a > b ? a : b; }
+// For doubles the comparison runs on the integer pipe (an FP64 compare takes
+// a slot of the FP64 pipe, which bounds these kernels): the bit patterns of
+// two doubles order like their values, in reverse when both are negative.
+// A NaN on either side selects b, as the comparison would.
+template <>
+__device__ __forceinline__ double dev_max<double>(double a, double b) {
+  const long long x = __double_as_longlong(a), y = __double_as_longlong(b);
+  const bool gt = (x & y) < 0 ? x < y : x > y;
+  const unsigned inf = 0x7ff00000u;
+  const bool ordered = ((unsigned)__double2hiint(a) & 0x7fffffffu) <= inf &&
+                       ((unsigned)__double2hiint(b) & 0x7fffffffu) <= inf;
+  return gt && ordered ? a : b;
+}
+
+// a*b + c in one rounding, and a*b in a rounding of its own: with these the
+// rounding of an expression does not depend on which products the compiler
+// contracts, so that a dual-number run rounds as the double run does.
+__device__ __forceinline__ double dev_fma(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ double dev_mul(double a, double b) { return __dmul_rn(a, b); }
 
 // ----------------------------------------------------------------- Philox
 // Philox4x32-10 (Salmon, Moraes, Dror, Shaw, SC'11): ten rounds of two

@@ -33,7 +33,7 @@ void launch_dt_finalize(const les_params& p, double* partials, DevScalars* sc, i
 void launch_mk_to_double(int precision, const Grid& g, const void* mk, int fields, double* out,
                          const Launch& L);
 
-// stage64.cu (FP64 form): node, viscosity, per-direction flux and update
+// stage64.cu (FP64 form): node, viscosity, flux and update
 // passes; each node quantity and interface flux is computed once.
 struct StageIO64 {
   const double* Qin;   // [5][N] stage input state
@@ -47,7 +47,7 @@ struct StageIO64 {
   DevScalars* sc;
   double* dtl = nullptr;  // [N] local steps (dt_mode LOCAL), else nullptr
   double* nu = nullptr;   // [3][N] pressure sensors along xi, eta, zeta
-                          // (k_sensor), or nullptr: k_flux evaluates them
+                          // (k_sensor; the reverse kernels read them)
   double* dyn = nullptr;  // [50][N] scratch of the dynamic SGS procedure
 };
 void launch_node64(const Grid& g, const les_params& p, const StageIO64& io, bool with_dt,
@@ -63,9 +63,9 @@ void launch_dynamic64(const Grid& g, const les_params& p, const StageIO64& io, d
 void launch_dynamic32(const Grid& g, const les_params& p, const float* Q, const float* M,
                       float* node, float* scratch, double* partials, DevScalars* sc,
                       const Launch& L);
-void launch_flux64(const Grid& g, const les_params& p, const StageIO64& io, int dir,
-                   const Launch& L);
-// the three pressure sensors of every node into io.nu (after launch_node64)
+void launch_flux64(const Grid& g, const les_params& p, const StageIO64& io, const Launch& L);
+// the three pressure sensors of every node into io.nu (after launch_node64),
+// for the reverse kernels
 void launch_sensor64(const Grid& g, const StageIO64& io, const Launch& L);
 // mode 0: RHS into out; 1: stage update into out; 2: last stage in place
 void launch_update64(const Grid& g, const StageIO64& io, const double* Q0, double alpha, int mode,

@@ -6,10 +6,10 @@
 //   k_node    per node: primitives u v w p T and the anisotropic spectral
 //             radii lbar (optionally the block minima of the CFL step);
 //   k_mu      per node: mu_eff, kappa_eff (Sutherland + SGS);
-//   k_flux<D> per interface (n, n + e_D): centred inviscid flux minus J^-1
-//             times the Turkel-Vatsa dissipation minus the viscous flux,
-//             stored as exactly twice its value (the interface means'
-//             factors 1/2 are folded away);
+//   k_flux3   per interface (n, n + e_D) of the three directions: centred
+//             inviscid flux minus J^-1 times the Turkel-Vatsa dissipation
+//             minus the viscous flux, stored as exactly twice its value (the
+//             interface means' factors 1/2 are folded away);
 //   k_update  per node: RHS = sum_D (F_{+1/2} - F_{-1/2}) and the stage
 //             update Q^(l) = Q^(0) - alpha_l dt J RHS (or RHS itself), with
 //             the factor 2 taken out once per node.
@@ -57,20 +57,11 @@ void launch_mu64(const Grid& g, const les_params& p, const StageIO64& io, const 
   }
 }
 
-void launch_flux64(const Grid& g, const les_params& p, const StageIO64& io, int dir,
-                   const Launch& L) {
-  const int th = 256, nb = blocks_for(g.N, th);
-  auto K = make_consts<double>(p);
-  double* F = io.flux + 5 * g.N * dir;
-  if (dir == 0)
-    k_flux<0, double, double, double><<<nb, th, 0, L.s>>>(g, K, io.Qin, io.M, io.node, io.mk, F,
-                                                          io.nu);
-  else if (dir == 1)
-    k_flux<1, double, double, double><<<nb, th, 0, L.s>>>(g, K, io.Qin, io.M, io.node, io.mk, F,
-                                                          io.nu);
-  else
-    k_flux<2, double, double, double><<<nb, th, 0, L.s>>>(g, K, io.Qin, io.M, io.node, io.mk, F,
-                                                          io.nu);
+void launch_flux64(const Grid& g, const les_params& p, const StageIO64& io, const Launch& L) {
+  const FluxPlan f = flux_plan(g);
+  const FluxIO<double, double, double> fio{io.Qin, io.M, io.node, io.mk, io.flux};
+  k_flux3<double, double, double><<<f.b2 + f.b0 + f.b1, kFluxThreads, 0, L.s>>>(
+      g, make_consts<double>(p), fio, f.b2, f.b0, f.len, f.len);
   ++*L.counter;
 }
 

@@ -34,6 +34,8 @@ inline int blocks_for(long long count, int threads, long long cap = 0) {
   return (int)b;
 }
 
+constexpr int kFluxThreads = 128;  // k_flux3's block
+
 // ------------------------------------------------------------------ k_node
 // Primitive recovery (System I energy), spectral radii lambda_d = |U_d| +
 // a |grad d| and lbar_xi = lambda_xi + sqrt(lambda_xi lambda_eta) +
@@ -229,8 +231,15 @@ __global__ void __launch_bounds__(256) k_mu(Grid g, Consts<R> K, const TQ* __res
 }
 
 // ------------------------------------------------------------------ k_flux
-// Pressure sensor |p+ - 2p + p-| / (p+ + 2p + p-) of node x along D; a face
-// node of a non-periodic direction takes its inward neighbour's value.
+// Pressure sensor |p+ - 2p + p-| / (p+ + 2p + p-) from the three pressures
+// around a node; a face node of a non-periodic direction takes its inward
+// neighbour's value.
+template <typename R>
+__device__ __forceinline__ R sensor3(R pm, R p0, R pp) {
+  const R s = pm + pp;
+  return dev_abs(dev_fma(R(-2), p0, s)) / dev_fma(R(2), p0, s);
+}
+
 template <int D, typename R>
 __device__ __forceinline__ R sensor(const Grid& g, const R* __restrict__ P, long long x, int cx) {
   const long long s = g.stride[D];
@@ -243,12 +252,11 @@ __device__ __forceinline__ R sensor(const Grid& g, const R* __restrict__ P, long
   }
   const long long xp = (cc == nd - 1) ? xc - (long long)(nd - 1) * s : xc + s;
   const long long xm = (cc == 0) ? xc + (long long)(nd - 1) * s : xc - s;
-  const R pp = P[xp], p0 = P[xc], pm = P[xm];
-  return dev_abs(pp - R(2) * p0 + pm) / (pp + R(2) * p0 + pm);
+  return sensor3(P[xm], P[xc], P[xp]);
 }
 
-// The three sensors of every node, once per residual evaluation (each node's
-// sensor along D is read by its two interfaces along D).
+// The three sensors of every node (the reverse kernels read them; k_flux3
+// evaluates them as it goes).
 template <typename R>
 __global__ void __launch_bounds__(256) k_sensor(Grid g, const R* __restrict__ P,
                                                 R* __restrict__ NU) {
@@ -263,195 +271,371 @@ __global__ void __launch_bounds__(256) k_sensor(Grid g, const R* __restrict__ P,
   }
 }
 
+template <typename R>
+__device__ __forceinline__ R dot3(const R& a0, const R& a1, const R& a2, const R& b0, const R& b1,
+                                  const R& b2) {
+  return dev_fma(a2, b2, dev_fma(a1, b1, dev_mul(a0, b0)));
+}
+
+// What an interface flux along D reads at one of its two nodes.
+template <typename R>
+struct FluxNode {
+  R W[5], p;         // rho, rho u, rho v, rho w, e + p; p
+  R u, v, w, T;
+  R m[9], J;         // metrics and J^-1
+  R lb, mu, ka, sg;  // lbar_D, mu_eff, kappa_eff, sigma_ll (dynamic model)
+  // per node, shared by its two interfaces along D:
+  R F[5];            // J^-1 times the inviscid flux (Eq. hat-flux-G, xi_t = 0)
+  R t1[4], t2[4];    // phi(+t) - phi(-t) of u, v, w, T along T1, T2
+};
+
+template <typename R, typename TQ, typename TM>
+struct FluxIO {
+  const TQ* Q;
+  const TM* M;
+  const R* node;
+  const R* mk;
+  R* F;
+};
+
+template <typename R, typename TQ, typename TM>
+__device__ __forceinline__ void flux_W(const FluxIO<R, TQ, TM>& io, long long N, long long n,
+                                       R W[5], R& p) {
+  p = io.node[3 * N + n];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) W[q] = (R)io.Q[q * N + n];
+  W[4] = (R)io.Q[4 * N + n] + p;
+}
+
+// The node's data but W and p, without the part its interfaces share.
 template <int D, typename R, typename TQ, typename TM>
-__global__ void __launch_bounds__(256) k_flux(Grid g, Consts<R> K, const TQ* __restrict__ Q,
-                                              const TM* __restrict__ M,
-                                              const R* __restrict__ node,
-                                              const R* __restrict__ mk, R* __restrict__ F,
-                                              const R* __restrict__ NU = nullptr) {
+__device__ __forceinline__ void flux_load(const FluxIO<R, TQ, TM>& io, long long N, bool dyn,
+                                          long long n, FluxNode<R>& x) {
+  x.u = io.node[n];
+  x.v = io.node[N + n];
+  x.w = io.node[2 * N + n];
+  x.T = io.node[4 * N + n];
+  x.lb = io.node[(5 + D) * N + n];
+#pragma unroll
+  for (int t = 0; t < 9; ++t) x.m[t] = (R)io.M[t * N + n];
+  x.J = (R)io.M[9 * N + n];
+  x.mu = io.mk[n];
+  x.ka = io.mk[N + n];
+  if (dyn) x.sg = io.mk[2 * N + n];
+}
+
+// The shared part: node flux and tangential differences (c: the node's
+// coordinates along T1 and T2, inside their faces).
+template <int D, typename R, typename TQ, typename TM>
+__device__ __forceinline__ void flux_shared(const Grid& g, const FluxIO<R, TQ, TM>& io,
+                                            long long n, const int c[3], FluxNode<R>& x) {
   constexpr int T1 = (D + 1) % 3, T2 = (D + 2) % 3;
   const long long N = g.N;
-  const R* __restrict__ U = node;
-  const R* __restrict__ V = node + N;
-  const R* __restrict__ Wv = node + 2 * N;
-  const R* __restrict__ P = node + 3 * N;
-  const R* __restrict__ Tt = node + 4 * N;
-  const R* __restrict__ LB = node + (5 + D) * N;
-  // The interface means are left as sums of the two nodes' values and their
-  // powers of two are folded into a few factors (exact in binary floating
-  // point): F is written as exactly 2x the interface flux, and k_update
-  // halves J once per node.
-  const R k2h = R(0.5) * K.k2, k4h = R(0.5) * K.k4;
-  for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N;
-       n += (long long)gridDim.x * blockDim.x) {
-    int c[3];
-    decompose(g, n, c);
-    if (!g.per[D] && c[D] == g.n[D] - 1) continue;
-    if (!g.per[T1] && (c[T1] == 0 || c[T1] == g.n[T1] - 1)) continue;
-    if (!g.per[T2] && (c[T2] == 0 || c[T2] == g.n[T2] - 1)) continue;
-    const long long a = n;
-    const long long b = step(g, n, c, D, 1);
-    const long long am = step(g, n, c, D, -1);
-    const long long bp = step(g, n, c, D, 2);
-    int cb[3] = {c[0], c[1], c[2]};
-    cb[D] = (c[D] + 1 == g.n[D]) ? 0 : c[D] + 1;
+  const long long p1 = step(g, n, c, T1, 1), m1 = step(g, n, c, T1, -1);
+  const long long p2 = step(g, n, c, T2, 1), m2 = step(g, n, c, T2, -1);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const R* phi = io.node + (q == 3 ? 4 : q) * N;
+    x.t1[q] = phi[p1] - phi[m1];
+    x.t2[q] = phi[p2] - phi[m2];
+  }
+  const R mx = x.m[3 * D], my = x.m[3 * D + 1], mz = x.m[3 * D + 2];
+  const R Jt = dev_mul(x.J, dot3(mx, my, mz, x.u, x.v, x.w)), Jp = dev_mul(x.J, x.p);
+  x.F[0] = dev_mul(x.W[0], Jt);
+  x.F[1] = dev_fma(x.W[1], Jt, dev_mul(Jp, mx));
+  x.F[2] = dev_fma(x.W[2], Jt, dev_mul(Jp, my));
+  x.F[3] = dev_fma(x.W[3], Jt, dev_mul(Jp, mz));
+  x.F[4] = dev_mul(x.W[4], Jt);
+}
 
-    // centred inviscid flux (Eq. hat-flux-G, xi_t = 0)
-    const R Ja = (R)M[9 * N + a], Jb = (R)M[9 * N + b];
-    const R ma0 = (R)M[(3 * D) * N + a], ma1 = (R)M[(3 * D + 1) * N + a],
-            ma2 = (R)M[(3 * D + 2) * N + a];
-    const R mb0 = (R)M[(3 * D) * N + b], mb1 = (R)M[(3 * D + 1) * N + b],
-            mb2 = (R)M[(3 * D + 2) * N + b];
-    const R pa = P[a], pb = P[b];
-    const R tha = ma0 * U[a] + ma1 * V[a] + ma2 * Wv[a];
-    const R thb = mb0 * U[b] + mb1 * V[b] + mb2 * Wv[b];
-    R Qa[5], Qb[5];
+// Exactly twice the flux through the interface (a, b = a + e_D): centred
+// inviscid flux minus J^-1 times the Turkel-Vatsa dissipation minus the
+// viscous + SGS flux.  The interface means are left as sums of the two
+// nodes' values and their powers of two are folded into a few factors
+// (exact in binary floating point); k_update halves J once per node.
+template <int D, typename R>
+__device__ __forceinline__ void flux_iface(const Consts<R>& K, const FluxNode<R>& a,
+                                           const FluxNode<R>& b, const R Wm[5], const R Wp[5],
+                                           R nua, R nub, R F[5]) {
+  constexpr int T1 = (D + 1) % 3, T2 = (D + 2) % 3;
+  // Turkel-Vatsa dissipation (Eqs. dissip_term, eps_2/4_dissip, W_dissip).
+  // With D1 = W_b - W_a and E = W_{b+1} - W_{a-1}, the third difference is
+  // E - 3 D1, so eps2 D1 - eps4 D3 = (eps2 + 3 eps4) D1 - eps4 E: two
+  // differences and two multiply-adds per component.  At a face the missing
+  // outside difference is minus the first inside one, i.e. the caller's
+  // W_{a-1} = W_b or W_{b+1} = W_a.
+  const R k2h = R(0.5) * K.k2, k4h = R(0.5) * K.k4, nu = dev_max(nua, nub);
+  const R eps2 = dev_mul(k2h, nu);                          // half of eps^(2)
+  const R eps4 = dev_max(R(0), dev_fma(-k2h, nu, k4h));     // half of eps^(4)
+  const R sJ = a.J + b.J;                                   // 2 J^-1 at the interface
+  const R lJ = dev_mul(a.lb + b.lb, sJ);                    // 4 lambda J^-1
+  const R d1 = dev_mul(lJ, dev_fma(R(3), eps4, eps2)), d3 = dev_mul(lJ, eps4);
 #pragma unroll
-    for (int q = 0; q < 5; ++q) {
-      Qa[q] = (R)Q[q * N + a];
-      Qb[q] = (R)Q[q * N + b];
-    }
-    R Fa[5], Fb[5];
-    Fa[0] = Ja * (Qa[0] * tha);
-    Fa[1] = Ja * (Qa[1] * tha + pa * ma0);
-    Fa[2] = Ja * (Qa[2] * tha + pa * ma1);
-    Fa[3] = Ja * (Qa[3] * tha + pa * ma2);
-    Fa[4] = Ja * ((Qa[4] + pa) * tha);
-    Fb[0] = Jb * (Qb[0] * thb);
-    Fb[1] = Jb * (Qb[1] * thb + pb * mb0);
-    Fb[2] = Jb * (Qb[2] * thb + pb * mb1);
-    Fb[3] = Jb * (Qb[3] * thb + pb * mb2);
-    Fb[4] = Jb * ((Qb[4] + pb) * thb);
+  for (int q = 0; q < 5; ++q)
+    F[q] = dev_fma(d3, Wp[q] - Wm[q], dev_fma(-d1, b.W[q] - a.W[q], a.F[q] + b.F[q]));
 
-    // Turkel-Vatsa dissipation (Eqs. dissip_term, eps_2/4_dissip, W_dissip)
-    const R nua = NU ? NU[D * N + a] : sensor<D>(g, P, a, c[D]);
-    const R nub = NU ? NU[D * N + b] : sensor<D>(g, P, b, cb[D]);
-    const R eps2 = k2h * dev_max(nua, nub);    // half of eps^(2)
-    const R eps4 = dev_max(R(0), k4h - eps2);  // half of eps^(4)
-    const R sJ = Ja + Jb;                      // 2 J^-1 at the interface
-    const R lJ = (LB[a] + LB[b]) * sJ;         // 4 lambda J^-1 at the interface
-    R Fq[5];                                   // 2x
+  // viscous + SGS flux with compact interface gradients (Eqs.
+  // hat-flux-Ev/Fv/Gv, tau_mod, q_mod with Fourier's sign): the normal
+  // differences, and 4x the tangential derivatives (the mean of the two
+  // nodes' central differences)
+  const R dn[4] = {b.u - a.u, b.v - a.v, b.w - a.w, b.T - a.T};
+  R s1[4], s2[4];
 #pragma unroll
-    for (int q = 0; q < 5; ++q) {
-      const R wa = (q == 4) ? Qa[4] + pa : Qa[q];
-      const R wb = (q == 4) ? Qb[4] + pb : Qb[q];
-      const R D1 = wb - wa;
-      R Dm, Dp;
-      if (am >= 0) {
-        const R wm = (q == 4) ? (R)Q[4 * N + am] + P[am] : (R)Q[q * N + am];
-        Dm = wa - wm;
-      } else {
-        Dm = -D1;
-      }
-      if (bp >= 0) {
-        const R wp = (q == 4) ? (R)Q[4 * N + bp] + P[bp] : (R)Q[q * N + bp];
-        Dp = wp - wb;
-      } else {
-        Dp = -D1;
-      }
-      const R D3 = Dp - R(2) * D1 + Dm;
-      Fq[q] = (Fa[q] + Fb[q]) - lJ * (eps2 * D1 - eps4 * D3);
-    }
+  for (int q = 0; q < 4; ++q) {
+    s1[q] = a.t1[q] + b.t1[q];
+    s2[q] = a.t2[q] + b.t2[q];
+  }
+  // interface metrics at 2x their mean
+  R mh[9];
+  if (K.axis) {
+    // a grid with an axis (Reading A27): the J^-1-weighted mean
+    // (J^-1_a m_a + J^-1_b m_b)/(J^-1_a + J^-1_b), kept at 2x like the
+    // plain sum; an axis node's stored metric is J^-1 m already
+    const R wa = (a.J == R(0)) ? R(1) : a.J, wb = (b.J == R(0)) ? R(1) : b.J;
+    const R r2 = R(2) / sJ;
+#pragma unroll
+    for (int t = 0; t < 9; ++t) mh[t] = dev_mul(dev_fma(wa, a.m[t], dev_mul(wb, b.m[t])), r2);
+  } else {
+#pragma unroll
+    for (int t = 0; t < 9; ++t) mh[t] = a.m[t] + b.m[t];
+  }
+  // The flux needs only m.tau and m.q (m = the interface metric of
+  // direction D), which follow from the contractions g_t = m . m_t and
+  // c_t = sum_j m_j dphi_j,t and the divergence without forming the
+  // gradient tensor:
+  //   m.tau_i / mu = sum_t g_t dphi_i,t + sum_t m_t,i c_t - 2/3 m_i div,
+  //   m.grad T     = sum_t g_t dphi_T,t,
+  // where the normal part of div is c_D itself.  With 2x metrics, 1x normal
+  // and 4x tangential differences every sum is 16x its value (g_D and c_D
+  // take the missing factor 4).
+  const R* m = mh + 3 * D;
+  const R* m1 = mh + 3 * T1;
+  const R* m2 = mh + 3 * T2;
+  const R gD = dev_mul(R(4), dot3(m[0], m[1], m[2], m[0], m[1], m[2]));
+  const R g1 = dot3(m[0], m[1], m[2], m1[0], m1[1], m1[2]);
+  const R g2 = dot3(m[0], m[1], m[2], m2[0], m2[1], m2[2]);
+  const R cD = dev_mul(R(4), dot3(m[0], m[1], m[2], dn[0], dn[1], dn[2]));
+  const R c1 = dot3(m[0], m[1], m[2], s1[0], s1[1], s1[2]);
+  const R c2 = dot3(m[0], m[1], m[2], s2[0], s2[1], s2[2]);
+  R div = cD;  // 8 div
+#pragma unroll
+  for (int i = 0; i < 3; ++i) div = dev_fma(m2[i], s2[i], dev_fma(m1[i], s1[i], div));
+  const R eD = dev_fma(R(-2.0 / 3.0), div, cD);
+  R sv[3];  // 16 m.tau_i / mu
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+    sv[i] = dev_fma(m2[i], c2, dev_fma(m1[i], c1, dev_fma(m[i], eD,
+                    dot3(gD, g1, g2, dn[i], s1[i], s2[i]))));
+  const R aT = dot3(gD, g1, g2, dn[3], s1[3], s2[3]);  // 16 m.grad T
+  const R uf[3] = {a.u + b.u, a.v + b.v, a.w + b.w};  // 2 u at the interface
+  // 2 J^-1 m.tau_i = sJ (2 mu) sv_i / 32; 2 J^-1 m.(tau u_f + kappa grad T) =
+  // sJ (2 mu) (2 u_f . sv) / 64 + sJ (2 kappa) aT / 32
+  const R sJ32 = dev_mul(sJ, R(1.0 / 32.0));
+  const R cm = dev_mul(sJ32, a.mu + b.mu), ck = dev_mul(sJ32, a.ka + b.ka);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) F[1 + i] = dev_fma(-cm, sv[i], F[1 + i]);
+  F[4] = dev_fma(dev_mul(R(-0.5), cm), dot3(uf[0], uf[1], uf[2], sv[0], sv[1], sv[2]), F[4]);
+  F[4] = dev_fma(-ck, aT, F[4]);
+  if (K.sgs == LES_SGS_DYNAMIC) {
+    // the modelled isotropic SGS stress sigma_ll/3 (Eq. yoshizawa) at the
+    // interface mean, subtracted from the normal stresses: m.tau_i gains
+    // -m_i sigma/3 and u_f.(m.tau) gains -(u_f . m) sigma/3
+    const R e = dev_mul(dev_mul(sJ, a.sg + b.sg), R(1.0 / 12.0));
+#pragma unroll
+    for (int i = 0; i < 3; ++i) F[1 + i] = dev_fma(e, m[i], F[1 + i]);
+    F[4] = dev_fma(dev_mul(R(0.5), e), dot3(uf[0], uf[1], uf[2], m[0], m[1], m[2]), F[4]);
+  }
+}
 
-    // viscous + SGS flux with compact interface gradients (Eqs.
-    // hat-flux-Ev/Fv/Gv, tau_mod, q_mod with Fourier's sign); the tangential
-    // derivatives are kept as 4x their value (the 1/4 of the mean of the two
-    // central differences is folded away)
-    const R* phi[4] = {U, V, Wv, Tt};
-    R dphi[4][3];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) dphi[q][D] = phi[q][b] - phi[q][a];
-    {
-      const long long ap = step(g, a, c, T1, 1), amm = step(g, a, c, T1, -1);
-      const long long bpp = step(g, b, cb, T1, 1), bm = step(g, b, cb, T1, -1);
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-        dphi[q][T1] = (phi[q][ap] - phi[q][amm]) + (phi[q][bpp] - phi[q][bm]);
-    }
-    {
-      const long long ap = step(g, a, c, T2, 1), amm = step(g, a, c, T2, -1);
-      const long long bpp = step(g, b, cb, T2, 1), bm = step(g, b, cb, T2, -1);
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-        dphi[q][T2] = (phi[q][ap] - phi[q][amm]) + (phi[q][bpp] - phi[q][bm]);
-    }
-    // interface metrics: 8x the mean along the normal, 2x along the
-    // tangents, so that every product with dphi is 8x its value
-    R mh[3][3];
-    if (K.axis) {
-      // a grid with an axis (Reading A27): the J^-1-weighted mean
-      // (J^-1_a m_a + J^-1_b m_b)/(J^-1_a + J^-1_b), kept at 2x like the
-      // plain sum; an axis node's stored metric is J^-1 m already
-      const R wa = (Ja == R(0)) ? R(1) : Ja, wb = (Jb == R(0)) ? R(1) : Jb;
-      const R s2 = R(2) / sJ;
-#pragma unroll
-      for (int t = 0; t < 3; ++t)
-#pragma unroll
-        for (int x = 0; x < 3; ++x)
-          mh[t][x] = (wa * (R)M[(3 * t + x) * N + a] + wb * (R)M[(3 * t + x) * N + b]) * s2;
+// Interfaces along xi (D = 0) or eta (D = 1): a thread walks a chunk of len
+// interfaces along D and keeps node b's data as the next interface's node
+// a, so the node flux, the tangential differences and the sensor are
+// evaluated once per node (plus one per chunk).
+template <int D, typename R, typename TQ, typename TM>
+__device__ __forceinline__ void flux_chain(const Grid& g, const Consts<R>& K,
+                                           const FluxIO<R, TQ, TM>& io, long long id, int len) {
+  constexpr int T1 = (D + 1) % 3, T2 = (D + 2) % 3;
+  const long long N = g.N;
+  const int nif = g.per[D] ? g.n[D] : g.n[D] - 1;  // interfaces of a line
+  const int nch = (nif + len - 1) / len;
+  // consecutive threads take consecutive k
+  int c[3];
+  const long long r = id / g.n[2];
+  c[2] = (int)(id - r * g.n[2]);
+  if (D == 0) {
+    c[0] = (int)(r / g.n[1]);
+    c[1] = (int)(r - (long long)c[0] * g.n[1]);
+  } else {
+    c[0] = (int)(r / nch);
+    c[1] = (int)(r - (long long)c[0] * nch);
+  }
+  if (c[0] >= (D == 0 ? nch : g.n[0])) return;
+  c[D] *= len;
+  if (!g.per[T1] && (c[T1] == 0 || c[T1] == g.n[T1] - 1)) return;
+  if (!g.per[T2] && (c[T2] == 0 || c[T2] == g.n[T2] - 1)) return;
+  const int end = c[D] + len < nif ? c[D] + len : nif;
+  const bool dyn = K.sgs == LES_SGS_DYNAMIC;
+  R* F = io.F + 5 * N * D;
+
+  long long na = idx3(g, c[0], c[1], c[2]);
+  FluxNode<R> a, b;
+  R Wm[5], pm = R(0);
+  const long long nm = step(g, na, c, D, -1);
+  bool has_m = nm >= 0;
+  if (has_m) flux_W(io, N, nm, Wm, pm);
+  flux_W(io, N, na, a.W, a.p);
+  flux_load<D>(io, N, dyn, na, a);
+  flux_shared<D>(g, io, na, c, a);
+  long long nb = step(g, na, c, D, 1);
+  flux_W(io, N, nb, b.W, b.p);
+  R nua = R(0);
+  if (has_m) nua = sensor3(pm, a.p, b.p);
+  for (int x = c[D]; x < end; ++x) {
+    c[D] = x;
+    const long long np = step(g, na, c, D, 2);
+    const bool has_p = np >= 0;
+    R Wp[5], pp = R(0);
+    if (has_p) flux_W(io, N, np, Wp, pp);
+    flux_load<D>(io, N, dyn, nb, b);
+    flux_shared<D>(g, io, nb, c, b);
+    R nub = nua;
+    if (has_p) {
+      nub = sensor3(a.p, b.p, pp);
     } else {
 #pragma unroll
-      for (int t = 0; t < 3; ++t)
-#pragma unroll
-        for (int x = 0; x < 3; ++x)
-          mh[t][x] = (R)M[(3 * t + x) * N + a] + (R)M[(3 * t + x) * N + b];
+      for (int q = 0; q < 5; ++q) Wp[q] = a.W[q];
     }
+    if (!has_m) {
+      nua = nub;
 #pragma unroll
-    for (int x = 0; x < 3; ++x) mh[D][x] = R(4) * mh[D][x];
-    // The flux needs only m.tau and m.q (m = the interface metric of
-    // direction D), which follow from the contractions g_t = m . m_t and
-    // c_t = sum_j m_j dphi_j,t and the divergence without forming the
-    // gradient tensor:
-    //   m.tau_i / mu = sum_t g_t dphi_i,t + sum_t m_t,i c_t - 2/3 m_i div,
-    //   m.grad T     = sum_t g_t dphi_T,t.
-    // With mh (8 m_D, 2 m_t) and dphi (1x along D, 4x along the tangents)
-    // every term below is 64x its value.
-    const R mx = mh[D][0], my = mh[D][1], mz = mh[D][2];  // 8 m
-    R G[3], Cc[3];
-#pragma unroll
-    for (int t = 0; t < 3; ++t) {
-      G[t] = mx * mh[t][0] + my * mh[t][1] + mz * mh[t][2];
-      Cc[t] = mx * dphi[0][t] + my * dphi[1][t] + mz * dphi[2][t];
+      for (int q = 0; q < 5; ++q) Wm[q] = b.W[q];
     }
-    R div = R(0);  // 8 div
+    R Fq[5];
+    flux_iface<D>(K, a, b, Wm, Wp, nua, nub, Fq);
 #pragma unroll
-    for (int t = 0; t < 3; ++t)
-      div += mh[t][0] * dphi[0][t] + mh[t][1] * dphi[1][t] + mh[t][2] * dphi[2][t];
-    const R d23 = R(2.0 / 3.0) * div;
-    const R mv[3] = {mx, my, mz};
-    R sv[3];  // 64 m.tau_i / mu
+    for (int q = 0; q < 5; ++q) F[q * N + na] = Fq[q];
 #pragma unroll
-    for (int i = 0; i < 3; ++i)
-      sv[i] = (G[0] * dphi[i][0] + G[1] * dphi[i][1] + G[2] * dphi[i][2]) +
-              (mh[0][i] * Cc[0] + mh[1][i] * Cc[1] + mh[2][i] * Cc[2]) - mv[i] * d23;
-    const R aT = G[0] * dphi[3][0] + G[1] * dphi[3][1] + G[2] * dphi[3][2];  // 64 m.grad T
-    const R mu = mk[a] + mk[b];                    // 2 mu
-    const R kap = R(2) * (mk[N + a] + mk[N + b]);  // 4 kappa
-    const R uf = U[a] + U[b];  // 2 u at the interface
-    const R vf = V[a] + V[b];
-    const R wf = Wv[a] + Wv[b];
-    // 2 J^-1 m.tau_i = sJ mu sv_i / 128; 2 J^-1 m.(tau u_f + kappa grad T) =
-    // sJ (mu (u_f . sv) + kap aT) / 256
-    const R c1 = sJ * mu * R(1.0 / 128.0), c2 = sJ * R(1.0 / 256.0);
-    R f1 = c1 * sv[0], f2 = c1 * sv[1], f3 = c1 * sv[2];
-    R f4 = c2 * (mu * (uf * sv[0] + vf * sv[1] + wf * sv[2]) + kap * aT);
-    if (K.sgs == LES_SGS_DYNAMIC) {
-      // the modelled isotropic SGS stress sigma_ll/3 (Eq. yoshizawa) at the
-      // interface mean, subtracted from the normal stresses: m.tau_i gains
-      // -m_i sigma/3 and u_f.(m.tau) gains -(u_f . m) sigma/3
-      const R ss = mk[2 * N + a] + mk[2 * N + b];  // 2 sigma_ll
-      const R e1 = sJ * ss * R(1.0 / 48.0);
-      f1 -= e1 * mx;
-      f2 -= e1 * my;
-      f3 -= e1 * mz;
-      f4 -= e1 * R(0.5) * (uf * mx + vf * my + wf * mz);
-    }
-    F[n] = Fq[0];
-    F[N + n] = Fq[1] - f1;
-    F[2 * N + n] = Fq[2] - f2;
-    F[3 * N + n] = Fq[3] - f3;
-    F[4 * N + n] = Fq[4] - f4;
+    for (int q = 0; q < 5; ++q) Wm[q] = a.W[q];
+    has_m = true;
+    a = b;
+    nua = nub;
+    na = nb;
+    nb = np;
+#pragma unroll
+    for (int q = 0; q < 5; ++q) b.W[q] = Wp[q];
+    b.p = pp;
   }
+}
+
+// Interfaces along zeta: one per thread over a block's run of consecutive
+// nodes, which share each node's part through shared memory; only the last
+// node of the run (and a wrap that leaves it) evaluates its neighbour's.
+template <typename R, typename TQ, typename TM>
+__device__ __forceinline__ void flux_zeta(const Grid& g, const Consts<R>& K,
+                                          const FluxIO<R, TQ, TM>& io, long long n0,
+                                          R (*sh)[kFluxThreads]) {
+  const long long N = g.N, n = n0 + threadIdx.x;
+  const R* P = io.node + 3 * N;
+  const bool dyn = K.sgs == LES_SGS_DYNAMIC;
+  int c[3] = {0, 0, 0};
+  bool in = n < N;
+  if (in) {
+    decompose(g, n, c);
+    in = (g.per[0] || (c[0] > 0 && c[0] < g.n[0] - 1)) &&
+         (g.per[1] || (c[1] > 0 && c[1] < g.n[1] - 1));
+  }
+  FluxNode<R> a, b;
+  R nua = R(0);
+  if (in) {
+    flux_W(io, N, n, a.W, a.p);
+    flux_load<2>(io, N, dyn, n, a);
+    flux_shared<2>(g, io, n, c, a);
+    nua = sensor<2>(g, P, n, c[2]);
+#pragma unroll
+    for (int q = 0; q < 5; ++q) sh[q][threadIdx.x] = a.F[q];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      sh[5 + q][threadIdx.x] = a.t1[q];
+      sh[9 + q][threadIdx.x] = a.t2[q];
+    }
+    sh[13][threadIdx.x] = nua;
+  }
+  __syncthreads();
+  if (!in) return;
+  const long long nb = step(g, n, c, 2, 1);
+  if (nb < 0) return;
+  flux_W(io, N, nb, b.W, b.p);
+  flux_load<2>(io, N, dyn, nb, b);
+  R nub;
+  if (nb >= n0 && nb < n0 + kFluxThreads) {
+    const int s = (int)(nb - n0);
+#pragma unroll
+    for (int q = 0; q < 5; ++q) b.F[q] = sh[q][s];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      b.t1[q] = sh[5 + q][s];
+      b.t2[q] = sh[9 + q][s];
+    }
+    nub = sh[13][s];
+  } else {
+    flux_shared<2>(g, io, nb, c, b);
+    nub = sensor<2>(g, P, nb, coord_step(g, c, 2, 1));
+  }
+  R Wm[5], Wp[5], unused;
+  const long long nm = step(g, n, c, 2, -1), np = step(g, n, c, 2, 2);
+  flux_W(io, N, nm >= 0 ? nm : nb, Wm, unused);  // at a face W_{a-1} = W_b
+  flux_W(io, N, np >= 0 ? np : n, Wp, unused);   // and W_{b+1} = W_a
+  R Fq[5];
+  flux_iface<2>(K, a, b, Wm, Wp, nua, nub, Fq);
+#pragma unroll
+  for (int q = 0; q < 5; ++q) io.F[(10 + q) * N + n] = Fq[q];
+}
+
+// The interface fluxes of the three directions in one launch (2x their
+// value, F[D][5][N] at the interface's node a): blocks [0, b2) take zeta,
+// the next b0 xi in chunks of len0, the rest eta in chunks of len1.  Bound by
+// the FP64 pipe, which issues one warp instruction per 64 cycles and
+// scheduler, so the shape is chosen for the fewest FP64 operations: about 145
+// per interface with chunks of 8 (205 before the node part was shared and
+// the dissipation and viscous sums regrouped).  Comparisons and absolute
+// values are done on the integer pipe (dev_max, dev_abs).  Against one launch
+// per direction with a sensor pass ahead of them: the 192 x 96 x 128 step
+// 18.3 -> 13.3 ms, the 48 x 24 x 32 step (three launches fewer per residual)
+// 0.50 -> 0.35 ms.
+template <typename R, typename TQ, typename TM>
+__global__ void __launch_bounds__(kFluxThreads, sizeof(R) == 8 ? 2 : 1)
+    k_flux3(Grid g, Consts<R> K, FluxIO<R, TQ, TM> io, unsigned b2, unsigned b0, int len0,
+            int len1) {
+  __shared__ R sh[14][kFluxThreads];
+  unsigned b = blockIdx.x;
+  if (b < b2) {
+    flux_zeta(g, K, io, (long long)b * kFluxThreads, sh);
+  } else if (b < b2 + b0) {
+    flux_chain<0>(g, K, io, (long long)(b - b2) * kFluxThreads + threadIdx.x, len0);
+  } else {
+    flux_chain<1>(g, K, io, (long long)(b - b2 - b0) * kFluxThreads + threadIdx.x, len1);
+  }
+}
+
+// Blocks of k_flux3 for chunks of at most len interfaces.
+struct FluxPlan {
+  unsigned b2, b0, b1;
+  int len;
+};
+inline FluxPlan flux_plan(const Grid& g) {
+  // Chunks as long as leaves a dozen waves of the two resident blocks per
+  // SM (a chunk repeats one node's part, 22 of its 142 FP64 operations per
+  // interface, so beyond 8 there is nothing left to gain).
+  const long long waves = 3 * g.N / ((long long)kFluxThreads * 2 * sm_count());
+  const int len = waves >= 96 ? 8 : (waves >= 48 ? 4 : (waves >= 24 ? 2 : 1));
+  auto blocks = [](long long t) { return (unsigned)((t + kFluxThreads - 1) / kFluxThreads); };
+  auto chunks = [&](int d) { return ((g.per[d] ? g.n[d] : g.n[d] - 1) + len - 1) / len; };
+  FluxPlan f;
+  f.len = len;
+  f.b2 = blocks(g.N);
+  f.b0 = blocks((long long)chunks(0) * g.n[1] * g.n[2]);
+  f.b1 = blocks((long long)g.n[0] * chunks(1) * g.n[2]);
+  return f;
 }
 
 // ---------------------------------------------------------------- k_update
@@ -485,20 +669,19 @@ __global__ void __launch_bounds__(256) k_update(Grid g, const R* __restrict__ F,
     const long long m0 = step(g, n, c, 0, -1);
     const long long m1 = step(g, n, c, 1, -1);
     const long long m2 = step(g, n, c, 2, -1);
-    // J once per node, halved: k_flux writes 2x the interface fluxes (jh
+    // J once per node, halved: k_flux3 writes 2x the interface fluxes (jh
     // holds the same quotient, taken at set-up)
     const double Jn = (MODE == 0) ? 0.0 : (jh ? jh[n] : 0.5 / (double)M[9 * N + n]);
     const double a = (MODE == 0) ? 0.0 : (dtl ? alpha * dtl[n] : adt);
+    const double aJ = a * Jn;
 #pragma unroll
     for (int q = 0; q < 5; ++q) {
-      R r = R(0);
-      r += F0[q * N + n] - F0[q * N + m0];
-      r += F1[q * N + n] - F1[q * N + m1];
-      r += F2[q * N + n] - F2[q * N + m2];
+      const R r = ((F0[q * N + n] - F0[q * N + m0]) + (F1[q * N + n] - F1[q * N + m1])) +
+                  (F2[q * N + n] - F2[q * N + m2]);
       if (MODE == 0) {
         out[q * N + n] = (TO)(R(0.5) * r);
       } else {
-        out[q * N + n] = (TO)(Q0[q * N + n] - a * (Jn * (double)r));
+        out[q * N + n] = (TO)(Q0[q * N + n] - aJ * (double)r);
       }
     }
   }
