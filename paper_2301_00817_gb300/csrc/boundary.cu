@@ -24,6 +24,8 @@ struct AccHL {
   }
 };
 
+constexpr int kBcThreads = 64;  // block of the boundary kernels
+
 struct JetBC {
   int mode;     // LES_BC_JET or LES_BC_JET_CHAR
   int forced;   // some forcing amplitude is non-zero
@@ -47,9 +49,10 @@ __device__ __forceinline__ void load_prim(const Acc& Q, long long N, long long n
                                           double& rho, double& u, double& v, double& w,
                                           double& p) {
   rho = Q.ld(n);
-  u = Q.ld(N + n) / rho;
-  v = Q.ld(2 * N + n) / rho;
-  w = Q.ld(3 * N + n) / rho;
+  const double ir = 1.0 / rho;
+  u = Q.ld(N + n) * ir;
+  v = Q.ld(2 * N + n) * ir;
+  w = Q.ld(3 * N + n) * ir;
   p = (gamma - 1.0) * (Q.ld(4 * N + n) - 0.5 * rho * (u * u + v * v + w * w));
 }
 
@@ -132,6 +135,20 @@ __device__ __forceinline__ void bc_inflow_part(const Grid& g, const JetBC& b,
   const long long N = g.N;
   const double t = use_host_t ? t_host : sc->t;
   const double two_pi = 6.283185307179586476925286766559;
+  // the four forcing phases are the same for every node: lane f of the warp
+  // takes phase f mod 4, and all lanes share the four
+  double sf[4] = {0.0, 0.0, 0.0, 0.0}, cf[4] = {0.0, 0.0, 0.0, 0.0};
+  if (b.forced) {
+    const int f = threadIdx.x & 3;
+    double s, c;
+    sincos(two_pi * (f == 0 ? b.St[0] : (f == 1 ? b.St[1] : (f == 2 ? b.St[2] : b.St[3]))) * b.Mj * t,
+           &s, &c);
+#pragma unroll
+    for (int l = 0; l < 4; ++l) {
+      sf[l] = __shfl_sync(0xffffffffu, s, l);
+      cf[l] = __shfl_sync(0xffffffffu, c, l);
+    }
+  }
   for (long long n = blk * (long long)blockDim.x + threadIdx.x; n < plane;
        n += (long long)nblk * blockDim.x) {
     const double r = rth[n], th = rth[plane + n];
@@ -149,9 +166,6 @@ __device__ __forceinline__ void bc_inflow_part(const Grid& g, const JetBC& b,
         cm[m] = cm[m - 1] * c1 - sm[m - 1] * s1;
         sm[m] = sm[m - 1] * c1 + cm[m - 1] * s1;
       }
-      double sf[4], cf[4];
-#pragma unroll
-      for (int f = 0; f < 4; ++f) sincos(two_pi * b.St[f] * b.Mj * t, &sf[f], &cf[f]);
       double acc = 0.0;
 #pragma unroll
       for (int m = 0; m < 4; ++m)
@@ -219,11 +233,6 @@ __device__ __forceinline__ void bc_farfield_part(const Grid& g, double gamma,
   }
 }
 
-template <class Acc, typename TM>
-__global__ void k_bc_farfield(Grid g, double gamma, const TM* __restrict__ M, Acc Q) {
-  bc_farfield_part(g, gamma, M, Q, blockIdx.x, gridDim.x);
-}
-
 // Inner ring j = 0 (0 < i < ni-1): azimuthal mean of the first interior
 // ring, one block per axial station, fixed-order tree (deterministic).
 template <class Acc>
@@ -258,21 +267,23 @@ __device__ __forceinline__ void bc_ring_part(const Grid& g, const Acc& Q, int bl
     for (int q = 0; q < 5; ++q) Q.st(q * N + base0 + k, red[q][0]);
 }
 
-template <class Acc>
-__global__ void k_bc_ring(Grid g, Acc Q) {
-  bc_ring_part(g, Q, blockIdx.x);
-}
-
 // The Dirichlet entrance, the far field and the inner ring in one launch
 // (blocks [0, nb_ff) the far field, then nb_in for the entrance, then one per
 // axial station for the ring).  They write disjoint surfaces (i = 0; j = nj-1
 // and j = 0 for 0 < i < ni-1) and read nothing another writes: the far field
 // reads j = nj-2 and the ring j = 1 (distinct for nj >= 3), and the
-// Dirichlet entrance reads no state.
+// Dirichlet entrance reads no state.  (The characteristic entrance reads the
+// plane i = 1 before its edges change: nb_in = 0, and a launch of its own
+// ahead of this one.)  A node takes 150 to 300 dependent FP64 operations, and
+// the FP64 pipe issues one warp instruction per 64 cycles and scheduler, so
+// a few nodes are bound by their latency: blocks of 64 threads, one warp for
+// each of two schedulers, spread them over the SMs (48 x 24 x 32: with blocks of
+// 256 this launch and the exit's had taken 24 + 14 us).
 template <class Acc, typename TM>
-__global__ void k_bc_sides(Grid g, JetBC b, const double* __restrict__ rth,
-                           const TM* __restrict__ M, const DevScalars* __restrict__ sc,
-                           int use_host_t, double t_host, Acc Q, int nb_ff, int nb_in) {
+__global__ void __launch_bounds__(kBcThreads)
+    k_bc_sides(Grid g, JetBC b, const double* __restrict__ rth, const TM* __restrict__ M,
+               const DevScalars* __restrict__ sc, int use_host_t, double t_host, Acc Q, int nb_ff,
+               int nb_in) {
   const int blk = blockIdx.x;
   if (blk < nb_ff)
     bc_farfield_part(g, b.gamma, M, Q, blk, nb_ff);
@@ -286,7 +297,8 @@ __global__ void k_bc_sides(Grid g, JetBC b, const double* __restrict__ rth,
 // the unit xi-normal) copies; subsonic takes p = 1/gamma and extrapolates the
 // velocity and the internal energy p/((gamma-1) rho).
 template <class Acc, typename TM>
-__global__ void k_bc_exit(Grid g, double gamma, const TM* __restrict__ M, Acc Q) {
+__global__ void __launch_bounds__(kBcThreads)
+    k_bc_exit(Grid g, double gamma, const TM* __restrict__ M, Acc Q) {
   const int ni = g.n[0];
   const long long plane = (long long)g.n[1] * g.n[2];
   const long long N = g.N;
@@ -307,13 +319,13 @@ __global__ void k_bc_exit(Grid g, double gamma, const TM* __restrict__ M, Acc Q)
 #pragma unroll
       for (int q = 0; q < 5; ++q) Q.st(q * N + nx_, Q.ld(q * N + ne));
     } else {
-      const double eint = p / (gm1 * rho);
-      const double rf = (1.0 / gamma) / (gm1 * eint);
+      // rho_f = p_inf/((gamma-1) e_int) = p_inf rho/p, e_int = p/((gamma-1) rho)
+      const double rf = rho / (gamma * p);
       Q.st(nx_, rf);
       Q.st(N + nx_, rf * u);
       Q.st(2 * N + nx_, rf * v);
       Q.st(3 * N + nx_, rf * w);
-      Q.st(4 * N + nx_, rf * (eint + 0.5 * (u * u + v * v + w * w)));
+      Q.st(4 * N + nx_, 1.0 / (gamma * gm1) + 0.5 * rf * (u * u + v * v + w * w));
     }
   }
 }
@@ -388,8 +400,8 @@ __global__ void k_set_time(DevScalars* sc, double t) {
 }
 
 static int nblocks(long long count) {
-  long long b = (count + 255) / 256;
-  const long long cap = 16LL * sm_count();
+  long long b = (count + kBcThreads - 1) / kBcThreads;
+  const long long cap = 64LL * sm_count();
   if (b > cap) b = cap;
   return (int)(b < 1 ? 1 : b);
 }
@@ -416,25 +428,19 @@ static void bc_jet(const Grid& g, const les_params& p, Acc Q, const TM* M,
   // and the exit only if it ends there (its far field and inner ring cover
   // its ghost planes too, which the next exchange overwrites)
   const int nb_ff = nblocks((long long)(g.n[0] - 2) * g.n[2]);
-  if (p.bc != LES_BC_JET_CHAR && g.n[1] >= 3) {
-    const int nb_in = g.glo == 0 ? nblocks(plane) : 0;
-    k_bc_sides<Acc, TM><<<nb_ff + nb_in + (g.n[0] - 2), 256, 0, L.s>>>(
-        g, b, rth, M, sc, use_host_t, t_host, Q, nb_ff, nb_in);
-    ++*L.counter;
-  } else {
+  int nb_in = g.glo == 0 ? nblocks(plane) : 0;
+  if (p.bc == LES_BC_JET_CHAR && nb_in > 0) {
     // the characteristic entrance reads the plane i = 1 before the far field
     // and the ring write its edges
-    if (g.glo == 0) {
-      k_bc_inflow<Acc, TM><<<nblocks(plane), 256, 0, L.s>>>(g, b, rth, M, sc, use_host_t, t_host,
-                                                             Q);
-      ++*L.counter;
-    }
-    k_bc_farfield<Acc, TM><<<nb_ff, 256, 0, L.s>>>(g, p.gamma, M, Q);
-    k_bc_ring<Acc><<<g.n[0] - 2, 256, 0, L.s>>>(g, Q);
-    *L.counter += 2;
+    k_bc_inflow<Acc, TM><<<nb_in, kBcThreads, 0, L.s>>>(g, b, rth, M, sc, use_host_t, t_host, Q);
+    ++*L.counter;
+    nb_in = 0;
   }
+  k_bc_sides<Acc, TM><<<nb_ff + nb_in + (g.n[0] - 2), kBcThreads, 0, L.s>>>(
+      g, b, rth, M, sc, use_host_t, t_host, Q, nb_ff, nb_in);
+  ++*L.counter;
   if (g.ghi == 0) {
-    k_bc_exit<Acc, TM><<<nblocks(plane), 256, 0, L.s>>>(g, p.gamma, M, Q);
+    k_bc_exit<Acc, TM><<<nblocks(plane), kBcThreads, 0, L.s>>>(g, p.gamma, M, Q);
     ++*L.counter;
   }
 }
