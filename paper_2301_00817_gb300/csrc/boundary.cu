@@ -382,11 +382,11 @@ __global__ void k_totals_partial(Grid g, View Q, const TM* __restrict__ M,
   }
 }
 
-__global__ void k_totals_final(const double* __restrict__ partials, DevScalars* sc) {
+__global__ void k_totals_final(const double* __restrict__ partials, int nb, DevScalars* sc) {
   const int q = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (q >= 5) return;
   double v = 0.0;
-  for (int b = lane; b < kRedBlocks; b += 32) v += partials[q * kRedBlocks + b];
+  for (int b = lane; b < nb; b += 32) v += partials[q * kRedBlocks + b];
   for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
   if (lane == 0) sc->totals[q] = v;
 }
@@ -470,8 +470,9 @@ void launch_bc_jet_hl(const Grid& g, const les_params& p, float* hi, float* lo, 
 template <class View, typename TM>
 static void totals_t(const Grid& g, View Q, const TM* M, double* partials, DevScalars* sc,
                      const Launch& L) {
-  k_totals_partial<View, TM><<<kRedBlocks, kRedThreads, 0, L.s>>>(g, Q, M, partials);
-  k_totals_final<<<1, 160, 0, L.s>>>(partials, sc);
+  const int nb = red_blocks(g.N);
+  k_totals_partial<View, TM><<<nb, kRedThreads, 0, L.s>>>(g, Q, M, partials);
+  k_totals_final<<<1, 160, 0, L.s>>>(partials, nb, sc);
   *L.counter += 2;
 }
 
@@ -498,9 +499,10 @@ void launch_totals_hl(const Grid& g, const float* hi, const float* lo, const flo
 template <typename TM>
 static void join_totals_t(const Grid& g, const float* hi, const float* lo, const TM* M, double* q,
                           double* partials, DevScalars* sc, const Launch& L) {
-  k_totals_partial<ViewHL, TM, true><<<kRedBlocks, kRedThreads, 0, L.s>>>(g, ViewHL{hi, lo}, M,
-                                                                        partials, q);
-  k_totals_final<<<1, 160, 0, L.s>>>(partials, sc);
+  const int nb = red_blocks(g.N);
+  k_totals_partial<ViewHL, TM, true><<<nb, kRedThreads, 0, L.s>>>(g, ViewHL{hi, lo}, M, partials,
+                                                                   q);
+  k_totals_final<<<1, 160, 0, L.s>>>(partials, nb, sc);
   *L.counter += 2;
 }
 

@@ -264,13 +264,13 @@ void launch_prestep(const Grid& g, const les_params& p, const float* Q0, const f
                       reinterpret_cast<uintptr_t>(mk) | reinterpret_cast<uintptr_t>(dtl)) &
                      15) == 0;
   if (p.sgs_model != LES_SGS_DYNAMIC && !p.axis && g.n[2] % 4 == 0 && al16)
-    k_prestep4<<<kRedBlocks, kRedThreads, 0, L.s>>>(g, K, Q0, M, mk, partials, sc, dtl,
+    k_prestep4<<<red_blocks(g.N / 4), kRedThreads, 0, L.s>>>(g, K, Q0, M, mk, partials, sc, dtl,
                                                      (float)p.cfl, fm, p.cfl, p.dt_fixed, finalize);
   else if (p.sgs_model == LES_SGS_DYNAMIC)
-    k_prestep<float, float, float, true><<<kRedBlocks, kRedThreads, 0, L.s>>>(
+    k_prestep<float, float, float, true><<<red_blocks(g.N), kRedThreads, 0, L.s>>>(
         g, K, Q0, M, mk, partials, sc, dtl, (float)p.cfl, dyn, fm, p.cfl, p.dt_fixed, finalize);
   else
-    k_prestep<float, float, float, false><<<kRedBlocks, kRedThreads, 0, L.s>>>(
+    k_prestep<float, float, float, false><<<red_blocks(g.N), kRedThreads, 0, L.s>>>(
         g, K, Q0, M, mk, partials, sc, dtl, (float)p.cfl, dyn, fm, p.cfl, p.dt_fixed, finalize);
   ++*L.counter;
   if (p.axis) {

@@ -187,6 +187,7 @@ template <typename R>
 __device__ __forceinline__ void prestep_finish(R local_min, int bad, double* __restrict__ partials,
                                                DevScalars* __restrict__ sc, int fin_mode,
                                                double fin_cfl, double fin_dt, int fin_advance) {
+  if (fin_mode < 0) fill_partials(partials);
   __shared__ R smin[32];
   __shared__ int sbad[32];
   for (int off = 16; off > 0; off >>= 1) {

@@ -60,6 +60,19 @@ struct DevScalars {
 constexpr int kRedBlocks = 1216;
 constexpr int kRedThreads = 256;
 constexpr int kMaxPartials = kRedBlocks;
+// Blocks of a reduction over n items: at most kRedBlocks, and none without an
+// item (on 48 x 24 x 32 most of the 1216 blocks had only queued for the
+// ticket or written an empty partial).  It depends on the grid alone.
+inline int red_blocks(long long n) {
+  const long long b = (n + kRedThreads - 1) / kRedThreads;
+  return b < kRedBlocks ? (int)(b < 1 ? 1 : b) : kRedBlocks;
+}
+// The partials that a smaller reduction grid leaves unwritten, as the
+// minimum's neutral element (by block 0).
+__device__ __forceinline__ void fill_partials(double* __restrict__ partials) {
+  if (blockIdx.x == 0)
+    for (int b = gridDim.x + threadIdx.x; b < kRedBlocks; b += blockDim.x) partials[b] = 1.0e300;
+}
 
 // Multiprocessor count of the current device (cached per device), for
 // sizing grid-stride launches in whole waves.

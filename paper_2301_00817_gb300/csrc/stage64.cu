@@ -28,7 +28,7 @@ namespace lesjet {
 void launch_node64(const Grid& g, const les_params& p, const StageIO64& io, bool with_dt,
                    const Launch& L) {
   const int th = 256;
-  const int nb = with_dt ? kRedBlocks : blocks_for(g.N, th);
+  const int nb = with_dt ? red_blocks(g.N) : blocks_for(g.N, th);
   auto K = make_consts<double>(p);
   if (with_dt)
     k_node<double, double, double, true><<<nb, th, 0, L.s>>>(g, K, io.Qin, io.M, io.gn, io.node,

@@ -106,6 +106,7 @@ __global__ void __launch_bounds__(256) k_node(Grid g, Consts<R> K, const TQ* __r
     }
   }
   if (WITH_DT) {
+    fill_partials(partials);
     __shared__ double smin[32];
     __shared__ int sbad;
     if (threadIdx.x == 0) sbad = 0;
