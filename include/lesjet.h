@@ -189,7 +189,7 @@ const char *les_last_error(const les_ctx *ctx);
 int les_set_params(les_ctx *ctx, const les_params *p);
 
 /* Bytes of the caller-owned device workspace this context needs: about
- * 416 B per point in FP64, 208 B mixed, 128 B compact mixed; plus one value
+ * 392 B per point in FP64, 208 B mixed, 128 B compact mixed; plus one value
  * per point with LES_DT_LOCAL and, with LES_SGS_DYNAMIC, 408 B per point
  * more (FP64) or 236 B per point more (mixed). */
 size_t les_workspace_bytes(const les_ctx *ctx);
@@ -321,9 +321,9 @@ const char *les_profile_name(int kind);
  * sgs_model LES_SGS_NONE, freeze_visc 1; LES_ERR_UNSUPPORTED otherwise.
  * Scratch lives in a caller-owned adjoint workspace of
  * les_adjoint_workspace_bytes(ctx, nsteps, ckpt_every) bytes: about
- * (300 + 5 ceil(nsteps/ckpt_every) + 72 ckpt_every) N doubles for a window
+ * (219 + 5 ceil(nsteps/ckpt_every) + 72 ckpt_every) N doubles for a window
  * (checkpoints, plus every stage state and stage-input node quantity of one
- * segment), 300 N for nsteps = 0 (residual and single-step calls only); 135
+ * segment), 219 N for nsteps = 0 (residual and single-step calls only); 66
  * N of it hold each interface's cotangent record, which a per-node gather
  * sums in a fixed order, so every adjoint result is bitwise reproducible
  * (no atomics).  At non-smooth

@@ -3,17 +3,15 @@
 // check it.
 //
 // Residual adjoint: for every interface I = (a, b) the flux F_I enters RHS_a
-// with + and RHS_b with -, so its cotangent is lamR_a - lamR_b.  The kernel
-// k_adj_iface<D> recomputes the forward intermediates of the interface flux
-// (centred inviscid flux, Turkel-Vatsa dissipation, compact viscous flux) and
-// runs them in reverse, accumulating cotangents of the node quantities it
-// read (conserved state, p, u, v, w, T, sensors, lbar, mu, kappa) into a
-// record of that interface (what it owes each node it read); k_adj_gather
-// then sums, per node and in a fixed order, the records of the interfaces
-// that read it, so the accumulation is bitwise reproducible (no atomics).
-// k_adj_sensor_terms / k_adj_sensor_gather move sensor cotangents to the
-// pressures they were computed from the same way, and k_adj_node reverses
-// the node quantities (radii, primitive recovery) into cotangents of Q.
+// with + and RHS_b with -, so its cotangent is lamR_a - lamR_b.  k_adj_flux3
+// recomputes what it needs of the interface's forward intermediates and runs
+// its dissipation and viscous flux in reverse into a record of that
+// interface (what it owes the nodes it read); k_adj_sensor_terms gathers the
+// sensors' cotangents; k_adj_node then sums, per node and in a fixed order,
+// the records of the interfaces that read it, adds the centred flux's part
+// (a node quantity: the cotangents of a node's two interfaces telescope) and
+// reverses the node quantities (radii, primitive recovery) into cotangents of
+// Q.  No atomics: the result is bitwise reproducible.
 //
 // Non-differentiable points follow the forward kernels' branch choices:
 // |x| has derivative -1 for x < 0 and +1 otherwise, max(a, b) passes the
@@ -36,35 +34,26 @@
 
 namespace lesjet {
 
-// accumulator slots (each [N] doubles)
-enum {
-  AQ0 = 0,   // AQ0..AQ0+4: direct cotangents of Q
-  AP = 5,    // p
-  AU = 6,    // u, v, w, T at AU..AU+3
-  ANU = 10,  // sensor of direction d at ANU + d
-  ALB = 13,  // lbar of direction d at ALB + d
-  AMU = 16,  // mu_eff, kappa_eff at AMU, AMU+1
-  NACC = 18
-};
-
 // Per-interface record (each [N] doubles, indexed by the interface's node a,
-// one record array per direction): the cotangents it owes each node it read.
+// one record array per direction): the cotangents it owes the nodes it read.
+// The conserved state's need no fields of their own: the dissipation owes
+// W_a d1 l, W_b -d1 l, W_{b+1} d3 l and W_{a-1} -d3 l, all multiples of l =
+// (lamR_a - lamR_b)/2, so the two coefficients are kept and k_adj_node forms
+// the products.
 enum {
-  RQA = 0,    // conserved state at a (5), then at b, a-1, b+1 (5 each)
-  RQB = 5,
-  RQM = 10,
-  RQP = 15,
-  RPA = 20,   // pressure at a, b, a-1, b+1
-  RUA = 24,   // u, v, w, T at a (4), then at b
-  RUB = 28,
-  RG1 = 32,   // tangential derivative cotangents g1 (T1) and g2 (T2): +g at
-  RG2 = 36,   //   a+t and b+t, -g at a-t and b-t, per component (4 each)
-  RNUA = 40,  // sensor of direction D at a, at b
-  RNUB = 41,
-  RLB = 42,   // half the lbar cotangent (a and b each)
-  RMU = 43,   // half the mu_eff and kappa_eff cotangents (a and b each)
-  RKA = 44,
-  NREC = 45
+  RUA = 0,    // u, v, w at a (3), then at b
+  RUB = 3,
+  RT = 6,     // T at b; minus it at a
+  RG1 = 7,    // tangential difference cotangents (T1, then T2): +g at a+t and
+  RG2 = 11,   //   b+t, -g at a-t and b-t, for u, v, w, T (4 each)
+  RNUA = 15,  // sensor of direction D at a, at b
+  RNUB = 16,
+  RLB = 17,   // lbar (a and b each)
+  RMU = 18,   // mu_eff and kappa_eff (a and b each)
+  RKA = 19,
+  RD1 = 20,   // d1 and d3
+  RD3 = 21,
+  NREC = kAdjRecords
 };
 
 // face-shifted centre triple of the pressure sensor of node x along D
@@ -88,354 +77,332 @@ __device__ __forceinline__ void sensor_triple(const Grid& g, long long x, int cx
   xm = (cc == 0) ? xc + (long long)(nd - 1) * s : xc - s;
 }
 
+__device__ __forceinline__ void sensor_triple_at(const Grid& g, int D, long long x, int cx,
+                                                 long long& xm, long long& xc, long long& xp) {
+  if (D == 0) sensor_triple<0>(g, x, cx, xm, xc, xp);
+  else if (D == 1) sensor_triple<1>(g, x, cx, xm, xc, xp);
+  else sensor_triple<2>(g, x, cx, xm, xc, xp);
+}
+
 __device__ __forceinline__ double sgn_abs(double x) { return x < 0.0 ? -1.0 : 1.0; }
 
 // ------------------------------------------------------------- interface
+struct AdjIO {
+  FluxIO<double, double, double> f;  // the stage input's state, metrics, node quantities, viscosity
+  const double* lamR;                // [5][N], 0 on the open faces
+  double* rec;                       // [3][NREC][N]
+};
+
+// Reverse of flux_iface for the cotangent l of the doubled flux (half the
+// flux's own), without the centred part: the dissipation and the viscous
+// flux, in flux_iface's terms and scaling.
 template <int D>
-__global__ void __launch_bounds__(256, 2) k_adj_iface(Grid g, Consts<double> K,
-                                                   const double* __restrict__ Q,
-                                                   const double* __restrict__ M,
-                                                   const double* __restrict__ node,
-                                                   const double* __restrict__ mk,
-                                                   const double* __restrict__ lamR,
-                                                   double* __restrict__ Rec,
-                                                   const double* __restrict__ NU) {
+__device__ __forceinline__ void adj_iface(const Consts<double>& K, const FluxNode<double>& a,
+                                          const FluxNode<double>& b, const double Wm[5],
+                                          const double Wp[5], double nua, double nub,
+                                          const double l[5], double out[NREC]) {
+  constexpr int T1 = (D + 1) % 3, T2 = (D + 2) % 3;
+  // ---- dissipation: -d1 D1 + d3 E, d1 = lJ (eps2 + 3 eps4), d3 = lJ eps4
+  const double k2h = 0.5 * K.k2, k4h = 0.5 * K.k4;
+  const double nu = dev_max(nua, nub);
+  // dev_max(nua, nub) = nua > nub ? nua : nub, and max(0, x) keeps x for x >= 0
+  const bool pick_b = !(nua > nub);
+  const double eps2 = k2h * nu, e4 = fma(-k2h, nu, k4h);
+  const bool e4on = !(0.0 > e4);
+  const double eps4 = e4on ? e4 : 0.0;
+  const double sJ = a.J + b.J, lJ = (a.lb + b.lb) * sJ, e23 = eps2 + 3.0 * eps4;
+  double ld1 = 0.0, ld3 = 0.0;
+#pragma unroll
+  for (int q = 0; q < 5; ++q) {
+    ld1 = fma(-l[q], b.W[q] - a.W[q], ld1);
+    ld3 = fma(l[q], Wp[q] - Wm[q], ld3);
+  }
+  out[RD1] = lJ * e23;
+  out[RD3] = lJ * eps4;
+  out[RLB] = sJ * (ld1 * e23 + ld3 * eps4);
+  const double leps4 = 3.0 * ld1 + ld3;
+  const double lnu = (k2h * lJ) * (e4on ? ld1 - leps4 : ld1);
+  out[RNUA] = pick_b ? 0.0 : lnu;
+  out[RNUB] = pick_b ? lnu : 0.0;
+
+  // ---- viscous flux, forward
+  const double dn[4] = {b.u - a.u, b.v - a.v, b.w - a.w, b.T - a.T};
+  double s1[4], s2[4], mh[9];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    s1[q] = a.t1[q] + b.t1[q];
+    s2[q] = a.t2[q] + b.t2[q];
+  }
+#pragma unroll
+  for (int t = 0; t < 9; ++t) mh[t] = a.m[t] + b.m[t];
+  const double* m = mh + 3 * D;
+  const double* m1 = mh + 3 * T1;
+  const double* m2 = mh + 3 * T2;
+  const double gD = 4.0 * dot3(m[0], m[1], m[2], m[0], m[1], m[2]);
+  const double g1 = dot3(m[0], m[1], m[2], m1[0], m1[1], m1[2]);
+  const double g2 = dot3(m[0], m[1], m[2], m2[0], m2[1], m2[2]);
+  const double cD = 4.0 * dot3(m[0], m[1], m[2], dn[0], dn[1], dn[2]);
+  const double c1 = dot3(m[0], m[1], m[2], s1[0], s1[1], s1[2]);
+  const double c2 = dot3(m[0], m[1], m[2], s2[0], s2[1], s2[2]);
+  double div = cD;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) div = fma(m2[i], s2[i], fma(m1[i], s1[i], div));
+  const double eD = fma(-2.0 / 3.0, div, cD);
+  double sv[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+    sv[i] = fma(m2[i], c2, fma(m1[i], c1, fma(m[i], eD, dot3(gD, g1, g2, dn[i], s1[i], s2[i]))));
+  const double aT = dot3(gD, g1, g2, dn[3], s1[3], s2[3]);
+  const double sJ32 = sJ * (1.0 / 32.0);
+  const double cm = sJ32 * (a.mu + b.mu), ck = sJ32 * (a.ka + b.ka);
+
+  // ---- reverse: F_i -= cm sv_i, F_4 -= cm/2 (u_a + u_b) . sv + ck aT
+  const double h4 = 0.5 * l[4];
+  const double rr[3] = {fma(h4, a.u + b.u, l[1]), fma(h4, a.v + b.v, l[2]), fma(h4, a.w + b.w, l[3])};
+  out[RMU] = -sJ32 * dot3(rr[0], rr[1], rr[2], sv[0], sv[1], sv[2]);
+  out[RKA] = -sJ32 * (l[4] * aT);
+  const double kf = -cm * h4;  // times sv: the interface velocity's
+  const double ls[3] = {-cm * rr[0], -cm * rr[1], -cm * rr[2]};  // sv's
+  const double lT = -ck * l[4];                                  // aT's
+  // sv_i = gD dn_i + g1 s1_i + g2 s2_i + m_i eD + m1_i c1 + m2_i c2
+  const double leD = dot3(ls[0], ls[1], ls[2], m[0], m[1], m[2]);
+  const double lc1 = dot3(ls[0], ls[1], ls[2], m1[0], m1[1], m1[2]);
+  const double lc2 = dot3(ls[0], ls[1], ls[2], m2[0], m2[1], m2[2]);
+  // eD = cD - 2/3 div and div = cD + ..., cD = 4 m . dn
+  const double l43 = (4.0 / 3.0) * leD, l23 = (-2.0 / 3.0) * leD;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const double ldn = fma(m[i], l43, gD * ls[i]);
+    out[RUA + i] = fma(kf, sv[i], -ldn);
+    out[RUB + i] = fma(kf, sv[i], ldn);
+    out[RG1 + i] = fma(m1[i], l23, fma(m[i], lc1, g1 * ls[i]));
+    out[RG2 + i] = fma(m2[i], l23, fma(m[i], lc2, g2 * ls[i]));
+  }
+  out[RT] = gD * lT;
+  out[RG1 + 3] = g1 * lT;
+  out[RG2 + 3] = g2 * lT;
+}
+
+template <int D>
+__device__ __forceinline__ void adj_put(const AdjIO& io, long long N, long long n,
+                                        const double out[NREC]) {
+  double* R = io.rec + (long long)D * NREC * N + n;
+#pragma unroll
+  for (int r = 0; r < NREC; ++r) R[r * N] = out[r];
+}
+
+template <int D>
+__device__ __forceinline__ void adj_empty(const AdjIO& io, long long N, long long n) {
+  double* R = io.rec + (long long)D * NREC * N + n;
+#pragma unroll 1
+  for (int r = 0; r < NREC; ++r) R[r * N] = 0.0;
+}
+
+// Tangential differences only (the centred flux is reversed per node).
+template <int D>
+__device__ __forceinline__ void adj_shared(const Grid& g, const double* node, long long n,
+                                           const int c[3], FluxNode<double>& x) {
   constexpr int T1 = (D + 1) % 3, T2 = (D + 2) % 3;
   const long long N = g.N;
-  const double* U = node;
-  const double* V = node + N;
-  const double* Wv = node + 2 * N;
-  const double* P = node + 3 * N;
-  const double* Tt = node + 4 * N;
-  const double* LB = node + (5 + D) * N;
-  for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N;
-       n += (long long)gridDim.x * blockDim.x) {
-    int c[3];
-    decompose(g, n, c);
-    // no interface here, or no cotangent on it: an empty record
-    auto empty = [&]() {
-#pragma unroll 1
-      for (int r = 0; r < NREC; ++r) Rec[(long long)r * N + n] = 0.0;
-    };
-    if ((!g.per[D] && c[D] == g.n[D] - 1) ||
-        (!g.per[T1] && (c[T1] == 0 || c[T1] == g.n[T1] - 1)) ||
-        (!g.per[T2] && (c[T2] == 0 || c[T2] == g.n[T2] - 1))) {
-      empty();
-      continue;
-    }
-    const long long a = n;
-    const long long b = step(g, n, c, D, 1);
-    int cb[3] = {c[0], c[1], c[2]};
-    cb[D] = (c[D] + 1 == g.n[D]) ? 0 : c[D] + 1;
-    // the residual is defined (and differentiated) on interior nodes only
-    const bool a_in = g.per[D] || (c[D] > 0 && c[D] < g.n[D] - 1);
-    const bool b_in = g.per[D] || (cb[D] > 0 && cb[D] < g.n[D] - 1);
-    double lF[5];
-    bool any = false;
+  const long long p1 = step(g, n, c, T1, 1), m1 = step(g, n, c, T1, -1);
+  const long long p2 = step(g, n, c, T2, 1), m2 = step(g, n, c, T2, -1);
 #pragma unroll
-    for (int q = 0; q < 5; ++q) {
-      lF[q] = (a_in ? lamR[q * N + a] : 0.0) - (b_in ? lamR[q * N + b] : 0.0);
-      any = any || lF[q] != 0.0;
-    }
-    if (!any) {
-      empty();
-      continue;
-    }
-    const long long am = step(g, n, c, D, -1);
-    const long long bp = step(g, n, c, D, 2);
-
-    // ---- forward recompute
-    const double Ja = M[9 * N + a], Jb = M[9 * N + b];
-    const double ma0 = M[(3 * D) * N + a], ma1 = M[(3 * D + 1) * N + a], ma2 = M[(3 * D + 2) * N + a];
-    const double mb0 = M[(3 * D) * N + b], mb1 = M[(3 * D + 1) * N + b], mb2 = M[(3 * D + 2) * N + b];
-    const double pa = P[a], pb = P[b];
-    const double tha = ma0 * U[a] + ma1 * V[a] + ma2 * Wv[a];
-    const double thb = mb0 * U[b] + mb1 * V[b] + mb2 * Wv[b];
-    double Qa[5], Qb[5];
-#pragma unroll
-    for (int q = 0; q < 5; ++q) {
-      Qa[q] = Q[q * N + a];
-      Qb[q] = Q[q * N + b];
-    }
-    // the two nodes' sensors, as the forward read them (k_sensor of this
-    // stage input)
-    const double nua = NU[D * N + a], nub = NU[D * N + b];
-    // forward: dev_max(nua, nub) = nua > nub ? nua : nub; max(0, x) keeps x for x >= 0
-    const bool pick_b = !(nua > nub);
-    const double eps2 = K.k2 * (pick_b ? nub : nua);
-    const bool e4on = !(0.0 > K.k4 - eps2);
-    const double eps4 = e4on ? K.k4 - eps2 : 0.0;
-    const double lam = 0.5 * (LB[a] + LB[b]);
-    const double Jh = 0.5 * (Ja + Jb);
-    double Wa[5], Wb[5], Wm[5], Wp[5], D1[5], D3[5];
-#pragma unroll
-    for (int q = 0; q < 5; ++q) {
-      Wa[q] = (q == 4) ? Qa[4] + pa : Qa[q];
-      Wb[q] = (q == 4) ? Qb[4] + pb : Qb[q];
-      Wm[q] = (am >= 0) ? ((q == 4) ? Q[4 * N + am] + P[am] : Q[q * N + am]) : 0.0;
-      Wp[q] = (bp >= 0) ? ((q == 4) ? Q[4 * N + bp] + P[bp] : Q[q * N + bp]) : 0.0;
-      D1[q] = Wb[q] - Wa[q];
-      const double Dm = (am >= 0) ? Wa[q] - Wm[q] : -D1[q];
-      const double Dp = (bp >= 0) ? Wp[q] - Wb[q] : -D1[q];
-      D3[q] = Dp - 2.0 * D1[q] + Dm;
-    }
-    const double* phi[4] = {U, V, Wv, Tt};
-    long long tn[2][4];  // tangential nodes: a+t, a-t, b+t, b-t for t = T1, T2
-    tn[0][0] = step(g, a, c, T1, 1);
-    tn[0][1] = step(g, a, c, T1, -1);
-    tn[0][2] = step(g, b, cb, T1, 1);
-    tn[0][3] = step(g, b, cb, T1, -1);
-    tn[1][0] = step(g, a, c, T2, 1);
-    tn[1][1] = step(g, a, c, T2, -1);
-    tn[1][2] = step(g, b, cb, T2, 1);
-    tn[1][3] = step(g, b, cb, T2, -1);
-    double dphi[4][3];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      dphi[q][D] = phi[q][b] - phi[q][a];
-      dphi[q][T1] = 0.25 * ((phi[q][tn[0][0]] - phi[q][tn[0][1]]) + (phi[q][tn[0][2]] - phi[q][tn[0][3]]));
-      dphi[q][T2] = 0.25 * ((phi[q][tn[1][0]] - phi[q][tn[1][1]]) + (phi[q][tn[1][2]] - phi[q][tn[1][3]]));
-    }
-    double mh[3][3];
-#pragma unroll
-    for (int t = 0; t < 3; ++t)
-#pragma unroll
-      for (int x = 0; x < 3; ++x) mh[t][x] = 0.5 * (M[(3 * t + x) * N + a] + M[(3 * t + x) * N + b]);
-    double gr[4][3];
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-#pragma unroll
-      for (int x = 0; x < 3; ++x)
-        gr[q][x] = mh[0][x] * dphi[q][0] + mh[1][x] * dphi[q][1] + mh[2][x] * dphi[q][2];
-    const double mu = 0.5 * (mk[a] + mk[b]);
-    const double kap = 0.5 * (mk[N + a] + mk[N + b]);
-    const double div = gr[0][0] + gr[1][1] + gr[2][2];
-    const double two3 = 2.0 / 3.0;
-    const double txx = mu * (2.0 * gr[0][0] - two3 * div);
-    const double tyy = mu * (2.0 * gr[1][1] - two3 * div);
-    const double tzz = mu * (2.0 * gr[2][2] - two3 * div);
-    const double txy = mu * (gr[0][1] + gr[1][0]);
-    const double txz = mu * (gr[0][2] + gr[2][0]);
-    const double tyz = mu * (gr[1][2] + gr[2][1]);
-    const double uf = 0.5 * (U[a] + U[b]), vf = 0.5 * (V[a] + V[b]), wf = 0.5 * (Wv[a] + Wv[b]);
-    const double mx = mh[D][0], my = mh[D][1], mz = mh[D][2];
-
-    // ---- reverse: F = Fq - Fv
-    // Fv_1..3 = Jh (m . tau_row), Fv_4 = Jh (m . beta)
-    const double lv1 = -lF[1], lv2 = -lF[2], lv3 = -lF[3], lv4 = -lF[4];
-    double ltxx = Jh * mx * lv1, ltyy = Jh * my * lv2, ltzz = Jh * mz * lv3;
-    double ltxy = Jh * (my * lv1 + mx * lv2), ltxz = Jh * (mz * lv1 + mx * lv3),
-           ltyz = Jh * (mz * lv2 + my * lv3);
-    const double lbx = Jh * mx * lv4, lby = Jh * my * lv4, lbz = Jh * mz * lv4;
-    // beta_x = txx uf + txy vf + txz wf + kap grT_x, ...
-    ltxx += lbx * uf;
-    ltxy += lbx * vf + lby * uf;
-    ltxz += lbx * wf + lbz * uf;
-    ltyy += lby * vf;
-    ltyz += lby * wf + lbz * vf;
-    ltzz += lbz * wf;
-    const double luf = lbx * txx + lby * txy + lbz * txz;
-    const double lvf = lbx * txy + lby * tyy + lbz * tyz;
-    const double lwf = lbx * txz + lby * tyz + lbz * tzz;
-    const double lkap = lbx * gr[3][0] + lby * gr[3][1] + lbz * gr[3][2];
-    double lgr[4][3];
-    lgr[3][0] = kap * lbx;
-    lgr[3][1] = kap * lby;
-    lgr[3][2] = kap * lbz;
-    // tau
-    double lmu = ltxx * (2.0 * gr[0][0] - two3 * div) + ltyy * (2.0 * gr[1][1] - two3 * div) +
-                 ltzz * (2.0 * gr[2][2] - two3 * div) + ltxy * (gr[0][1] + gr[1][0]) +
-                 ltxz * (gr[0][2] + gr[2][0]) + ltyz * (gr[1][2] + gr[2][1]);
-    const double ldiv = -two3 * mu * (ltxx + ltyy + ltzz);
-    lgr[0][0] = 2.0 * mu * ltxx + ldiv;
-    lgr[1][1] = 2.0 * mu * ltyy + ldiv;
-    lgr[2][2] = 2.0 * mu * ltzz + ldiv;
-    lgr[0][1] = mu * ltxy;
-    lgr[1][0] = mu * ltxy;
-    lgr[0][2] = mu * ltxz;
-    lgr[2][0] = mu * ltxz;
-    lgr[1][2] = mu * ltyz;
-    lgr[2][1] = mu * ltyz;
-    // gr[q][x] = sum_t mh[t][x] dphi[q][t]
-    double ldphi[4][3];
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-#pragma unroll
-      for (int t = 0; t < 3; ++t)
-        ldphi[q][t] = mh[t][0] * lgr[q][0] + mh[t][1] * lgr[q][1] + mh[t][2] * lgr[q][2];
-
-    // Fq = (Fa + Fb)/2 - Jh lam (eps2 D1 - eps4 D3)
-    double lWa[5] = {0, 0, 0, 0, 0}, lWb[5] = {0, 0, 0, 0, 0}, lWm[5] = {0, 0, 0, 0, 0},
-           lWp[5] = {0, 0, 0, 0, 0};
-    double llam = 0.0, leps2 = 0.0, leps4 = 0.0;
-#pragma unroll
-    for (int q = 0; q < 5; ++q) {
-      const double ld = -Jh * lF[q];
-      llam += ld * (eps2 * D1[q] - eps4 * D3[q]);
-      leps2 += ld * lam * D1[q];
-      leps4 -= ld * lam * D3[q];
-      double lD1 = ld * lam * eps2;
-      const double lD3 = -ld * lam * eps4;
-      lD1 += -2.0 * lD3;
-      if (am >= 0) {
-        lWa[q] += lD3;
-        lWm[q] -= lD3;
-      } else {
-        lD1 -= lD3;
-      }
-      if (bp >= 0) {
-        lWp[q] += lD3;
-        lWb[q] -= lD3;
-      } else {
-        lD1 -= lD3;
-      }
-      lWb[q] += lD1;
-      lWa[q] -= lD1;
-    }
-    if (e4on) leps2 -= leps4;
-    const double lnu = K.k2 * leps2;
-    // centred flux: Fa_q = Ja (Qa_q tha + pa ma_q') ; Fa_4 = Ja (Qa4 + pa) tha
-    double lQa[5], lQb[5];
-    const double hFa[5] = {0.5 * lF[0], 0.5 * lF[1], 0.5 * lF[2], 0.5 * lF[3], 0.5 * lF[4]};
-#pragma unroll
-    for (int q = 0; q < 5; ++q) {
-      lQa[q] = Ja * tha * hFa[q];
-      lQb[q] = Jb * thb * hFa[q];
-    }
-    const double lpa_f = Ja * (ma0 * hFa[1] + ma1 * hFa[2] + ma2 * hFa[3] + tha * hFa[4]);
-    const double lpb_f = Jb * (mb0 * hFa[1] + mb1 * hFa[2] + mb2 * hFa[3] + thb * hFa[4]);
-    const double ltha = Ja * (Qa[0] * hFa[0] + Qa[1] * hFa[1] + Qa[2] * hFa[2] + Qa[3] * hFa[3] +
-                              (Qa[4] + pa) * hFa[4]);
-    const double lthb = Jb * (Qb[0] * hFa[0] + Qb[1] * hFa[1] + Qb[2] * hFa[2] + Qb[3] * hFa[3] +
-                              (Qb[4] + pb) * hFa[4]);
-
-    // ---- the record: conserved state and pressure (W4 = Q4 + p)
-    auto put = [&](int r, double v) { Rec[(long long)r * N + n] = v; };
-#pragma unroll
-    for (int q = 0; q < 5; ++q) {
-      put(RQA + q, lQa[q] + lWa[q]);
-      put(RQB + q, lQb[q] + lWb[q]);
-      put(RQM + q, am >= 0 ? lWm[q] : 0.0);
-      put(RQP + q, bp >= 0 ? lWp[q] : 0.0);
-    }
-    put(RPA, lpa_f + lWa[4]);
-    put(RPA + 1, lpb_f + lWb[4]);
-    put(RPA + 2, am >= 0 ? lWm[4] : 0.0);
-    put(RPA + 3, bp >= 0 ? lWp[4] : 0.0);
-    // velocities: contravariant velocity and interface mean
-    put(RUA + 0, ma0 * ltha + 0.5 * luf - ldphi[0][D]);
-    put(RUA + 1, ma1 * ltha + 0.5 * lvf - ldphi[1][D]);
-    put(RUA + 2, ma2 * ltha + 0.5 * lwf - ldphi[2][D]);
-    put(RUA + 3, -ldphi[3][D]);
-    put(RUB + 0, mb0 * lthb + 0.5 * luf + ldphi[0][D]);
-    put(RUB + 1, mb1 * lthb + 0.5 * lvf + ldphi[1][D]);
-    put(RUB + 2, mb2 * lthb + 0.5 * lwf + ldphi[2][D]);
-    put(RUB + 3, ldphi[3][D]);
-    // tangential derivatives: 1/4 (phi(a+t) - phi(a-t) + phi(b+t) - phi(b-t))
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      put(RG1 + q, 0.25 * ldphi[q][T1]);
-      put(RG2 + q, 0.25 * ldphi[q][T2]);
-    }
-    // sensor, spectral radius, viscosity
-    put(RNUA, pick_b ? 0.0 : lnu);
-    put(RNUB, pick_b ? lnu : 0.0);
-    put(RLB, 0.5 * llam);
-    put(RMU, 0.5 * lmu);
-    put(RKA, 0.5 * lkap);
+  for (int q = 0; q < 4; ++q) {
+    const double* phi = node + (q == 3 ? 4 : q) * N;
+    x.t1[q] = phi[p1] - phi[m1];
+    x.t2[q] = phi[p2] - phi[m2];
   }
 }
 
-// Per node, in a fixed order (direction 0, 1, 2; then the roles), the sum of
-// what the interface records owe it: as node a of the interface at n, as b
-// of the one at n - e_D, as a - 1 of the one at n + e_D, as b + 1 of the one
-// at n - 2 e_D, and as a tangential neighbour (a + t, a - t, b + t, b - t)
-// of the interfaces at n - e_t, n + e_t, n - e_t - e_D, n + e_t - e_D.
-// Writes every accumulator slot of every node (the sensor pass adds to the
-// pressure slot afterwards).  One output slot at a time (its own fixed
-// order of terms), so few accumulators are live and the kernel keeps
-// enough warps resident to cover its memory latency.
-__global__ void __launch_bounds__(256) k_adj_gather(Grid g, const double* __restrict__ R0,
-                                                   const double* __restrict__ R1,
-                                                   const double* __restrict__ R2,
-                                                   double* __restrict__ A) {
+// Records of the interfaces along xi or eta: chunks of len interfaces per
+// thread, as flux_chain walks them.  An interface without a cotangent (a
+// window's cotangent spreads from one ring) gets an empty record.
+template <int D>
+__device__ __forceinline__ void adj_chain(const Grid& g, const Consts<double>& K, const AdjIO& io,
+                                          long long id, int len) {
+  constexpr int T1 = (D + 1) % 3, T2 = (D + 2) % 3;
   const long long N = g.N;
-  const double* Rd[3] = {R0, R1, R2};
-  for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N;
-       n += (long long)gridDim.x * blockDim.x) {
-    int c[3];
-    decompose(g, n, c);
-    long long mB[3], mM[3], mP[3];  // interfaces whose b, a - 1, b + 1 is n
-#pragma unroll
-    for (int D = 0; D < 3; ++D) {
-      mB[D] = step(g, n, c, D, -1);
-      mM[D] = step(g, n, c, D, 1);
-      mP[D] = step(g, n, c, D, -2);
-    }
-    auto rec = [&](int D, int r, long long m) { return m >= 0 ? Rd[D][(long long)r * N + m] : 0.0; };
-    // conserved state (k < 5) and pressure (k = 5): four roles per direction
-#pragma unroll 1
-    for (int k = 0; k < 6; ++k) {
-      const int ra = k < 5 ? RQA + k : RPA, rb = k < 5 ? RQB + k : RPA + 1;
-      const int rm = k < 5 ? RQM + k : RPA + 2, rp = k < 5 ? RQP + k : RPA + 3;
-      double acc = 0.0;
-#pragma unroll
-      for (int D = 0; D < 3; ++D)
-        acc += ((rec(D, ra, n) + rec(D, rb, mB[D])) + rec(D, rm, mM[D])) + rec(D, rp, mP[D]);
-      A[(k < 5 ? AQ0 + k : AP) * N + n] = acc;
-    }
-    // u, v, w, T: as a and b, then as a tangential neighbour along T1, T2
-#pragma unroll 1
-    for (int k = 0; k < 4; ++k) {
-      double acc = 0.0;
-#pragma unroll
-      for (int D = 0; D < 3; ++D) {
-        acc += rec(D, RUA + k, n) + rec(D, RUB + k, mB[D]);
-#pragma unroll
-        for (int s = 1; s <= 2; ++s) {
-          const int t = (D + s) % 3;
-          const int G = (s == 1) ? RG1 : RG2;
-          const long long tm = step(g, n, c, t, -1), tp = step(g, n, c, t, 1);
-          long long tmb = -1, tpb = -1;  // n - e_t - e_D, n + e_t - e_D
-          if (tm >= 0) {
-            int ct[3] = {c[0], c[1], c[2]};
-            ct[t] = coord_step(g, c, t, -1);
-            tmb = step(g, tm, ct, D, -1);
-          }
-          if (tp >= 0) {
-            int ct[3] = {c[0], c[1], c[2]};
-            ct[t] = coord_step(g, c, t, 1);
-            tpb = step(g, tp, ct, D, -1);
-          }
-          acc += ((rec(D, G + k, tm) - rec(D, G + k, tp)) + rec(D, G + k, tmb)) - rec(D, G + k, tpb);
-        }
-      }
-      A[(AU + k) * N + n] = acc;
-    }
-    // sensor and lbar of each direction; mu_eff and kappa_eff over the three
-#pragma unroll
-    for (int D = 0; D < 3; ++D) {
-      A[(ANU + D) * N + n] = rec(D, RNUA, n) + rec(D, RNUB, mB[D]);
-      A[(ALB + D) * N + n] = rec(D, RLB, n) + rec(D, RLB, mB[D]);
-    }
-    double mu = 0.0, ka = 0.0;
-#pragma unroll
-    for (int D = 0; D < 3; ++D) {
-      mu += rec(D, RMU, n) + rec(D, RMU, mB[D]);
-      ka += rec(D, RKA, n) + rec(D, RKA, mB[D]);
-    }
-    A[AMU * N + n] = mu;
-    A[(AMU + 1) * N + n] = ka;
+  const int nd = g.n[D];  // entries of a line (the last one empty on an open line)
+  const int nch = (nd + len - 1) / len;
+  int c[3];
+  const long long r = id / g.n[2];
+  c[2] = (int)(id - r * g.n[2]);
+  if (D == 0) {
+    c[0] = (int)(r / g.n[1]);
+    c[1] = (int)(r - (long long)c[0] * g.n[1]);
+  } else {
+    c[0] = (int)(r / nch);
+    c[1] = (int)(r - (long long)c[0] * nch);
   }
+  if (c[0] >= (D == 0 ? nch : g.n[0])) return;
+  c[D] *= len;
+  const int end = c[D] + len < nd ? c[D] + len : nd;
+  long long na = idx3(g, c[0], c[1], c[2]);
+  if ((!g.per[T1] && (c[T1] == 0 || c[T1] == g.n[T1] - 1)) ||
+      (!g.per[T2] && (c[T2] == 0 || c[T2] == g.n[T2] - 1))) {
+    for (int x = c[D]; x < end; ++x, na += g.stride[D]) adj_empty<D>(io, N, na);
+    return;
+  }
+  FluxNode<double> a, b;
+  double Wm[5], pm = 0.0, la[5];
+  const long long nm = step(g, na, c, D, -1);
+  bool has_m = nm >= 0;
+  if (has_m) flux_W(io.f, N, nm, Wm, pm);
+  flux_W(io.f, N, na, a.W, a.p);
+  flux_load<D>(io.f, N, false, na, a);
+  adj_shared<D>(g, io.f.node, na, c, a);
+#pragma unroll
+  for (int q = 0; q < 5; ++q) la[q] = io.lamR[q * N + na];
+  long long nb = step(g, na, c, D, 1);
+  double nua = 0.0;
+  if (nb >= 0) {
+    flux_W(io.f, N, nb, b.W, b.p);
+    if (has_m) nua = sensor3(pm, a.p, b.p);
+  }
+  for (int x = c[D]; x < end; ++x) {
+    if (nb < 0) {  // past the last interface of an open line
+      adj_empty<D>(io, N, na);
+      return;
+    }
+    c[D] = x;
+    const long long np = step(g, na, c, D, 2);
+    const bool has_p = np >= 0;
+    double Wp[5], pp = 0.0, l[5], lb[5];
+    if (has_p) flux_W(io.f, N, np, Wp, pp);
+    flux_load<D>(io.f, N, false, nb, b);
+    adj_shared<D>(g, io.f.node, nb, c, b);
+    double nub = nua;
+    if (has_p) {
+      nub = sensor3(a.p, b.p, pp);
+    } else {
+#pragma unroll
+      for (int q = 0; q < 5; ++q) Wp[q] = a.W[q];
+    }
+    if (!has_m) {
+      nua = nub;
+#pragma unroll
+      for (int q = 0; q < 5; ++q) Wm[q] = b.W[q];
+    }
+    bool any = false;
+#pragma unroll
+    for (int q = 0; q < 5; ++q) {
+      lb[q] = io.lamR[q * N + nb];
+      l[q] = 0.5 * (la[q] - lb[q]);
+      any = any || l[q] != 0.0;
+      la[q] = lb[q];
+    }
+    if (any) {
+      double out[NREC];
+      adj_iface<D>(K, a, b, Wm, Wp, nua, nub, l, out);
+      adj_put<D>(io, N, na, out);
+    } else {
+      adj_empty<D>(io, N, na);
+    }
+#pragma unroll
+    for (int q = 0; q < 5; ++q) Wm[q] = a.W[q];
+    has_m = true;
+    a = b;
+    nua = nub;
+    na = nb;
+    nb = np;
+#pragma unroll
+    for (int q = 0; q < 5; ++q) b.W[q] = Wp[q];
+    b.p = pp;
+  }
+}
+
+// Records of the zeta interfaces, one per thread; a block's run of nodes
+// shares their tangential differences and sensors, as flux_zeta.
+__device__ __forceinline__ void adj_zeta(const Grid& g, const Consts<double>& K, const AdjIO& io,
+                                         long long n0, double (*sh)[kFluxThreads]) {
+  const long long N = g.N, n = n0 + threadIdx.x;
+  const double* P = io.f.node + 3 * N;
+  int c[3] = {0, 0, 0};
+  bool in = n < N;
+  if (in) {
+    decompose(g, n, c);
+    in = (g.per[0] || (c[0] > 0 && c[0] < g.n[0] - 1)) &&
+         (g.per[1] || (c[1] > 0 && c[1] < g.n[1] - 1));
+    if (!in) adj_empty<2>(io, N, n);
+  }
+  FluxNode<double> a, b;
+  double nua = 0.0;
+  if (in) {
+    flux_W(io.f, N, n, a.W, a.p);
+    flux_load<2>(io.f, N, false, n, a);
+    adj_shared<2>(g, io.f.node, n, c, a);
+    nua = sensor<2>(g, P, n, c[2]);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      sh[q][threadIdx.x] = a.t1[q];
+      sh[4 + q][threadIdx.x] = a.t2[q];
+    }
+    sh[8][threadIdx.x] = nua;
+  }
+  __syncthreads();
+  if (!in) return;
+  const long long nb = step(g, n, c, 2, 1);
+  double l[5];
+  bool any = false;
+  if (nb >= 0) {
+#pragma unroll
+    for (int q = 0; q < 5; ++q) {
+      l[q] = 0.5 * (io.lamR[q * N + n] - io.lamR[q * N + nb]);
+      any = any || l[q] != 0.0;
+    }
+  }
+  if (!any) {
+    adj_empty<2>(io, N, n);
+    return;
+  }
+  flux_W(io.f, N, nb, b.W, b.p);
+  flux_load<2>(io.f, N, false, nb, b);
+  double nub;
+  if (nb >= n0 && nb < n0 + kFluxThreads) {
+    const int s = (int)(nb - n0);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      b.t1[q] = sh[q][s];
+      b.t2[q] = sh[4 + q][s];
+    }
+    nub = sh[8][s];
+  } else {
+    adj_shared<2>(g, io.f.node, nb, c, b);
+    nub = sensor<2>(g, P, nb, coord_step(g, c, 2, 1));
+  }
+  double Wm[5], Wp[5], unused;
+  const long long nm = step(g, n, c, 2, -1), np = step(g, n, c, 2, 2);
+  flux_W(io.f, N, nm >= 0 ? nm : nb, Wm, unused);
+  flux_W(io.f, N, np >= 0 ? np : n, Wp, unused);
+  double out[NREC];
+  adj_iface<2>(K, a, b, Wm, Wp, nua, nub, l, out);
+  adj_put<2>(io, N, n, out);
+}
+
+// The three directions' records in one launch, split as k_flux3's.  Bound by
+// the FP64 pipe like the forward kernel: about 165 operations per interface
+// (some 420 when the gradient tensor was formed, the stress reversed term by
+// term and the centred flux reversed twice per node).
+__global__ void __launch_bounds__(kFluxThreads, 2)
+    k_adj_flux3(Grid g, Consts<double> K, AdjIO io, unsigned b2, unsigned b0, int len) {
+  __shared__ double sh[9][kFluxThreads];
+  const unsigned b = blockIdx.x;
+  if (b < b2)
+    adj_zeta(g, K, io, (long long)b * kFluxThreads, sh);
+  else if (b < b2 + b0)
+    adj_chain<0>(g, K, io, (long long)(b - b2) * kFluxThreads + threadIdx.x, len);
+  else
+    adj_chain<1>(g, K, io, (long long)(b - b2 - b0) * kFluxThreads + threadIdx.x, len);
 }
 
 // Sensor cotangents to the pressures of the (face-shifted) centre triple:
 // per node x and direction d the two terms it owes (ls + lden to its outer
-// pair, -2 ls + 2 lden to its centre) into ST[2 d], ST[2 d + 1]; then each
-// node gathers, in a fixed order, the terms of the nodes whose triple holds
-// it (x within two nodes along d).
-__global__ void k_adj_sensor_terms(Grid g, const double* __restrict__ node,
-                                   const double* __restrict__ A, double* __restrict__ ST) {
+// pair, -2 ls + 2 lden to its centre) into ST[2 d], ST[2 d + 1]; k_adj_node
+// gathers, in a fixed order, the terms of the nodes whose triple holds a
+// node (x within two nodes along d).
+__global__ void __launch_bounds__(256) k_adj_sensor_terms(Grid g, const double* __restrict__ node,
+                                                          const double* __restrict__ rec,
+                                                          double* __restrict__ ST) {
   const long long N = g.N;
   const double* P = node + 3 * N;
   for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N;
@@ -444,17 +411,17 @@ __global__ void k_adj_sensor_terms(Grid g, const double* __restrict__ node,
     decompose(g, n, c);
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-      const double ln = A[(ANU + d) * N + n];
+      const double* R = rec + (long long)d * NREC * N;
+      const long long mB = step(g, n, c, d, -1);
+      const double ln = R[RNUA * N + n] + (mB >= 0 ? R[RNUB * N + mB] : 0.0);
       double outer = 0.0, centre = 0.0;
       if (ln != 0.0) {
         long long xm, xc, xp;
-        if (d == 0) sensor_triple<0>(g, n, c[0], xm, xc, xp);
-        else if (d == 1) sensor_triple<1>(g, n, c[1], xm, xc, xp);
-        else sensor_triple<2>(g, n, c[2], xm, xc, xp);
+        sensor_triple_at(g, d, n, c[d], xm, xc, xp);
         // nu = |s| / den, rounded as sensor3 does (the sign of s decides the
         // branch where the pressure is uniform to rounding)
         const double pm = P[xm] + P[xp];
-        const double s = pm - 2.0 * P[xc], den = pm + 2.0 * P[xc];
+        const double s = fma(-2.0, P[xc], pm), den = fma(2.0, P[xc], pm);
         const double iden = 1.0 / den;
         const double ls = ln * sgn_abs(s) * iden;
         const double lden = -ln * fabs(s) * iden * iden;
@@ -467,103 +434,167 @@ __global__ void k_adj_sensor_terms(Grid g, const double* __restrict__ node,
   }
 }
 
-__global__ void k_adj_sensor_gather(Grid g, const double* __restrict__ ST, double* __restrict__ A) {
+// Per node, in a fixed order: what the interface records owe it, the centred
+// flux's part, the sensors' part, then the node quantities back to Q: radii
+// lbar(lambda_d), lambda_d = |m_d.u| + sqrt(T)|grad d|, u = Q1/rho, p =
+// (g-1)(Q4 - rho|u|^2/2), T = g p/rho.  mu/kappa cotangents are added to
+// lamMK.  |grad d| comes from gn ([3][N], set-up).
+// A node reads about 240 values (its interfaces' records and lamR within two
+// nodes along each direction), few of them twice by one thread, and does
+// about 500 FP64 operations, whose pipe bounds it; gathering straight into
+// the node's reverse saves the 18 accumulator fields of a pass of their own.
+__global__ void __launch_bounds__(128, 3)
+    k_adj_node(Grid g, Consts<double> K, const double* __restrict__ Q,
+               const double* __restrict__ M, const double* __restrict__ gn,
+               const double* __restrict__ node, const double* __restrict__ lamR,
+               const double* __restrict__ rec, const double* __restrict__ ST,
+               double* __restrict__ lamQ, double* __restrict__ lamMK) {
   const long long N = g.N;
   for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N;
        n += (long long)gridDim.x * blockDim.x) {
     int c[3];
     decompose(g, n, c);
-    double add = 0.0;
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-#pragma unroll
-      for (int off = -2; off <= 2; ++off) {
-        const long long x = step(g, n, c, d, off);
-        if (x < 0) continue;
-        int cx[3] = {c[0], c[1], c[2]};
-        cx[d] = coord_step(g, c, d, off);
-        long long xm, xc, xp;
-        if (d == 0) sensor_triple<0>(g, x, cx[0], xm, xc, xp);
-        else if (d == 1) sensor_triple<1>(g, x, cx[1], xm, xc, xp);
-        else sensor_triple<2>(g, x, cx[2], xm, xc, xp);
-        if (xp == n) add += ST[(2 * d) * N + x];
-        if (xc == n) add += ST[(2 * d + 1) * N + x];
-        if (xm == n) add += ST[(2 * d) * N + x];
-      }
-    }
-    A[AP * N + n] += add;
-  }
-}
-
-// Node quantities back to Q: radii lbar(lambda_d), lambda_d = |m_d.u| +
-// sqrt(T)|grad d|, then u = Q1/rho, p = (g-1)(Q4 - rho|u|^2/2), T = g p/rho.
-// lamQ = direct + chained; mu/kappa cotangents are added to lamMK.  |grad d|
-// comes from gn ([3][N], set-up) when given, else from M.
-__global__ void __launch_bounds__(256, 2) k_adj_node(Grid g, Consts<double> K, const double* __restrict__ Q,
-                           const double* __restrict__ M, const double* __restrict__ gn,
-                           const double* __restrict__ node,
-                           const double* __restrict__ A, double* __restrict__ lamQ,
-                           double* __restrict__ lamMK) {
-  const long long N = g.N;
-  for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N;
-       n += (long long)gridDim.x * blockDim.x) {
-    const double rho = Q[n];
-    const double ir = 1.0 / rho;
     const double u = node[n], v = node[N + n], w = node[2 * N + n], p = node[3 * N + n],
                  T = node[4 * N + n];
-    double lu = A[(AU + 0) * N + n], lv = A[(AU + 1) * N + n], lw = A[(AU + 2) * N + n];
-    double lT = A[(AU + 3) * N + n], lp = A[AP * N + n];
+    const double Jv = M[9 * N + n];
+    double lW[5] = {0.0, 0.0, 0.0, 0.0, 0.0};   // twice the cotangents of W
+    double lv[4] = {0.0, 0.0, 0.0, 0.0};        // u, v, w, T
+    double lp = 0.0, lmu = 0.0, lka = 0.0, llb[3], th[3];
+#pragma unroll
+    for (int D = 0; D < 3; ++D) {
+      const double* R = rec + (long long)D * NREC * N;
+      const long long m1 = step(g, n, c, D, -1), p1 = step(g, n, c, D, 1);
+      const long long m2 = step(g, n, c, D, -2), p2 = step(g, n, c, D, 2);
+      // interfaces (m2, m1), (m1, n), (n, p1), (p1, p2), by their node a
+      double kB = 0.0, kA = 0.0, kP = 0.0, kM = 0.0;
+      if (m1 >= 0) kB = R[RD1 * N + m1];
+      if (p1 >= 0) kA = R[RD1 * N + n];
+      if (m2 >= 0) kP = R[RD3 * N + m2];
+      else if (m1 >= 0) kB += R[RD3 * N + m1];  // its W_{a-1} was W_b, this node
+      if (p2 >= 0) kM = R[RD3 * N + p1];
+      else if (p1 >= 0) kA += R[RD3 * N + n];   // its W_{b+1} was W_a, this node
+      const double mx = M[(3 * D) * N + n], my = M[(3 * D + 1) * N + n], mz = M[(3 * D + 2) * N + n];
+      th[D] = dot3(mx, my, mz, u, v, w);
+      const double Jt = Jv * th[D];
+      double lJt = 0.0, lF[5];
+#pragma unroll
+      for (int q = 0; q < 5; ++q) {
+        const double* L = lamR + q * N;
+        const double l0 = L[n];
+        const double lm = m1 >= 0 ? L[m1] : l0, lq = p1 >= 0 ? L[p1] : l0;
+        const double eB = lm - l0, eA = l0 - lq;  // 0 where there is no interface
+        const double eP = m2 >= 0 ? L[m2] - lm : 0.0, eM = p2 >= 0 ? lq - L[p2] : 0.0;
+        lW[q] = fma(kP, eP, fma(Jt - kB, eB, fma(Jt + kA, eA, fma(-kM, eM, lW[q]))));
+        lF[q] = eB + eA;  // twice the cotangent of the node's flux along D
+        const double W = Q[q * N + n] + (q == 4 ? p : 0.0);
+        lJt = fma(W, lF[q], lJt);
+      }
+      // node flux: W Jt (+ Jp m in the momentum), Jt = J^-1 m . u, Jp = J^-1 p
+      const double hJ = 0.5 * Jv, lth = hJ * lJt;
+      lp = fma(hJ, dot3(mx, my, mz, lF[1], lF[2], lF[3]), lp);
+      lv[0] = fma(mx, lth, lv[0]);
+      lv[1] = fma(my, lth, lv[1]);
+      lv[2] = fma(mz, lth, lv[2]);
+      // as a, as b
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        lv[k] += R[(RUA + k) * N + n];
+        if (m1 >= 0) lv[k] += R[(RUB + k) * N + m1];
+      }
+      lv[3] -= R[RT * N + n];
+      if (m1 >= 0) lv[3] += R[RT * N + m1];
+      llb[D] = R[RLB * N + n];
+      lmu += R[RMU * N + n];
+      lka += R[RKA * N + n];
+      if (m1 >= 0) {
+        llb[D] += R[RLB * N + m1];
+        lmu += R[RMU * N + m1];
+        lka += R[RKA * N + m1];
+      }
+      // as a tangential neighbour (a + t, b + t, a - t, b - t) of the
+      // interfaces at n - e_t, n - e_t - e_D, n + e_t, n + e_t - e_D
+#pragma unroll
+      for (int s = 1; s <= 2; ++s) {
+        const int t = (D + s) % 3;
+        const double* G = R + (s == 1 ? RG1 : RG2) * N;
+        const long long tm = step(g, n, c, t, -1), tp = step(g, n, c, t, 1);
+        const long long dB = m1 - n;  // to the interface's node a when n + t is its b
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          if (tm >= 0) lv[k] += G[k * N + tm];
+          if (tp >= 0) lv[k] -= G[k * N + tp];
+          if (m1 >= 0) {
+            if (tm >= 0) lv[k] += G[k * N + tm + dB];
+            if (tp >= 0) lv[k] -= G[k * N + tp + dB];
+          }
+        }
+      }
+      // the sensors along D whose triple holds this node
+#pragma unroll
+      for (int off = -2; off <= 2; ++off) {
+        const long long x = off == 0 ? n : (off == -2 ? m2 : (off == -1 ? m1 : (off == 1 ? p1 : p2)));
+        if (x < 0) continue;
+        const int cx = off == 0 ? c[D] : coord_step(g, c, D, off);
+        if ((off == -2 || off == 2) && (g.per[D] || (cx != 0 && cx != g.n[D] - 1))) continue;
+        long long xm, xc, xp;
+        sensor_triple_at(g, D, x, cx, xm, xc, xp);
+        if (xp == n) lp += ST[(2 * D) * N + x];
+        if (xc == n) lp += ST[(2 * D + 1) * N + x];
+        if (xm == n) lp += ST[(2 * D) * N + x];
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 5; ++q) lW[q] *= 0.5;
+    lp += lW[4];  // W4 = Q4 + p
+    double lT = lv[3];
     // lbar -> lambda
-    const double llb0 = A[(ALB + 0) * N + n], llb1 = A[(ALB + 1) * N + n], llb2 = A[(ALB + 2) * N + n];
-    if (llb0 != 0.0 || llb1 != 0.0 || llb2 != 0.0) {
-      const double a = sqrt(T);
-      double l[3], th[3], gm[3];
+    if (llb[0] != 0.0 || llb[1] != 0.0 || llb[2] != 0.0) {
+      const double ra = rsqrt(T), a = T * ra;
+      double l[3], gm[3];
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
-        const double mx = M[(3 * d) * N + n], my = M[(3 * d + 1) * N + n], mz = M[(3 * d + 2) * N + n];
-        th[d] = mx * u + my * v + mz * w;
-        gm[d] = gn ? gn[d * N + n] : sqrt(mx * mx + my * my + mz * mz);
-        l[d] = fabs(th[d]) + a * gm[d];
+        gm[d] = gn[d * N + n];
+        l[d] = fma(a, gm[d], fabs(th[d]));
       }
-      const double s01 = sqrt(l[0] * l[1]), s02 = sqrt(l[0] * l[2]), s12 = sqrt(l[1] * l[2]);
-      const double c01 = llb0 + llb1, c02 = llb0 + llb2, c12 = llb1 + llb2;
-      // d sqrt(l_a l_b)/d l_a = l_b/(2 sqrt(l_a l_b)): one reciprocal per pair
-      const double h01 = c01 / (2.0 * s01), h02 = c02 / (2.0 * s02), h12 = c12 / (2.0 * s12);
+      // d sqrt(l_a l_b)/d l_a = l_b/(2 sqrt(l_a l_b)): one reciprocal root per pair
+      const double h01 = 0.5 * (llb[0] + llb[1]) * rsqrt(l[0] * l[1]);
+      const double h02 = 0.5 * (llb[0] + llb[2]) * rsqrt(l[0] * l[2]);
+      const double h12 = 0.5 * (llb[1] + llb[2]) * rsqrt(l[1] * l[2]);
       double ll[3];
-      ll[0] = llb0 + h01 * l[1] + h02 * l[2];
-      ll[1] = llb1 + h01 * l[0] + h12 * l[2];
-      ll[2] = llb2 + h02 * l[0] + h12 * l[1];
+      ll[0] = llb[0] + h01 * l[1] + h02 * l[2];
+      ll[1] = llb[1] + h01 * l[0] + h12 * l[2];
+      ll[2] = llb[2] + h02 * l[0] + h12 * l[1];
       double la = 0.0;
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
         const double lth = ll[d] * sgn_abs(th[d]);
-        lu += M[(3 * d) * N + n] * lth;
-        lv += M[(3 * d + 1) * N + n] * lth;
-        lw += M[(3 * d + 2) * N + n] * lth;
-        la += ll[d] * gm[d];
+        lv[0] = fma(M[(3 * d) * N + n], lth, lv[0]);
+        lv[1] = fma(M[(3 * d + 1) * N + n], lth, lv[1]);
+        lv[2] = fma(M[(3 * d + 2) * N + n], lth, lv[2]);
+        la = fma(ll[d], gm[d], la);
       }
-      lT += la / (2.0 * a);
+      lT = fma(0.5 * la, ra, lT);
     }
+    const double rho = Q[n], ir = 1.0 / rho;
     // T = gamma p / rho
-    lp += K.gamma * ir * lT;
-    double lrho = -K.gamma * p * ir * ir * lT;
+    const double gT = K.gamma * ir * lT;
+    lp += gT;
+    double lrho = -(p * ir) * gT;
     // p = (gamma-1)(Q4 - rho |u|^2 / 2)
-    double lQ4 = K.gm1 * lp;
-    lrho += -0.5 * K.gm1 * (u * u + v * v + w * w) * lp;
-    lu += -K.gm1 * rho * u * lp;
-    lv += -K.gm1 * rho * v * lp;
-    lw += -K.gm1 * rho * w * lp;
+    const double lQ4 = K.gm1 * lp;
+    lrho = fma(-0.5 * lQ4, dot3(u, v, w, u, v, w), lrho);
+    const double rl = rho * lQ4;
+    const double lu = fma(-rl, u, lv[0]), lvv = fma(-rl, v, lv[1]), lw = fma(-rl, w, lv[2]);
     // u = Q1 / rho
-    const double lQ1 = ir * lu, lQ2 = ir * lv, lQ3 = ir * lw;
-    lrho += -ir * (u * lu + v * lv + w * lw);
-    lamQ[n] = A[AQ0 * N + n] + lrho;
-    lamQ[N + n] = A[(AQ0 + 1) * N + n] + lQ1;
-    lamQ[2 * N + n] = A[(AQ0 + 2) * N + n] + lQ2;
-    lamQ[3 * N + n] = A[(AQ0 + 3) * N + n] + lQ3;
-    lamQ[4 * N + n] = A[(AQ0 + 4) * N + n] + lQ4;
+    lrho = fma(-ir, dot3(u, v, w, lu, lvv, lw), lrho);
+    lamQ[n] = lW[0] + lrho;
+    lamQ[N + n] = fma(ir, lu, lW[1]);
+    lamQ[2 * N + n] = fma(ir, lvv, lW[2]);
+    lamQ[3 * N + n] = fma(ir, lw, lW[3]);
+    lamQ[4 * N + n] = lW[4] + lQ4;
     if (lamMK) {
-      lamMK[n] += A[AMU * N + n];
-      lamMK[N + n] += A[(AMU + 1) * N + n];
+      lamMK[n] += lmu;
+      lamMK[N + n] += lka;
     }
   }
 }
@@ -617,6 +648,21 @@ __global__ void k_adj_stage_prep(Grid g, const double* __restrict__ M, double co
       lamQ0[q * N + n] += ls;
       lamR[q * N + n] = in ? -coef * Jn * ls : 0.0;
     }
+  }
+}
+
+// out = lam, 0 on the faces of non-periodic directions (where the residual is 0)
+__global__ void k_mask_faces(Grid g, const double* __restrict__ lam, double* __restrict__ out) {
+  const long long N = g.N;
+  for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N;
+       n += (long long)gridDim.x * blockDim.x) {
+    int c[3];
+    decompose(g, n, c);
+    bool in = true;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) in = in && (g.per[d] || (c[d] > 0 && c[d] < g.n[d] - 1));
+#pragma unroll
+    for (int q = 0; q < 5; ++q) out[q * N + n] = in ? lam[q * N + n] : 0.0;
   }
 }
 
@@ -694,22 +740,22 @@ __device__ void exit_formula(const T qe[5], double ex, double ey, double ez, dou
   qo[4] = rf * (eint + 0.5 * (u * u + v * v + w * w));
 }
 
-// out += J^T lam for a 5 -> 5 map evaluated by forward-mode dual numbers
+// Component i of J^T lam for a 5 -> 5 map evaluated by forward-mode dual
+// numbers.
 template <int KIND>
-__device__ void local_vjp(const double qe[5], double a0, double a1, double a2, double gamma,
-                          const double lam[5], double out[5]) {
-#pragma unroll 1
-  for (int i = 0; i < 5; ++i) {
-    Dual x[5], y[5];
-    for (int q = 0; q < 5; ++q) x[q] = Dual(qe[q], q == i ? 1.0 : 0.0);
-    if (KIND == 0)
-      farfield_formula<Dual>(x, a0, a1, a2, gamma, y);
-    else
-      exit_formula<Dual>(x, a0, a1, a2, gamma, y);
-    double s = 0.0;
-    for (int q = 0; q < 5; ++q) s += y[q].d * lam[q];
-    out[i] += s;
-  }
+__device__ double local_vjp(int i, const double qe[5], double a0, double a1, double a2,
+                            double gamma, const double lam[5]) {
+  Dual x[5], y[5];
+#pragma unroll
+  for (int q = 0; q < 5; ++q) x[q] = Dual(qe[q], q == i ? 1.0 : 0.0);
+  if (KIND == 0)
+    farfield_formula<Dual>(x, a0, a1, a2, gamma, y);
+  else
+    exit_formula<Dual>(x, a0, a1, a2, gamma, y);
+  double s = 0.0;
+#pragma unroll
+  for (int q = 0; q < 5; ++q) s += y[q].d * lam[q];
+  return s;
 }
 
 // lamS = lamNext on interior nodes, 0 on boundary nodes (their stage values
@@ -728,35 +774,45 @@ __global__ void k_adjbc_init(Grid g, const double* __restrict__ lamNext, double*
 
 // exit: the plane i = ni-1 copies / extrapolates the post-phase-1 column
 // i = ni-2 (taken from Qnext).  Interior rows go straight into lamS; the two
-// face rows (j = 0, nj-1) go to E for the ring / far-field reverse.
-__global__ void k_adjbc_exit(Grid g, double gamma, const double* __restrict__ M,
-                             const double* __restrict__ Qnext, const double* __restrict__ lamNext,
-                             double* __restrict__ lamS, double* __restrict__ E) {
-  const int ni = g.n[0], nj = g.n[1], nk = g.n[2];
+// face rows (j = 0, nj-1) go to E for the ring / far-field reverse.  Block row
+// y takes component y of every node: a node's five derivatives are
+// independent, each a chain of a few hundred dependent FP64 operations, and
+// a face has too few nodes to fill the SMs with all five in one thread
+// (the far field's launch took 191 us whatever its size, most of it two pows).
+__global__ void __launch_bounds__(64) k_adjbc_exit(Grid g, double gamma,
+                                                   const double* __restrict__ M,
+                                                   const double* __restrict__ Qnext,
+                                                   const double* __restrict__ lamNext,
+                                                   double* __restrict__ lamS,
+                                                   double* __restrict__ E) {
+  const int ni = g.n[0], nj = g.n[1], nk = g.n[2], i5 = blockIdx.y;
   const long long plane = (long long)nj * nk, N = g.N;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < plane;
        e += (long long)gridDim.x * blockDim.x) {
     const int j = (int)(e / nk);
     const long long nx_ = (long long)(ni - 1) * plane + e, ne = nx_ - plane;
-    double qe[5], lam[5], out[5] = {0, 0, 0, 0, 0};
+    double qe[5], lam[5];
+#pragma unroll
     for (int q = 0; q < 5; ++q) {
       qe[q] = Qnext[q * N + ne];
       lam[q] = lamNext[q * N + nx_];
     }
-    local_vjp<1>(qe, M[nx_], M[N + nx_], M[2 * N + nx_], gamma, lam, out);
-    if (j == 0 || j == nj - 1) {
-      for (int q = 0; q < 5; ++q) E[q * plane + e] = out[q];
-    } else {
-      for (int q = 0; q < 5; ++q) lamS[q * N + ne] += out[q];
-    }
+    const double out = local_vjp<1>(i5, qe, M[nx_], M[N + nx_], M[2 * N + nx_], gamma, lam);
+    if (j == 0 || j == nj - 1)
+      E[i5 * plane + e] = out;
+    else
+      lamS[i5 * N + ne] += out;
   }
 }
 
 // far field: node (i, nj-1, k) from (i, nj-2, k) of the stage-5 state
-__global__ void k_adjbc_farfield(Grid g, double gamma, const double* __restrict__ M,
-                                 const double* __restrict__ S5, const double* __restrict__ lamNext,
-                                 const double* __restrict__ E, double* __restrict__ lamS) {
-  const int ni = g.n[0], nj = g.n[1], nk = g.n[2];
+__global__ void __launch_bounds__(64) k_adjbc_farfield(Grid g, double gamma,
+                                                       const double* __restrict__ M,
+                                                       const double* __restrict__ S5,
+                                                       const double* __restrict__ lamNext,
+                                                       const double* __restrict__ E,
+                                                       double* __restrict__ lamS) {
+  const int ni = g.n[0], nj = g.n[1], nk = g.n[2], i5 = blockIdx.y;
   const long long count = (long long)(ni - 2) * nk, N = g.N, plane = (long long)nj * nk;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < count;
        e += (long long)gridDim.x * blockDim.x) {
@@ -764,13 +820,13 @@ __global__ void k_adjbc_farfield(Grid g, double gamma, const double* __restrict_
     const long long nf = idx3(g, i, nj - 1, k), ne = idx3(g, i, nj - 2, k);
     const double ex = M[3 * N + nf], ey = M[4 * N + nf], ez = M[5 * N + nf];
     const double inv = 1.0 / sqrt(ex * ex + ey * ey + ez * ez);
-    double qe[5], lam[5], out[5] = {0, 0, 0, 0, 0};
+    double qe[5], lam[5];
+#pragma unroll
     for (int q = 0; q < 5; ++q) {
       qe[q] = S5[q * N + ne];
       lam[q] = lamNext[q * N + nf] + (i == ni - 2 ? E[q * plane + (long long)(nj - 1) * nk + k] : 0.0);
     }
-    local_vjp<0>(qe, ex * inv, ey * inv, ez * inv, gamma, lam, out);
-    for (int q = 0; q < 5; ++q) lamS[q * N + ne] += out[q];
+    lamS[i5 * N + ne] += local_vjp<0>(i5, qe, ex * inv, ey * inv, ez * inv, gamma, lam);
   }
 }
 
@@ -806,50 +862,79 @@ __global__ void k_adjbc_ring(Grid g, const double* __restrict__ lamNext, const d
 // entrance: Q = (1, u, 0, 0, p/(g-1) + u^2/2), u = profile + sum a_mf g(r)
 // cos(m theta - 2 pi St_f Mj t): grad_mf += sum over the plane of
 // (lam1 + u lam4) g(r) cos(...); one partial per block and mode.
-__global__ void k_adjbc_inflow(Grid g, double Mj, double r_jet, double theta_m, double width,
-                               const double* __restrict__ St, const double* __restrict__ amp,
-                               const double* __restrict__ rth, double t,
-                               const double* __restrict__ lamNext, double* __restrict__ partials) {
+struct AdjInflow {
+  double Mj, r_jet, theta_m, width, t;
+  double St[4], amp[16];
+};
+
+__global__ void __launch_bounds__(64) k_adjbc_inflow(Grid g, AdjInflow b,
+                                                     const double* __restrict__ rth,
+                                                     const double* __restrict__ lamNext,
+                                                     double* __restrict__ partials) {
   const long long plane = (long long)g.n[1] * g.n[2], N = g.N;
   const double two_pi = 6.283185307179586476925286766559;
+  // cos(m theta - phi_f) = cos(m theta) cos(phi_f) + sin(m theta) sin(phi_f), as
+  // the forward entrance forms it; lane f of the warp takes phase f mod 4
+  double sf[4], cf[4];
+  {
+    const int f = threadIdx.x & 3;
+    double s, c;
+    sincos(two_pi * (f == 0 ? b.St[0] : (f == 1 ? b.St[1] : (f == 2 ? b.St[2] : b.St[3]))) * b.Mj * b.t,
+           &s, &c);
+#pragma unroll
+    for (int l = 0; l < 4; ++l) {
+      sf[l] = __shfl_sync(0xffffffffu, s, l);
+      cf[l] = __shfl_sync(0xffffffffu, c, l);
+    }
+  }
   double acc[16];
+#pragma unroll
   for (int m = 0; m < 16; ++m) acc[m] = 0.0;
   for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < plane;
        n += (long long)gridDim.x * blockDim.x) {
     const double r = rth[n], th = rth[plane + n];
-    double u = 0.5 * Mj * (1.0 + tanh((r_jet - r) / (2.0 * theta_m)));
-    const double x = (r - r_jet) / width;
+    double u = 0.5 * b.Mj * (1.0 + tanh((b.r_jet - r) / (2.0 * b.theta_m)));
+    const double x = (r - b.r_jet) / b.width;
     const double gr = exp(-(x * x));
-    double cs[16];
-    for (int m = 0; m < 4; ++m)
-      for (int f = 0; f < 4; ++f) {
-        cs[m * 4 + f] = cos(m * th - two_pi * St[f] * Mj * t);
-        u += amp[m * 4 + f] * gr * cs[m * 4 + f];
-      }
-    const double lu = lamNext[N + n] + u * lamNext[4 * N + n];
-    for (int m = 0; m < 16; ++m) acc[m] += lu * gr * cs[m];
+    double s1, c1;
+    sincos(th, &s1, &c1);
+    double cm[4] = {1.0, c1, 0.0, 0.0}, sm[4] = {0.0, s1, 0.0, 0.0};
+#pragma unroll
+    for (int m = 2; m < 4; ++m) {
+      cm[m] = cm[m - 1] * c1 - sm[m - 1] * s1;
+      sm[m] = sm[m - 1] * c1 + cm[m - 1] * s1;
+    }
+    double cs[16], f = 0.0;
+#pragma unroll
+    for (int m = 0; m < 16; ++m) {
+      cs[m] = cm[m >> 2] * cf[m & 3] + sm[m >> 2] * sf[m & 3];
+      f += b.amp[m] * cs[m];
+    }
+    u += gr * f;
+    const double lu = gr * (lamNext[N + n] + u * lamNext[4 * N + n]);
+#pragma unroll
+    for (int m = 0; m < 16; ++m) acc[m] += lu * cs[m];
   }
-  __shared__ double red[16][32];
+  __shared__ double red[16][2];
+#pragma unroll
   for (int m = 0; m < 16; ++m) {
     double v = acc[m];
     for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
     if ((threadIdx.x & 31) == 0) red[m][threadIdx.x >> 5] = v;
   }
   __syncthreads();
-  if (threadIdx.x < 16) {
-    double v = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += red[threadIdx.x][w];
-    partials[blockIdx.x * 16 + threadIdx.x] = v;
-  }
+  if (threadIdx.x < 16) partials[blockIdx.x * 16 + threadIdx.x] = red[threadIdx.x][0] + red[threadIdx.x][1];
 }
 
-// grad[m] += sum of the block partials (fixed order)
-__global__ void k_sum_partials16(const double* __restrict__ partials, int nb, double* __restrict__ grad) {
-  const int m = threadIdx.x;
-  if (m >= 16) return;
+// out[m] += sum of the block partials of item m = this block's, in a fixed
+// order (a warp per item; lanes take the blocks in turn)
+__global__ void k_sum_partials(const double* __restrict__ partials, int nb, int items,
+                               double* __restrict__ out) {
+  const int m = blockIdx.x, lane = threadIdx.x;
   double s = 0.0;
-  for (int b = 0; b < nb; ++b) s += partials[b * 16 + m];
-  grad[m] += s;
+  for (int b = lane; b < nb; b += 32) s += partials[b * items + m];
+  for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+  if (lane == 0) out[m] += s;
 }
 
 // ------------------------------------------------------------ functional
@@ -893,13 +978,6 @@ __global__ void k_functional(Grid g, double gamma, int j5, double dt, const TM* 
   }
 }
 
-__global__ void k_sum_partials1(const double* __restrict__ partials, int nb, double* __restrict__ out) {
-  if (threadIdx.x != 0) return;
-  double s = 0.0;
-  for (int b = 0; b < nb; ++b) s += partials[b];
-  out[0] += s;
-}
-
 __global__ void k_pack_dual(long long count, const double* __restrict__ v,
                             const double* __restrict__ d, Dual* __restrict__ out) {
   for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < count;
@@ -927,23 +1005,28 @@ static int nb_for(long long count) {
 }
 
 void launch_rhs_vjp(const Grid& g, const les_params& p, const double* Q, const double* M,
-                    const double* gn, const double* node, const double* mk, const double* lamR, double* acc,
-                    double* lamQ, double* lamMK, const Launch& L, const double* nu) {
-  // nu: the three sensors of the stage input (launch_sensor64 on node)
+                    const double* gn, const double* node, const double* mk, const double* lamR,
+                    double* acc, double* lamQ, double* lamMK, const Launch& L) {
   const Consts<double> K = make_consts<double>(p);
-  const int nb = nb_for(g.N);
-  // acc holds the NACC accumulator slots, then the three directions' records
-  double* rec = acc + (size_t)NACC * g.N;
-  const size_t rs = (size_t)NREC * g.N;
-  k_adj_iface<0><<<nb, 256, 0, L.s>>>(g, K, Q, M, node, mk, lamR, rec, nu);
-  k_adj_iface<1><<<nb, 256, 0, L.s>>>(g, K, Q, M, node, mk, lamR, rec + rs, nu);
-  k_adj_iface<2><<<nb, 256, 0, L.s>>>(g, K, Q, M, node, mk, lamR, rec + 2 * rs, nu);
-  k_adj_gather<<<nb, 256, 0, L.s>>>(g, rec, rec + rs, rec + 2 * rs, acc);
-  // the records are consumed: their space holds the sensor terms
-  k_adj_sensor_terms<<<nb, 256, 0, L.s>>>(g, node, acc, rec);
-  k_adj_sensor_gather<<<nb, 256, 0, L.s>>>(g, rec, acc);
-  k_adj_node<<<nb, 256, 0, L.s>>>(g, K, Q, M, gn, node, acc, lamQ, lamMK);
-  *L.counter += 7;
+  // acc holds the sensor terms, then the three directions' records
+  double* ST = acc;
+  double* rec = acc + (size_t)kAdjSensorTerms * g.N;
+  // chunk lengths as the forward's; a line has an entry for every node
+  const FluxPlan f = flux_plan(g);
+  auto blocks = [](long long t) { return (unsigned)((t + kFluxThreads - 1) / kFluxThreads); };
+  auto chunks = [&](int d) { return (g.n[d] + f.len - 1) / f.len; };
+  const unsigned b0 = blocks((long long)chunks(0) * g.n[1] * g.n[2]);
+  const unsigned b1 = blocks((long long)g.n[0] * chunks(1) * g.n[2]);
+  const AdjIO io{FluxIO<double, double, double>{Q, M, node, mk, nullptr}, lamR, rec};
+  k_adj_flux3<<<f.b2 + b0 + b1, kFluxThreads, 0, L.s>>>(g, K, io, f.b2, b0, f.len);
+  k_adj_sensor_terms<<<nb_for(g.N), 256, 0, L.s>>>(g, node, rec, ST);
+  k_adj_node<<<blocks_for(g.N, 128), 128, 0, L.s>>>(g, K, Q, M, gn, node, lamR, rec, ST, lamQ, lamMK);
+  *L.counter += 3;
+}
+
+void launch_mask_faces(const Grid& g, const double* lam, double* out, const Launch& L) {
+  k_mask_faces<<<nb_for(g.N), 256, 0, L.s>>>(g, lam, out);
+  ++*L.counter;
 }
 
 void launch_rhs_jvp(const Grid& g, const les_params& p, const Dual* Q, const double* M,
@@ -990,20 +1073,25 @@ void launch_bc_vjp(const Grid& g, const les_params& p, const double* M, const do
                    double* lamS, double* E, double* partials, double* grad, const Launch& L) {
   const long long plane = (long long)g.n[1] * g.n[2];
   k_adjbc_init<<<nb_for(g.N), 256, 0, L.s>>>(g, lamNext, lamS);
-  k_adjbc_exit<<<nb_for(plane), 256, 0, L.s>>>(g, p.gamma, M, Qnext, lamNext, lamS, E);
-  k_adjbc_farfield<<<nb_for((long long)(g.n[0] - 2) * g.n[2]), 256, 0, L.s>>>(g, p.gamma, M, S5,
-                                                                               lamNext, E, lamS);
+  auto nb64 = [](long long count) {
+    const long long b = (count + 63) / 64;
+    return (unsigned)(b < kAdjBlocks ? b : kAdjBlocks);
+  };
+  k_adjbc_exit<<<dim3(nb64(plane), 5), 64, 0, L.s>>>(g, p.gamma, M, Qnext, lamNext, lamS, E);
+  k_adjbc_farfield<<<dim3(nb64((long long)(g.n[0] - 2) * g.n[2]), 5), 64, 0, L.s>>>(
+      g, p.gamma, M, S5, lamNext, E, lamS);
   k_adjbc_ring<<<g.n[0] - 2, 256, 0, L.s>>>(g, lamNext, E, lamS);
-  // forcing parameters in a small device block after the partials
-  double* par = partials + kAdjBlocks * 16;
-  double hostpar[20];
-  for (int i = 0; i < 4; ++i) hostpar[i] = p.St[i];
-  for (int i = 0; i < 16; ++i) hostpar[4 + i] = p.amp[i];
-  cudaMemcpyAsync(par, hostpar, sizeof(hostpar), cudaMemcpyHostToDevice, L.s);
-  const int nbi = nb_for(plane) < kAdjBlocks ? nb_for(plane) : kAdjBlocks;
-  k_adjbc_inflow<<<nbi, 256, 0, L.s>>>(g, p.Mj, p.r_jet, p.theta_m, p.force_width, par, par + 4,
-                                       rth, t_next, lamNext, partials);
-  k_sum_partials16<<<1, 32, 0, L.s>>>(partials, nbi, grad);
+  AdjInflow in;
+  in.Mj = p.Mj;
+  in.r_jet = p.r_jet;
+  in.theta_m = p.theta_m;
+  in.width = p.force_width;
+  in.t = t_next;
+  for (int i = 0; i < 4; ++i) in.St[i] = p.St[i];
+  for (int i = 0; i < 16; ++i) in.amp[i] = p.amp[i];
+  const unsigned nbi = nb64(plane);
+  k_adjbc_inflow<<<nbi, 64, 0, L.s>>>(g, in, rth, lamNext, partials);
+  k_sum_partials<<<16, 32, 0, L.s>>>(partials, (int)nbi, 16, grad);
   *L.counter += 6;
 }
 
@@ -1013,7 +1101,7 @@ void launch_functional(const Grid& g, const les_params& p, int j5, double dt, co
   const long long count = (long long)g.n[0] * g.n[2];
   const int nb = nb_for(count) < kAdjBlocks ? nb_for(count) : kAdjBlocks;
   k_functional<double><<<nb, 256, 0, L.s>>>(g, p.gamma, j5, dt, M, Q, lam, partials);
-  k_sum_partials1<<<1, 32, 0, L.s>>>(partials, nb, Jout);
+  k_sum_partials<<<1, 32, 0, L.s>>>(partials, nb, 1, Jout);
   *L.counter += 2;
 }
 
@@ -1022,7 +1110,7 @@ void launch_functional(const Grid& g, const les_params& p, int j5, double dt, co
   const long long count = (long long)g.n[0] * g.n[2];
   const int nb = nb_for(count) < kAdjBlocks ? nb_for(count) : kAdjBlocks;
   k_functional<float><<<nb, 256, 0, L.s>>>(g, p.gamma, j5, dt, M, Q, nullptr, partials);
-  k_sum_partials1<<<1, 32, 0, L.s>>>(partials, nb, Jout);
+  k_sum_partials<<<1, 32, 0, L.s>>>(partials, nb, 1, Jout);
   *L.counter += 2;
 }
 

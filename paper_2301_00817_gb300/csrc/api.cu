@@ -39,7 +39,7 @@ struct les_ctx {
   les_params p;
   Grid g;
   // workspace layout (byte offsets, 256-byte aligned)
-  size_t off_m64, off_m32, off_mk, off_sa, off_sb, off_hi, off_lo, off_node, off_flux, off_nu, off_gn, off_rth,
+  size_t off_m64, off_m32, off_mk, off_sa, off_sb, off_hi, off_lo, off_node, off_flux, off_gn, off_rth,
       off_sc, off_part, off_dtl, off_dyn;
   size_t total;
   bool local_dt;  // the workspace holds per-node steps (dt_mode LOCAL at creation)
@@ -207,7 +207,6 @@ void layout(les_ctx* c) {
   // node fields: FP64 form; FP32 for the mixed forms' dynamic procedure
   c->off_node = o; o = align256(o + (mixed ? (c->dyn_ws ? 8 * N * sizeof(float) : 0) : 8 * N * sizeof(double)));
   c->off_flux = o; o = align256(o + (mixed ? 0 : 15 * N * sizeof(double)));
-  c->off_nu = o; o = align256(o + (mixed ? 0 : 3 * N * sizeof(double)));
   c->off_gn = o; o = align256(o + (mixed ? 0 : 4 * N * sizeof(double)));
   c->off_rth = o; o = align256(o + 2 * (size_t)c->g.n[1] * c->g.n[2] * sizeof(double));
   c->off_sc = o; o = align256(o + sizeof(DevScalars));
@@ -248,7 +247,6 @@ lesjet::StageIO64 io64(les_ctx* c, const double* Qin) {
   io.sc = at<DevScalars>(c, c->off_sc);
   io.dtl = c->p.dt_mode == LES_DT_LOCAL ? at<double>(c, c->off_dtl) : nullptr;
   io.dyn = c->dyn_ws ? at<double>(c, c->off_dyn) : nullptr;
-  io.nu = at<double>(c, c->off_nu);
   return io;
 }
 
@@ -1055,7 +1053,7 @@ AdjLayout adj_layout(const les_ctx* c, int nsteps, int K) {
     o = align256(o + bytes);
     return at_;
   };
-  L.acc = take((18 + 3 * 45) * N * d);  // accumulators, then the interface records
+  L.acc = take((lesjet::kAdjSensorTerms + 3 * lesjet::kAdjRecords) * N * d);
   L.node = take(8 * N * d);
   L.mk = take(2 * N * d);
   L.lamMK = take(2 * N * d);
@@ -1117,7 +1115,6 @@ lesjet::StageIO64 adj_io(les_ctx* c, void* aw, const AdjLayout& Ly, const double
   io.Qin = Qin;
   io.M = at<double>(c, c->off_m64);
   io.gn = at<double>(c, c->off_gn);
-  io.nu = at<double>(c, c->off_nu);
   io.node = aw_at<double>(aw, Ly.node);
   io.mk = aw_at<double>(aw, Ly.mk);
   io.flux = at<double>(c, c->off_flux);
@@ -1188,9 +1185,8 @@ void adj_reverse(les_ctx* c, void* aw, const AdjLayout& Ly, double* const S[6], 
       io.node = const_cast<double*>(nodes) + (size_t)(l - 1) * 8 * g.N;  // kept by adj_forward
     else
       lesjet::launch_node64(g, c->p, io, false, L);
-    lesjet::launch_sensor64(g, io, L);
     lesjet::launch_rhs_vjp(g, c->p, S[l - 1], M, io.gn, io.node, io.mk, lamR, aw_at<double>(aw, Ly.acc),
-                           lamS, lamMK, L, io.nu);
+                           lamS, lamMK, L);
   }
   lesjet::launch_axpy(5 * g.N, 1.0, lamS, lamQ0, L);
   lesjet::launch_mu_vjp(g, c->p, S[0], lamMK, lamQ0, L);
@@ -1246,9 +1242,11 @@ int les_rhs_vjp(les_ctx* c, const double* Q, const double* lamR, double* lamQ, d
   lesjet::launch_node64(c->g, c->p, io, false, L);
   lesjet::launch_mu64(c->g, c->p, io, L);
   cudaMemsetAsync(lamMK, 0, 2 * (size_t)c->g.N * sizeof(double), s);
-  lesjet::launch_sensor64(c->g, io, L);
-  lesjet::launch_rhs_vjp(c->g, c->p, Q, io.M, io.gn, io.node, io.mk, lamR, aw_at<double>(aw, Ly.acc), lamQ,
-                         lamMK, L, io.nu);
+  // boundary entries of lamR are ignored: the kernels read a copy without them
+  double* lR = aw_at<double>(aw, Ly.lamR);
+  lesjet::launch_mask_faces(c->g, lamR, lR, L);
+  lesjet::launch_rhs_vjp(c->g, c->p, Q, io.M, io.gn, io.node, io.mk, lR, aw_at<double>(aw, Ly.acc), lamQ,
+                         lamMK, L);
   return cuda_check(c, "les_rhs_vjp");
 }
 
@@ -1267,8 +1265,11 @@ int les_adjoint_step(les_ctx* c, const double* Qn, double t_n, const double* lam
   for (int l = 0; l < 6; ++l) S[l] = aw_at<double>(aw, Ly.S) + (size_t)l * 5 * c->g.N;
   cudaMemcpyAsync(S[0], Qn, 5 * (size_t)c->g.N * sizeof(double), cudaMemcpyDeviceToDevice, s);
   double* mk = aw_at<double>(aw, Ly.mk);
-  adj_forward(c, aw, Ly, S, mk, nullptr, s);
-  adj_reverse(c, aw, Ly, S, mk, nullptr, t_n, lam_next, lam_out, gdev, s);
+  // the five stage inputs' node quantities are kept for the reverse, in the
+  // space of the tangent's dual numbers
+  double* nodes = aw_at<double>(aw, Ly.qd);
+  adj_forward(c, aw, Ly, S, mk, nodes, s);
+  adj_reverse(c, aw, Ly, S, mk, nodes, t_n, lam_next, lam_out, gdev, s);
   if ((rc = cuda_check(c, "les_adjoint_step")) != LES_OK) return rc;
   double h[16];
   cudaMemcpyAsync(h, gdev, sizeof(h), cudaMemcpyDeviceToHost, s);

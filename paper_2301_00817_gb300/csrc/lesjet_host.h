@@ -46,8 +46,6 @@ struct StageIO64 {
   double* partials;    // [kRedBlocks] block minima (dt)
   DevScalars* sc;
   double* dtl = nullptr;  // [N] local steps (dt_mode LOCAL), else nullptr
-  double* nu = nullptr;   // [3][N] pressure sensors along xi, eta, zeta
-                          // (k_sensor; the reverse kernels read them)
   double* dyn = nullptr;  // [50][N] scratch of the dynamic SGS procedure
 };
 void launch_node64(const Grid& g, const les_params& p, const StageIO64& io, bool with_dt,
@@ -64,9 +62,6 @@ void launch_dynamic32(const Grid& g, const les_params& p, const float* Q, const 
                       float* node, float* scratch, double* partials, DevScalars* sc,
                       const Launch& L);
 void launch_flux64(const Grid& g, const les_params& p, const StageIO64& io, const Launch& L);
-// the three pressure sensors of every node into io.nu (after launch_node64),
-// for the reverse kernels
-void launch_sensor64(const Grid& g, const StageIO64& io, const Launch& L);
 // mode 0: RHS into out; 1: stage update into out; 2: last stage in place
 void launch_update64(const Grid& g, const StageIO64& io, const double* Q0, double alpha, int mode,
                      double* out, const Launch& L);
@@ -101,8 +96,14 @@ void launch_join(long long count, const float* hi, const float* lo, double* q, c
 // bookkeeping, boundary-condition adjoint and the surface functional
 struct Dual;
 void launch_rhs_vjp(const Grid& g, const les_params& p, const double* Q, const double* M,
-                    const double* gn, const double* node, const double* mk, const double* lamR, double* acc,
-                    double* lamQ, double* lamMK, const Launch& L, const double* nu);
+                    const double* gn, const double* node, const double* mk, const double* lamR,
+                    double* acc, double* lamQ, double* lamMK, const Launch& L);
+// out = lam, 0 on the faces of non-periodic directions ([5][N]), as
+// launch_rhs_vjp wants lamR
+void launch_mask_faces(const Grid& g, const double* lam, double* out, const Launch& L);
+// scratch of launch_rhs_vjp (acc): sensor terms, then one record of
+// kAdjRecords fields per interface of each direction
+constexpr int kAdjSensorTerms = 6, kAdjRecords = 22;
 void launch_rhs_jvp(const Grid& g, const les_params& p, const Dual* Q, const double* M,
                     const Dual* mk, Dual* node, Dual* flux, Dual* R, const Launch& L);
 void launch_mu_vjp(const Grid& g, const les_params& p, const double* Q, const double* lamMK,

@@ -65,13 +65,6 @@ void launch_flux64(const Grid& g, const les_params& p, const StageIO64& io, cons
   ++*L.counter;
 }
 
-void launch_sensor64(const Grid& g, const StageIO64& io, const Launch& L) {
-  if (!io.nu) return;
-  const int th = 256, nb = blocks_for(g.N, th);
-  k_sensor<double><<<nb, th, 0, L.s>>>(g, io.node + 3 * g.N, io.nu);
-  ++*L.counter;
-}
-
 void launch_update64(const Grid& g, const StageIO64& io, const double* Q0, double alpha, int mode,
                      double* out, const Launch& L) {
   const int th = 256, nb = blocks_for(g.N, th);

@@ -256,22 +256,6 @@ __device__ __forceinline__ R sensor(const Grid& g, const R* __restrict__ P, long
   return sensor3(P[xm], P[xc], P[xp]);
 }
 
-// The three sensors of every node (the reverse kernels read them; k_flux3
-// evaluates them as it goes).
-template <typename R>
-__global__ void __launch_bounds__(256) k_sensor(Grid g, const R* __restrict__ P,
-                                                R* __restrict__ NU) {
-  const long long N = g.N;
-  for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N;
-       n += (long long)gridDim.x * blockDim.x) {
-    int c[3];
-    decompose(g, n, c);
-    NU[n] = sensor<0>(g, P, n, c[0]);
-    NU[N + n] = sensor<1>(g, P, n, c[1]);
-    NU[2 * N + n] = sensor<2>(g, P, n, c[2]);
-  }
-}
-
 template <typename R>
 __device__ __forceinline__ R dot3(const R& a0, const R& a1, const R& a2, const R& b0, const R& b1,
                                   const R& b2) {
