@@ -55,13 +55,16 @@ __device__ __forceinline__ void cp_async_wait() {
 }
 
 // ----------------------------------------------------------- interface flux
-// Flux through the interface between nodes a and b (b = a + e_D): centred
-// inviscid flux (Eqs. hat-flux-G, inv_flux_vec) minus J^-1 d (Eqs.
+// Twice the flux through the interface between nodes a and b (b = a + e_D):
+// centred inviscid flux (Eqs. hat-flux-G, inv_flux_vec) minus J^-1 d (Eqs.
 // dissip_term, eps_2/4_dissip with the boundary closure of the centerline
 // section) minus the viscous + SGS flux (Eqs. hat-flux-Ev/Fv/Gv, tau_mod,
 // q_mod with Fourier's sign) from compact interface gradients.
 // m*[0..8] = xi_x .. zeta_z, m*[9] = J^-1; W* = (rho, rho u, rho v, rho w,
-// e + p); dphi[q][t] = computational derivative of u, v, w, T along t.
+// e + p); dphi[q][t] = the difference of u, v, w, T along the normal (t = D)
+// and four times the computational derivative along a tangent.  The interface
+// means stay sums of the two nodes' values, their powers of two collected in
+// a few constants; the epilogue halves once per node.
 template <int D, typename R, bool AXIS, bool DYN>
 __device__ __forceinline__ void iface_flux(const Consts<R>& K, const R* Wm, const R* Wa,
                                            const R* Wb, const R* Wp, bool has_m, bool has_p,
@@ -69,34 +72,35 @@ __device__ __forceinline__ void iface_flux(const Consts<R>& K, const R* Wm, cons
                                            R pa, R pb, R ua, R va, R wa, R ub, R vb, R wb,
                                            const R (&dphi)[4][3], R mua, R mub, R kaa, R kab,
                                            R sga, R sgb, R F[5]) {
-  const R tha = ma[3 * D] * ua + ma[3 * D + 1] * va + ma[3 * D + 2] * wa;
-  const R thb = mb[3 * D] * ub + mb[3 * D + 1] * vb + mb[3 * D + 2] * wb;
+  constexpr int T1 = (D + 1) % 3, T2 = (D + 2) % 3;
   const R Ja = ma[9], Jb = mb[9];
-  R Fc[5];
   // W[0..3] = Q[0..3]; W[4] = e + p, so (e + p) Th = W[4] Th
-  Fc[0] = Ja * (Wa[0] * tha) + Jb * (Wb[0] * thb);
-  Fc[1] = Ja * (Wa[1] * tha + pa * ma[3 * D]) + Jb * (Wb[1] * thb + pb * mb[3 * D]);
-  Fc[2] = Ja * (Wa[2] * tha + pa * ma[3 * D + 1]) + Jb * (Wb[2] * thb + pb * mb[3 * D + 1]);
-  Fc[3] = Ja * (Wa[3] * tha + pa * ma[3 * D + 2]) + Jb * (Wb[3] * thb + pb * mb[3 * D + 2]);
-  Fc[4] = Ja * (Wa[4] * tha) + Jb * (Wb[4] * thb);
+  const R Ta = Ja * (ma[3 * D] * ua + ma[3 * D + 1] * va + ma[3 * D + 2] * wa);
+  const R Tb = Jb * (mb[3 * D] * ub + mb[3 * D + 1] * vb + mb[3 * D + 2] * wb);
+  const R qa = Ja * pa, qb = Jb * pb;
+  // Dissipation: with D1 = W_b - W_a and E = W_{b+1} - W_{a-1} the third
+  // difference is E - 3 D1, so eps2 D1 - eps4 D3 = (eps2 + 3 eps4) D1 - eps4 E;
+  // a missing outside difference, minus the first inside one, means W_{a-1} =
+  // W_b or W_{b+1} = W_a
   const R eps2 = K.k2 * dev_max(nua, nub);
   const R eps4 = dev_max(R(0), K.k4 - eps2);
-  const R Jh = R(0.5) * (Ja + Jb);
-  const R lJ = R(0.5) * (lba + lbb) * Jh;
+  const R sJ = Ja + Jb;
+  const R lJ = R(0.5) * (lba + lbb) * sJ;  // 2 lambda J^-1
+  const R d1 = lJ * (eps2 + R(3) * eps4), d3 = lJ * eps4;
 #pragma unroll
   for (int q = 0; q < 5; ++q) {
-    const R D1 = Wb[q] - Wa[q];
-    const R Dm = has_m ? Wa[q] - Wm[q] : -D1;
-    const R Dp = has_p ? Wp[q] - Wb[q] : -D1;
-    const R D3 = Dp - R(2) * D1 + Dm;
-    F[q] = R(0.5) * Fc[q] - lJ * (eps2 * D1 - eps4 * D3);
+    R f = Wa[q] * Ta + Wb[q] * Tb;
+    if (q >= 1 && q <= 3) f += qa * ma[3 * D + q - 1] + qb * mb[3 * D + q - 1];
+    const R E = (has_p ? Wp[q] : Wa[q]) - (has_m ? Wm[q] : Wb[q]);
+    F[q] = f - d1 * (Wb[q] - Wa[q]) + d3 * E;
   }
   // Viscous part from the interface metric vectors m_t (kept at twice
   // their mean): with m = m_D, the flux needs only m.tau and m.q, and
   //   m.tau_i / mu = sum_t g_t dphi_i,t + sum_t m_t,i c_t - 2/3 m_i div,
   //   m.grad T     = sum_t g_t dphi_T,t,
   // where g_t = m . m_t, c_t = sum_j m_j dphi_j,t and div = sum_t m_t .
-  // dphi_.,t (every factor 2 of the sums is collected in the constants).
+  // dphi_.,t, whose normal part is c_D itself.  g_D and c_D take the factor 4
+  // that the normal difference lacks: every sum is 16x its value.
   R mt[9];
   if (AXIS) {
     // a grid with an axis (Reading A27): the J^-1-weighted mean of the two
@@ -109,41 +113,41 @@ __device__ __forceinline__ void iface_flux(const Consts<R>& K, const R* Wm, cons
 #pragma unroll
     for (int t = 0; t < 9; ++t) mt[t] = ma[t] + mb[t];
   }
-  const R mx = mt[3 * D], my = mt[3 * D + 1], mz = mt[3 * D + 2];  // 2 m
+  const R m0 = mt[3 * D], m1 = mt[3 * D + 1], m2 = mt[3 * D + 2];  // 2 m
   R g[3], c[3];
 #pragma unroll
   for (int t = 0; t < 3; ++t) {
-    g[t] = mx * mt[3 * t] + my * mt[3 * t + 1] + mz * mt[3 * t + 2];        // 4 g_t
-    c[t] = mx * dphi[0][t] + my * dphi[1][t] + mz * dphi[2][t];             // 2 c_t
+    g[t] = m0 * mt[3 * t] + m1 * mt[3 * t + 1] + m2 * mt[3 * t + 2];
+    c[t] = m0 * dphi[0][t] + m1 * dphi[1][t] + m2 * dphi[2][t];
   }
-  R div = R(0);  // 2 div
-#pragma unroll
-  for (int t = 0; t < 3; ++t)
-    div += mt[3 * t] * dphi[0][t] + mt[3 * t + 1] * dphi[1][t] + mt[3 * t + 2] * dphi[2][t];
-  const R d23 = R(2.0 / 3.0) * div;
-  const R mm[3] = {mx, my, mz};
-  R sv[3];  // 4 m.tau_i / mu
+  g[D] *= R(4);
+  c[D] *= R(4);
+  R div = c[D];  // 8 div
+  div += mt[3 * T1] * dphi[0][T1] + mt[3 * T1 + 1] * dphi[1][T1] + mt[3 * T1 + 2] * dphi[2][T1];
+  div += mt[3 * T2] * dphi[0][T2] + mt[3 * T2 + 1] * dphi[1][T2] + mt[3 * T2 + 2] * dphi[2][T2];
+  c[D] -= R(2.0 / 3.0) * div;
+  R sv[3];  // 16 m.tau_i / mu
 #pragma unroll
   for (int i = 0; i < 3; ++i)
-    sv[i] = (g[0] * dphi[i][0] + g[1] * dphi[i][1] + g[2] * dphi[i][2]) +
-            (mt[i] * c[0] + mt[3 + i] * c[1] + mt[6 + i] * c[2]) - mm[i] * d23;
-  const R aT = g[0] * dphi[3][0] + g[1] * dphi[3][1] + g[2] * dphi[3][2];  // 4 m.grad T
-  const R sJ = Ja + Jb, smu = mua + mub, skap = kaa + kab;  // 2x the means
-  const R cf = sJ * smu * R(1.0 / 16.0);
-  F[1] -= cf * sv[0];
-  F[2] -= cf * sv[1];
-  F[3] -= cf * sv[2];
-  const R us = (ua + ub) * sv[0] + (va + vb) * sv[1] + (wa + wb) * sv[2];  // 8 u_f . m.tau / mu
-  F[4] -= sJ * (smu * us * R(1.0 / 32.0) + skap * aT * R(1.0 / 16.0));
+    sv[i] = g[0] * dphi[i][0] + g[1] * dphi[i][1] + g[2] * dphi[i][2] + mt[i] * c[0] +
+            mt[3 + i] * c[1] + mt[6 + i] * c[2];
+  const R aT = g[0] * dphi[3][0] + g[1] * dphi[3][1] + g[2] * dphi[3][2];  // 16 m.grad T
+  const R sJ32 = sJ * R(1.0 / 32.0);
+  const R cm = sJ32 * (mua + mub), ck = sJ32 * (kaa + kab);
+  F[1] -= cm * sv[0];
+  F[2] -= cm * sv[1];
+  F[3] -= cm * sv[2];
+  F[4] -= R(0.5) * cm * ((ua + ub) * sv[0] + (va + vb) * sv[1] + (wa + wb) * sv[2]);
+  F[4] -= ck * aT;
   if (DYN) {
     // the modelled isotropic SGS stress sigma_ll/3 (Eq. yoshizawa) at the
     // interface mean, subtracted from the normal stresses: m.tau_i gains
     // -m_i sigma/3 and u_f.(m.tau) gains -(u_f . m) sigma/3
-    const R e1 = sJ * (sga + sgb) * R(1.0 / 24.0);
-    F[1] += e1 * mx;
-    F[2] += e1 * my;
-    F[3] += e1 * mz;
-    F[4] += e1 * R(0.5) * ((ua + ub) * mx + (va + vb) * my + (wa + wb) * mz);
+    const R e1 = sJ * (sga + sgb) * R(1.0 / 12.0);
+    F[1] += e1 * m0;
+    F[2] += e1 * m1;
+    F[3] += e1 * m2;
+    F[4] += e1 * R(0.5) * ((ua + ub) * m0 + (va + vb) * m1 + (wa + wb) * m2);
   }
 }
 
@@ -462,10 +466,10 @@ struct FLayout {
 };
 static_assert(FLayout<true>::FLOATS * 4 <= 227 * 1024, "shared memory plan exceeds 227 KB");
 
-// Computational derivatives of (u, v, w, T) at an interface from node
-// records (float4 u, v, w, T): along the interface normal, phi_b - phi_a;
-// along a tangent t, the mean of the two nodes' central differences,
-// 1/4 [(phi_{a+t} - phi_{a-t}) + (phi_{b+t} - phi_{b-t})].
+// Differences of (u, v, w, T) at an interface from node records (float4 u, v,
+// w, T): along the interface normal, phi_b - phi_a; along a tangent t, four
+// times the mean of the two nodes' central differences,
+// (phi_{a+t} - phi_{a-t}) + (phi_{b+t} - phi_{b-t}).
 template <int D>
 __device__ __forceinline__ void dphi_normal(const float4 a, const float4 b, float (&dphi)[4][3]) {
   dphi[0][D] = b.x - a.x;
@@ -476,10 +480,10 @@ __device__ __forceinline__ void dphi_normal(const float4 a, const float4 b, floa
 template <int T>
 __device__ __forceinline__ void dphi_tangent(const float4 ap, const float4 am, const float4 bp,
                                              const float4 bm, float (&dphi)[4][3]) {
-  dphi[0][T] = 0.25f * ((ap.x - am.x) + (bp.x - bm.x));
-  dphi[1][T] = 0.25f * ((ap.y - am.y) + (bp.y - bm.y));
-  dphi[2][T] = 0.25f * ((ap.z - am.z) + (bp.z - bm.z));
-  dphi[3][T] = 0.25f * ((ap.w - am.w) + (bp.w - bm.w));
+  dphi[0][T] = (ap.x - am.x) + (bp.x - bm.x);
+  dphi[1][T] = (ap.y - am.y) + (bp.y - bm.y);
+  dphi[2][T] = (ap.z - am.z) + (bp.z - bm.z);
+  dphi[3][T] = (ap.w - am.w) + (bp.w - bm.w);
 }
 
 __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
@@ -997,7 +1001,8 @@ __global__ void __launch_bounds__(FNT, 1)
   float Fx_prev[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
   if (own && jint && kint && (per_i || ib - 1 >= 0))
     xi_flux(ib - 1, s_m, s_c, s_m, s_c, l_p, l_c, nullptr, nullptr, nullptr, nullptr, Fx_prev);
-  const float adt = (MODE == FMODE_RHS) ? 0.f : (float)(alpha * sc->dt);
+  // the fluxes are twice their value
+  const float adt = (MODE == FMODE_RHS) ? 0.f : (float)(0.5 * alpha * sc->dt);
   // plane ib+1 has landed (this thread's copies; the barrier makes everyone's
   // visible) and the xi flux above is done with the slots of plane ib-1
   cp_async_wait<0>();
@@ -1102,7 +1107,9 @@ __global__ void __launch_bounds__(FNT, 1)
       const int n = (ig * nj + jown) * nk + kown;
       if (iint && jint && kint) {
         const float Jn = frcp_fast(mo[9]);
-        const float an = LOCAL ? (float)alpha * dc : adt;
+        // alpha dt J / 2
+        const float an = LOCAL ? (float)(0.5 * alpha) * dc : adt;
+        const float aJ = an * Jn;
 #pragma unroll
         for (int c = 0; c < 5; ++c) {
           float r = 0.f;
@@ -1111,13 +1118,13 @@ __global__ void __launch_bounds__(FNT, 1)
           r += dz[c];
           if (tx == 0) r -= sFz[c * FTJ + ty];
           if (MODE == FMODE_RHS) {
-            P.outd[c][n] = (double)r;
+            P.outd[c][n] = (double)(0.5f * r);
           } else if (MODE == FMODE_STAGE) {
-            P.out[c][n] = hc[c] - an * (Jn * r);
+            P.out[c][n] = hc[c] - aJ * r;
           } else {
             // compensated update of the pair (hi, lo) by d (TwoSum, then
             // renormalisation), all in FP32
-            const float d = -an * (Jn * r);
+            const float d = -aJ * r;
             const float hi = hc[c], lo = lc[c];
             const float s = hi + d;
             const float bb = s - hi;
