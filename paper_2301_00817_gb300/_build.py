@@ -23,7 +23,8 @@ NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xptxas"
 # Per-file flags: the FP32-mixed kernels use approximate FP32 division and
 # square root (FP64 code is unaffected by these flags).
 _FAST_FP32 = ["-prec-div=false", "-prec-sqrt=false", "-ftz=true"]
-FILE_FLAGS = {f: _FAST_FP32 for f in ("fused.cu", "fused_jet4.cu", "fused_jet12.cu", "fused_jet28.cu")}
+FILE_FLAGS = {f: _FAST_FP32 for f in ("fused.cu", "fused_jet4.cu", "fused_jet4s.cu", "fused_jet12.cu",
+                                   "fused_jet12s.cu", "fused_jet28.cu")}
 
 
 def _nvcc() -> str:

@@ -336,6 +336,20 @@ void launch_prestep(const Grid& g, const les_params& p, const float* Q0, const f
   }
 }
 
+// Rows of the fused stage's tiles.  A plane of an 8-row tile costs 0.66 of a
+// 16-row one's (its warps wait less for one another, but its halo is twice
+// the share), so 8 rows win where they let the schedule finish earlier by
+// that factor: on grids with about a plane per SM or less, whose stage is
+// mostly latency (us a step with 16 and with 8 rows: 48 x 24 x 32 94 and 76, 96
+// x 24 x 32 122 and 93, 96 x 32 x 32 121 and 109; 64 x 64 x 64 178 and 178, 192
+// x 64 x 64 375 and 422).  Both give the same bits.
+static int tile_rows(const FusedGeom& G) {
+  const int sms = sm_count(), tk = (G.nk + FTK - 1) / FTK;
+  const int t16 = tk * ((G.nj + 15) / 16), t8 = tk * ((G.nj + 7) / 8);
+  if ((long long)t16 * G.ni > 4LL * sms) return 16;  // (no grid of that size gains)
+  return 0.66 * choose_chunks(G.ni, t8, sms).t < choose_chunks(G.ni, t16, sms).t ? 8 : 16;
+}
+
 void launch_stage_fused(int mode, const Grid& g, const les_params& p, const FusedIO& io,
                         double alpha, const Launch& L) {
   FusedGeom G;
@@ -374,9 +388,14 @@ void launch_stage_fused(int mode, const Grid& g, const les_params& p, const Fuse
   // PM = 12 with that staging alone, PM = 4 for the other row lengths.
   // Other grids read them at run time (PM = -1).
   const bool jet = !g.per[0] && !g.per[1] && g.per[2];
-  const bool full = g.n[1] % FTJ == 0 && g.n[2] % FTK == 0;
+  const bool full = g.n[1] % 16 == 0 && g.n[2] % FTK == 0;
   const int pm = !jet ? -1 : (!G.vec16 ? 4 : (full ? 28 : 12));
-  if (pm == 28)
+  const bool small = jet && tile_rows(G) == 8;
+  if (small && G.vec16)
+    launch_stage_jet12s(mode, local, p.axis != 0, dyn, G, K, P, io.sc, alpha, L);
+  else if (small)
+    launch_stage_jet4s(mode, local, p.axis != 0, dyn, G, K, P, io.sc, alpha, L);
+  else if (pm == 28)
     launch_stage_jet28(mode, local, p.axis != 0, dyn, G, K, P, io.sc, alpha, L);
   else if (pm == 12)
     launch_stage_jet12(mode, local, p.axis != 0, dyn, G, K, P, io.sc, alpha, L);

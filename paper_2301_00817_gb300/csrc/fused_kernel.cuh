@@ -2,7 +2,7 @@
 // fused), its helpers and launch templates; fused.cu holds the launchers,
 // fused_jet4.cu, fused_jet12.cu and fused_jet28.cu the jet-grid instantiations.
 //
-// A CTA owns a TJ x TK = 16 x 32 tile of (eta, zeta) columns and marches along
+// A CTA owns a 16 x 32 (small grids: 8 x 32) tile of (eta, zeta) columns and marches along
 // xi over a chunk of axial planes.  Per plane it stages the conserved state
 // of the tile plus a two-node halo in shared memory with cp.async (one plane
 // ahead), derives the primitives and the anisotropic spectral radii once per
@@ -429,8 +429,10 @@ __global__ void __launch_bounds__(256) k_prestep(Grid g, Consts<R> K, const TQ* 
 // ------------------------------------------------------------ fused stage
 enum { FMODE_RHS = 0, FMODE_STAGE = 1, FMODE_LAST = 2 };
 
-// Tile of FTJ x FTK (eta, zeta) columns, one thread per column.
-constexpr int FTJ = 16, FTK = 32, FNT = FTJ * FTK;
+// Tile of TJ x FTK (eta, zeta) columns, one thread per column: TJ = 16, or 8
+// on grids with so few planes and columns that most of a stage is latency
+// (tile_rows).
+constexpr int FTK = 32;
 // Shared-memory rows hold the tile's FTK columns and a two-column halo on
 // each side: tile column kk in [-2, FTK+1] lives at row column kk + 2.  When
 // zeta is periodic and nk % 4 == 0 the tiles are shifted by two columns
@@ -438,8 +440,6 @@ constexpr int FTJ = 16, FTK = 32, FNT = FTJ * FTK;
 // whole row, halos included, is the 16-byte-aligned global range
 // [32 t, 32 t + 36): nine 16-byte copies and no separate halo copy.
 constexpr int SK = FTK + 4;
-constexpr int R2 = FTJ + 4, R1 = FTJ + 2;  // rows with a 2-node / 1-node halo
-constexpr int PL2 = R2 * SK, PL1 = R1 * SK;
 __host__ __device__ constexpr int colk(int kk) { return kk + 2; }
 
 // Shared-memory plan (floats):
@@ -449,22 +449,24 @@ __host__ __device__ constexpr int colk(int kk) { return kk + 2; }
 //   sM[3][10][PL1] metrics of planes i, i+1, i+2 (1-node halo)
 //   sK[3][2][PL1]  mu_eff kappa_eff of planes i, i+1, i+2
 //   sL[2][3][PL1]  lbar of planes i, i+1
-//   sFe[5][FTJ+1][FTK]  eta interface fluxes (rows -1 .. FTJ-1 of the tile)
-//   sFz[5][FTJ]         the tile's left-edge zeta interface fluxes (the
+//   sFe[5][TJ+1][FTK]   eta interface fluxes (rows -1 .. TJ-1 of the tile)
+//   sFz[5][TJ]          the tile's left-edge zeta interface fluxes (the
 //                       others pass between neighbouring lanes by shuffle)
-constexpr int OFF_PR = 3 * 5 * PL2, OFF_PW = OFF_PR + 3 * 4 * PL2,
-              OFF_M = OFF_PW + 3 * 2 * PL2, OFF_K = OFF_M + 3 * 10 * PL1;
 // With the dynamic SGS model the viscosity slots hold a third field, the
 // Yoshizawa sigma_ll (sK[3][3][PL1]); the regions after sK move up.
-template <bool DYN>
+template <int TJ, bool DYN>
 struct FLayout {
+  static constexpr int R2 = TJ + 4, R1 = TJ + 2;  // rows with a 2-node / 1-node halo
+  static constexpr int PL2 = R2 * SK, PL1 = R1 * SK;
+  static constexpr int PR = 3 * 5 * PL2, PW = PR + 3 * 4 * PL2, M = PW + 3 * 2 * PL2;
+  static constexpr int K = M + 3 * 10 * PL1;
   static constexpr int NKF = DYN ? 3 : 2;  // fields per viscosity slot
-  static constexpr int L = OFF_K + 3 * NKF * PL1;
+  static constexpr int L = K + 3 * NKF * PL1;
   static constexpr int FE = L + 2 * 3 * PL1;
-  static constexpr int FZ = FE + 5 * (FTJ + 1) * FTK;
-  static constexpr int FLOATS = FZ + 5 * FTJ;
+  static constexpr int FZ = FE + 5 * (TJ + 1) * FTK;
+  static constexpr int FLOATS = FZ + 5 * TJ;
 };
-static_assert(FLayout<true>::FLOATS * 4 <= 227 * 1024, "shared memory plan exceeds 227 KB");
+static_assert(FLayout<16, true>::FLOATS * 4 <= 227 * 1024, "shared memory plan exceeds 227 KB");
 
 // Differences of (u, v, w, T) at an interface from node records (float4 u, v,
 // w, T): along the interface normal, phi_b - phi_a; along a tangent t, four
@@ -536,20 +538,22 @@ __device__ __forceinline__ int wrap_fast(int v, int n, int per) {
 // one-sided-difference tests fold away: bits 0-2, direction d periodic;
 // bit 3, the shifted 16-byte staging (G.vec16); bit 4, tiles that cover eta
 // and zeta exactly (every thread owns a column).  PM = -1 reads them from G.
-template <int MODE, bool LOCAL, bool AXIS, bool DYN, int PM>
-__global__ void __launch_bounds__(FNT, 1)
+template <int MODE, bool LOCAL, bool AXIS, bool DYN, int PM, int FTJ>
+__global__ void __launch_bounds__(FTJ * FTK, 1)
     k_stage_fused(const FusedGeom G, const Consts<float> K, const FusedPtrs P,
                   const DevScalars* __restrict__ sc, double alpha) {
   extern __shared__ __align__(16) float smem[];
+  using Y = FLayout<FTJ, DYN>;
+  constexpr int FNT = FTJ * FTK, R2 = Y::R2, R1 = Y::R1, PL2 = Y::PL2, PL1 = Y::PL1;
   float* sQ = smem;
-  float4* sPr = reinterpret_cast<float4*>(smem + OFF_PR);
-  float2* sPw = reinterpret_cast<float2*>(smem + OFF_PW);
-  float* sM = smem + OFF_M;
-  float* sK = smem + OFF_K;
-  constexpr int NKF = FLayout<DYN>::NKF;
-  float* sL = smem + FLayout<DYN>::L;
-  float* sFe = smem + FLayout<DYN>::FE;
-  float* sFz = smem + FLayout<DYN>::FZ;
+  float4* sPr = reinterpret_cast<float4*>(smem + Y::PR);
+  float2* sPw = reinterpret_cast<float2*>(smem + Y::PW);
+  float* sM = smem + Y::M;
+  float* sK = smem + Y::K;
+  constexpr int NKF = Y::NKF;
+  float* sL = smem + Y::L;
+  float* sFe = smem + Y::FE;
+  float* sFz = smem + Y::FZ;
   const int ni = G.ni, nj = G.nj, nk = G.nk;
   // periodicity of xi, eta, zeta: fixed at compile time for PM >= 0 (bit d:
   // direction d periodic), else the grid's flags
@@ -1201,6 +1205,7 @@ static Consts<R> fused_consts(const les_params& p) {
 // SMs, simulated once per grid shape and cached.
 struct Chunks {
   int nch, n1, a1;
+  double t;  // the schedule's finishing time, in planes
 };
 
 static double chunk_schedule(int ni, int n1, int a1, int n2, int tiles, int slots, double pro) {
@@ -1241,17 +1246,19 @@ static Chunks choose_chunks(int ni, int tiles, int slots) {
   }
   const double pro = 1.5;
   const long long cap = 24LL * slots;  // at most 24 waves of CTAs
-  Chunks best{1, 0, 0};
+  Chunks best{1, 0, 0, 0.0};
   double best_t = 1e300;
   auto consider = [&](int n1, int a1, int n2) {
     const double t = chunk_schedule(ni, n1, a1, n2, tiles, slots, pro);
     if (t < best_t - 1e-9) {
       best_t = t;
-      best = Chunks{n1 + n2, n1, a1};
+      best = Chunks{n1 + n2, n1, a1, t};
     }
   };
   const int max_nch = ni < 64 ? ni : 64;
-  for (int n2 = 1; n2 <= max_nch; ++n2) {
+  // equal chunks: up to one plane each while that leaves a CTA per SM
+  const int max_eq = ni < 64 ? ni : (slots / tiles > 64 ? (slots / tiles < ni ? slots / tiles : ni) : 64);
+  for (int n2 = 1; n2 <= max_eq; ++n2) {
     if (n2 > 1 && (long long)tiles * n2 > cap) break;
     consider(0, 0, n2);
   }
@@ -1280,11 +1287,11 @@ static Chunks choose_chunks(int ni, int tiles, int slots) {
   return best;
 }
 
-template <int MODE, bool LOCAL, bool AXIS, bool DYN, int PM>
+template <int MODE, bool LOCAL, bool AXIS, bool DYN, int PM, int TJ>
 static void launch_stage_t(const FusedGeom& G0, const Consts<float>& K, const FusedPtrs& P,
                            const DevScalars* sc, double alpha, const Launch& L) {
   FusedGeom G = G0;
-  const size_t smem = (size_t)FLayout<DYN>::FLOATS * sizeof(float);
+  const size_t smem = (size_t)FLayout<TJ, DYN>::FLOATS * sizeof(float);
   // the shared-memory opt-in is a per-device function attribute: set it once
   // for each device this process launches on
   static std::atomic<unsigned long long> attr_set{0};
@@ -1292,38 +1299,45 @@ static void launch_stage_t(const FusedGeom& G0, const Consts<float>& K, const Fu
   cudaGetDevice(&dev);
   const unsigned long long bit = 1ull << (dev & 63);
   if (!(attr_set.load(std::memory_order_acquire) & bit)) {
-    cudaFuncSetAttribute(k_stage_fused<MODE, LOCAL, AXIS, DYN, PM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)smem);
+    cudaFuncSetAttribute(k_stage_fused<MODE, LOCAL, AXIS, DYN, PM, TJ>,
+                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     attr_set.fetch_or(bit, std::memory_order_acq_rel);
   }
-  const int tk = (G.nk + FTK - 1) / FTK, tj = (G.nj + FTJ - 1) / FTJ;
+  const int tk = (G.nk + FTK - 1) / FTK, tj = (G.nj + TJ - 1) / TJ;
   const Chunks ch = choose_chunks(G.ni, tk * tj, sm_count());  // one CTA per SM
   G.nch = ch.nch;
   G.n1 = ch.n1;
   G.a1 = ch.a1;
   dim3 grid(tk, tj, G.nch);
-  k_stage_fused<MODE, LOCAL, AXIS, DYN, PM><<<grid, FNT, smem, L.s>>>(G, K, P, sc, alpha);
+  k_stage_fused<MODE, LOCAL, AXIS, DYN, PM, TJ><<<grid, TJ * FTK, smem, L.s>>>(G, K, P, sc, alpha);
   ++*L.counter;
 }
 
-template <bool AXIS, bool DYN, int PM>
+template <bool AXIS, bool DYN, int PM, int TJ = 16>
 static void launch_stage_dispatch(int mode, bool local, const FusedGeom& G, const Consts<float>& K,
                                   const FusedPtrs& P, const DevScalars* sc, double alpha,
                                   const Launch& L) {
   if (mode == FMODE_RHS)
-    launch_stage_t<FMODE_RHS, false, AXIS, DYN, PM>(G, K, P, sc, alpha, L);
+    launch_stage_t<FMODE_RHS, false, AXIS, DYN, PM, TJ>(G, K, P, sc, alpha, L);
   else if (mode == FMODE_STAGE && !local)
-    launch_stage_t<FMODE_STAGE, false, AXIS, DYN, PM>(G, K, P, sc, alpha, L);
+    launch_stage_t<FMODE_STAGE, false, AXIS, DYN, PM, TJ>(G, K, P, sc, alpha, L);
   else if (mode == FMODE_STAGE)
-    launch_stage_t<FMODE_STAGE, true, AXIS, DYN, PM>(G, K, P, sc, alpha, L);
+    launch_stage_t<FMODE_STAGE, true, AXIS, DYN, PM, TJ>(G, K, P, sc, alpha, L);
   else if (!local)
-    launch_stage_t<FMODE_LAST, false, AXIS, DYN, PM>(G, K, P, sc, alpha, L);
+    launch_stage_t<FMODE_LAST, false, AXIS, DYN, PM, TJ>(G, K, P, sc, alpha, L);
   else
-    launch_stage_t<FMODE_LAST, true, AXIS, DYN, PM>(G, K, P, sc, alpha, L);
+    launch_stage_t<FMODE_LAST, true, AXIS, DYN, PM, TJ>(G, K, P, sc, alpha, L);
 }
 
-// The jet-grid instantiations (PM = 4, 12 and 28), each compiled in a
-// translation unit of its own so the build compiles them in parallel.
+// The jet-grid instantiations (PM = 4, 12 and 28; PM = 4 and 12 also with
+// tiles of 8 rows), each compiled in a translation unit of its own so the
+// build compiles them in parallel.
+void launch_stage_jet4s(int mode, bool local, bool axis, bool dyn, const FusedGeom& G,
+                        const Consts<float>& K, const FusedPtrs& P, const DevScalars* sc,
+                        double alpha, const Launch& L);
+void launch_stage_jet12s(int mode, bool local, bool axis, bool dyn, const FusedGeom& G,
+                         const Consts<float>& K, const FusedPtrs& P, const DevScalars* sc,
+                         double alpha, const Launch& L);
 void launch_stage_jet4(int mode, bool local, bool axis, bool dyn, const FusedGeom& G,
                        const Consts<float>& K, const FusedPtrs& P, const DevScalars* sc,
                        double alpha, const Launch& L);
