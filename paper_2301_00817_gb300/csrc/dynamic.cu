@@ -23,6 +23,8 @@
 // dynamic kappa_sgs and the Yoshizawa sigma_ll = 2 C_I rho Delta^2 |S|^2.
 // Test filter: the (1/4, 1/2, 1/4) trapezoidal filter along each direction
 // (width 2 Delta), identity along a non-periodic direction at its faces.
+#include <type_traits>
+
 #include "stage64_kernels.cuh"
 
 namespace lesjet {
@@ -32,18 +34,58 @@ namespace {
 constexpr int kDynFields = 25;
 constexpr int kDynSums = 7;  // six weighted sums and the sum of the weights
 
-// Cartesian gradient of a node field through the node's metrics.
-template <typename R, typename TM>
-__device__ __forceinline__ void grad_of(const Grid& g, const TM* __restrict__ M,
-                                        const R* __restrict__ f, long long n, const int c[3],
-                                        R out[3]) {
-  const long long N = g.N;
+// The neighbours that a node's central differences read, found once per node
+// for all fields (mode 0; at an open face the two of the one-sided
+// difference: mode 1 at the low face, n + s and n + 2 s, mode 2 at the high
+// one, n - 2 s and n - s).
+// (The mixed forms' fields, FP32, have fewer than 2^31 points.)
+template <typename R>
+struct Stencil {
+  using I = typename std::conditional<sizeof(R) == 4, int, long long>::type;
+  I p[3], m[3];
+  int mode[3];
+};
+
+template <typename R>
+__device__ __forceinline__ Stencil<R> stencil_of(const Grid& g, long long node, const int c[3]) {
+  using I = typename Stencil<R>::I;
+  Stencil<R> t;
+  const I n = (I)node;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    const I s = (I)g.stride[d];
+    const int last = g.n[d] - 1;
+    t.mode[d] = 0;
+    t.p[d] = c[d] == last ? n - last * s : n + s;
+    t.m[d] = c[d] == 0 ? n + last * s : n - s;
+    if (!g.per[d] && c[d] == 0) {
+      t.m[d] = n + 2 * s;
+      t.mode[d] = 1;
+    } else if (!g.per[d] && c[d] == last) {
+      t.p[d] = n - 2 * s;
+      t.mode[d] = 2;
+    }
+  }
+  return t;
+}
+
+// Cartesian gradient of a node field; mh: half the node's metrics (the
+// differences are twice the derivatives).  INTERIOR: mode 0 in every direction.
+template <bool INTERIOR, typename R>
+__device__ __forceinline__ void grad_of(const R* __restrict__ f, long long n, const Stencil<R>& t,
+                                        const R mh[9], R out[3]) {
   R dd[3];
 #pragma unroll
-  for (int d = 0; d < 3; ++d) dd[d] = node_deriv(g, f, n, c, d);
+  for (int d = 0; d < 3; ++d) {
+    const R fp = f[t.p[d]], fm = f[t.m[d]];
+    dd[d] = fp - fm;
+    if (!INTERIOR) {
+      if (t.mode[d] == 1) dd[d] = R(-3) * f[n] + R(4) * fp - fm;
+      if (t.mode[d] == 2) dd[d] = R(3) * f[n] - R(4) * fm + fp;
+    }
+  }
 #pragma unroll
-  for (int x = 0; x < 3; ++x)
-    out[x] = (R)M[x * N + n] * dd[0] + (R)M[(3 + x) * N + n] * dd[1] + (R)M[(6 + x) * N + n] * dd[2];
+  for (int x = 0; x < 3; ++x) out[x] = mh[x] * dd[0] + mh[3 + x] * dd[1] + mh[6 + x] * dd[2];
 }
 
 // S_ij from a velocity gradient gr[i][x] = d u_i/d x_x; returns |S|.
@@ -60,8 +102,28 @@ __device__ __forceinline__ R strain(const R gr[3][3], R S[3][3]) {
   return dev_sqrt(R(2) * ss);
 }
 
-__constant__ int kI6[6] = {0, 1, 2, 0, 0, 1};
-__constant__ int kJ6[6] = {0, 1, 2, 1, 2, 2};
+// Component k of a symmetric tensor: (0,0) (1,1) (2,2) (0,1) (0,2) (1,2).
+// (Functions, so that the unrolled loops index registers: a table in constant
+// memory had put the tensors into local memory.)
+__device__ constexpr int i6(int k) { return k < 3 ? k : (k == 5 ? 1 : 0); }
+__device__ constexpr int j6(int k) { return k < 3 ? k : (k == 3 ? 1 : 2); }
+
+// u, v, w, T of the mixed forms' float state (node fields 0, 1, 2 and 4; the
+// procedure reads no other).
+__global__ void __launch_bounds__(256) k_dyn_node(long long N, float gamma, float gm1,
+                                                  const float* __restrict__ Q,
+                                                  float* __restrict__ node) {
+  for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N;
+       n += (long long)gridDim.x * blockDim.x) {
+    const float rho = Q[n], ir = 1.f / rho;
+    const float u = Q[N + n] * ir, v = Q[2 * N + n] * ir, w = Q[3 * N + n] * ir;
+    const float p = gm1 * (Q[4 * N + n] - 0.5f * rho * (u * u + v * v + w * w));
+    node[n] = u;
+    node[N + n] = v;
+    node[2 * N + n] = w;
+    node[4 * N + n] = gamma * p * ir;
+  }
+}
 
 // Register bounds (here and on k_dyn_sums): left free, the compiler gave
 // these kernels 230-254 registers, one 256-thread block per SM for a
@@ -79,10 +141,13 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_dyn_products(Gr
     const R rho = (R)Q[n];
     const R vel[3] = {node[n], node[N + n], node[2 * N + n]};
     const R T = node[4 * N + n];
-    R gr[3][3], S[3][3], dT[3];
+    const Stencil<R> st = stencil_of<R>(g, n, c);
+    R mh[9], gr[3][3], S[3][3], dT[3];
 #pragma unroll
-    for (int q = 0; q < 3; ++q) grad_of(g, M, node + q * N, n, c, gr[q]);
-    grad_of(g, M, node + 4 * N, n, c, dT);
+    for (int t = 0; t < 9; ++t) mh[t] = R(0.5) * (R)M[t * N + n];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) grad_of<false>(node + q * N, n, st, mh, gr[q]);
+    grad_of<false>(node + 4 * N, n, st, mh, dT);
     const R Sm = strain(gr, S);
     D[n] = rho;
 #pragma unroll
@@ -90,7 +155,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_dyn_products(Gr
     D[4 * N + n] = rho * T;
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
-      const int i = kI6[k], j = kJ6[k];
+      const int i = i6(k), j = j6(k);
       D[(5 + k) * N + n] = rho * vel[i] * vel[j];
       D[(11 + k) * N + n] = rho * Sm * S[i][j];
     }
@@ -130,89 +195,85 @@ __global__ void __launch_bounds__(256) k_dyn_filter1(Grid g, const R* __restrict
   }
 }
 
-// The test filter's three directions in one kernel.  A CTA owns a tile of
-// kF3J x kF3K (eta, zeta) columns and a range of planes [i0, i1), and takes
-// the fields NB at a time.  For each group it marches along xi over planes
-// i0 - 1 .. i1: it stages the plane's tile with a one-node halo in shared
-// memory, filters along zeta over the halo rows, then along eta, and keeps
-// the last three of its column's 2-D-filtered values in registers to
+// The test filter's three directions in one kernel (blockIdx.z: field, then
+// axial chunk).  A thread owns kF3R rows of one column and marches along xi
+// over planes i0 - 1 .. i1: it reads the plane's kF3R + 2 rows at its column
+// and the two beside it (the next plane's while it works on this one), filters
+// along zeta, then eta, and keeps the last two planes' values in registers to
 // filter along xi.  Each output takes the same operations in the same order
-// as three one-direction passes would (zeta, eta, xi; identity at the faces
-// of a non-periodic direction).  Traffic: each field read once (with the
-// tile and chunk halos) and written once, against three reads and three
-// writes for separate passes; the NB fields of a group share the barriers
-// and keep several loads in flight per thread (one field at a time was
-// latency-bound: 40% slower than three passes).
-constexpr int kF3J = 8, kF3K = 32;  // tile rows (eta) x columns (zeta); 256 threads
+// as three one-direction passes would (zeta, eta, xi; identity at the faces of
+// a non-periodic direction).  Bound by the latency of those loads, most of
+// them L1 hits, so it is shaped for many resident threads: one field per
+// block, about 40 registers, no shared memory and no barriers.
+constexpr int kF3J = 4, kF3K = 32, kF3R = 2;  // 128 threads: 8 rows x 32 columns
 
-template <typename R, int NB>
+template <typename R>
 __global__ void __launch_bounds__(kF3J * kF3K) k_dyn_filter3(Grid g, const R* __restrict__ src,
-                                                             int count, int nch,
-                                                             R* __restrict__ dst) {
-  __shared__ R S[NB][kF3J + 2][kF3K + 2];  // the plane's tile with a one-node halo
-  __shared__ R Z[NB][kF3J + 2][kF3K];      // filtered along zeta, rows -1 .. kF3J
+                                                             int fields, R* __restrict__ dst) {
   const long long N = g.N;
   const int ni = g.n[0], nj = g.n[1], nk = g.n[2];
   const int tx = threadIdx.x % kF3K, ty = threadIdx.x / kF3K;
-  const int k0 = blockIdx.x * kF3K, j0 = blockIdx.y * kF3J;
-  const int i0 = (int)((long long)blockIdx.z * ni / nch);
-  const int i1 = (int)((long long)(blockIdx.z + 1) * ni / nch);
-  const int j = j0 + ty, k = k0 + tx;
-  const bool own = j < nj && k < nk;
-  auto wrap = [](int v, int n, int per) {  // -1 outside a non-periodic range
-    if (per) return ((v % n) + n) % n;     // (a tile may span several periods)
-    return (v >= 0 && v < n) ? v : -1;
+  const int k = blockIdx.x * kF3K + tx, j0 = (blockIdx.y * kF3J + ty) * kF3R;
+  const int f = blockIdx.z % fields, ch = blockIdx.z / fields, nch = gridDim.z / fields;
+  const int i0 = (int)((long long)ch * ni / nch), i1 = (int)((long long)(ch + 1) * ni / nch);
+  if (k >= nk || j0 >= nj) return;
+  src += (long long)f * N;
+  dst += (long long)f * N;
+  // a missing neighbour (an open face's) is the node itself, and not used
+  const bool kface = !g.per[2] && (k == 0 || k == nk - 1);
+  const int km = kface ? k : (k == 0 ? nk - 1 : k - 1), kp = kface ? k : (k == nk - 1 ? 0 : k + 1);
+  int row[kF3R + 2];  // offsets of rows j0 - 1 .. j0 + kF3R within a plane
+  bool jface[kF3R];
+#pragma unroll
+  for (int q = 0; q < kF3R + 2; ++q) {
+    int j = j0 - 1 + q;
+    if (j < 0) j = g.per[1] ? nj - 1 : 0;
+    if (j >= nj) j = g.per[1] ? j % nj : nj - 1;
+    row[q] = j * nk;
+  }
+#pragma unroll
+  for (int q = 0; q < kF3R; ++q) jface[q] = !g.per[1] && (j0 + q == 0 || j0 + q == nj - 1);
+  R s[kF3R + 2][3];  // the raw values of the plane to come
+  auto fetch = [&](int x) {
+    const int ig = (x >= 0 && x < ni) ? x : (g.per[0] ? (x < 0 ? ni - 1 : 0) : -1);
+    if (ig < 0) return;  // outside an open xi: read by no output
+    const R* S = src + (long long)ig * g.stride[0];
+#pragma unroll
+    for (int q = 0; q < kF3R + 2; ++q) {
+      s[q][0] = S[row[q] + km];
+      s[q][1] = S[row[q] + k];
+      s[q][2] = S[row[q] + kp];
+    }
   };
-  const bool jface = !g.per[1] && (j == 0 || j == nj - 1);
-  for (int f0 = 0; f0 < count; f0 += NB) {  // NB fields at a time (count % NB == 0)
-    R em[NB], ec[NB];  // 2-D-filtered values of planes x - 2, x - 1
 #pragma unroll
-    for (int b = 0; b < NB; ++b) em[b] = ec[b] = R(0);
-    for (int x = i0 - 1; x <= i1; ++x) {
-      const int ig = wrap(x, ni, g.per[0]);
-      R e[NB];
+  for (int q = 0; q < kF3R + 2; ++q) s[q][0] = s[q][1] = s[q][2] = R(0);
+  fetch(i0 - 1);
+  R em[kF3R], ec[kF3R];  // 2-D-filtered values of planes x - 2, x - 1
 #pragma unroll
-      for (int b = 0; b < NB; ++b) e[b] = R(0);
-      if (ig >= 0) {  // (uniform over the CTA)
-        const long long pbase = (long long)ig * nj * nk;
-        for (int q = threadIdx.x; q < (kF3J + 2) * (kF3K + 2); q += blockDim.x) {
-          const int r = q / (kF3K + 2), c = q - r * (kF3K + 2);
-          const int jg = wrap(j0 - 1 + r, nj, g.per[1]), kg = wrap(k0 - 1 + c, nk, g.per[2]);
-          const bool in = jg >= 0 && kg >= 0;
-          const long long off = pbase + (long long)jg * nk + kg;
+  for (int q = 0; q < kF3R; ++q) em[q] = ec[q] = R(0);
+  for (int x = i0 - 1; x <= i1; ++x) {
+    R z[kF3R + 2], e[kF3R];
 #pragma unroll
-          for (int b = 0; b < NB; ++b) S[b][r][c] = in ? src[(long long)(f0 + b) * N + off] : R(0);
-        }
-        __syncthreads();
-        for (int q = threadIdx.x; q < (kF3J + 2) * kF3K; q += blockDim.x) {
-          const int r = q / kF3K, c = q - r * kF3K;
-          const int kk = k0 + c;
-          const bool face = !g.per[2] && (kk == 0 || kk == nk - 1);
+    for (int q = 0; q < kF3R + 2; ++q)
+      z[q] = kface ? s[q][1] : R(0.25) * s[q][0] + R(0.5) * s[q][1] + R(0.25) * s[q][2];
+    if (x < i1) fetch(x + 1);
 #pragma unroll
-          for (int b = 0; b < NB; ++b)
-            Z[b][r][c] = face ? S[b][r][c + 1]
-                              : R(0.25) * S[b][r][c] + R(0.5) * S[b][r][c + 1] + R(0.25) * S[b][r][c + 2];
-        }
-        __syncthreads();
+    for (int q = 0; q < kF3R; ++q)
+      e[q] = jface[q] ? z[q + 1] : R(0.25) * z[q] + R(0.5) * z[q + 1] + R(0.25) * z[q + 2];
+    // plane x - 1 has both xi neighbours now
+    const int xo = x - 1;
+    if (xo >= i0) {
+      const bool face = !g.per[0] && (xo == 0 || xo == ni - 1);
+      const long long o = (long long)xo * g.stride[0] + (long long)j0 * nk + k;
 #pragma unroll
-        for (int b = 0; b < NB; ++b)
-          e[b] = jface ? Z[b][ty + 1][tx]
-                       : R(0.25) * Z[b][ty][tx] + R(0.5) * Z[b][ty + 1][tx] + R(0.25) * Z[b][ty + 2][tx];
-      }
-      // plane x - 1 has both xi neighbours now
-      const int xo = x - 1;
-      if (xo >= i0 && xo < i1 && own) {
-        const bool face = !g.per[0] && (xo == 0 || xo == ni - 1);
-        const long long o = (long long)xo * nj * nk + (long long)j * nk + k;
+      for (int q = 0; q < kF3R; ++q)
+        if (j0 + q < nj)
+          dst[o + q * nk] = face ? ec[q] : R(0.25) * em[q] + R(0.5) * ec[q] + R(0.25) * e[q];
+    }
 #pragma unroll
-        for (int b = 0; b < NB; ++b)
-          dst[(long long)(f0 + b) * N + o] = face ? ec[b] : R(0.25) * em[b] + R(0.5) * ec[b] + R(0.25) * e[b];
-      }
-#pragma unroll
-      for (int b = 0; b < NB; ++b) {
-        em[b] = ec[b];
-        ec[b] = e[b];
-      }
+    for (int q = 0; q < kF3R; ++q) {
+      em[q] = ec[q];
+      ec[q] = e[q];
     }
   }
 }
@@ -224,9 +285,9 @@ __global__ void __launch_bounds__(256) k_dyn_favre(long long N, const R* __restr
                                                    R* __restrict__ H) {
   for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N;
        n += (long long)gridDim.x * blockDim.x) {
-    const R r = F[n];
+    const R ir = R(1) / F[n];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) H[q * N + n] = F[(1 + q) * N + n] / r;
+    for (int q = 0; q < 4; ++q) H[q * N + n] = F[(1 + q) * N + n] * ir;
   }
 }
 
@@ -245,29 +306,32 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 1) k_dyn_sums(Grid g
     int c[3];
     decompose(g, n, c);
     if (!is_interior(g, c)) continue;
-    const double wgt = (double)M[9 * N + n];
+    const double wgt = widen(M[9 * N + n]);
     const R Delta = cbrt((R)M[9 * N + n]);
     const R D2 = Delta * Delta, Dh2 = R(4) * D2;
-    R gr[3][3], S[3][3], dT[3], grh[3][3], Sh[3][3], dTh[3];
+    const Stencil<R> st = stencil_of<R>(g, n, c);
+    R mm[9], gr[3][3], S[3][3], dT[3], grh[3][3], Sh[3][3], dTh[3];
 #pragma unroll
-    for (int q = 0; q < 3; ++q) grad_of(g, M, node + q * N, n, c, gr[q]);
-    grad_of(g, M, node + 4 * N, n, c, dT);
+    for (int t = 0; t < 9; ++t) mm[t] = R(0.5) * (R)M[t * N + n];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) grad_of<true>(node + q * N, n, st, mm, gr[q]);
+    grad_of<true>(node + 4 * N, n, st, mm, dT);
     strain(gr, S);
 #pragma unroll
-    for (int q = 0; q < 3; ++q) grad_of(g, M, H + q * N, n, c, grh[q]);
-    grad_of(g, M, H + 3 * N, n, c, dTh);
+    for (int q = 0; q < 3; ++q) grad_of<true>(H + q * N, n, st, mm, grh[q]);
+    grad_of<true>(H + 3 * N, n, st, mm, dTh);
     const R Shm = strain(grh, Sh);
     // the filtered fields at this node (Fh holds all 25)
     R fh[kDynFields];
 #pragma unroll
     for (int q = 5; q < kDynFields; ++q) fh[q] = Fh[q * N + n];
-    const R rh = Fh[n];
+    const R rh = Fh[n], irh = R(1) / rh;  // one division per node
     const R mh[3] = {Fh[N + n], Fh[2 * N + n], Fh[3 * N + n]};
     R L[3][3], Fs[3][3];
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
-      const int i = kI6[k], j = kJ6[k];
-      L[i][j] = L[j][i] = fh[5 + k] - mh[i] * mh[j] / rh;
+      const int i = i6(k), j = j6(k);
+      L[i][j] = L[j][i] = fh[5 + k] - mh[i] * mh[j] * irh;
       Fs[i][j] = Fs[j][i] = fh[11 + k];
     }
     const R trS = S[0][0] + S[1][1] + S[2][2];
@@ -282,23 +346,24 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 1) k_dyn_sums(Grid g
         ShS += Sh[i][j] * S[i][j];
       }
     const R Lkk = L[0][0] + L[1][1] + L[2][2];
-    const R numC = LS - Lkk * trS / R(3);
-    const R denC = R(2) * D2 * (FS - fh[17] * trS / R(3)) -
-                   R(2) * Dh2 * (rh * Shm * ShS - rh * Shm * trSh * trS / R(3));
+    const R tr3 = trS * R(1.0 / 3.0);
+    const R numC = LS - Lkk * tr3;
+    const R denC = R(2) * D2 * (FS - fh[17] * tr3) -
+                   R(2) * Dh2 * (rh * Shm * ShS - rh * Shm * trSh * tr3);
     const R denI = R(2) * Dh2 * rh * Shm * Shm - R(2) * D2 * fh[18];
     R numP = R(0), denP = R(0);
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
-      const R K = fh[19 + j] - mh[j] * Fh[4 * N + n] / rh;
+      const R K = fh[19 + j] - mh[j] * Fh[4 * N + n] * irh;
       numP += D2 * fh[22 + j] * dT[j] - Dh2 * rh * Shm * dTh[j] * dT[j];
       denP += K * dT[j];
     }
-    acc[0] += wgt * (double)numC;
-    acc[1] += wgt * (double)denC;
-    acc[2] += wgt * (double)Lkk;
-    acc[3] += wgt * (double)denI;
-    acc[4] += wgt * (double)numP;
-    acc[5] += wgt * (double)denP;
+    acc[0] += wgt * widen(numC);
+    acc[1] += wgt * widen(denC);
+    acc[2] += wgt * widen(Lkk);
+    acc[3] += wgt * widen(denI);
+    acc[4] += wgt * widen(numP);
+    acc[5] += wgt * widen(denP);
     acc[6] += wgt;
   }
   __shared__ double red[kDynSums][32];
@@ -326,6 +391,7 @@ __global__ void k_dyn_final(const double* __restrict__ partials, double pr_defau
   const int q = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (q < kDynSums) {
     double v = 0.0;
+#pragma unroll 19
     for (int b = lane; b < kRedBlocks; b += 32) v += partials[q * kRedBlocks + b];
     for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
     if (lane == 0) tot[q] = v;
@@ -357,13 +423,16 @@ static void dynamic_t(const Grid& g, const les_params& p, const TQ* Q, const TM*
   k_dyn_products<R, TQ, TM><<<nb, th, 0, L.s>>>(g, Q, M, node, D);
   if constexpr (sizeof(R) == 4) {
     // FP32 fields: the test filter in one pass (k_dyn_filter3), with enough
-    // axial chunks for about eight CTAs per SM
-    const int tk = (g.n[2] + kF3K - 1) / kF3K, tj = (g.n[1] + kF3J - 1) / kF3J;
-    const long long want = 8LL * sm_count();
-    int nch = (int)((want + (long long)tk * tj - 1) / ((long long)tk * tj));
-    nch = nch < 1 ? 1 : (nch > g.n[0] ? g.n[0] : nch);
-    static_assert(kDynFields % 5 == 0, "the filter takes the fields five at a time");
-    k_dyn_filter3<R, 5><<<dim3(tk, tj, nch), kF3J * kF3K, 0, L.s>>>(g, D, kDynFields, nch, T);
+    // axial chunks for some sixty CTAs per SM (each reads two planes more
+    // than it writes)
+    const long long tk = (g.n[2] + kF3K - 1) / kF3K,
+                    tj = (g.n[1] + kF3J * kF3R - 1) / (kF3J * kF3R), tiles = tk * tj * kDynFields;
+    const long long want = 64LL * sm_count();
+    const long long most = g.n[0] / 12 > 1 ? g.n[0] / 12 : 1;
+    long long nch = (want + tiles - 1) / tiles;
+    nch = nch < 1 ? 1 : (nch > most ? most : nch);
+    k_dyn_filter3<R><<<dim3((unsigned)tk, (unsigned)tj, (unsigned)(nch * kDynFields)), kF3J * kF3K, 0,
+                       L.s>>>(g, D, kDynFields, T);
     *L.counter += 1;
   } else {
     // FP64 fields: three one-direction passes (the one-pass kernel is bound
@@ -387,10 +456,8 @@ void launch_dynamic64(const Grid& g, const les_params& p, const StageIO64& io, d
 void launch_dynamic32(const Grid& g, const les_params& p, const float* Q, const float* M,
                       float* node, float* scratch, double* partials, DevScalars* sc,
                       const Launch& L) {
-  // the FP32 node fields (u v w p T; the radii are not used) of the float state
   const int th = 256, nb = blocks_for(g.N, th);
-  k_node<float, float, float, false><<<nb, th, 0, L.s>>>(g, make_consts<float>(p), Q, M, nullptr, node,
-                                                        partials, sc);
+  k_dyn_node<<<nb, th, 0, L.s>>>(g.N, (float)p.gamma, (float)(p.gamma - 1.0), Q, node);
   ++*L.counter;
   dynamic_t<float, float, float>(g, p, Q, M, node, scratch, partials, sc, L);
 }

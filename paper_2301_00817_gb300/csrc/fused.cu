@@ -42,15 +42,6 @@ __device__ __forceinline__ void split_value(double v, float& h, float& l) {
   }
 }
 
-// (double)x on the integer pipe (exact; zeros, denormals, infinities and NaN
-// take the conversion).
-__device__ __forceinline__ double widen(float x) {
-  const unsigned b = __float_as_uint(x), mag = b & 0x7fffffffu;
-  if (mag - 0x00800000u < 0x7f000000u)
-    return __hiloint2double((int)((b & 0x80000000u) | ((mag >> 3) + 0x38000000u)), (int)(b << 29));
-  return mag == 0u ? __hiloint2double((int)b, 0) : (double)x;
-}
-
 // Four values per thread and iteration where the arrays are 16-byte aligned
 // (the workspace's are, and the entry points ask it of Q); the last count % 4
 // one by one.

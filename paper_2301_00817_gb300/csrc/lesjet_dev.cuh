@@ -170,6 +170,16 @@ __device__ __forceinline__ double dev_max<double>(double a, double b) {
   return gt && ordered ? a : b;
 }
 
+// (double)x on the integer pipe (exact; zeros, denormals, infinities and NaN
+// take the conversion).
+__device__ __forceinline__ double widen(float x) {
+  const unsigned b = __float_as_uint(x), mag = b & 0x7fffffffu;
+  if (mag - 0x00800000u < 0x7f000000u)
+    return __hiloint2double((int)((b & 0x80000000u) | ((mag >> 3) + 0x38000000u)), (int)(b << 29));
+  return mag == 0u ? __hiloint2double((int)b, 0) : (double)x;
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+
 // a*b + c in one rounding, and a*b in a rounding of its own: with these the
 // rounding of an expression does not depend on which products the compiler
 // contracts, so that a dual-number run rounds as the double run does.
