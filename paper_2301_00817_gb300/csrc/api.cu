@@ -207,7 +207,7 @@ void layout(les_ctx* c) {
   // node fields: FP64 form; FP32 for the mixed forms' dynamic procedure
   c->off_node = o; o = align256(o + (mixed ? (c->dyn_ws ? 8 * N * sizeof(float) : 0) : 8 * N * sizeof(double)));
   c->off_flux = o; o = align256(o + (mixed ? 0 : 15 * N * sizeof(double)));
-  c->off_gn = o; o = align256(o + (mixed ? 0 : 4 * N * sizeof(double)));
+  c->off_gn = o; o = align256(o + (mixed ? 0 : 5 * N * sizeof(double)));
   c->off_rth = o; o = align256(o + 2 * (size_t)c->g.n[1] * c->g.n[2] * sizeof(double));
   c->off_sc = o; o = align256(o + sizeof(DevScalars));
   c->off_part = o; o = align256(o + 8 * (size_t)lesjet::kMaxPartials * sizeof(double));

@@ -154,9 +154,10 @@ __global__ void k_to_float(long long count, const double* __restrict__ a, float*
 
 // Grid constants the FP64 form takes once here instead of per residual:
 // |grad d| = |(d_x, d_y, d_z)| of the three computational coordinates (the
-// metric norms of the spectral radii lambda_d = |U_d| + a |grad d|), and
+// metric norms of the spectral radii lambda_d = |U_d| + a |grad d|),
 // J/2 = 0.5 / J^-1 of the stage update (0 where J^-1 = 0: an axis node,
-// which the stages do not update).
+// which the stages do not update), and the squared filter width
+// Delta^2 = (J^-1)^(2/3) of the SGS models.
 __global__ void k_grad_norms(long long N, const double* __restrict__ M, double* __restrict__ gn) {
   for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N;
        n += (long long)gridDim.x * blockDim.x) {
@@ -167,6 +168,8 @@ __global__ void k_grad_norms(long long N, const double* __restrict__ M, double* 
     }
     const double Ji = M[9 * N + n];
     gn[3 * N + n] = Ji == 0.0 ? 0.0 : 0.5 / Ji;
+    const double delta = cbrt(Ji);
+    gn[4 * N + n] = delta * delta;
   }
 }
 

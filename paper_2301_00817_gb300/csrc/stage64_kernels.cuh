@@ -128,21 +128,26 @@ __global__ void __launch_bounds__(256) k_node(Grid g, Consts<R> K, const TQ* __r
 }
 
 // -------------------------------------------------------------------- k_mu
-// Node-centred computational derivative (central; one-sided second order at
-// non-periodic faces).
+// Twice the node-centred computational derivative (central; one-sided second
+// order at non-periodic faces).
 template <typename R>
-__device__ __forceinline__ R node_deriv(const Grid& g, const R* __restrict__ f, long long n,
-                                        const int c[3], int d) {
+__device__ __forceinline__ R node_diff(const Grid& g, const R* __restrict__ f, long long n,
+                                       const int c[3], int d) {
   const long long s = g.stride[d];
   const int nd = g.n[d];
   if (g.per[d]) {
     const long long np = (c[d] == nd - 1) ? n - (long long)(nd - 1) * s : n + s;
     const long long nm = (c[d] == 0) ? n + (long long)(nd - 1) * s : n - s;
-    return R(0.5) * (f[np] - f[nm]);
+    return f[np] - f[nm];
   }
-  if (c[d] == 0) return R(0.5) * (R(-3) * f[n] + R(4) * f[n + s] - f[n + 2 * s]);
-  if (c[d] == nd - 1) return R(0.5) * (R(3) * f[n] - R(4) * f[n - s] + f[n - 2 * s]);
-  return R(0.5) * (f[n + s] - f[n - s]);
+  if (c[d] == 0) return R(-3) * f[n] + R(4) * f[n + s] - f[n + 2 * s];
+  if (c[d] == nd - 1) return R(3) * f[n] - R(4) * f[n - s] + f[n - 2 * s];
+  return f[n + s] - f[n - s];
+}
+template <typename R>
+__device__ __forceinline__ R node_deriv(const Grid& g, const R* __restrict__ f, long long n,
+                                        const int c[3], int d) {
+  return R(0.5) * node_diff(g, f, n, c, d);
 }
 
 // mu_eff = (Mj/Re) T^1.5 (1+S)/(T+S) + mu_sgs; kappa_eff = mu_lam/((g-1)Pr)
@@ -150,11 +155,15 @@ __device__ __forceinline__ R node_deriv(const Grid& g, const R* __restrict__ f, 
 // rho c sqrt(B_beta/alpha:alpha) (0 when alpha:alpha = 0, B_beta >= 0);
 // dynamic: C_ds rho Delta^2 |S| with the dynamic Pr_sgs and the Yoshizawa
 // sigma_ll = 2 C_I rho Delta^2 |S|^2 as a third field (coefficients dyn[6..8]
-// from the dynamic procedure); Delta = (J^-1)^(1/3).
+// from the dynamic procedure); Delta = (J^-1)^(1/3), Delta^2 from del2 (set-up).
+// The gradient is kept at twice its value and the strain at four times, whose
+// powers of two leave with one constant (FP64-pipe bound: 158 operations per
+// node with Smagorinsky before, when it also took the cube root, about 90 now).
 template <typename R, typename TQ, typename TM>
 __global__ void __launch_bounds__(256) k_mu(Grid g, Consts<R> K, const TQ* __restrict__ Q,
                                             const TM* __restrict__ M,
                                             const R* __restrict__ node, R* __restrict__ mk,
+                                            const double* __restrict__ del2,
                                             const double* __restrict__ dyn = nullptr) {
   const long long N = g.N;
   for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N;
@@ -167,63 +176,49 @@ __global__ void __launch_bounds__(256) k_mu(Grid g, Consts<R> K, const TQ* __res
     if (K.sgs != LES_SGS_NONE) {
       int c[3];
       decompose(g, n, c);
-      R gr[3][3];  // gr[i][x] = d u_i / d x_x
+      R gr[3][3];  // 2 d u_i / d x_x
 #pragma unroll
       for (int q = 0; q < 3; ++q) {
         R dd[3];
 #pragma unroll
-        for (int d = 0; d < 3; ++d) dd[d] = node_deriv(g, node + q * N, n, c, d);
+        for (int d = 0; d < 3; ++d) dd[d] = node_diff(g, node + q * N, n, c, d);
 #pragma unroll
         for (int x = 0; x < 3; ++x)
           gr[q][x] = (R)M[x * N + n] * dd[0] + (R)M[(3 + x) * N + n] * dd[1] +
                      (R)M[(6 + x) * N + n] * dd[2];
       }
-      const R Jinv = (R)M[9 * N + n];
-      const R delta = cbrt(Jinv);
-      const R rho = (R)Q[n];
-      if (K.sgs == LES_SGS_SMAGORINSKY) {
-        R ss = R(0);
-#pragma unroll
-        for (int i = 0; i < 3; ++i)
-#pragma unroll
-          for (int j = 0; j < 3; ++j) {
-            const R sij = R(0.5) * (gr[i][j] + gr[j][i]);
-            ss += sij * sij;
-          }
-        mu_s = rho * (delta * delta) * K.cs2 * dev_sqrt(R(2) * ss);
-      } else if (K.sgs == LES_SGS_DYNAMIC) {
-        R ss = R(0);
-#pragma unroll
-        for (int i = 0; i < 3; ++i)
-#pragma unroll
-          for (int j = 0; j < 3; ++j) {
-            const R sij = R(0.5) * (gr[i][j] + gr[j][i]);
-            ss += sij * sij;
-          }
-        const R smag = dev_sqrt(R(2) * ss);
-        const R d2 = delta * delta;
-        mu_s = R(dyn[6]) * rho * d2 * smag;
-        kap_s = mu_s / (K.gm1 * R(dyn[8]));
-        kap_set = true;
-        mk[2 * N + n] = R(2) * R(dyn[7]) * rho * d2 * smag * smag;
+      const R rd2 = (R)Q[n] * (R)del2[n];  // rho Delta^2
+      if (K.sgs == LES_SGS_SMAGORINSKY || K.sgs == LES_SGS_DYNAMIC) {
+        // |S|^2 = 2 S:S = 2 sum_i g_ii^2 + sum_{i<j} (g_ij + g_ji)^2 of the
+        // gradient g = gr/2
+        const R d = gr[0][0] * gr[0][0] + gr[1][1] * gr[1][1] + gr[2][2] * gr[2][2];
+        const R s01 = gr[0][1] + gr[1][0], s02 = gr[0][2] + gr[2][0], s12 = gr[1][2] + gr[2][1];
+        const R o = s01 * s01 + s02 * s02 + s12 * s12;
+        const R smag2 = R(0.25) * (R(2) * d + o);  // |S|^2
+        const R smag = dev_sqrt(smag2);
+        if (K.sgs == LES_SGS_SMAGORINSKY) {
+          mu_s = rd2 * K.cs2 * smag;
+        } else {
+          mu_s = R(dyn[6]) * rd2 * smag;
+          kap_s = mu_s / (K.gm1 * R(dyn[8]));
+          kap_set = true;
+          mk[2 * N + n] = R(2) * R(dyn[7]) * rd2 * smag2;
+        }
       } else {
-        // alpha_ij = d u_j / d x_i = gr[j][i]; beta_ij = Delta^2 alpha_mi alpha_mj
-        R aa = R(0);
+        // alpha_ij = d u_j / d x_i = gr[j][i]; beta_ij = Delta^2 alpha_mi alpha_mj:
+        // sqrt(B_beta/alpha:alpha) = Delta^2 sqrt(B_gg/alpha:alpha) with gg =
+        // alpha_mi alpha_mj, here 4x (B_gg 16x, alpha:alpha 4x)
+        R b[3][3], aa = R(0);
 #pragma unroll
         for (int i = 0; i < 3; ++i)
 #pragma unroll
-          for (int j = 0; j < 3; ++j) aa += gr[i][j] * gr[i][j];
-        R be[3][3];
-#pragma unroll
-        for (int i = 0; i < 3; ++i)
-#pragma unroll
-          for (int j = 0; j < 3; ++j)
-            be[i][j] = delta * delta *
-                       (gr[i][0] * gr[j][0] + gr[i][1] * gr[j][1] + gr[i][2] * gr[j][2]);
-        R B = be[0][0] * be[1][1] - be[0][1] * be[0][1] + be[0][0] * be[2][2] -
-              be[0][2] * be[0][2] + be[1][1] * be[2][2] - be[1][2] * be[1][2];
+          for (int j = i; j < 3; ++j)
+            b[i][j] = gr[i][0] * gr[j][0] + gr[i][1] * gr[j][1] + gr[i][2] * gr[j][2];
+        aa = b[0][0] + b[1][1] + b[2][2];
+        R B = b[0][0] * b[1][1] - b[0][1] * b[0][1] + b[0][0] * b[2][2] - b[0][2] * b[0][2] +
+              b[1][1] * b[2][2] - b[1][2] * b[1][2];
         B = B > R(0) ? B : R(0);
-        mu_s = (aa == R(0)) ? R(0) : rho * K.cs2 * dev_sqrt(B / aa);
+        mu_s = (aa == R(0)) ? R(0) : rd2 * K.cs2 * R(0.5) * dev_sqrt(B / aa);
       }
     }
     mk[n] = mu_l + mu_s;
