@@ -321,9 +321,9 @@ const char *les_profile_name(int kind);
  * sgs_model LES_SGS_NONE, freeze_visc 1; LES_ERR_UNSUPPORTED otherwise.
  * Scratch lives in a caller-owned adjoint workspace of
  * les_adjoint_workspace_bytes(ctx, nsteps, ckpt_every) bytes: about
- * (219 + 5 ceil(nsteps/ckpt_every) + 72 ckpt_every) N doubles for a window
+ * (234 + 5 ceil(nsteps/ckpt_every) + 72 ckpt_every) N doubles for a window
  * (checkpoints, plus every stage state and stage-input node quantity of one
- * segment), 219 N for nsteps = 0 (residual and single-step calls only); 66
+ * segment), 234 N for nsteps = 0 (residual and single-step calls only); 81
  * N of it hold each interface's cotangent record, which a per-node gather
  * sums in a fixed order, so every adjoint result is bitwise reproducible
  * (no atomics).  At non-smooth

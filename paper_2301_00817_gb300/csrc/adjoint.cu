@@ -36,10 +36,9 @@ namespace lesjet {
 
 // Per-interface record (each [N] doubles, indexed by the interface's node a,
 // one record array per direction): the cotangents it owes the nodes it read.
-// The conserved state's need no fields of their own: the dissipation owes
-// W_a d1 l, W_b -d1 l, W_{b+1} d3 l and W_{a-1} -d3 l, all multiples of l =
-// (lamR_a - lamR_b)/2, so the two coefficients are kept and k_adj_node forms
-// the products.
+// The conserved state's are products that k_adj_node forms: the dissipation
+// owes W_a d1 l, W_b -d1 l, W_{b+1} d3 l and W_{a-1} -d3 l, with l = (lamR_a -
+// lamR_b)/2, so the two coefficients and l are kept.
 enum {
   RUA = 0,    // u, v, w at a (3), then at b
   RUB = 3,
@@ -53,6 +52,7 @@ enum {
   RKA = 19,
   RD1 = 20,   // d1 and d3
   RD3 = 21,
+  RL = 22,    // l (5)
   NREC = kAdjRecords
 };
 
@@ -178,6 +178,8 @@ __device__ __forceinline__ void adj_iface(const Consts<double>& K, const FluxNod
     out[RG1 + i] = fma(m1[i], l23, fma(m[i], lc1, g1 * ls[i]));
     out[RG2 + i] = fma(m2[i], l23, fma(m[i], lc2, g2 * ls[i]));
   }
+#pragma unroll
+  for (int q = 0; q < 5; ++q) out[RL + q] = l[q];
   out[RT] = gD * lT;
   out[RG1 + 3] = g1 * lT;
   out[RG2 + 3] = g2 * lT;
@@ -439,15 +441,15 @@ __global__ void __launch_bounds__(256) k_adj_sensor_terms(Grid g, const double* 
 // lbar(lambda_d), lambda_d = |m_d.u| + sqrt(T)|grad d|, u = Q1/rho, p =
 // (g-1)(Q4 - rho|u|^2/2), T = g p/rho.  mu/kappa cotangents are added to
 // lamMK.  |grad d| comes from gn ([3][N], set-up).
-// A node reads about 240 values (its interfaces' records and lamR within two
-// nodes along each direction), few of them twice by one thread, and does
-// about 500 FP64 operations, whose pipe bounds it; gathering straight into
+// A node reads about 240 values (its interfaces' records within two nodes
+// along each direction), few of them twice by one thread, and does about 400
+// FP64 operations, whose pipe bounds it; gathering straight into
 // the node's reverse saves the 18 accumulator fields of a pass of their own.
 __global__ void __launch_bounds__(128, 3)
     k_adj_node(Grid g, Consts<double> K, const double* __restrict__ Q,
                const double* __restrict__ M, const double* __restrict__ gn,
-               const double* __restrict__ node, const double* __restrict__ lamR,
-               const double* __restrict__ rec, const double* __restrict__ ST,
+               const double* __restrict__ node, const double* __restrict__ rec,
+               const double* __restrict__ ST,
                double* __restrict__ lamQ, double* __restrict__ lamMK) {
   const long long N = g.N;
   for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N;
@@ -457,7 +459,7 @@ __global__ void __launch_bounds__(128, 3)
     const double u = node[n], v = node[N + n], w = node[2 * N + n], p = node[3 * N + n],
                  T = node[4 * N + n];
     const double Jv = M[9 * N + n];
-    double lW[5] = {0.0, 0.0, 0.0, 0.0, 0.0};   // twice the cotangents of W
+    double lW[5] = {0.0, 0.0, 0.0, 0.0, 0.0};   // the cotangents of W
     double lv[4] = {0.0, 0.0, 0.0, 0.0};        // u, v, w, T
     double lp = 0.0, lmu = 0.0, lka = 0.0, llb[3], th[3];
 #pragma unroll
@@ -479,19 +481,17 @@ __global__ void __launch_bounds__(128, 3)
       double lJt = 0.0, lF[5];
 #pragma unroll
       for (int q = 0; q < 5; ++q) {
-        const double* L = lamR + q * N;
-        const double l0 = L[n];
-        const double lm = m1 >= 0 ? L[m1] : l0, lq = p1 >= 0 ? L[p1] : l0;
-        const double eB = lm - l0, eA = l0 - lq;  // 0 where there is no interface
-        const double eP = m2 >= 0 ? L[m2] - lm : 0.0, eM = p2 >= 0 ? lq - L[p2] : 0.0;
+        const double* L = R + (RL + q) * N;
+        const double eA = L[n], eB = m1 >= 0 ? L[m1] : 0.0;
+        const double eP = m2 >= 0 ? L[m2] : 0.0, eM = p1 >= 0 ? L[p1] : 0.0;
         lW[q] = fma(kP, eP, fma(Jt - kB, eB, fma(Jt + kA, eA, fma(-kM, eM, lW[q]))));
-        lF[q] = eB + eA;  // twice the cotangent of the node's flux along D
+        lF[q] = eB + eA;  // the cotangent of the node's flux along D
         const double W = Q[q * N + n] + (q == 4 ? p : 0.0);
         lJt = fma(W, lF[q], lJt);
       }
       // node flux: W Jt (+ Jp m in the momentum), Jt = J^-1 m . u, Jp = J^-1 p
-      const double hJ = 0.5 * Jv, lth = hJ * lJt;
-      lp = fma(hJ, dot3(mx, my, mz, lF[1], lF[2], lF[3]), lp);
+      const double lth = Jv * lJt;
+      lp = fma(Jv, dot3(mx, my, mz, lF[1], lF[2], lF[3]), lp);
       lv[0] = fma(mx, lth, lv[0]);
       lv[1] = fma(my, lth, lv[1]);
       lv[2] = fma(mz, lth, lv[2]);
@@ -543,8 +543,6 @@ __global__ void __launch_bounds__(128, 3)
         if (xm == n) lp += ST[(2 * D) * N + x];
       }
     }
-#pragma unroll
-    for (int q = 0; q < 5; ++q) lW[q] *= 0.5;
     lp += lW[4];  // W4 = Q4 + p
     double lT = lv[3];
     // lbar -> lambda
@@ -1020,7 +1018,7 @@ void launch_rhs_vjp(const Grid& g, const les_params& p, const double* Q, const d
   const AdjIO io{FluxIO<double, double, double>{Q, M, node, mk, nullptr}, lamR, rec};
   k_adj_flux3<<<f.b2 + b0 + b1, kFluxThreads, 0, L.s>>>(g, K, io, f.b2, b0, f.len);
   k_adj_sensor_terms<<<nb_for(g.N), 256, 0, L.s>>>(g, node, rec, ST);
-  k_adj_node<<<blocks_for(g.N, 128), 128, 0, L.s>>>(g, K, Q, M, gn, node, lamR, rec, ST, lamQ, lamMK);
+  k_adj_node<<<blocks_for(g.N, 128), 128, 0, L.s>>>(g, K, Q, M, gn, node, rec, ST, lamQ, lamMK);
   *L.counter += 3;
 }
 

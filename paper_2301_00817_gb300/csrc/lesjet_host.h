@@ -103,7 +103,7 @@ void launch_rhs_vjp(const Grid& g, const les_params& p, const double* Q, const d
 void launch_mask_faces(const Grid& g, const double* lam, double* out, const Launch& L);
 // scratch of launch_rhs_vjp (acc): sensor terms, then one record of
 // kAdjRecords fields per interface of each direction
-constexpr int kAdjSensorTerms = 6, kAdjRecords = 22;
+constexpr int kAdjSensorTerms = 6, kAdjRecords = 27;
 void launch_rhs_jvp(const Grid& g, const les_params& p, const Dual* Q, const double* M,
                     const Dual* mk, Dual* node, Dual* flux, Dual* R, const Launch& L);
 void launch_mu_vjp(const Grid& g, const les_params& p, const double* Q, const double* lamMK,
