@@ -167,10 +167,11 @@ __device__ __forceinline__ void node_lbar(const R* m, R u, R v, R w, R T, R lb[3
     const R mx = m[3 * d], my = m[3 * d + 1], mz = m[3 * d + 2];
     l[d] = dev_abs(mx * u + my * v + mz * w) + a * dev_sqrt(mx * mx + my * my + mz * mz);
   }
-  const R s01 = dev_sqrt(l[0] * l[1]), s02 = dev_sqrt(l[0] * l[2]), s12 = dev_sqrt(l[1] * l[2]);
-  lb[0] = l[0] + s01 + s02;
-  lb[1] = l[1] + s01 + s12;
-  lb[2] = l[2] + s02 + s12;
+  // l_0 + sqrt(l_0 l_1) + sqrt(l_0 l_2) = r_0 (r_0 + r_1 + r_2), r_d = sqrt(l_d)
+  const R r0 = dev_sqrt(l[0]), r1 = dev_sqrt(l[1]), r2 = dev_sqrt(l[2]), rs = r0 + r1 + r2;
+  lb[0] = r0 * rs;
+  lb[1] = r1 * rs;
+  lb[2] = r2 * rs;
 }
 
 template <typename TM, typename R>

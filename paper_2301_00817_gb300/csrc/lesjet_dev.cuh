@@ -152,10 +152,20 @@ template <typename T>
 __device__ __forceinline__ T dev_abs(T x) { return x < T(0) ? -x : x; }
 template <>
 __device__ __forceinline__ double dev_abs<double>(double x) { return fabs(x); }  // no FP64 compare
+template <>
+__device__ __forceinline__ float dev_abs<float>(float x) { return fabsf(x); }  // a source modifier
 
 // a > b ? a : b
 template <typename T>
 __device__ __forceinline__ T dev_max(T a, T b) { return a > b ? a : b; }
+// For floats one instruction, which gives NaN if either operand is one (the
+// comparison would select b and could hide a NaN in a).
+template <>
+__device__ __forceinline__ float dev_max<float>(float a, float b) {
+  float m;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(m) : "f"(a), "f"(b));
+  return m;
+}
 // For doubles the comparison runs on the integer pipe (an FP64 compare takes
 // a slot of the FP64 pipe, which bounds these kernels): the bit patterns of
 // two doubles order like their values, in reverse when both are negative.
