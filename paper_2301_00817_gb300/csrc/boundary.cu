@@ -24,36 +24,42 @@ struct AccHL {
   }
 };
 
-constexpr int kBcThreads = 64;  // block of the boundary kernels
+constexpr int kBcThreads = 128;  // block of the boundary kernels: a warp per scheduler
 
 struct JetBC {
   int mode;     // LES_BC_JET or LES_BC_JET_CHAR
   int forced;   // some forcing amplitude is non-zero
   double gamma, Mj, r_jet, theta_m, force_width;
+  double gm1, igm1, ig;  // gamma - 1 and the reciprocals of it and of gamma
   double St[4];
   double amp[16];
 };
 
+// (The boundary nodes' chains of dependent FP64 operations are what their
+// launches take, and a division is ten of them: constants are multiplied by
+// their reciprocals, a node's density is inverted once, the sound speed and
+// its reciprocal come from one root, and Mach numbers are compared without
+// being formed.)
 template <class Acc>
-__device__ __forceinline__ void store_prim(const Acc& Q, long long N, long long n, double gamma,
+__device__ __forceinline__ void store_prim(const Acc& Q, long long N, long long n, double igm1,
                                            double rho, double u, double v, double w, double p) {
   Q.st(n, rho);
   Q.st(N + n, rho * u);
   Q.st(2 * N + n, rho * v);
   Q.st(3 * N + n, rho * w);
-  Q.st(4 * N + n, p / (gamma - 1.0) + 0.5 * rho * (u * u + v * v + w * w));
+  Q.st(4 * N + n, p * igm1 + 0.5 * rho * (u * u + v * v + w * w));
 }
 
 template <class Acc>
-__device__ __forceinline__ void load_prim(const Acc& Q, long long N, long long n, double gamma,
-                                          double& rho, double& u, double& v, double& w,
+__device__ __forceinline__ void load_prim(const Acc& Q, long long N, long long n, double gm1,
+                                          double& rho, double& ir, double& u, double& v, double& w,
                                           double& p) {
   rho = Q.ld(n);
-  const double ir = 1.0 / rho;
+  ir = 1.0 / rho;
   u = Q.ld(N + n) * ir;
   v = Q.ld(2 * N + n) * ir;
   w = Q.ld(3 * N + n) * ir;
-  p = (gamma - 1.0) * (Q.ld(4 * N + n) - 0.5 * rho * (u * u + v * v + w * w));
+  p = gm1 * (Q.ld(4 * N + n) - 0.5 * rho * (u * u + v * v + w * w));
 }
 
 // Riemann-invariant state of a far-field node from its interior neighbour's
@@ -77,40 +83,39 @@ __device__ __forceinline__ double pow_entropy(double x, double e) {
   return pow(x, e);
 }
 
-__device__ __forceinline__ bool far_field_state(double gamma, double rho, double u, double v,
-                                                double w, double p, double nx, double ny,
+__device__ __forceinline__ bool far_field_state(const JetBC& b, double rho, double ir, double u,
+                                                double v, double w, double p, double nx, double ny,
                                                 double nz, double f[5]) {
-  const double gm1 = gamma - 1.0;
-  const double ae = sqrt(gamma * p / rho);
+  const double T = b.gamma * p * ir, ra = rsqrt(T), ae = T * ra;
   const double qne = u * nx + v * ny + w * nz;
-  const double Rp = qne + 2.0 * ae / gm1;
-  const double Rm = 0.0 - 2.0 * 1.0 / gm1;
+  const double Rp = qne + 2.0 * ae * b.igm1;
+  const double Rm = -2.0 * b.igm1;
   const double qnf = 0.5 * (Rp + Rm);
-  const double af = 0.25 * gm1 * (Rp - Rm);
-  const double Mn = qne / ae;
-  if (Mn >= 1.0) return true;
-  if (Mn >= 0.0) {
+  const double af = 0.25 * b.gm1 * (Rp - Rm);
+  // q_n,e/a_e >= 1, >= 0, > -1
+  if (qne >= ae) return true;
+  if (qne >= 0.0) {
     // entropy of the interior node: rho_f = (rho_e^gamma a_f^2/(gamma p_e))^(1/(gamma-1))
     // = rho_e (a_f/a_e)^(2/(gamma-1)), one power instead of two
     const double dq = qnf - qne;
-    const double rf = rho * pow_entropy(af / ae, 2.0 / gm1);
+    const double rf = rho * pow_entropy(af * ra, 2.0 * b.igm1);
     f[0] = rf;
     f[1] = u + dq * nx;
     f[2] = v + dq * ny;
     f[3] = w + dq * nz;
-    f[4] = rf * af * af / gamma;
-  } else if (Mn > -1.0) {
+    f[4] = rf * af * af * b.ig;
+  } else if (qne > -ae) {
     // free-stream entropy (rho = 1, p = 1/gamma): rho_f = a_f^(2/(gamma-1))
-    const double rf = pow_entropy(af, 2.0 / gm1);
+    const double rf = pow_entropy(af, 2.0 * b.igm1);
     f[0] = rf;
     f[1] = qnf * nx;
     f[2] = qnf * ny;
     f[3] = qnf * nz;
-    f[4] = rf * af * af / gamma;
+    f[4] = rf * af * af * b.ig;
   } else {
     f[0] = 1.0;
     f[1] = f[2] = f[3] = 0.0;
-    f[4] = 1.0 / gamma;
+    f[4] = b.ig;
   }
   return false;
 }
@@ -135,72 +140,89 @@ __device__ __forceinline__ void bc_inflow_part(const Grid& g, const JetBC& b,
   const long long N = g.N;
   const double t = use_host_t ? t_host : sc->t;
   const double two_pi = 6.283185307179586476925286766559;
-  // the four forcing phases are the same for every node: lane f of the warp
-  // takes phase f mod 4, and all lanes share the four
-  double sf[4] = {0.0, 0.0, 0.0, 0.0}, cf[4] = {0.0, 0.0, 0.0, 0.0};
-  if (b.forced) {
-    const int f = threadIdx.x & 3;
-    double s, c;
-    sincos(two_pi * (f == 0 ? b.St[0] : (f == 1 ? b.St[1] : (f == 2 ? b.St[2] : b.St[3]))) * b.Mj * t,
-           &s, &c);
-#pragma unroll
-    for (int l = 0; l < 4; ++l) {
-      sf[l] = __shfl_sync(0xffffffffu, s, l);
-      cf[l] = __shfl_sync(0xffffffffu, c, l);
-    }
-  }
-  for (long long n = blk * (long long)blockDim.x + threadIdx.x; n < plane;
-       n += (long long)nblk * blockDim.x) {
-    const double r = rth[n], th = rth[plane + n];
-    double u = 0.5 * b.Mj * (1.0 + tanh((b.r_jet - r) / (2.0 * b.theta_m)));
+  // 32 nodes per block and iteration.  A node's profile and forcing are four
+  // independent chains of 40 to 80 FP64 operations, and a warp's operations
+  // follow one another at 64 cycles each, so the block's four warps, on four
+  // schedulers, take one chain each: tanh, exp, sin and cos of theta, and the
+  // four forcing phases (lane f of warp 3 takes phase f mod 4); then one m each.
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  __shared__ double su[32], sg[32], sc1[4][32], ss1[4][32], sf[4], cf[4], sa[4][32];
+  for (long long n0 = blk * 32LL; n0 < plane; n0 += nblk * 32LL) {
+    const long long n = n0 + lane;
+    const bool in = n < plane;
+    const double r = in ? rth[n] : 1.0;
+    if (warp == 0) su[lane] = 0.5 * b.Mj * (1.0 + tanh((b.r_jet - r) / (2.0 * b.theta_m)));
     if (b.forced) {
       // cos(m theta - phi_f) = cos(m theta) cos(phi_f) + sin(m theta) sin(phi_f),
       // with cos/sin(m theta) by the angle-addition recurrence from theta
-      const double x = (r - b.r_jet) / b.force_width;
-      const double gr = exp(-(x * x));
-      double s1, c1;
-      sincos(th, &s1, &c1);
-      double cm[4] = {1.0, c1, 0.0, 0.0}, sm[4] = {0.0, s1, 0.0, 0.0};
-#pragma unroll
-      for (int m = 2; m < 4; ++m) {
-        cm[m] = cm[m - 1] * c1 - sm[m - 1] * s1;
-        sm[m] = sm[m - 1] * c1 + cm[m - 1] * s1;
+      if (warp == 1) {
+        const double x = (r - b.r_jet) / b.force_width;
+        sg[lane] = exp(-(x * x));
+      } else if (warp == 2) {
+        double s1, c1;
+        sincos(in ? rth[plane + n] : 0.0, &s1, &c1);
+        const double c2 = c1 * c1 - s1 * s1, s2 = s1 * c1 + c1 * s1;
+        sc1[0][lane] = 1.0;
+        ss1[0][lane] = 0.0;
+        sc1[1][lane] = c1;
+        ss1[1][lane] = s1;
+        sc1[2][lane] = c2;
+        ss1[2][lane] = s2;
+        sc1[3][lane] = c2 * c1 - s2 * s1;
+        ss1[3][lane] = s2 * c1 + c2 * s1;
+      } else if (warp == 3) {
+        const int f = lane & 3;
+        double s, c;
+        sincos(two_pi * (f == 0 ? b.St[0] : (f == 1 ? b.St[1] : (f == 2 ? b.St[2] : b.St[3]))) * b.Mj * t,
+               &s, &c);
+        if (lane < 4) {
+          sf[lane] = s;
+          cf[lane] = c;
+        }
       }
+      __syncthreads();
       double acc = 0.0;
 #pragma unroll
-      for (int m = 0; m < 4; ++m)
-#pragma unroll
-        for (int f = 0; f < 4; ++f) acc += b.amp[m * 4 + f] * (cm[m] * cf[f] + sm[m] * sf[f]);
-      u += gr * acc;
-    }
-    const long long ne = n + plane;  // node (1, j, k)
-    if (b.mode == LES_BC_JET_CHAR && r > b.r_jet) {
-      const double ex = (double)M[n], ey = (double)M[N + n], ez = (double)M[2 * N + n];
-      const double inv = 1.0 / sqrt(ex * ex + ey * ey + ez * ez);
-      double rho, ue, ve, we, p, f[5];
-      load_prim(Q, N, ne, b.gamma, rho, ue, ve, we, p);
-      if (far_field_state(b.gamma, rho, ue, ve, we, p, -ex * inv, -ey * inv, -ez * inv, f)) {
-#pragma unroll
-        for (int q = 0; q < 5; ++q) Q.st(q * N + n, Q.ld(q * N + ne));
-      } else {
-        store_prim(Q, N, n, b.gamma, f[0], f[1], f[2], f[3], f[4]);
+      for (int f = 0; f < 4; ++f) {
+        const double a = warp == 0 ? b.amp[f] : (warp == 1 ? b.amp[4 + f] : (warp == 2 ? b.amp[8 + f] : b.amp[12 + f]));
+        acc += a * (sc1[warp][lane] * cf[f] + ss1[warp][lane] * sf[f]);
       }
-    } else if (b.mode == LES_BC_JET_CHAR && b.Mj < 1.0) {
-      const double gm1 = b.gamma - 1.0;
-      double rho, ue, ve, we, p;
-      load_prim(Q, N, ne, b.gamma, rho, ue, ve, we, p);
-      const double Tt = 1.0 + 0.5 * gm1 * b.Mj * b.Mj;
-      const double T = Tt / (1.0 + 0.5 * gm1 * (u * u + ve * ve + we * we));
-      const double pf = pow(T, b.gamma / gm1) / b.gamma;
-      store_prim(Q, N, n, b.gamma, b.gamma * pf / T, u, ve, we, pf);
-    } else {
-      store_prim(Q, N, n, b.gamma, 1.0, u, 0.0, 0.0, 1.0 / b.gamma);
+      sa[warp][lane] = acc;
+      __syncthreads();
     }
+    if (warp == 0 && in) {
+      double u = su[lane];
+      if (b.forced) u += sg[lane] * (((sa[0][lane] + sa[1][lane]) + sa[2][lane]) + sa[3][lane]);
+      const long long ne = n + plane;  // node (1, j, k)
+      if (b.mode == LES_BC_JET_CHAR && r > b.r_jet) {
+        const double ex = (double)M[n], ey = (double)M[N + n], ez = (double)M[2 * N + n];
+        const double inv = rsqrt(ex * ex + ey * ey + ez * ez);
+        double rho, ir, ue, ve, we, p, f[5];
+        load_prim(Q, N, ne, b.gm1, rho, ir, ue, ve, we, p);
+        if (far_field_state(b, rho, ir, ue, ve, we, p, -ex * inv, -ey * inv, -ez * inv, f)) {
+#pragma unroll
+          for (int q = 0; q < 5; ++q) Q.st(q * N + n, Q.ld(q * N + ne));
+        } else {
+          store_prim(Q, N, n, b.igm1, f[0], f[1], f[2], f[3], f[4]);
+        }
+      } else if (b.mode == LES_BC_JET_CHAR && b.Mj < 1.0) {
+        const double gm1 = b.gm1;
+        double rho, ir, ue, ve, we, p;
+        load_prim(Q, N, ne, gm1, rho, ir, ue, ve, we, p);
+        const double Tt = 1.0 + 0.5 * gm1 * b.Mj * b.Mj;
+        const double T = Tt / (1.0 + 0.5 * gm1 * (u * u + ve * ve + we * we));
+        const double pf = pow(T, b.gamma / gm1) / b.gamma;
+        store_prim(Q, N, n, b.igm1, b.gamma * pf / T, u, ve, we, pf);
+      } else {
+        store_prim(Q, N, n, b.igm1, 1.0, u, 0.0, 0.0, b.ig);
+      }
+    }
+    __syncthreads();  // the next 32 nodes' values replace these
   }
 }
 
 template <class Acc, typename TM>
-__global__ void k_bc_inflow(Grid g, JetBC b, const double* __restrict__ rth,
+__global__ void __launch_bounds__(kBcThreads) k_bc_inflow(Grid g, JetBC b, const double* __restrict__ rth,
                             const TM* __restrict__ M, const DevScalars* __restrict__ sc,
                             int use_host_t, double t_host, Acc Q) {
   bc_inflow_part(g, b, rth, M, sc, use_host_t, t_host, Q, blockIdx.x, gridDim.x);
@@ -210,7 +232,7 @@ __global__ void k_bc_inflow(Grid g, JetBC b, const double* __restrict__ rth,
 // eta-normal with R+ from the adjacent interior node and R- from the free
 // stream at rest (rho = 1, p = 1/gamma, a = 1); four branches by q_n/a.
 template <class Acc, typename TM>
-__device__ __forceinline__ void bc_farfield_part(const Grid& g, double gamma,
+__device__ __forceinline__ void bc_farfield_part(const Grid& g, const JetBC& b,
                                                  const TM* __restrict__ M, const Acc& Q, int blk,
                                                  int nblk) {
   const int ni = g.n[0], nj = g.n[1], nk = g.n[2];
@@ -221,14 +243,14 @@ __device__ __forceinline__ void bc_farfield_part(const Grid& g, double gamma,
     const int i = 1 + (int)(e / nk), k = (int)(e % nk);
     const long long nf = idx3(g, i, nj - 1, k), ne = idx3(g, i, nj - 2, k);
     const double ex = (double)M[3 * N + nf], ey = (double)M[4 * N + nf], ez = (double)M[5 * N + nf];
-    const double inv = 1.0 / sqrt(ex * ex + ey * ey + ez * ez);
-    double rho, u, v, w, p, f[5];
-    load_prim(Q, N, ne, gamma, rho, u, v, w, p);
-    if (far_field_state(gamma, rho, u, v, w, p, ex * inv, ey * inv, ez * inv, f)) {
+    const double inv = rsqrt(ex * ex + ey * ey + ez * ez);
+    double rho, ir, u, v, w, p, f[5];
+    load_prim(Q, N, ne, b.gm1, rho, ir, u, v, w, p);
+    if (far_field_state(b, rho, ir, u, v, w, p, ex * inv, ey * inv, ez * inv, f)) {
 #pragma unroll
       for (int q = 0; q < 5; ++q) Q.st(q * N + nf, Q.ld(q * N + ne));
     } else {
-      store_prim(Q, N, nf, gamma, f[0], f[1], f[2], f[3], f[4]);
+      store_prim(Q, N, nf, b.igm1, f[0], f[1], f[2], f[3], f[4]);
     }
   }
 }
@@ -276,9 +298,9 @@ __device__ __forceinline__ void bc_ring_part(const Grid& g, const Acc& Q, int bl
 // plane i = 1 before its edges change: nb_in = 0, and a launch of its own
 // ahead of this one.)  A node takes 150 to 300 dependent FP64 operations, and
 // the FP64 pipe issues one warp instruction per 64 cycles and scheduler, so
-// a few nodes are bound by their latency: blocks of 64 threads, one warp for
-// each of two schedulers, spread them over the SMs (48 x 24 x 32: with blocks of
-// 256 this launch and the exit's had taken 24 + 14 us).
+// a few nodes are bound by their latency: blocks of 128 threads, one warp per
+// scheduler, spread them over the SMs (48 x 24 x 32: with blocks of 256 this
+// launch and the exit's had taken 24 + 14 us).
 template <class Acc, typename TM>
 __global__ void __launch_bounds__(kBcThreads)
     k_bc_sides(Grid g, JetBC b, const double* __restrict__ rth, const TM* __restrict__ M,
@@ -286,7 +308,7 @@ __global__ void __launch_bounds__(kBcThreads)
                int nb_in) {
   const int blk = blockIdx.x;
   if (blk < nb_ff)
-    bc_farfield_part(g, b.gamma, M, Q, blk, nb_ff);
+    bc_farfield_part(g, b, M, Q, blk, nb_ff);
   else if (blk < nb_ff + nb_in)
     bc_inflow_part(g, b, rth, M, sc, use_host_t, t_host, Q, blk - nb_ff, nb_in);
   else
@@ -298,11 +320,10 @@ __global__ void __launch_bounds__(kBcThreads)
 // velocity and the internal energy p/((gamma-1) rho).
 template <class Acc, typename TM>
 __global__ void __launch_bounds__(kBcThreads)
-    k_bc_exit(Grid g, double gamma, const TM* __restrict__ M, Acc Q) {
+    k_bc_exit(Grid g, JetBC b, const TM* __restrict__ M, Acc Q) {
   const int ni = g.n[0];
   const long long plane = (long long)g.n[1] * g.n[2];
   const long long N = g.N;
-  const double gm1 = gamma - 1.0;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < plane;
        e += (long long)gridDim.x * blockDim.x) {
     const long long nx_ = (long long)(ni - 1) * plane + e, ne = nx_ - plane;
@@ -310,22 +331,22 @@ __global__ void __launch_bounds__(kBcThreads)
     // outward normal of (ni-1, 1, k) (Reading A27)
     const long long nm = (e < g.n[2] && (double)M[9 * N + nx_] == 0.0) ? nx_ + g.n[2] : nx_;
     const double ex = (double)M[nm], ey = (double)M[N + nm], ez = (double)M[2 * N + nm];
-    const double inv = 1.0 / sqrt(ex * ex + ey * ey + ez * ez);
-    double rho, u, v, w, p;
-    load_prim(Q, N, ne, gamma, rho, u, v, w, p);
-    const double ae = sqrt(gamma * p / rho);
-    const double qn = (u * ex + v * ey + w * ez) * inv;
-    if (qn / ae >= 1.0) {
+    const double gn = sqrt(ex * ex + ey * ey + ez * ez);
+    double rho, ir, u, v, w, p;
+    load_prim(Q, N, ne, b.gm1, rho, ir, u, v, w, p);
+    const double ae = sqrt(b.gamma * p * ir);
+    // q_n >= a_e, q_n = u . e/|e|
+    if (u * ex + v * ey + w * ez >= ae * gn) {
 #pragma unroll
       for (int q = 0; q < 5; ++q) Q.st(q * N + nx_, Q.ld(q * N + ne));
     } else {
       // rho_f = p_inf/((gamma-1) e_int) = p_inf rho/p, e_int = p/((gamma-1) rho)
-      const double rf = rho / (gamma * p);
+      const double rf = rho / (b.gamma * p);
       Q.st(nx_, rf);
       Q.st(N + nx_, rf * u);
       Q.st(2 * N + nx_, rf * v);
       Q.st(3 * N + nx_, rf * w);
-      Q.st(4 * N + nx_, 1.0 / (gamma * gm1) + 0.5 * rf * (u * u + v * v + w * w));
+      Q.st(4 * N + nx_, b.ig * b.igm1 + 0.5 * rf * (u * u + v * v + w * w));
     }
   }
 }
@@ -413,6 +434,9 @@ static void bc_jet(const Grid& g, const les_params& p, Acc Q, const TM* M,
   JetBC b;
   b.mode = p.bc;
   b.gamma = p.gamma;
+  b.gm1 = p.gamma - 1.0;
+  b.igm1 = 1.0 / b.gm1;
+  b.ig = 1.0 / p.gamma;
   b.Mj = p.Mj;
   b.r_jet = p.r_jet;
   b.theta_m = p.theta_m;
@@ -428,7 +452,7 @@ static void bc_jet(const Grid& g, const les_params& p, Acc Q, const TM* M,
   // and the exit only if it ends there (its far field and inner ring cover
   // its ghost planes too, which the next exchange overwrites)
   const int nb_ff = nblocks((long long)(g.n[0] - 2) * g.n[2]);
-  int nb_in = g.glo == 0 ? nblocks(plane) : 0;
+  int nb_in = g.glo == 0 ? nblocks(4 * plane) : 0;  // 32 nodes per block
   if (p.bc == LES_BC_JET_CHAR && nb_in > 0) {
     // the characteristic entrance reads the plane i = 1 before the far field
     // and the ring write its edges
@@ -440,7 +464,7 @@ static void bc_jet(const Grid& g, const les_params& p, Acc Q, const TM* M,
       g, b, rth, M, sc, use_host_t, t_host, Q, nb_ff, nb_in);
   ++*L.counter;
   if (g.ghi == 0) {
-    k_bc_exit<Acc, TM><<<nblocks(plane), kBcThreads, 0, L.s>>>(g, p.gamma, M, Q);
+    k_bc_exit<Acc, TM><<<nblocks(plane), kBcThreads, 0, L.s>>>(g, b, M, Q);
     ++*L.counter;
   }
 }
