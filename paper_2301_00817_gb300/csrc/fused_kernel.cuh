@@ -712,47 +712,45 @@ __global__ void __launch_bounds__(FTJ * FTK, 1)
   };
 
   // ---- primitives (2-node halo) and lbar (1-node halo) of a staged plane
-  auto derive_plane = [&](int qs, int ps, int ms, int ls) {
+  auto derive_node = [&](int r, int qs, int ps, int ms, int ls) {
     const float* q = sQ + qs * 5 * PL2;
     float4* pr = sPr + ps * PL2;
     float2* pw = sPw + ps * PL2;
     const float* mm = sM + ms * 10 * PL1;
     float* ll = sL + ls * 3 * PL1;
-    for (int r = tid; r < PL2; r += FNT) {
-      const float rho = q[r];
-      const float ir = frcp_fast(rho);
-      const float u = q[PL2 + r] * ir, v = q[2 * PL2 + r] * ir, w = q[3 * PL2 + r] * ir;
-      const float p = K.gm1 * (q[4 * PL2 + r] - 0.5f * rho * (u * u + v * v + w * w));
-      const float T = K.gamma * p * ir;
-      pr[r] = make_float4(u, v, w, T);
-      pw[r] = make_float2(p, q[4 * PL2 + r] + p);
-      const int row = r / SK, col = r - row * SK;
-      // 1-node halo: rows 1 .. R2-2 of the 2-node layout, columns kk in [-1, FTK]
-      if (row >= 1 && row <= R2 - 2 && col >= colk(-1) && col <= colk(FTK)) {
-        const int r1 = r - SK;
-        float m[10];
+    const float rho = q[r];
+    const float ir = frcp_fast(rho);
+    const float u = q[PL2 + r] * ir, v = q[2 * PL2 + r] * ir, w = q[3 * PL2 + r] * ir;
+    const float p = K.gm1 * (q[4 * PL2 + r] - 0.5f * rho * (u * u + v * v + w * w));
+    const float T = K.gamma * p * ir;
+    pr[r] = make_float4(u, v, w, T);
+    pw[r] = make_float2(p, q[4 * PL2 + r] + p);
+    const int row = r / SK, col = r - row * SK;
+    // 1-node halo: rows 1 .. R2-2 of the 2-node layout, columns kk in [-1, FTK]
+    if (row >= 1 && row <= R2 - 2 && col >= colk(-1) && col <= colk(FTK)) {
+      const int r1 = r - SK;
+      float m[10];
 #pragma unroll
-        for (int t = 0; t < 10; ++t) m[t] = mm[t * PL1 + r1];
-        float lb[3];
-        if (AXIS && m[9] == 0.f && j0 + row - 2 == 0) {
-          // an axis node (Reading A27) takes the radii of its inward
-          // neighbour (i, 1, k): the next row of the same plane
-          const int s = r + SK;
-          const float rho1 = q[s];
-          const float ir1 = frcp_fast(rho1);
-          const float u1 = q[PL2 + s] * ir1, v1 = q[2 * PL2 + s] * ir1, w1 = q[3 * PL2 + s] * ir1;
-          const float p1 = K.gm1 * (q[4 * PL2 + s] - 0.5f * rho1 * (u1 * u1 + v1 * v1 + w1 * w1));
-          float m1[10];
+      for (int t = 0; t < 10; ++t) m[t] = mm[t * PL1 + r1];
+      float lb[3];
+      if (AXIS && m[9] == 0.f && j0 + row - 2 == 0) {
+        // an axis node (Reading A27) takes the radii of its inward
+        // neighbour (i, 1, k): the next row of the same plane
+        const int s = r + SK;
+        const float rho1 = q[s];
+        const float ir1 = frcp_fast(rho1);
+        const float u1 = q[PL2 + s] * ir1, v1 = q[2 * PL2 + s] * ir1, w1 = q[3 * PL2 + s] * ir1;
+        const float p1 = K.gm1 * (q[4 * PL2 + s] - 0.5f * rho1 * (u1 * u1 + v1 * v1 + w1 * w1));
+        float m1[10];
 #pragma unroll
-          for (int t = 0; t < 10; ++t) m1[t] = mm[t * PL1 + r1 + SK];
-          node_lbar(m1, u1, v1, w1, K.gamma * p1 * ir1, lb);
-        } else {
-          node_lbar(m, u, v, w, T, lb);
-        }
-        ll[r1] = lb[0];
-        ll[PL1 + r1] = lb[1];
-        ll[2 * PL1 + r1] = lb[2];
+        for (int t = 0; t < 10; ++t) m1[t] = mm[t * PL1 + r1 + SK];
+        node_lbar(m1, u1, v1, w1, K.gamma * p1 * ir1, lb);
+      } else {
+        node_lbar(m, u, v, w, T, lb);
       }
+      ll[r1] = lb[0];
+      ll[PL1 + r1] = lb[1];
+      ll[2 * PL1 + r1] = lb[2];
     }
   };
 
@@ -1000,8 +998,12 @@ __global__ void __launch_bounds__(FTJ * FTK, 1)
   fetch_h(ib);
   cp_async_wait<1>();
   __syncthreads();
-  derive_plane(s_m, s_m, s_m, l_p);  // m2(ib - 1) == m2(ib + 1)
-  derive_plane(s_c, s_c, s_c, l_c);
+  // planes ib - 1 and ib in one loop over the threads: m2(ib - 1) == m2(ib + 1)
+  for (int t = tid; t < 2 * PL2; t += FNT) {
+    const bool lo = t < PL2;
+    const int s = lo ? s_m : s_c;
+    derive_node(lo ? t : t - PL2, s, s, s, lo ? l_p : l_c);
+  }
   __syncthreads();
   float Fx_prev[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
   if (own && jint && kint && (per_i || ib - 1 >= 0))
@@ -1030,7 +1032,7 @@ __global__ void __launch_bounds__(FTJ * FTK, 1)
     // those slots and plane i+1 derived without a barrier of their own.
     stage_plane(s_m, i + 2);
     cp_async_commit();
-    derive_plane(s_p, s_p, s_p, l_p);
+    for (int r = tid; r < PL2; r += FNT) derive_node(r, s_p, s_p, s_p, l_p);
     __syncthreads();
 
     const int ig = wrap_fast(i, ni, per0);
