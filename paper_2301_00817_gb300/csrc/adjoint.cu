@@ -422,8 +422,8 @@ __global__ void __launch_bounds__(256) k_adj_sensor_terms(Grid g, const double* 
         sensor_triple_at(g, d, n, c[d], xm, xc, xp);
         // nu = |s| / den, rounded as sensor3 does (the sign of s decides the
         // branch where the pressure is uniform to rounding)
-        const double pm = P[xm] + P[xp];
-        const double s = fma(-2.0, P[xc], pm), den = fma(2.0, P[xc], pm);
+        const double p0 = P[xc];
+        const double s = (P[xp] - p0) - (p0 - P[xm]), den = fma(4.0, p0, s);
         const double iden = 1.0 / den;
         const double ls = ln * sgn_abs(s) * iden;
         const double lden = -ln * fabs(s) * iden * iden;
