@@ -387,6 +387,7 @@ __device__ __forceinline__ void adj_zeta(const Grid& g, const Consts<double>& K,
 // term and the centred flux reversed twice per node).
 __global__ void __launch_bounds__(kFluxThreads, 2)
     k_adj_flux3(Grid g, Consts<double> K, AdjIO io, unsigned b2, unsigned b0, int len) {
+  begin_dependent();
   __shared__ double sh[9][kFluxThreads];
   const unsigned b = blockIdx.x;
   if (b < b2)
@@ -405,6 +406,7 @@ __global__ void __launch_bounds__(kFluxThreads, 2)
 __global__ void __launch_bounds__(256) k_adj_sensor_terms(Grid g, const double* __restrict__ node,
                                                           const double* __restrict__ rec,
                                                           double* __restrict__ ST) {
+  begin_dependent();
   const long long N = g.N;
   const double* P = node + 3 * N;
   for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N;
@@ -451,6 +453,7 @@ __global__ void __launch_bounds__(128, 3)
                const double* __restrict__ node, const double* __restrict__ rec,
                const double* __restrict__ ST,
                double* __restrict__ lamQ, double* __restrict__ lamMK) {
+  begin_dependent();
   const long long N = g.N;
   for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N;
        n += (long long)gridDim.x * blockDim.x) {
@@ -601,6 +604,7 @@ __global__ void __launch_bounds__(128, 3)
 // mu/((g-1)Pr), T = g p/rho of Q^n; adds the Q cotangent to lamQ.
 __global__ void k_adj_mu(Grid g, Consts<double> K, const double* __restrict__ Q,
                          const double* __restrict__ lamMK, double* __restrict__ lamQ) {
+  begin_dependent();
   const long long N = g.N;
   for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N;
        n += (long long)gridDim.x * blockDim.x) {
@@ -633,6 +637,7 @@ __global__ void k_adj_mu(Grid g, Consts<double> K, const double* __restrict__ Q,
 __global__ void k_adj_stage_prep(Grid g, const double* __restrict__ M, double coef,
                                  const double* __restrict__ lamS, double* __restrict__ lamR,
                                  double* __restrict__ lamQ0) {
+  begin_dependent();
   const long long N = g.N;
   for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N;
        n += (long long)gridDim.x * blockDim.x) {
@@ -651,6 +656,7 @@ __global__ void k_adj_stage_prep(Grid g, const double* __restrict__ M, double co
 
 // out = lam, 0 on the faces of non-periodic directions (where the residual is 0)
 __global__ void k_mask_faces(Grid g, const double* __restrict__ lam, double* __restrict__ out) {
+  begin_dependent();
   const long long N = g.N;
   for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N;
        n += (long long)gridDim.x * blockDim.x) {
@@ -665,6 +671,7 @@ __global__ void k_mask_faces(Grid g, const double* __restrict__ lam, double* __r
 }
 
 __global__ void k_axpy(long long count, double a, const double* __restrict__ x, double* __restrict__ y) {
+  begin_dependent();
   for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < count;
        n += (long long)gridDim.x * blockDim.x)
     y[n] += a * x[n];
@@ -759,6 +766,7 @@ __device__ double local_vjp(int i, const double qe[5], double a0, double a1, dou
 // lamS = lamNext on interior nodes, 0 on boundary nodes (their stage values
 // are overwritten by the boundary conditions)
 __global__ void k_adjbc_init(Grid g, const double* __restrict__ lamNext, double* __restrict__ lamS) {
+  begin_dependent();
   const long long N = g.N;
   for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N;
        n += (long long)gridDim.x * blockDim.x) {
@@ -783,6 +791,7 @@ __global__ void __launch_bounds__(64) k_adjbc_exit(Grid g, double gamma,
                                                    const double* __restrict__ lamNext,
                                                    double* __restrict__ lamS,
                                                    double* __restrict__ E) {
+  begin_dependent();
   const int ni = g.n[0], nj = g.n[1], nk = g.n[2], i5 = blockIdx.y;
   const long long plane = (long long)nj * nk, N = g.N;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < plane;
@@ -810,6 +819,7 @@ __global__ void __launch_bounds__(64) k_adjbc_farfield(Grid g, double gamma,
                                                        const double* __restrict__ lamNext,
                                                        const double* __restrict__ E,
                                                        double* __restrict__ lamS) {
+  begin_dependent();
   const int ni = g.n[0], nj = g.n[1], nk = g.n[2], i5 = blockIdx.y;
   const long long count = (long long)(ni - 2) * nk, N = g.N, plane = (long long)nj * nk;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < count;
@@ -831,6 +841,7 @@ __global__ void __launch_bounds__(64) k_adjbc_farfield(Grid g, double gamma,
 // inner ring: Q(i,0,k) = mean_k S5(i,1,k), one block per axial station
 __global__ void k_adjbc_ring(Grid g, const double* __restrict__ lamNext, const double* __restrict__ E,
                              double* __restrict__ lamS) {
+  begin_dependent();
   const int i = 1 + blockIdx.x;
   const int ni = g.n[0], nk = g.n[2];
   const long long N = g.N;
@@ -869,6 +880,7 @@ __global__ void __launch_bounds__(64) k_adjbc_inflow(Grid g, AdjInflow b,
                                                      const double* __restrict__ rth,
                                                      const double* __restrict__ lamNext,
                                                      double* __restrict__ partials) {
+  begin_dependent();
   const long long plane = (long long)g.n[1] * g.n[2], N = g.N;
   const double two_pi = 6.283185307179586476925286766559;
   // cos(m theta - phi_f) = cos(m theta) cos(phi_f) + sin(m theta) sin(phi_f), as
@@ -928,6 +940,7 @@ __global__ void __launch_bounds__(64) k_adjbc_inflow(Grid g, AdjInflow b,
 // order (a warp per item; lanes take the blocks in turn)
 __global__ void k_sum_partials(const double* __restrict__ partials, int nb, int items,
                                double* __restrict__ out) {
+  begin_dependent();
   const int m = blockIdx.x, lane = threadIdx.x;
   double s = 0.0;
   for (int b = lane; b < nb; b += 32) s += partials[b * items + m];
@@ -942,6 +955,7 @@ template <typename TM>
 __global__ void k_functional(Grid g, double gamma, int j5, double dt, const TM* __restrict__ M,
                              const double* __restrict__ Q, double* __restrict__ lam,
                              double* __restrict__ partials) {
+  begin_dependent();
   const int ni = g.n[0], nk = g.n[2];
   const long long count = (long long)ni * nk, N = g.N;
   const double gm1 = gamma - 1.0;
@@ -1016,14 +1030,15 @@ void launch_rhs_vjp(const Grid& g, const les_params& p, const double* Q, const d
   const unsigned b0 = blocks((long long)chunks(0) * g.n[1] * g.n[2]);
   const unsigned b1 = blocks((long long)g.n[0] * chunks(1) * g.n[2]);
   const AdjIO io{FluxIO<double, double, double>{Q, M, node, mk, nullptr}, lamR, rec};
-  k_adj_flux3<<<f.b2 + b0 + b1, kFluxThreads, 0, L.s>>>(g, K, io, f.b2, b0, f.len);
-  k_adj_sensor_terms<<<nb_for(g.N), 256, 0, L.s>>>(g, node, rec, ST);
-  k_adj_node<<<blocks_for(g.N, 128), 128, 0, L.s>>>(g, K, Q, M, gn, node, rec, ST, lamQ, lamMK);
+  launch_dependent(k_adj_flux3, f.b2 + b0 + b1, kFluxThreads, 0, L, g, K, io, f.b2, b0, f.len);
+  launch_dependent(k_adj_sensor_terms, nb_for(g.N), 256, 0, L, g, node, rec, ST);
+  launch_dependent(k_adj_node, blocks_for(g.N, 128), 128, 0, L, g, K, Q, M, gn, node, rec, ST, lamQ,
+                   lamMK);
   *L.counter += 3;
 }
 
 void launch_mask_faces(const Grid& g, const double* lam, double* out, const Launch& L) {
-  k_mask_faces<<<nb_for(g.N), 256, 0, L.s>>>(g, lam, out);
+  launch_dependent(k_mask_faces, nb_for(g.N), 256, 0, L, g, lam, out);
   ++*L.counter;
 }
 
@@ -1031,11 +1046,13 @@ void launch_rhs_jvp(const Grid& g, const les_params& p, const Dual* Q, const dou
                     const Dual* mk, Dual* node, Dual* flux, Dual* R, const Launch& L) {
   const Consts<Dual> K = make_consts<Dual>(p);
   const int nb = nb_for(g.N);
-  k_node<Dual, Dual, double, false><<<nb, 256, 0, L.s>>>(g, K, Q, M, nullptr, node, nullptr, nullptr);
+  launch_dependent(k_node<Dual, Dual, double, false>, nb, 256, 0, L, g, K, Q, M, nullptr, node,
+                   nullptr, nullptr, nullptr, 0.0);
   const FluxPlan f = flux_plan(g);
-  k_flux3<Dual, Dual, double><<<f.b2 + f.b0 + f.b1, kFluxThreads, 0, L.s>>>(
-      g, K, FluxIO<Dual, Dual, double>{Q, M, node, mk, flux}, f.b2, f.b0, f.len, f.len);
-  k_update<Dual, double, Dual, 0><<<nb, 256, 0, L.s>>>(g, flux, nullptr, M, nullptr, 0.0, R);
+  launch_dependent(k_flux3<Dual, Dual, double>, f.b2 + f.b0 + f.b1, kFluxThreads, 0, L, g, K,
+                   FluxIO<Dual, Dual, double>{Q, M, node, mk, flux}, f.b2, f.b0, f.len, f.len);
+  launch_dependent(k_update<Dual, double, Dual, 0>, nb, 256, 0, L, g, flux, nullptr, M, nullptr,
+                   0.0, R, nullptr, nullptr);
   *L.counter += 3;
 }
 
@@ -1051,18 +1068,18 @@ void launch_unpack_dual(long long count, const Dual* in, double* v, double* d, c
 
 void launch_mu_vjp(const Grid& g, const les_params& p, const double* Q, const double* lamMK,
                    double* lamQ, const Launch& L) {
-  k_adj_mu<<<nb_for(g.N), 256, 0, L.s>>>(g, make_consts<double>(p), Q, lamMK, lamQ);
+  launch_dependent(k_adj_mu, nb_for(g.N), 256, 0, L, g, make_consts<double>(p), Q, lamMK, lamQ);
   ++*L.counter;
 }
 
 void launch_stage_prep(const Grid& g, const double* M, double coef, const double* lamS,
                        double* lamR, double* lamQ0, const Launch& L) {
-  k_adj_stage_prep<<<nb_for(g.N), 256, 0, L.s>>>(g, M, coef, lamS, lamR, lamQ0);
+  launch_dependent(k_adj_stage_prep, nb_for(g.N), 256, 0, L, g, M, coef, lamS, lamR, lamQ0);
   ++*L.counter;
 }
 
 void launch_axpy(long long count, double a, const double* x, double* y, const Launch& L) {
-  k_axpy<<<nb_for(count), 256, 0, L.s>>>(count, a, x, y);
+  launch_dependent(k_axpy, nb_for(count), 256, 0, L, count, a, x, y);
   ++*L.counter;
 }
 
@@ -1070,15 +1087,16 @@ void launch_bc_vjp(const Grid& g, const les_params& p, const double* M, const do
                    const double* S5, const double* Qnext, const double* lamNext, double t_next,
                    double* lamS, double* E, double* partials, double* grad, const Launch& L) {
   const long long plane = (long long)g.n[1] * g.n[2];
-  k_adjbc_init<<<nb_for(g.N), 256, 0, L.s>>>(g, lamNext, lamS);
+  launch_dependent(k_adjbc_init, nb_for(g.N), 256, 0, L, g, lamNext, lamS);
   auto nb64 = [](long long count) {
     const long long b = (count + 63) / 64;
     return (unsigned)(b < kAdjBlocks ? b : kAdjBlocks);
   };
-  k_adjbc_exit<<<dim3(nb64(plane), 5), 64, 0, L.s>>>(g, p.gamma, M, Qnext, lamNext, lamS, E);
-  k_adjbc_farfield<<<dim3(nb64((long long)(g.n[0] - 2) * g.n[2]), 5), 64, 0, L.s>>>(
-      g, p.gamma, M, S5, lamNext, E, lamS);
-  k_adjbc_ring<<<g.n[0] - 2, 256, 0, L.s>>>(g, lamNext, E, lamS);
+  launch_dependent(k_adjbc_exit, dim3(nb64(plane), 5), 64, 0, L, g, p.gamma, M, Qnext, lamNext,
+                   lamS, E);
+  launch_dependent(k_adjbc_farfield, dim3(nb64((long long)(g.n[0] - 2) * g.n[2]), 5), 64, 0, L, g,
+                   p.gamma, M, S5, lamNext, E, lamS);
+  launch_dependent(k_adjbc_ring, g.n[0] - 2, 256, 0, L, g, lamNext, E, lamS);
   AdjInflow in;
   in.Mj = p.Mj;
   in.r_jet = p.r_jet;
@@ -1088,8 +1106,8 @@ void launch_bc_vjp(const Grid& g, const les_params& p, const double* M, const do
   for (int i = 0; i < 4; ++i) in.St[i] = p.St[i];
   for (int i = 0; i < 16; ++i) in.amp[i] = p.amp[i];
   const unsigned nbi = nb64(plane);
-  k_adjbc_inflow<<<nbi, 64, 0, L.s>>>(g, in, rth, lamNext, partials);
-  k_sum_partials<<<16, 32, 0, L.s>>>(partials, (int)nbi, 16, grad);
+  launch_dependent(k_adjbc_inflow, nbi, 64, 0, L, g, in, rth, lamNext, partials);
+  launch_dependent(k_sum_partials, 16, 32, 0, L, partials, (int)nbi, 16, grad);
   *L.counter += 6;
 }
 
@@ -1098,8 +1116,8 @@ void launch_functional(const Grid& g, const les_params& p, int j5, double dt, co
                        const Launch& L) {
   const long long count = (long long)g.n[0] * g.n[2];
   const int nb = nb_for(count) < kAdjBlocks ? nb_for(count) : kAdjBlocks;
-  k_functional<double><<<nb, 256, 0, L.s>>>(g, p.gamma, j5, dt, M, Q, lam, partials);
-  k_sum_partials<<<1, 32, 0, L.s>>>(partials, nb, 1, Jout);
+  launch_dependent(k_functional<double>, nb, 256, 0, L, g, p.gamma, j5, dt, M, Q, lam, partials);
+  launch_dependent(k_sum_partials, 1, 32, 0, L, partials, nb, 1, Jout);
   *L.counter += 2;
 }
 
@@ -1107,8 +1125,8 @@ void launch_functional(const Grid& g, const les_params& p, int j5, double dt, co
                        const double* Q, double* partials, double* Jout, const Launch& L) {
   const long long count = (long long)g.n[0] * g.n[2];
   const int nb = nb_for(count) < kAdjBlocks ? nb_for(count) : kAdjBlocks;
-  k_functional<float><<<nb, 256, 0, L.s>>>(g, p.gamma, j5, dt, M, Q, nullptr, partials);
-  k_sum_partials<<<1, 32, 0, L.s>>>(partials, nb, 1, Jout);
+  launch_dependent(k_functional<float>, nb, 256, 0, L, g, p.gamma, j5, dt, M, Q, nullptr, partials);
+  launch_dependent(k_sum_partials, 1, 32, 0, L, partials, nb, 1, Jout);
   *L.counter += 2;
 }
 

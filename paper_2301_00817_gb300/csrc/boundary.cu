@@ -225,6 +225,7 @@ template <class Acc, typename TM>
 __global__ void __launch_bounds__(kBcThreads) k_bc_inflow(Grid g, JetBC b, const double* __restrict__ rth,
                             const TM* __restrict__ M, const DevScalars* __restrict__ sc,
                             int use_host_t, double t_host, Acc Q) {
+  begin_dependent();
   bc_inflow_part(g, b, rth, M, sc, use_host_t, t_host, Q, blockIdx.x, gridDim.x);
 }
 
@@ -306,6 +307,7 @@ __global__ void __launch_bounds__(kBcThreads)
     k_bc_sides(Grid g, JetBC b, const double* __restrict__ rth, const TM* __restrict__ M,
                const DevScalars* __restrict__ sc, int use_host_t, double t_host, Acc Q, int nb_ff,
                int nb_in) {
+  begin_dependent();
   const int blk = blockIdx.x;
   if (blk < nb_ff)
     bc_farfield_part(g, b, M, Q, blk, nb_ff);
@@ -321,6 +323,7 @@ __global__ void __launch_bounds__(kBcThreads)
 template <class Acc, typename TM>
 __global__ void __launch_bounds__(kBcThreads)
     k_bc_exit(Grid g, JetBC b, const TM* __restrict__ M, Acc Q) {
+  begin_dependent();
   const int ni = g.n[0];
   const long long plane = (long long)g.n[1] * g.n[2];
   const long long N = g.N;
@@ -369,6 +372,7 @@ struct ViewHL {
 template <class View, typename TM, bool JOIN = false>
 __global__ void k_totals_partial(Grid g, View Q, const TM* __restrict__ M,
                                  double* __restrict__ partials, double* __restrict__ qout = nullptr) {
+  begin_dependent();
   const long long N = g.N;
   double s[5] = {0, 0, 0, 0, 0};
   for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N;
@@ -404,6 +408,7 @@ __global__ void k_totals_partial(Grid g, View Q, const TM* __restrict__ M,
 }
 
 __global__ void k_totals_final(const double* __restrict__ partials, int nb, DevScalars* sc) {
+  begin_dependent();
   const int q = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (q >= 5) return;
   double v = 0.0;
@@ -456,15 +461,16 @@ static void bc_jet(const Grid& g, const les_params& p, Acc Q, const TM* M,
   if (p.bc == LES_BC_JET_CHAR && nb_in > 0) {
     // the characteristic entrance reads the plane i = 1 before the far field
     // and the ring write its edges
-    k_bc_inflow<Acc, TM><<<nb_in, kBcThreads, 0, L.s>>>(g, b, rth, M, sc, use_host_t, t_host, Q);
+    launch_dependent(k_bc_inflow<Acc, TM>, nb_in, kBcThreads, 0, L, g, b, rth, M, sc, use_host_t,
+                     t_host, Q);
     ++*L.counter;
     nb_in = 0;
   }
-  k_bc_sides<Acc, TM><<<nb_ff + nb_in + (g.n[0] - 2), kBcThreads, 0, L.s>>>(
-      g, b, rth, M, sc, use_host_t, t_host, Q, nb_ff, nb_in);
+  launch_dependent(k_bc_sides<Acc, TM>, nb_ff + nb_in + (g.n[0] - 2), kBcThreads, 0, L, g, b, rth,
+                   M, sc, use_host_t, t_host, Q, nb_ff, nb_in);
   ++*L.counter;
   if (g.ghi == 0) {
-    k_bc_exit<Acc, TM><<<nblocks(plane), kBcThreads, 0, L.s>>>(g, b, M, Q);
+    launch_dependent(k_bc_exit<Acc, TM>, nblocks(plane), kBcThreads, 0, L, g, b, M, Q);
     ++*L.counter;
   }
 }
@@ -495,8 +501,8 @@ template <class View, typename TM>
 static void totals_t(const Grid& g, View Q, const TM* M, double* partials, DevScalars* sc,
                      const Launch& L) {
   const int nb = red_blocks(g.N);
-  k_totals_partial<View, TM><<<nb, kRedThreads, 0, L.s>>>(g, Q, M, partials);
-  k_totals_final<<<1, 160, 0, L.s>>>(partials, nb, sc);
+  launch_dependent(k_totals_partial<View, TM>, nb, kRedThreads, 0, L, g, Q, M, partials, nullptr);
+  launch_dependent(k_totals_final, 1, 160, 0, L, partials, nb, sc);
   *L.counter += 2;
 }
 
@@ -524,9 +530,9 @@ template <typename TM>
 static void join_totals_t(const Grid& g, const float* hi, const float* lo, const TM* M, double* q,
                           double* partials, DevScalars* sc, const Launch& L) {
   const int nb = red_blocks(g.N);
-  k_totals_partial<ViewHL, TM, true><<<nb, kRedThreads, 0, L.s>>>(g, ViewHL{hi, lo}, M, partials,
-                                                                   q);
-  k_totals_final<<<1, 160, 0, L.s>>>(partials, nb, sc);
+  launch_dependent(k_totals_partial<ViewHL, TM, true>, nb, kRedThreads, 0, L, g, ViewHL{hi, lo}, M,
+                   partials, q);
+  launch_dependent(k_totals_final, 1, 160, 0, L, partials, nb, sc);
   *L.counter += 2;
 }
 

@@ -113,6 +113,7 @@ __device__ constexpr int j6(int k) { return k < 3 ? k : (k == 3 ? 1 : 2); }
 __global__ void __launch_bounds__(256) k_dyn_node(long long N, float gamma, float gm1,
                                                   const float* __restrict__ Q,
                                                   float* __restrict__ node) {
+  begin_dependent();
   for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N;
        n += (long long)gridDim.x * blockDim.x) {
     const float rho = Q[n], ir = 1.f / rho;
@@ -133,6 +134,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_dyn_products(Gr
                                                       const TM* __restrict__ M,
                                                       const R* __restrict__ node,
                                                       R* __restrict__ D) {
+  begin_dependent();
   const long long N = g.N;
   for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N;
        n += (long long)gridDim.x * blockDim.x) {
@@ -175,6 +177,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_dyn_products(Gr
 template <int D, typename R>
 __global__ void __launch_bounds__(256) k_dyn_filter1(Grid g, const R* __restrict__ src,
                                                      int count, R* __restrict__ dst) {
+  begin_dependent();
   const long long N = g.N;
   const long long s = g.stride[D];
   const int nd = g.n[D];
@@ -210,6 +213,7 @@ constexpr int kF3J = 4, kF3K = 32, kF3R = 2;  // 128 threads: 8 rows x 32 column
 template <typename R>
 __global__ void __launch_bounds__(kF3J * kF3K) k_dyn_filter3(Grid g, const R* __restrict__ src,
                                                              int fields, R* __restrict__ dst) {
+  begin_dependent();
   const long long N = g.N;
   const int ni = g.n[0], nj = g.n[1], nk = g.n[2];
   const int tx = threadIdx.x % kF3K, ty = threadIdx.x / kF3K;
@@ -283,6 +287,7 @@ __global__ void __launch_bounds__(kF3J * kF3K) k_dyn_filter3(Grid g, const R* __
 template <typename R>
 __global__ void __launch_bounds__(256) k_dyn_favre(long long N, const R* __restrict__ F,
                                                    R* __restrict__ H) {
+  begin_dependent();
   for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N;
        n += (long long)gridDim.x * blockDim.x) {
     const R ir = R(1) / F[n];
@@ -299,6 +304,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 1) k_dyn_sums(Grid g
                                                   const R* __restrict__ Fh,
                                                   const R* __restrict__ H,
                                                   double* __restrict__ partials) {
+  begin_dependent();
   const long long N = g.N;
   double acc[kDynSums] = {0, 0, 0, 0, 0, 0, 0};
   for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N;
@@ -387,6 +393,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 1) k_dyn_sums(Grid g
 // One block of kDynSums warps: warp q totals partial array q in a fixed order.
 __global__ void k_dyn_final(const double* __restrict__ partials, double pr_default,
                             DevScalars* __restrict__ sc) {
+  begin_dependent();
   __shared__ double tot[kDynSums];
   const int q = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (q < kDynSums) {
@@ -420,7 +427,7 @@ static void dynamic_t(const Grid& g, const les_params& p, const TQ* Q, const TM*
   const int th = 256, nb = blocks_for(g.N, th);
   R* D = scratch;                                 // products, then the eta pass
   R* T = scratch + (long long)kDynFields * g.N;  // zeta pass, then the filtered fields
-  k_dyn_products<R, TQ, TM><<<nb, th, 0, L.s>>>(g, Q, M, node, D);
+  launch_dependent(k_dyn_products<R, TQ, TM>, nb, th, 0, L, g, Q, M, node, D);
   if constexpr (sizeof(R) == 4) {
     // FP32 fields: the test filter in one pass (k_dyn_filter3), with enough
     // axial chunks for some sixty CTAs per SM (each reads two planes more
@@ -431,20 +438,20 @@ static void dynamic_t(const Grid& g, const les_params& p, const TQ* Q, const TM*
     const long long most = g.n[0] / 12 > 1 ? g.n[0] / 12 : 1;
     long long nch = (want + tiles - 1) / tiles;
     nch = nch < 1 ? 1 : (nch > most ? most : nch);
-    k_dyn_filter3<R><<<dim3((unsigned)tk, (unsigned)tj, (unsigned)(nch * kDynFields)), kF3J * kF3K, 0,
-                       L.s>>>(g, D, kDynFields, T);
+    launch_dependent(k_dyn_filter3<R>, dim3((unsigned)tk, (unsigned)tj,
+                     (unsigned)(nch * kDynFields)), kF3J * kF3K, 0, L, g, D, kDynFields, T);
     *L.counter += 1;
   } else {
     // FP64 fields: three one-direction passes (the one-pass kernel is bound
     // by its FP64 work and latency there: 1.24 against 0.86 ms on 1.97M points)
-    k_dyn_filter1<2, R><<<nb, th, 0, L.s>>>(g, D, kDynFields, T);
-    k_dyn_filter1<1, R><<<nb, th, 0, L.s>>>(g, T, kDynFields, D);
-    k_dyn_filter1<0, R><<<nb, th, 0, L.s>>>(g, D, kDynFields, T);
+    launch_dependent(k_dyn_filter1<2, R>, nb, th, 0, L, g, D, kDynFields, T);
+    launch_dependent(k_dyn_filter1<1, R>, nb, th, 0, L, g, T, kDynFields, D);
+    launch_dependent(k_dyn_filter1<0, R>, nb, th, 0, L, g, D, kDynFields, T);
     *L.counter += 3;
   }
-  k_dyn_favre<R><<<nb, th, 0, L.s>>>(g.N, T, D);  // D is free again: u^, v^, w^, T^
-  k_dyn_sums<R, TM><<<kRedBlocks, kRedThreads, 0, L.s>>>(g, M, node, T, D, partials);
-  k_dyn_final<<<1, 32 * kDynSums, 0, L.s>>>(partials, p.Pr_sgs, sc);
+  launch_dependent(k_dyn_favre<R>, nb, th, 0, L, g.N, T, D);  // D is free again: u^, v^, w^, T^
+  launch_dependent(k_dyn_sums<R, TM>, kRedBlocks, kRedThreads, 0, L, g, M, node, T, D, partials);
+  launch_dependent(k_dyn_final, 1, 32 * kDynSums, 0, L, partials, p.Pr_sgs, sc);
   *L.counter += 4;
 }
 
@@ -457,7 +464,7 @@ void launch_dynamic32(const Grid& g, const les_params& p, const float* Q, const 
                       float* node, float* scratch, double* partials, DevScalars* sc,
                       const Launch& L) {
   const int th = 256, nb = blocks_for(g.N, th);
-  k_dyn_node<<<nb, th, 0, L.s>>>(g.N, (float)p.gamma, (float)(p.gamma - 1.0), Q, node);
+  launch_dependent(k_dyn_node, nb, th, 0, L, g.N, (float)p.gamma, (float)(p.gamma - 1.0), Q, node);
   ++*L.counter;
   dynamic_t<float, float, float>(g, p, Q, M, node, scratch, partials, sc, L);
 }

@@ -196,6 +196,13 @@ __device__ __forceinline__ double widen(double x) { return x; }
 __device__ __forceinline__ double dev_fma(double a, double b, double c) { return fma(a, b, c); }
 __device__ __forceinline__ double dev_mul(double a, double b) { return __dmul_rn(a, b); }
 
+// First statement of every kernel that launch_dependent starts: nothing runs on
+// before the kernel ahead of it has finished and its writes are visible.  (In
+// a launch without the attribute it returns at once.)
+__device__ __forceinline__ void begin_dependent() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // ----------------------------------------------------------------- Philox
 // Philox4x32-10 (Salmon, Moraes, Dror, Shaw, SC'11): ten rounds of two
 // 32x32->64 multiplies with the round multipliers, word swap, xor with the
@@ -227,6 +234,32 @@ struct Launch {
   unsigned long long* counter;
 };
 
+// A launch whose blocks may take their places, and fetch their code and
+// arguments, while the kernel ahead of it in the stream drains; they wait for
+// its end in begin_dependent.  For the FP64 and adjoint paths, 18 launches and
+// more a step in series: the gap between two was a tenth of the 48 x 24 x 32
+// step (323 -> 285 us; the adjoint window on 64 x 40 x 48 30.8 -> 29.5 ms).
+// Letting the next kernel start before the last block of this one (an early
+// trigger) was slower everywhere, its waiting blocks taking SM places, and
+// the mixed step's graph, whose edges are cheap, gains nothing: its kernels
+// are launched plainly.  Every kernel that is launched so begins with
+// begin_dependent, so the end of one implies that of all before it.
+template <typename... P, typename... A>
+inline void launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
+                             const Launch& L, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = L.s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // On a grid with an axis (Reading A27) an axis node's SGS viscosity is the
 // azimuthal mean of ring 1's at its plane, summed in increasing k; its
 // laminar part is its own.  One block per plane i, after k_mu (or the mixed
@@ -239,6 +272,7 @@ __device__ __forceinline__ R mu_laminar(const Consts<R>& K, R T) {
 
 template <typename R, class TempOf>
 __global__ void k_mu_axis(Grid g, Consts<R> K, TempOf T, R* __restrict__ mk) {
+  begin_dependent();
   extern __shared__ __align__(16) unsigned char smu_raw[];
   R* smu = reinterpret_cast<R*>(smu_raw);
   const int nk = g.n[2];

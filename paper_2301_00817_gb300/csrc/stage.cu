@@ -16,6 +16,7 @@ static int blocks_for(long long count, int threads, long long cap = 0) {
 // Fixed-order minimum over the block partials, then dt and t^{n+1}.
 __global__ void k_dt_finalize(const double* __restrict__ partials, int nparts, int mode,
                               double cfl, double dt_fixed, int advance, DevScalars* sc) {
+  begin_dependent();
   __shared__ double sm[32];
   double m = 1.0e300;
   for (int i = threadIdx.x; i < nparts; i += blockDim.x) m = fmin(m, partials[i]);
@@ -43,6 +44,7 @@ __global__ void k_dt_finalize(const double* __restrict__ partials, int nparts, i
 }
 
 __global__ void k_set_dt(DevScalars* sc, double dt) {
+  begin_dependent();
   if (threadIdx.x == 0 && blockIdx.x == 0) {
     sc->dt = dt;
     sc->t += dt;
@@ -51,7 +53,7 @@ __global__ void k_set_dt(DevScalars* sc, double dt) {
 }
 
 void launch_set_dt(DevScalars* sc, double dt, const Launch& L) {
-  k_set_dt<<<1, 32, 0, L.s>>>(sc, dt);
+  launch_dependent(k_set_dt, 1, 32, 0, L, sc, dt);
   ++*L.counter;
 }
 
@@ -66,8 +68,8 @@ __global__ void k_cast_to_double(long long count, const R* __restrict__ a, doubl
 
 void launch_dt_finalize(const les_params& p, double* partials, DevScalars* sc, int advance,
                         const Launch& L) {
-  k_dt_finalize<<<1, 1024, 0, L.s>>>(partials, kRedBlocks, p.dt_mode, p.cfl, p.dt_fixed, advance,
-                                     sc);
+  launch_dependent(k_dt_finalize, 1, 1024, 0, L, partials, kRedBlocks, p.dt_mode, p.cfl, p.dt_fixed,
+                   advance, sc);
   ++*L.counter;
 }
 

@@ -31,11 +31,11 @@ void launch_node64(const Grid& g, const les_params& p, const StageIO64& io, bool
   const int nb = with_dt ? red_blocks(g.N) : blocks_for(g.N, th);
   auto K = make_consts<double>(p);
   if (with_dt)
-    k_node<double, double, double, true><<<nb, th, 0, L.s>>>(g, K, io.Qin, io.M, io.gn, io.node,
-                                                             io.partials, io.sc, io.dtl, p.cfl);
+    launch_dependent(k_node<double, double, double, true>, nb, th, 0, L, g, K, io.Qin, io.M, io.gn,
+                     io.node, io.partials, io.sc, io.dtl, p.cfl);
   else
-    k_node<double, double, double, false><<<nb, th, 0, L.s>>>(g, K, io.Qin, io.M, io.gn, io.node,
-                                                              io.partials, io.sc);
+    launch_dependent(k_node<double, double, double, false>, nb, th, 0, L, g, K, io.Qin, io.M, io.gn,
+                     io.node, io.partials, io.sc, nullptr, 0.0);
   ++*L.counter;
 }
 
@@ -47,12 +47,12 @@ void launch_mu64(const Grid& g, const les_params& p, const StageIO64& io, const 
     dyn = reinterpret_cast<const double*>(reinterpret_cast<const char*>(io.sc) +
                                           offsetof(DevScalars, dyn));
   }
-  k_mu<double, double, double><<<nb, th, 0, L.s>>>(g, make_consts<double>(p), io.Qin, io.M,
-                                                    io.node, io.mk, io.gn + 4 * g.N, dyn);
+  launch_dependent(k_mu<double, double, double>, nb, th, 0, L, g, make_consts<double>(p), io.Qin,
+                   io.M, io.node, io.mk, io.gn + 4 * g.N, dyn);
   ++*L.counter;
   if (p.axis) {
-    k_mu_axis<double, TempFromNode<double>><<<g.n[0], 128, g.n[2] * sizeof(double), L.s>>>(
-        g, make_consts<double>(p), TempFromNode<double>{io.node, g.N}, io.mk);
+    launch_dependent(k_mu_axis<double, TempFromNode<double>>, g.n[0], 128, g.n[2] * sizeof(double),
+                     L, g, make_consts<double>(p), TempFromNode<double>{io.node, g.N}, io.mk);
     ++*L.counter;
   }
 }
@@ -60,8 +60,8 @@ void launch_mu64(const Grid& g, const les_params& p, const StageIO64& io, const 
 void launch_flux64(const Grid& g, const les_params& p, const StageIO64& io, const Launch& L) {
   const FluxPlan f = flux_plan(g);
   const FluxIO<double, double, double> fio{io.Qin, io.M, io.node, io.mk, io.flux};
-  k_flux3<double, double, double><<<f.b2 + f.b0 + f.b1, kFluxThreads, 0, L.s>>>(
-      g, make_consts<double>(p), fio, f.b2, f.b0, f.len, f.len);
+  launch_dependent(k_flux3<double, double, double>, f.b2 + f.b0 + f.b1, kFluxThreads, 0, L, g,
+                   make_consts<double>(p), fio, f.b2, f.b0, f.len, f.len);
   ++*L.counter;
 }
 
@@ -69,13 +69,14 @@ void launch_update64(const Grid& g, const StageIO64& io, const double* Q0, doubl
                      double* out, const Launch& L) {
   const int th = 256, nb = blocks_for(g.N, th);
   if (mode == 0)
-    k_update<double, double, double, 0><<<nb, th, 0, L.s>>>(g, io.flux, Q0, io.M, io.sc, alpha, out, io.dtl);
+    launch_dependent(k_update<double, double, double, 0>, nb, th, 0, L, g, io.flux, Q0, io.M, io.sc,
+                     alpha, out, io.dtl, nullptr);
   else if (mode == 1)
-    k_update<double, double, double, 1><<<nb, th, 0, L.s>>>(g, io.flux, Q0, io.M, io.sc, alpha, out, io.dtl,
-                                                            io.gn ? io.gn + 3 * g.N : nullptr);
+    launch_dependent(k_update<double, double, double, 1>, nb, th, 0, L, g, io.flux, Q0, io.M, io.sc,
+                     alpha, out, io.dtl, io.gn ? io.gn + 3 * g.N : nullptr);
   else
-    k_update<double, double, double, 2><<<nb, th, 0, L.s>>>(g, io.flux, Q0, io.M, io.sc, alpha, out, io.dtl,
-                                                            io.gn ? io.gn + 3 * g.N : nullptr);
+    launch_dependent(k_update<double, double, double, 2>, nb, th, 0, L, g, io.flux, Q0, io.M, io.sc,
+                     alpha, out, io.dtl, io.gn ? io.gn + 3 * g.N : nullptr);
   ++*L.counter;
 }
 

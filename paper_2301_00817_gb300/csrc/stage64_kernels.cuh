@@ -58,6 +58,7 @@ __global__ void __launch_bounds__(256) k_node(Grid g, Consts<R> K, const TQ* __r
                                               DevScalars* __restrict__ sc,
                                               double* __restrict__ dtl = nullptr,
                                               double cfl = 0.0) {
+  begin_dependent();
   const long long N = g.N;
   double local_min = 1.0e300;
   int bad = 0;
@@ -175,6 +176,7 @@ __global__ void __launch_bounds__(256) k_mu(Grid g, Consts<R> K, const TQ* __res
                                             const R* __restrict__ node, R* __restrict__ mk,
                                             const double* __restrict__ del2,
                                             const double* __restrict__ dyn = nullptr) {
+  begin_dependent();
   const long long N = g.N;
   for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N;
        n += (long long)gridDim.x * blockDim.x) {
@@ -608,6 +610,7 @@ template <typename R, typename TQ, typename TM>
 __global__ void __launch_bounds__(kFluxThreads, sizeof(R) == 8 ? 2 : 1)
     k_flux3(Grid g, Consts<R> K, FluxIO<R, TQ, TM> io, unsigned b2, unsigned b0, int len0,
             int len1) {
+  begin_dependent();
   __shared__ R sh[14][kFluxThreads];
   unsigned b = blockIdx.x;
   if (b < b2) {
@@ -649,6 +652,7 @@ __global__ void __launch_bounds__(256) k_update(Grid g, const R* __restrict__ F,
                                                 TO* __restrict__ out,
                                                 const double* __restrict__ dtl = nullptr,
                                                 const double* __restrict__ jh = nullptr) {
+  begin_dependent();
   const long long N = g.N;
   const R* F0 = F;
   const R* F1 = F + 5 * N;
