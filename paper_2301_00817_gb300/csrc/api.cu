@@ -1179,7 +1179,7 @@ void adj_reverse(les_ctx* c, void* aw, const AdjLayout& Ly, double* const S[6], 
   cudaMemsetAsync(lamQ0, 0, bytes, s);
   cudaMemsetAsync(lamMK, 0, 2 * (size_t)g.N * sizeof(double), s);
   for (int l = 5; l >= 1; --l) {
-    lesjet::launch_stage_prep(g, M, kAlpha[l - 1] * dt, lamS, lamR, lamQ0, L);
+    lesjet::launch_stage_prep(g, io.gn + 3 * g.N, kAlpha[l - 1] * dt, lamS, lamR, lamQ0, L);
     io.Qin = S[l - 1];
     if (nodes)
       io.node = const_cast<double*>(nodes) + (size_t)(l - 1) * 8 * g.N;  // kept by adj_forward

@@ -108,7 +108,7 @@ void launch_rhs_jvp(const Grid& g, const les_params& p, const Dual* Q, const dou
                     const Dual* mk, Dual* node, Dual* flux, Dual* R, const Launch& L);
 void launch_mu_vjp(const Grid& g, const les_params& p, const double* Q, const double* lamMK,
                    double* lamQ, const Launch& L);
-void launch_stage_prep(const Grid& g, const double* M, double coef, const double* lamS,
+void launch_stage_prep(const Grid& g, const double* jh, double coef, const double* lamS,
                        double* lamR, double* lamQ0, const Launch& L);
 void launch_axpy(long long count, double a, const double* x, double* y, const Launch& L);
 void launch_bc_vjp(const Grid& g, const les_params& p, const double* M, const double* rth,
