@@ -27,6 +27,7 @@
 #include <map>
 #include <mutex>
 #include <queue>
+#include <type_traits>
 #include <utility>
 #include <vector>
 
@@ -496,6 +497,10 @@ __device__ __forceinline__ void dphi_tangent(const float4 ap, const float4 am, c
   dphi[3][T] = (ap.w - am.w) + (bp.w - bm.w);
 }
 
+__device__ __forceinline__ void cp_async8(void* smem, const void* gmem) {
+  const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(s), "l"(gmem) : "memory");
+}
 __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
   const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(gmem) : "memory");
@@ -595,127 +600,76 @@ __global__ void __launch_bounds__(FTJ * FTK, 1)
   const int o1 = (ty + 1) * SK + tx + 2;  // own node, 1-node-halo planes
 
   // ---- stage plane x (state: 2-node halo; metrics, mu/kappa: 1-node halo)
-  // Rows that cannot go as 16-byte pieces (nk % 4 != 0, an open zeta, nk <
-  // FTK): a warp copies a row, one 4-byte cp.async per lane, so a request
-  // covers 128 contiguous bytes; the halo columns of all rows follow, spread
-  // over the threads.  (One thread per row, 36 copies in series and none of
-  // them coalesced, had made such a grid's stage four times the time per
-  // point of an aligned one: 242 us on 131 x 75 x 83.)  The lane's wrapped
-  // columns and the warp's rows do not change from plane to plane.
-  const int jr_q = vec_ok ? 0 : wrap_fast(j0 + ty - 2, nj, per1);
-  const int jr_m = vec_ok ? 0 : wrap_fast(j0 + ty - 1, nj, per1);
-  const int kr = vec_ok ? 0 : wrap_fast(k0 + tx, nk, per2);
-  auto put = [&](float* dst, const float* src, int ig, int jg, int kg, float benign) {
-    if (ig >= 0 && jg >= 0 && kg >= 0)
-      cp_async4(dst, src + ((ig * nj + jg) * nk + kg));
-    else
-      *dst = benign;
-  };
-  auto stage_rows = [&](int slot, int ig) {
-    float* dq = sQ + slot * 5 * PL2;
-    float* dm = sM + slot * 10 * PL1;
-    float* dk = sK + slot * NKF * PL1;
-    // tile rows -2 .. FTJ - 3 (state) and -1 .. FTJ - 2 (metrics, mu/kappa)
-    const int c2 = ty * SK + colk(tx);
+  // A lane takes one piece of a row, of the five state fields, of metrics 0 ..
+  // 5 or of metrics 6 .. 9 and the viscosities: neighbouring lanes copy
+  // neighbouring pieces, so a request covers whole rows, and a row's address
+  // is formed once for five or six copies.  (One thread a row, nine copies in
+  // series and 32 rows to a request, had taken 288 x 160 x 128 2.26 ms a step
+  // and 48 x 24 x 32 71 us, this 2.01 ms and 61.)  Pieces are of VW floats: 4
+  // with the shifted tiles, else 2 where nk is even (no piece straddles the
+  // ends of a row then) or 1.  An incomplete round is left to the highest-
+  // numbered threads: the lowest ones derive a second node record in the same
+  // phase.
+  auto stage_pieces = [&](auto vw, int slot, int ig) {
+    constexpr int VW = decltype(vw)::value;
+    constexpr int PC = SK / VW, UQ = R2 * PC, UM = R1 * PC, NU = UQ + 2 * UM;
+#pragma unroll 1
+    for (int b = NU - FNT; b > -FNT; b -= FNT) {
+      const int u = b + tid;
+      if (u < 0) continue;
+      const bool st = u < UQ, hi = u >= UQ + UM;
+      const int x = st ? u : (hi ? u - UQ - UM : u - UQ);
+      const int row = x / PC, pc = x - row * PC;
+      const int jg = wrap_fast(j0 + row - (st ? 2 : 1), nj, per1);
+      // shifted tiles: columns kt .. kt + SK - 1, which in the last tile wrap
+      // at nk (kt + SK < 2 nk because nk >= FTK); else kt - 2 .. kt + SK - 3
+      int kg;
+      if (VW == 4)
+        kg = kt + 4 * pc < nk ? kt + 4 * pc : kt + 4 * pc - nk;
+      else
+        kg = wrap_fast(kt - 2 + VW * pc, nk, per2);
+      const bool in = ig >= 0 && jg >= 0 && kg >= 0;
+      const int n = (ig * nj + jg) * nk + kg, d = row * SK + VW * pc;
+      auto piece = [&](float* dst, const float* src, float benign) {
+        if (in) {
+          if (VW == 4)
+            cp_async16(dst, src);
+          else if (VW == 2)
+            cp_async8(dst, src);
+          else
+            cp_async4(dst, src);
+        } else {
 #pragma unroll
-    for (int f = 0; f < 5; ++f)
-      put(dq + f * PL2 + c2, P.qin[0] + (long long)f * G.N, ig, jr_q, kr,
-          (f == 0 || f == 4) ? 1.f : 0.f);
+          for (int c = 0; c < VW; ++c) dst[c] = benign;
+        }
+      };
+      if (st) {
 #pragma unroll
-    for (int f = 0; f < 10; ++f)
-      put(dm + f * PL1 + c2, P.m[0] + (long long)f * G.N, ig, jr_m, kr, 1.f);
+        for (int f = 0; f < 5; ++f)
+          piece(sQ + (slot * 5 + f) * PL2 + d, P.qin[0] + (long long)f * G.N + n,
+                (f == 0 || f == 4) ? 1.f : 0.f);
+      } else if (!hi) {
 #pragma unroll
-    for (int f = 0; f < NKF; ++f)
-      put(dk + f * PL1 + c2, P.mk[0] + (long long)f * G.N, ig, jr_m, kr, 0.f);
-    // the rows left: four of each state field, two of each other one
-    constexpr int XQ = 4 * 5, XM = 2 * 10, XK = 2 * NKF;
-    for (int r = ty; r < XQ + XM + XK; r += FTJ) {
-      if (r < XQ) {
-        const int f = r >> 2, jj = FTJ - 2 + (r & 3);
-        put(dq + f * PL2 + (jj + 2) * SK + colk(tx), P.qin[0] + (long long)f * G.N, ig,
-            wrap_fast(j0 + jj, nj, per1), kr, (f == 0 || f == 4) ? 1.f : 0.f);
+        for (int f = 0; f < 6; ++f)
+          piece(sM + (slot * 10 + f) * PL1 + d, P.m[0] + (long long)f * G.N + n, 1.f);
       } else {
-        const bool met = r < XQ + XM;
-        const int u = met ? r - XQ : r - XQ - XM, f = u >> 1, jj = FTJ - 1 + (u & 1);
-        put((met ? dm : dk) + f * PL1 + (jj + 1) * SK + colk(tx),
-            (met ? P.m[0] : P.mk[0]) + (long long)f * G.N, ig, wrap_fast(j0 + jj, nj, per1), kr,
-            met ? 1.f : 0.f);
-      }
-    }
-    // halo columns: -2, -1, FTK, FTK + 1 of the state rows, -1 and FTK of the others
-    constexpr int HQ = 5 * R2 * 4, HM = 10 * R1 * 2, HK = NKF * R1 * 2;
-    for (int e = tid; e < HQ + HM + HK; e += FNT) {
-      if (e < HQ) {
-        const int h = e & 3, row = e >> 2, f = row / R2, jj = row - f * R2 - 2;
-        const int kk = h < 2 ? h - 2 : FTK + h - 2;
-        put(dq + f * PL2 + (jj + 2) * SK + colk(kk), P.qin[0] + (long long)f * G.N, ig,
-            wrap_fast(j0 + jj, nj, per1), wrap_fast(k0 + kk, nk, per2),
-            (f == 0 || f == 4) ? 1.f : 0.f);
-      } else {
-        const bool met = e < HQ + HM;
-        const int u = met ? e - HQ : e - HQ - HM;
-        const int row = u >> 1, f = row / R1, jj = row - f * R1 - 1, kk = (u & 1) ? FTK : -1;
-        put((met ? dm : dk) + f * PL1 + (jj + 1) * SK + colk(kk),
-            (met ? P.m[0] : P.mk[0]) + (long long)f * G.N, ig, wrap_fast(j0 + jj, nj, per1),
-            wrap_fast(k0 + kk, nk, per2), met ? 1.f : 0.f);
+#pragma unroll
+        for (int f = 6; f < 10; ++f)
+          piece(sM + (slot * 10 + f) * PL1 + d, P.m[0] + (long long)f * G.N + n, 1.f);
+#pragma unroll
+        for (int f = 0; f < NKF; ++f)
+          piece(sK + (slot * NKF + f) * PL1 + d, P.mk[0] + (long long)f * G.N + n, 0.f);
       }
     }
   };
   auto stage_plane = [&](int slot, int x) {
     const int ig = wrap_fast(x, ni, per0);
-    if (!vec_ok) {
-      stage_rows(slot, ig);
-      return;
-    }
-    constexpr int JQ = 5 * R2, JM = 10 * R1, JK = NKF * R1;
-    // one row per thread, taken by the highest-numbered threads: the lowest
-    // ones derive a second node record in the same phase
-    const int tid = threadIdx.x - (FNT - (JQ + JM + JK));
-    if (tid < 0) return;
-    const float* src;
-    float* dst;
-    int jj;
-    float benign;
-    if (tid < JQ) {
-      const int f = tid / R2;
-      jj = tid - f * R2 - 2;
-      src = P.qin[0] + (long long)f * G.N;
-      dst = sQ + (slot * 5 + f) * PL2 + (jj + 2) * SK;
-      benign = (f == 0 || f == 4) ? 1.f : 0.f;
-    } else if (tid < JQ + JM) {
-      const int u = tid - JQ, f = u / R1;
-      jj = u - f * R1 - 1;
-      src = P.m[0] + (long long)f * G.N;
-      dst = sM + (slot * 10 + f) * PL1 + (jj + 1) * SK;
-      benign = 1.f;
-    } else {
-      const int u = tid - JQ - JM, f = u / R1;
-      jj = u - f * R1 - 1;
-      src = P.mk[0] + (long long)f * G.N;
-      dst = sK + (slot * NKF + f) * PL1 + (jj + 1) * SK;
-      benign = 0.f;
-    }
-    const int jg = wrap_fast(j0 + jj, nj, per1);
-    if (ig < 0 || jg < 0) {
-      for (int c = 0; c < SK; ++c) dst[c] = benign;
-      return;
-    }
-    const float* row = src + (ig * nj + jg) * nk;
-    if (kt + SK <= nk) {
-      // the row's global columns kt .. kt + SK - 1, inside the row
-      const float* rk = row + kt;
-#pragma unroll
-      for (int v = 0; v < SK / 4; ++v) cp_async16(dst + 4 * v, rk + 4 * v);
-    } else {
-      // the last tile: columns kt .. kt + SK - 1 wrapped at nk (a multiple
-      // of 4, so no 16-byte piece straddles the wrap; kt + SK < 2 nk because
-      // nk >= FTK)
-#pragma unroll
-      for (int v = 0; v < SK / 4; ++v) {
-        const int kg = (kt + 4 * v < nk) ? kt + 4 * v : kt + 4 * v - nk;
-        cp_async16(dst + 4 * v, row + kg);
-      }
-    }
+    if (vec_ok)
+      stage_pieces(std::integral_constant<int, 4>{}, slot, ig);
+    else if ((nk & 1) == 0)
+      stage_pieces(std::integral_constant<int, 2>{}, slot, ig);
+    else
+      stage_pieces(std::integral_constant<int, 1>{}, slot, ig);
   };
 
   // ---- primitives (2-node halo) and lbar (1-node halo) of a staged plane
