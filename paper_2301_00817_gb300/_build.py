@@ -24,7 +24,7 @@ NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xptxas"
 # square root (FP64 code is unaffected by these flags).
 _FAST_FP32 = ["-prec-div=false", "-prec-sqrt=false", "-ftz=true"]
 FILE_FLAGS = {f: _FAST_FP32 for f in ("fused.cu", "fused_jet4.cu", "fused_jet4s.cu", "fused_jet12.cu",
-                                   "fused_jet12s.cu", "fused_jet28.cu")}
+                                   "fused_jet28.cu")}
 
 
 def _nvcc() -> str:

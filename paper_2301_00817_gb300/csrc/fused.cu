@@ -1,6 +1,5 @@
 // fused.cu -- launchers of the FP32-mixed form: the fused stage kernel
-// (fused_kernel.cuh; the jet-grid instantiations in fused_jet4.cu,
-// fused_jet12.cu and fused_jet28.cu), the once-per-step viscosity/CFL pass (k_prestep, and
+// (fused_kernel.cuh; the jet-grid instantiations in fused_jet*.cu), the once-per-step viscosity/CFL pass (k_prestep, and
 // its four-node form k_prestep4 here) and the split and join of the
 // float-pair state.  Built with approximate FP32 division and
 // square root.
@@ -327,18 +326,38 @@ void launch_prestep(const Grid& g, const les_params& p, const float* Q0, const f
   }
 }
 
-// Rows of the fused stage's tiles.  A plane of an 8-row tile costs 0.66 of a
-// 16-row one's (its warps wait less for one another, but its halo is twice
-// the share), so 8 rows win where they let the schedule finish earlier by
-// that factor: on grids with about a plane per SM or less, whose stage is
-// mostly latency (us a step with 16 and with 8 rows: 48 x 24 x 32 94 and 76, 96
-// x 24 x 32 122 and 93, 96 x 32 x 32 121 and 109; 64 x 64 x 64 178 and 178, 192
-// x 64 x 64 375 and 422).  Both give the same bits.
-static int tile_rows(const FusedGeom& G) {
+// Tile rows of the fused stage and the CTAs per SM its chunks are scheduled for.
+// - Two 8-row CTAs march through two planes in the time that one 16-row CTA
+//   takes for one, or less: their halo is a greater share, but one's barriers
+//   and staging hide behind the other, and they cover eta with fewer rows
+//   (us a step with 16 and with 2 x 8 rows: 64 x 64 x 64 150 and 149, 192 x 64 x 64
+//   324 and 318, 288 x 160 x 128 2010 and 1958, 576 x 320 x 256 15392 and 14375; 300
+//   x 120 x 96 1355 and 1168).
+// - One 16-row CTA where rows take no 16-byte pieces, the schedule is no
+//   longer for it and the grid is small (131 x 75 x 83 466 and 480, 97 x 40 x 61
+//   184 and 189; but 250 x 96 x 111 1390 and 1379, 300 x 250 x 510 16181 and 15396,
+//   96 x 56 x 75, whose schedule is longer, 296 and 277).
+// - One 8-row CTA on grids with about a plane per SM or less, whose stage is
+//   mostly latency: its plane costs 0.69 of one of two CTAs' (2 x 8 and 8: 64 x
+//   24 x 32 75 and 73, 96 x 32 x 32 98 and 88, 40 x 40 x 64 100 and 92; 64 x 64 x 64 149
+//   and 152, 128 x 64 x 64 221 and 297).
+// All give the same bits.
+struct TileForm {
+  int rows, ctas;
+};
+
+static TileForm tile_form(const FusedGeom& G) {
   const int sms = sm_count(), tk = (G.nk + FTK - 1) / FTK;
-  const int t16 = tk * ((G.nj + 15) / 16), t8 = tk * ((G.nj + 7) / 8);
-  if ((long long)t16 * G.ni > 4LL * sms) return 16;  // (no grid of that size gains)
-  return 0.66 * choose_chunks(G.ni, t8, sms).t < choose_chunks(G.ni, t16, sms).t ? 8 : 16;
+  const int r16 = (G.nj + 15) / 16, r8 = (G.nj + 7) / 8;
+  TileForm f{8, 2};
+  if (!G.vec16 && G.N < 1 << 20 &&
+      choose_chunks(G.ni, tk * r8, 2 * sms).t >= choose_chunks(G.ni, tk * r16, sms).t)
+    f = {16, 1};
+  if ((long long)tk * r8 * G.ni <= 8LL * sms &&
+      0.69 * choose_chunks(G.ni, tk * r8, sms).t <
+          choose_chunks(G.ni, tk * (f.rows == 8 ? r8 : r16), f.ctas * sms).t)
+    return {8, 1};
+  return f;
 }
 
 void launch_stage_fused(int mode, const Grid& g, const les_params& p, const FusedIO& io,
@@ -379,17 +398,16 @@ void launch_stage_fused(int mode, const Grid& g, const les_params& p, const Fuse
   // PM = 12 with that staging alone, PM = 4 for the other row lengths.
   // Other grids read them at run time (PM = -1).
   const bool jet = !g.per[0] && !g.per[1] && g.per[2];
-  const bool full = g.n[1] % 16 == 0 && g.n[2] % FTK == 0;
+  const TileForm tf = jet ? tile_form(G) : TileForm{16, 1};
+  G.ctas = tf.ctas;
+  const bool full = g.n[1] % tf.rows == 0 && g.n[2] % FTK == 0;
   const int pm = !jet ? -1 : (!G.vec16 ? 4 : (full ? 28 : 12));
-  const bool small = jet && tile_rows(G) == 8;
-  if (small && G.vec16)
-    launch_stage_jet12s(mode, local, p.axis != 0, dyn, G, K, P, io.sc, alpha, L);
-  else if (small)
-    launch_stage_jet4s(mode, local, p.axis != 0, dyn, G, K, P, io.sc, alpha, L);
-  else if (pm == 28)
+  if (pm == 28)
     launch_stage_jet28(mode, local, p.axis != 0, dyn, G, K, P, io.sc, alpha, L);
   else if (pm == 12)
     launch_stage_jet12(mode, local, p.axis != 0, dyn, G, K, P, io.sc, alpha, L);
+  else if (pm == 4 && tf.rows == 8)
+    launch_stage_jet4s(mode, local, p.axis != 0, dyn, G, K, P, io.sc, alpha, L);
   else if (pm == 4)
     launch_stage_jet4(mode, local, p.axis != 0, dyn, G, K, P, io.sc, alpha, L);
   else if (dyn)  // (not with an axis: rejected at creation)

@@ -1,9 +1,10 @@
 // fused_kernel.cuh -- one kernel per Runge-Kutta stage (residual + update
 // fused), its helpers and launch templates; fused.cu holds the launchers,
-// fused_jet4.cu, fused_jet12.cu and fused_jet28.cu the jet-grid instantiations.
+// fused_jet4.cu, fused_jet4s.cu, fused_jet12.cu and fused_jet28.cu the jet-grid
+// instantiations.
 //
-// A CTA owns a 16 x 32 (small grids: 8 x 32) tile of (eta, zeta) columns and marches along
-// xi over a chunk of axial planes.  Per plane it stages the conserved state
+// A CTA owns a 16 x 32 or 8 x 32 tile of (eta, zeta) columns (tile_form in
+// fused.cu) and marches along xi over a chunk of axial planes.  Per plane it stages the conserved state
 // of the tile plus a two-node halo in shared memory with cp.async (one plane
 // ahead), derives the primitives and the anisotropic spectral radii once per
 // node, and keeps the own column's data of the neighbouring planes in
@@ -22,6 +23,7 @@
 // (their error is inside the form's measured error budget).
 #pragma once
 
+#include <array>
 #include <atomic>
 #include <functional>
 #include <map>
@@ -438,9 +440,7 @@ __global__ void __launch_bounds__(256) k_prestep(Grid g, Consts<R> K, const TQ* 
 // ------------------------------------------------------------ fused stage
 enum { FMODE_RHS = 0, FMODE_STAGE = 1, FMODE_LAST = 2 };
 
-// Tile of TJ x FTK (eta, zeta) columns, one thread per column: TJ = 16, or 8
-// on grids with so few planes and columns that most of a stage is latency
-// (tile_rows).
+// Tile of TJ x FTK (eta, zeta) columns, one thread per column: TJ = 16 or 8.
 constexpr int FTK = 32;
 // Shared-memory rows hold the tile's FTK columns and a two-column halo on
 // each side: tile column kk in [-2, FTK+1] lives at row column kk + 2.  When
@@ -453,28 +453,42 @@ __host__ __device__ constexpr int colk(int kk) { return kk + 2; }
 
 // Shared-memory plan (floats):
 //   sQ[3][5][PL2]  conserved state of planes i, i+1, i+2 (2-node halo)
-//   sPr[3][PL2]    float4 (u, v, w, T) of planes i-1, i, i+1
-//   sPw[3][PL2]    float2 (p, e + p) of the same planes
+//   sPr[3][PL1]    float4 (u, v, w, T) of planes i-1, i, i+1 (1-node halo)
+//   sPw[2][PL2]    float2 (p, e + p) of planes i, i+1 (2-node halo)
 //   sM[3][10][PL1] metrics of planes i, i+1, i+2 (1-node halo)
 //   sK[3][2][PL1]  mu_eff kappa_eff of planes i, i+1, i+2
-//   sL[2][3][PL1]  lbar of planes i, i+1
+//   sL[2][LS]      lbar of planes i, i+1: lbar_xi of the tile's own columns
+//                  [TJ][FTK], lbar_eta and lbar_zeta [PL1] each
 //   sFe[5][TJ+1][FTK]   eta interface fluxes (rows -1 .. TJ-1 of the tile)
 //   sFz[5][TJ]          the tile's left-edge zeta interface fluxes (the
 //                       others pass between neighbouring lanes by shuffle)
 // With the dynamic SGS model the viscosity slots hold a third field, the
-// Yoshizawa sigma_ll (sK[3][3][PL1]); the regions after sK move up.
+// Yoshizawa sigma_ll; the 8-row form then has two slots, of planes i and i+1
+// (sK[2][3][PL1]), and plane i+1's viscosities, which only the flux phase
+// reads, are staged while that plane is derived.
 template <int TJ, bool DYN>
 struct FLayout {
   static constexpr int R2 = TJ + 4, R1 = TJ + 2;  // rows with a 2-node / 1-node halo
   static constexpr int PL2 = R2 * SK, PL1 = R1 * SK;
-  static constexpr int PR = 3 * 5 * PL2, PW = PR + 3 * 4 * PL2, M = PW + 3 * 2 * PL2;
+  static constexpr int PR = 3 * 5 * PL2, PW = PR + 3 * 4 * PL1, M = PW + 2 * 2 * PL2;
   static constexpr int K = M + 3 * 10 * PL1;
   static constexpr int NKF = DYN ? 3 : 2;  // fields per viscosity slot
-  static constexpr int L = K + 3 * NKF * PL1;
-  static constexpr int FE = L + 2 * 3 * PL1;
+  static constexpr int KS = DYN && TJ <= 8 ? 2 : 3;  // viscosity slots
+  static constexpr int L = K + KS * NKF * PL1;
+  static constexpr int LS = TJ * FTK + 2 * PL1;
+  static constexpr int FE = L + 2 * LS;
   static constexpr int FZ = FE + 5 * (TJ + 1) * FTK;
   static constexpr int FLOATS = FZ + 5 * TJ;
 };
+// CTAs per SM: the primitives without a second halo node, two slots for
+// (p, e + p), lbar_xi of the own columns alone and the dynamic model's two
+// viscosity slots bring two 8-row CTAs under the 228 KB (a kilobyte of each is
+// the system's).
+template <int TJ>
+constexpr int kStageCtas = TJ <= 8 ? 2 : 1;
+static_assert(2 * (FLayout<8, false>::FLOATS * 4 + 1024) <= 228 * 1024 &&
+                  2 * (FLayout<8, true>::FLOATS * 4 + 1024) <= 228 * 1024,
+              "two 8-row CTAs per SM");
 static_assert(FLayout<16, true>::FLOATS * 4 <= 227 * 1024, "shared memory plan exceeds 227 KB");
 
 // Differences of (u, v, w, T) at an interface from node records (float4 u, v,
@@ -525,6 +539,7 @@ struct FusedGeom {
   // axial chunks: the first n1 hold a1 planes each, the other nch - n1
   // split the remaining planes evenly (n1 = 0: nch chunks of equal length)
   int nch, n1, a1;
+  int ctas;   // CTAs per SM that the chunks are scheduled for
   int vec16;  // zeta periodic, nk % 4 == 0 and nk >= FTK: tiles shifted by
               // two columns, rows staged as 16-byte copies
   int ilo, ihi;  // planes the stage updates along a non-periodic xi: [ilo, ihi)
@@ -552,7 +567,7 @@ __device__ __forceinline__ int wrap_fast(int v, int n, int per) {
 // bit 3, the shifted 16-byte staging (G.vec16); bit 4, tiles that cover eta
 // and zeta exactly (every thread owns a column).  PM = -1 reads them from G.
 template <int MODE, bool LOCAL, bool AXIS, bool DYN, int PM, int FTJ>
-__global__ void __launch_bounds__(FTJ * FTK, 1)
+__global__ void __launch_bounds__(FTJ * FTK, kStageCtas<FTJ>)
     k_stage_fused(const FusedGeom G, const Consts<float> K, const FusedPtrs P,
                   const DevScalars* __restrict__ sc, double alpha) {
   extern __shared__ __align__(16) float smem[];
@@ -563,7 +578,7 @@ __global__ void __launch_bounds__(FTJ * FTK, 1)
   float2* sPw = reinterpret_cast<float2*>(smem + Y::PW);
   float* sM = smem + Y::M;
   float* sK = smem + Y::K;
-  constexpr int NKF = Y::NKF;
+  constexpr int NKF = Y::NKF, KS = Y::KS, LS = Y::LS;
   float* sL = smem + Y::L;
   float* sFe = smem + Y::FE;
   float* sFz = smem + Y::FZ;
@@ -656,9 +671,11 @@ __global__ void __launch_bounds__(FTJ * FTK, 1)
 #pragma unroll
         for (int f = 6; f < 10; ++f)
           piece(sM + (slot * 10 + f) * PL1 + d, P.m[0] + (long long)f * G.N + n, 1.f);
+        if (KS == 3) {
 #pragma unroll
-        for (int f = 0; f < NKF; ++f)
-          piece(sK + (slot * NKF + f) * PL1 + d, P.mk[0] + (long long)f * G.N + n, 0.f);
+          for (int f = 0; f < NKF; ++f)
+            piece(sK + (slot * NKF + f) * PL1 + d, P.mk[0] + (long long)f * G.N + n, 0.f);
+        }
       }
     }
   };
@@ -671,25 +688,48 @@ __global__ void __launch_bounds__(FTJ * FTK, 1)
     else
       stage_pieces(std::integral_constant<int, 1>{}, slot, ig);
   };
+  // the viscosities of plane x where they have two slots (float by float
+  // where the rows do not take 16-byte pieces)
+  auto stage_visc = [&](int slot, int x) {
+    const int ig = wrap_fast(x, ni, per0), vw = vec_ok ? 4 : 1, pcs = SK / vw;
+    for (int u = tid; u < R1 * pcs; u += FNT) {
+      const int row = u / pcs, pc = u - row * pcs, jg = wrap_fast(j0 + row - 1, nj, per1);
+      const int kg = vec_ok ? (kt + 4 * pc < nk ? kt + 4 * pc : kt + 4 * pc - nk)
+                            : wrap_fast(kt - 2 + pc, nk, per2);
+      const int n = (ig * nj + jg) * nk + kg;
+#pragma unroll
+      for (int f = 0; f < NKF; ++f) {
+        float* dst = sK + (slot * NKF + f) * PL1 + row * SK + vw * pc;
+        const float* src = P.mk[0] + (long long)f * G.N + n;
+        if (ig < 0 || jg < 0 || kg < 0) {
+          for (int c = 0; c < vw; ++c) dst[c] = 0.f;
+        } else if (vec_ok) {
+          cp_async16(dst, src);
+        } else {
+          cp_async4(dst, src);
+        }
+      }
+    }
+  };
 
   // ---- primitives (2-node halo) and lbar (1-node halo) of a staged plane
   auto derive_node = [&](int r, int qs, int ps, int ms, int ls) {
     const float* q = sQ + qs * 5 * PL2;
-    float4* pr = sPr + ps * PL2;
-    float2* pw = sPw + ps * PL2;
+    float4* pr = sPr + ps * PL1;
+    float2* pw = sPw + ls * PL2;
     const float* mm = sM + ms * 10 * PL1;
-    float* ll = sL + ls * 3 * PL1;
+    float* ll = sL + ls * LS;
     const float rho = q[r];
     const float ir = frcp_fast(rho);
     const float u = q[PL2 + r] * ir, v = q[2 * PL2 + r] * ir, w = q[3 * PL2 + r] * ir;
     const float p = K.gm1 * (q[4 * PL2 + r] - 0.5f * rho * (u * u + v * v + w * w));
     const float T = K.gamma * p * ir;
-    pr[r] = make_float4(u, v, w, T);
     pw[r] = make_float2(p, q[4 * PL2 + r] + p);
     const int row = r / SK, col = r - row * SK;
     // 1-node halo: rows 1 .. R2-2 of the 2-node layout, columns kk in [-1, FTK]
     if (row >= 1 && row <= R2 - 2 && col >= colk(-1) && col <= colk(FTK)) {
       const int r1 = r - SK;
+      pr[r1] = make_float4(u, v, w, T);
       float m[10];
 #pragma unroll
       for (int t = 0; t < 10; ++t) m[t] = mm[t * PL1 + r1];
@@ -709,9 +749,10 @@ __global__ void __launch_bounds__(FTJ * FTK, 1)
       } else {
         node_lbar(m, u, v, w, T, lb);
       }
-      ll[r1] = lb[0];
-      ll[PL1 + r1] = lb[1];
-      ll[2 * PL1 + r1] = lb[2];
+      if (row >= 2 && row < FTJ + 2 && col >= colk(0) && col < colk(FTK))
+        ll[(row - 2) * FTK + col - colk(0)] = lb[0];
+      ll[FNT + r1] = lb[1];
+      ll[FNT + PL1 + r1] = lb[2];
     }
   };
 
@@ -769,8 +810,8 @@ __global__ void __launch_bounds__(FTJ * FTK, 1)
   // xi interface (x, x+1) of the own column: sPr/sPw/sM/sK/sL slots of both planes
   auto xi_flux = [&](int x, int p0, int p1, int m0, int m1, int l0, int l1, const float* mown,
                      const float4* rown, const float4* rpm, const float2* wown, float F[5]) {
-    const float4* A0 = sPr + p0 * PL2;
-    const float4* A1 = sPr + p1 * PL2;
+    const float4* A0 = sPr + p0 * PL1;
+    const float4* A1 = sPr + p1 * PL1;
     float nua, nub;
     if (!per_i && x == 0)
       nua = sensor3(pq[1], pq[2], pq[3]);
@@ -780,9 +821,9 @@ __global__ void __launch_bounds__(FTJ * FTK, 1)
       nub = sensor3(pq[0], pq[1], pq[2]);
     else
       nub = sensor3(pq[1], pq[2], pq[3]);
-    const float4 a0 = rown ? rown[0] : A0[o2], b0 = rpm ? rpm[0] : A1[o2];
-    const float4 an = A0[o2 + SK], as = A0[o2 - SK], bn = A1[o2 + SK], bs = A1[o2 - SK];
-    const float4 ae = A0[o2 + 1], aw = A0[o2 - 1], be = A1[o2 + 1], bw = A1[o2 - 1];
+    const float4 a0 = rown ? rown[0] : A0[o1], b0 = rpm ? rpm[0] : A1[o1];
+    const float4 an = A0[o1 + SK], as = A0[o1 - SK], bn = A1[o1 + SK], bs = A1[o1 - SK];
+    const float4 ae = A0[o1 + 1], aw = A0[o1 - 1], be = A1[o1 + 1], bw = A1[o1 - 1];
     float dphi[4][3];
     dphi_normal<0>(a0, b0, dphi);
     dphi_tangent<1>(an, as, bn, bs, dphi);
@@ -793,12 +834,12 @@ __global__ void __launch_bounds__(FTJ * FTK, 1)
       ma[t] = mown ? mown[t] : sM[(m0 * 10 + t) * PL1 + o1];
       mb[t] = sM[(m1 * 10 + t) * PL1 + o1];
     }
-    const float* Ka = sK + m0 * NKF * PL1;
-    const float* Kb = sK + m1 * NKF * PL1;
+    const float* Ka = sK + (KS == 2 ? l0 : m0) * NKF * PL1;
+    const float* Kb = sK + (KS == 2 ? l1 : m1) * NKF * PL1;
     iface_flux<0, float, AXIS, DYN>(K, Wq[0], Wq[1], Wq[2], Wq[3], vq[0], vq[3], nua, nub,
-                         sL[l0 * 3 * PL1 + o1], sL[l1 * 3 * PL1 + o1], ma, mb,
-                         wown ? wown->x : sPw[p0 * PL2 + o2].x,
-                         sPw[p1 * PL2 + o2].x, a0.x, a0.y, a0.z, b0.x, b0.y, b0.z, dphi, Ka[o1],
+                         sL[l0 * LS + tid], sL[l1 * LS + tid], ma, mb,
+                         wown ? wown->x : sPw[l0 * PL2 + o2].x,
+                         sPw[l1 * PL2 + o2].x, a0.x, a0.y, a0.z, b0.x, b0.y, b0.z, dphi, Ka[o1],
                          Kb[o1], Ka[PL1 + o1], Kb[PL1 + o1], DYN ? Ka[2 * PL1 + o1] : 0.f,
                          DYN ? Kb[2 * PL1 + o1] : 0.f, F);
   };
@@ -808,10 +849,10 @@ __global__ void __launch_bounds__(FTJ * FTK, 1)
   auto eta_flux = [&](int ra, int qs, int pm, int ps, int pp, int ms, int ls, const float* mown,
                       const float4* rown, const float4* rpm, const float2* wown, float F[5]) {
     const float* Qs = sQ + qs * 5 * PL2;
-    const float4* Pc = sPr + ps * PL2;
-    const float4* Pm = sPr + pm * PL2;
-    const float4* Pp = sPr + pp * PL2;
-    const float2* Pw = sPw + ps * PL2;
+    const float4* Pc = sPr + ps * PL1;
+    const float4* Pm = sPr + pm * PL1;
+    const float4* Pp = sPr + pp * PL1;
+    const float2* Pw = sPw + ls * PL2;
     const int a2 = (ra + 2) * SK + colk(tx), b2 = a2 + SK;
     const int a1 = (ra + 1) * SK + colk(tx), b1 = a1 + SK;
     const int jga = j0 + ra;
@@ -840,20 +881,19 @@ __global__ void __launch_bounds__(FTJ * FTK, 1)
       nub = sensor3(wm.x, wa.x, wb.x);
     else
       nub = sensor3(wa.x, wb.x, wp.x);
-    const int am1 = a2 - 1, bm1 = b2 - 1;
-    const float4 ca = rown ? rown[0] : Pc[a2], cb = Pc[b2];
+    const float4 ca = rown ? rown[0] : Pc[a1], cb = Pc[b1];
     float dphi[4][3];
     dphi_normal<1>(ca, cb, dphi);
-    dphi_tangent<0>(rpm ? rpm[0] : Pp[a2], rpm ? rpm[1] : Pm[a2], Pp[b2], Pm[b2], dphi);
-    dphi_tangent<2>(Pc[a2 + 1], Pc[am1], Pc[b2 + 1], Pc[bm1], dphi);
+    dphi_tangent<0>(rpm ? rpm[0] : Pp[a1], rpm ? rpm[1] : Pm[a1], Pp[b1], Pm[b1], dphi);
+    dphi_tangent<2>(Pc[a1 + 1], Pc[a1 - 1], Pc[b1 + 1], Pc[b1 - 1], dphi);
     float ma[10], mb[10];
 #pragma unroll
     for (int t = 0; t < 10; ++t) {
       ma[t] = mown ? mown[t] : sM[(ms * 10 + t) * PL1 + a1];
       mb[t] = sM[(ms * 10 + t) * PL1 + b1];
     }
-    const float* Kc = sK + ms * NKF * PL1;
-    const float* L = sL + ls * 3 * PL1 + PL1;
+    const float* Kc = sK + (KS == 2 ? ls : ms) * NKF * PL1;
+    const float* L = sL + ls * LS + FNT;
     iface_flux<1, float, AXIS, DYN>(K, Wm, Wa, Wb, Wp, has_m, has_p, nua, nub, L[a1], L[b1], ma, mb, wa.x,
                          wb.x, ca.x, ca.y, ca.z, cb.x, cb.y, cb.z, dphi, Kc[a1], Kc[b1],
                          Kc[PL1 + a1], Kc[PL1 + b1], DYN ? Kc[2 * PL1 + a1] : 0.f,
@@ -866,10 +906,10 @@ __global__ void __launch_bounds__(FTJ * FTK, 1)
                        const float* mown, const float4* rown, const float4* rpm, const float2* wown,
                        float F[5]) {
     const float* Qs = sQ + qs * 5 * PL2;
-    const float4* Pc = sPr + ps * PL2;
-    const float4* Pm = sPr + pm * PL2;
-    const float4* Pp = sPr + pp * PL2;
-    const float2* Pw = sPw + ps * PL2;
+    const float4* Pc = sPr + ps * PL1;
+    const float4* Pm = sPr + pm * PL1;
+    const float4* Pp = sPr + pp * PL1;
+    const float2* Pw = sPw + ls * PL2;
     const int rb2 = (rr + 2) * SK, rb1 = (rr + 1) * SK;
     const int ca_c = colk(ca), cb_c = colk(ca + 1), cm_c = colk(ca - 1), cp_c = colk(ca + 2);
     const int a2 = rb2 + ca_c, b2 = rb2 + cb_c, m2 = rb2 + cm_c, q2 = rb2 + cp_c;
@@ -899,19 +939,19 @@ __global__ void __launch_bounds__(FTJ * FTK, 1)
       nub = sensor3(wm.x, wa.x, wb.x);
     else
       nub = sensor3(wa.x, wb.x, wp.x);
-    const float4 pa = rown ? rown[0] : Pc[a2], pb = Pc[b2];
+    const float4 pa = rown ? rown[0] : Pc[a1], pb = Pc[b1];
     float dphi[4][3];
     dphi_normal<2>(pa, pb, dphi);
-    dphi_tangent<0>(rpm ? rpm[0] : Pp[a2], rpm ? rpm[1] : Pm[a2], Pp[b2], Pm[b2], dphi);
-    dphi_tangent<1>(Pc[a2 + SK], Pc[a2 - SK], Pc[b2 + SK], Pc[b2 - SK], dphi);
+    dphi_tangent<0>(rpm ? rpm[0] : Pp[a1], rpm ? rpm[1] : Pm[a1], Pp[b1], Pm[b1], dphi);
+    dphi_tangent<1>(Pc[a1 + SK], Pc[a1 - SK], Pc[b1 + SK], Pc[b1 - SK], dphi);
     float ma[10], mb[10];
 #pragma unroll
     for (int t = 0; t < 10; ++t) {
       ma[t] = mown ? mown[t] : sM[(ms * 10 + t) * PL1 + a1];
       mb[t] = sM[(ms * 10 + t) * PL1 + b1];
     }
-    const float* Kc = sK + ms * NKF * PL1;
-    const float* L = sL + ls * 3 * PL1 + 2 * PL1;
+    const float* Kc = sK + (KS == 2 ? ls : ms) * NKF * PL1;
+    const float* L = sL + ls * LS + FNT + PL1;
     iface_flux<2, float, AXIS, DYN>(K, Wm, Wa, Wb, Wp, has_m, has_p, nua, nub, L[a1], L[b1], ma, mb, wa.x,
                          wb.x, pa.x, pa.y, pa.z, pb.x, pb.y, pb.z, dphi, Kc[a1], Kc[b1],
                          Kc[PL1 + a1], Kc[PL1 + b1], DYN ? Kc[2 * PL1 + a1] : 0.f,
@@ -921,14 +961,18 @@ __global__ void __launch_bounds__(FTJ * FTK, 1)
   auto m3 = [](int x) { return ((x % 3) + 3) % 3; };
   auto m2 = [](int x) { return ((x % 2) + 2) % 2; };
   // ---------------------------------------------------------- prologue
-  // sQ/sM/sK slot of plane x: x mod 3 (planes i, i+1, i+2 live); sP slot:
-  // x mod 3 (planes i-1, i, i+1); sL slot: x mod 2 (planes i, i+1).
+  // sQ/sM/sK slot of plane x: x mod 3 (planes i, i+1, i+2 live); sPr slot:
+  // x mod 3 (planes i-1, i, i+1); sPw and sL slot: x mod 2 (planes i, i+1).
   // rotating slots: planes i-1, i, i+1 (plane i+2 is staged into the slot of
   // plane i-1) and the lbar slots of planes i, i+1
   int s_m = m3(ib - 1), s_c = m3(ib), s_p = m3(ib + 1);
   int l_c = m2(ib), l_p = m2(ib + 1);
   stage_plane(s_m, ib - 1);
   stage_plane(s_c, ib);
+  if (KS == 2) {
+    stage_visc(l_p, ib - 1);
+    stage_visc(l_c, ib);
+  }
   cp_async_commit();
   stage_plane(s_p, ib + 1);
   cp_async_commit();
@@ -992,9 +1036,14 @@ __global__ void __launch_bounds__(FTJ * FTK, 1)
     // plane i-1 any more: both were settled by the barrier that closed the
     // previous flux phase (or the prologue), so plane i+2 is staged into
     // those slots and plane i+1 derived without a barrier of their own.
+    if (KS == 2) {
+      stage_visc(l_p, i + 1);
+      cp_async_commit();
+    }
     stage_plane(s_m, i + 2);
     cp_async_commit();
     for (int r = tid; r < PL2; r += FNT) derive_node(r, s_p, s_p, s_p, l_p);
+    if (KS == 2) cp_async_wait<1>();  // plane i+1's viscosities
     __syncthreads();
 
     const int ig = wrap_fast(i, ni, per0);
@@ -1008,13 +1057,13 @@ __global__ void __launch_bounds__(FTJ * FTK, 1)
     // those of planes i+1 and i-1 of the own column (the last stage and the
     // local-step variants keep them in shared memory: their epilogues need
     // the registers)
-    const float4 ro = sPr[s_c * PL2 + o2];
-    const float2 wo = sPw[s_c * PL2 + o2];
+    const float4 ro = sPr[s_c * PL1 + o1];
+    const float2 wo = sPw[l_c * PL2 + o2];
     constexpr bool keep_pm = MODE != FMODE_LAST && !LOCAL;
     float4 rq[2];
     if (keep_pm) {
-      rq[0] = sPr[s_p * PL2 + o2];
-      rq[1] = sPr[s_m * PL2 + o2];
+      rq[0] = sPr[s_p * PL1 + o1];
+      rq[1] = sPr[s_m * PL1 + o1];
     }
     const float4* rpm = keep_pm ? rq : nullptr;
     if (own && jint && kint && (per_i || i + 1 <= ni - 1))
@@ -1167,7 +1216,7 @@ static Consts<R> fused_consts(const les_params& p) {
 // the other planes split evenly over n2 chunks (n1 = 0: equal chunks).  Long
 // chunks first leave the short ones to fill the last wave.  The choice
 // minimises the finishing time of a greedy list schedule of the CTAs on the
-// SMs, simulated once per grid shape and cached.
+// slots (SMs times CTAs per SM), simulated once per grid shape and cached.
 struct Chunks {
   int nch, n1, a1;
   double t;  // the schedule's finishing time, in planes
@@ -1203,10 +1252,10 @@ static double chunk_schedule(int ni, int n1, int a1, int n2, int tiles, int slot
 
 static Chunks choose_chunks(int ni, int tiles, int slots) {
   static std::mutex mu;
-  static std::map<std::pair<int, int>, Chunks> cache;
+  static std::map<std::array<int, 3>, Chunks> cache;
   {
     std::lock_guard<std::mutex> lk(mu);
-    auto it = cache.find({ni, tiles});
+    auto it = cache.find({ni, tiles, slots});
     if (it != cache.end()) return it->second;
   }
   const double pro = 1.5;
@@ -1214,6 +1263,8 @@ static Chunks choose_chunks(int ni, int tiles, int slots) {
   Chunks best{1, 0, 0, 0.0};
   double best_t = 1e300;
   auto consider = [&](int n1, int a1, int n2) {
+    // no schedule ends before its work divided by the slots
+    if ((ni + (n1 + n2) * pro) * tiles / slots >= best_t - 1e-9) return;
     const double t = chunk_schedule(ni, n1, a1, n2, tiles, slots, pro);
     if (t < best_t - 1e-9) {
       best_t = t;
@@ -1248,7 +1299,7 @@ static Chunks choose_chunks(int ni, int tiles, int slots) {
     }
   }
   std::lock_guard<std::mutex> lk(mu);
-  cache[{ni, tiles}] = best;
+  cache[{ni, tiles, slots}] = best;
   return best;
 }
 
@@ -1266,10 +1317,13 @@ static void launch_stage_t(const FusedGeom& G0, const Consts<float>& K, const Fu
   if (!(attr_set.load(std::memory_order_acquire) & bit)) {
     cudaFuncSetAttribute(k_stage_fused<MODE, LOCAL, AXIS, DYN, PM, TJ>,
                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaFuncSetAttribute(k_stage_fused<MODE, LOCAL, AXIS, DYN, PM, TJ>,
+                         cudaFuncAttributePreferredSharedMemoryCarveout,
+                         cudaSharedmemCarveoutMaxShared);
     attr_set.fetch_or(bit, std::memory_order_acq_rel);
   }
   const int tk = (G.nk + FTK - 1) / FTK, tj = (G.nj + TJ - 1) / TJ;
-  const Chunks ch = choose_chunks(G.ni, tk * tj, sm_count());  // one CTA per SM
+  const Chunks ch = choose_chunks(G.ni, tk * tj, G.ctas * sm_count());
   G.nch = ch.nch;
   G.n1 = ch.n1;
   G.a1 = ch.a1;
@@ -1294,15 +1348,12 @@ static void launch_stage_dispatch(int mode, bool local, const FusedGeom& G, cons
     launch_stage_t<FMODE_LAST, true, AXIS, DYN, PM, TJ>(G, K, P, sc, alpha, L);
 }
 
-// The jet-grid instantiations (PM = 4, 12 and 28; PM = 4 and 12 also with
-// tiles of 8 rows), each compiled in a translation unit of its own so the
-// build compiles them in parallel.
+// The jet-grid instantiations (PM = 12 and 28 with tiles of 8 rows, PM = 4 with
+// 16 and with 8), each compiled in a translation unit of its own so the build
+// compiles them in parallel.
 void launch_stage_jet4s(int mode, bool local, bool axis, bool dyn, const FusedGeom& G,
                         const Consts<float>& K, const FusedPtrs& P, const DevScalars* sc,
                         double alpha, const Launch& L);
-void launch_stage_jet12s(int mode, bool local, bool axis, bool dyn, const FusedGeom& G,
-                         const Consts<float>& K, const FusedPtrs& P, const DevScalars* sc,
-                         double alpha, const Launch& L);
 void launch_stage_jet4(int mode, bool local, bool axis, bool dyn, const FusedGeom& G,
                        const Consts<float>& K, const FusedPtrs& P, const DevScalars* sc,
                        double alpha, const Launch& L);

@@ -1,15 +1,17 @@
-"""The fused stage kernel's two tile heights: 16 rows on grids large enough to
-give every SM several planes (with the tiles covering eta and zeta exactly, with
-eta cut, with rows that take no 16-byte staging), 8 rows on grids of about a
-plane per SM, at eta extents around a multiple of 8.  Every variant of the
-stage, three steps within 1e-5 (relative L2) of the FP64 oracle's."""
+"""The fused stage kernel's tile forms: two CTAs of 8 rows per SM (with the tiles
+covering eta and zeta exactly, with eta or zeta cut, with rows in 8-byte pieces),
+one of 16 rows (small grids with rows that take no 16-byte pieces, of even and of
+odd length), one of 8 rows on grids of about a plane per SM, at eta extents
+around a multiple of 8.  Every variant of the stage, three steps within 1e-5
+(relative L2) of the FP64 oracle's."""
 import pytest
 
 from gpu_helpers import device_ctx, oracle_params, rel_l2
 
 pytestmark = pytest.mark.gpu
 
-TALL = [(64, 64, 64), (70, 60, 64), (70, 60, 63)]
+PAIRS = [(64, 64, 64), (70, 60, 64), (21, 49, 64), (61, 17, 68), (61, 17, 66)]
+TALL = [(70, 60, 63), (70, 60, 66)]
 SHORT = [(31, 7, 32), (31, 8, 36), (31, 9, 35), (21, 17, 64)]
 
 
@@ -29,7 +31,7 @@ def torch():
     return torch
 
 
-@pytest.mark.parametrize("shape", TALL + SHORT)
+@pytest.mark.parametrize("shape", PAIRS + TALL + SHORT)
 @pytest.mark.parametrize("option", ["plain", "local", "axis", "dynamic", "entrance"])
 def test_stage_variants(orc, lj, torch, shape, option):
     kw = dict(sgs_model=3 if option == "dynamic" else 1, axis=int(option == "axis"),
