@@ -300,8 +300,9 @@ __device__ __forceinline__ void bc_ring_part(const Grid& g, const Acc& Q, int bl
 // ahead of this one.)  A node takes 150 to 300 dependent FP64 operations, and
 // the FP64 pipe issues one warp instruction per 64 cycles and scheduler, so
 // a few nodes are bound by their latency: blocks of 128 threads, one warp per
-// scheduler, spread them over the SMs (48 x 24 x 32: with blocks of 256 this
-// launch and the exit's had taken 24 + 14 us).
+// scheduler, spread them over the SMs (288 x 160 x 128: this launch and the
+// exit's 33 + 15 us with blocks of 256, 25 + 10 now; 24 + 14 on 48 x 24 x 32
+// then).
 template <class Acc, typename TM>
 __global__ void __launch_bounds__(kBcThreads)
     k_bc_sides(Grid g, JetBC b, const double* __restrict__ rth, const TM* __restrict__ M,

@@ -12,7 +12,7 @@ namespace lesjet {
 // rounded to nearest, lo the rest rounded to nearest.  The conversions and
 // the subtraction would each take a slot of the FP64 pipe, which made the
 // split four times slower than its memory traffic (320 us for 5.9M points,
-// 71 at the memory rate), so they are done on the bits: hi takes the top 24
+// 71 at the memory rate; 67 now, the join 161 -> 74), so they are done on the bits: hi takes the top 24
 // bits of the significand, rounded to nearest even, and the signed rest of
 // at most 2^28 units is exact in an int, whose float (rounded to nearest)
 // times the unit is lo.  Values that the bit form does not cover (the

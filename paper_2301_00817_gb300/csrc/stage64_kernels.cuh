@@ -169,7 +169,8 @@ __device__ __forceinline__ R node_deriv(const Grid& g, const R* __restrict__ f, 
 // from the dynamic procedure); Delta = (J^-1)^(1/3), Delta^2 from del2 (set-up).
 // The gradient is kept at twice its value and the strain at four times, whose
 // powers of two leave with one constant (FP64-pipe bound: 158 operations per
-// node with Smagorinsky before, when it also took the cube root, about 90 now).
+// node with Smagorinsky before, when it also took the cube root, 82 now; 192 x
+// 96 x 128 593 -> 448 us).
 template <typename R, typename TQ, typename TM>
 __global__ void __launch_bounds__(256) k_mu(Grid g, Consts<R> K, const TQ* __restrict__ Q,
                                             const TM* __restrict__ M,
@@ -599,9 +600,9 @@ __device__ __forceinline__ void flux_zeta(const Grid& g, const Consts<R>& K,
 // value, F[D][5][N] at the interface's node a): blocks [0, b2) take zeta,
 // the next b0 xi in chunks of len0, the rest eta in chunks of len1.  Bound by
 // the FP64 pipe, which issues one warp instruction per 64 cycles and
-// scheduler, so the shape is chosen for the fewest FP64 operations: about 145
+// scheduler, so the shape is chosen for the fewest FP64 operations: about 157
 // per interface with chunks of 8 (205 before the node part was shared and
-// the dissipation and viscous sums regrouped).  Comparisons and absolute
+// the dissipation and viscous sums regrouped); 85 to 87 % of the pipe's rate.  Comparisons and absolute
 // values are done on the integer pipe (dev_max, dev_abs).  Against one launch
 // per direction with a sensor pass ahead of them: the 192 x 96 x 128 step
 // 18.3 -> 13.3 ms, the 48 x 24 x 32 step (three launches fewer per residual)
