@@ -128,7 +128,9 @@ __global__ void __launch_bounds__(256) k_dyn_node(long long N, float gamma, floa
 
 // Register bounds (here and on k_dyn_sums): left free, the compiler gave
 // these kernels 230-254 registers, one 256-thread block per SM for a
-// latency-bound pass; the FP32 forms fit 64 (80 for the sums) registers.
+// latency-bound pass; the FP32 forms run at 64 (the sums spill 276 bytes there
+// and 108 at 80, but the fourth block per SM is worth more: two mixed steps on
+// 192 x 96 x 128 2.61 and 2.59 ms; five blocks 2.71).
 template <typename R, typename TQ, typename TM>
 __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 2) k_dyn_products(Grid g, const TQ* __restrict__ Q,
                                                       const TM* __restrict__ M,
@@ -205,10 +207,10 @@ __global__ void __launch_bounds__(256) k_dyn_filter1(Grid g, const R* __restrict
 // along zeta, then eta, and keeps the last two planes' values in registers to
 // filter along xi.  Each output takes the same operations in the same order
 // as three one-direction passes would (zeta, eta, xi; identity at the faces of
-// a non-periodic direction).  Bound by the latency of those loads, most of
-// them L1 hits, so it is shaped for many resident threads: one field per
-// block, about 40 registers, no shared memory and no barriers.
-constexpr int kF3J = 4, kF3K = 32, kF3R = 2;  // 128 threads: 8 rows x 32 columns
+// a non-periodic direction).  Bound by those loads, most of them L1 hits: one
+// field per block, no shared memory and no barriers, and four rows per thread,
+// whose 18 loads give four outputs (12 gave two).
+constexpr int kF3J = 2, kF3K = 32, kF3R = 4;  // 64 threads: 8 rows x 32 columns
 
 template <typename R>
 __global__ void __launch_bounds__(kF3J * kF3K) k_dyn_filter3(Grid g, const R* __restrict__ src,
@@ -299,7 +301,7 @@ __global__ void __launch_bounds__(256) k_dyn_favre(long long N, const R* __restr
 // Per interior node the six terms (numerators and denominators of the
 // three coefficients), in R; their J^-1-weighted sums in FP64.
 template <typename R, typename TM>
-__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 3 : 1) k_dyn_sums(Grid g, const TM* __restrict__ M,
+__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 1) k_dyn_sums(Grid g, const TM* __restrict__ M,
                                                   const R* __restrict__ node,
                                                   const R* __restrict__ Fh,
                                                   const R* __restrict__ H,
