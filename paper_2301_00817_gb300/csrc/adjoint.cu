@@ -386,16 +386,16 @@ __device__ __forceinline__ void adj_zeta(const Grid& g, const Consts<double>& K,
 // (some 420 when the gradient tensor was formed, the stress reversed term by
 // term and the centred flux reversed twice per node).
 __global__ void __launch_bounds__(kFluxThreads, 2)
-    k_adj_flux3(Grid g, Consts<double> K, AdjIO io, unsigned b2, unsigned b0, int len) {
+    k_adj_flux3(Grid g, Consts<double> K, AdjIO io, unsigned b0, unsigned b1, int len) {
   begin_dependent();
   __shared__ double sh[9][kFluxThreads];
   const unsigned b = blockIdx.x;
-  if (b < b2)
-    adj_zeta(g, K, io, (long long)b * kFluxThreads, sh);
-  else if (b < b2 + b0)
-    adj_chain<0>(g, K, io, (long long)(b - b2) * kFluxThreads + threadIdx.x, len);
+  if (b < b0)
+    adj_chain<0>(g, K, io, (long long)b * kFluxThreads + threadIdx.x, len);
+  else if (b < b0 + b1)
+    adj_chain<1>(g, K, io, (long long)(b - b0) * kFluxThreads + threadIdx.x, len);
   else
-    adj_chain<1>(g, K, io, (long long)(b - b2 - b0) * kFluxThreads + threadIdx.x, len);
+    adj_zeta(g, K, io, (long long)(b - b0 - b1) * kFluxThreads, sh);
 }
 
 // Sensor cotangents to the pressures of the (face-shifted) centre triple:
@@ -1046,7 +1046,7 @@ void launch_rhs_vjp(const Grid& g, const les_params& p, const double* Q, const d
   const unsigned b0 = blocks((long long)chunks(0) * g.n[1] * g.n[2]);
   const unsigned b1 = blocks((long long)g.n[0] * chunks(1) * g.n[2]);
   const AdjIO io{FluxIO<double, double, double>{Q, M, node, mk, nullptr}, lamR, rec};
-  launch_dependent(k_adj_flux3, f.b2 + b0 + b1, kFluxThreads, 0, L, g, K, io, f.b2, b0, f.len);
+  launch_dependent(k_adj_flux3, f.b2 + b0 + b1, kFluxThreads, 0, L, g, K, io, b0, b1, f.len);
   launch_dependent(k_adj_sensor_terms, nb_for(g.N), 256, 0, L, g, node, rec, ST);
   launch_dependent(k_adj_node, blocks_for(g.N, 128), 128, 0, L, g, K, Q, M, gn, node, rec, ST, lamQ,
                    lamMK);
@@ -1066,7 +1066,7 @@ void launch_rhs_jvp(const Grid& g, const les_params& p, const Dual* Q, const dou
                    nullptr, nullptr, nullptr, 0.0);
   const FluxPlan f = flux_plan(g);
   launch_dependent(k_flux3<Dual, Dual, double>, f.b2 + f.b0 + f.b1, kFluxThreads, 0, L, g, K,
-                   FluxIO<Dual, Dual, double>{Q, M, node, mk, flux}, f.b2, f.b0, f.len, f.len);
+                   FluxIO<Dual, Dual, double>{Q, M, node, mk, flux}, f.b0, f.b1, f.len, f.len);
   launch_dependent(k_update<Dual, double, Dual, 0>, nb, 256, 0, L, g, flux, nullptr, M, nullptr,
                    0.0, R, nullptr, nullptr);
   *L.counter += 3;

@@ -597,29 +597,29 @@ __device__ __forceinline__ void flux_zeta(const Grid& g, const Consts<R>& K,
 }
 
 // The interface fluxes of the three directions in one launch (2x their
-// value, F[D][5][N] at the interface's node a): blocks [0, b2) take zeta,
-// the next b0 xi in chunks of len0, the rest eta in chunks of len1.  Bound by
+// value, F[D][5][N] at the interface's node a): blocks [0, b0) take xi in
+// chunks of len0, the next b1 eta in chunks of len1, the rest zeta.  Bound by
 // the FP64 pipe, which issues one warp instruction per 64 cycles and
 // scheduler, so the shape is chosen for the fewest FP64 operations: about 157
 // per interface with chunks of 8 (205 before the node part was shared and
-// the dissipation and viscous sums regrouped); 85 to 87 % of the pipe's rate.  Comparisons and absolute
-// values are done on the integer pipe (dev_max, dev_abs).  Against one launch
-// per direction with a sensor pass ahead of them: the 192 x 96 x 128 step
-// 18.3 -> 13.3 ms, the 48 x 24 x 32 step (three launches fewer per residual)
-// 0.50 -> 0.35 ms.
+// the dissipation and viscous sums regrouped); 85 to 87 % of the pipe's rate.
+// Comparisons and absolute values are done on the integer pipe (dev_max,
+// dev_abs).  Against one launch per direction with a sensor pass ahead of
+// them: the 192 x 96 x 128 step 18.3 -> 13.1 ms, the 48 x 24 x 32 step (three
+// launches fewer per residual) 0.50 -> 0.27 ms.
 template <typename R, typename TQ, typename TM>
 __global__ void __launch_bounds__(kFluxThreads, sizeof(R) == 8 ? 2 : 1)
-    k_flux3(Grid g, Consts<R> K, FluxIO<R, TQ, TM> io, unsigned b2, unsigned b0, int len0,
+    k_flux3(Grid g, Consts<R> K, FluxIO<R, TQ, TM> io, unsigned b0, unsigned b1, int len0,
             int len1) {
   begin_dependent();
   __shared__ R sh[14][kFluxThreads];
-  unsigned b = blockIdx.x;
-  if (b < b2) {
-    flux_zeta(g, K, io, (long long)b * kFluxThreads, sh);
-  } else if (b < b2 + b0) {
-    flux_chain<0>(g, K, io, (long long)(b - b2) * kFluxThreads + threadIdx.x, len0);
+  const unsigned b = blockIdx.x;
+  if (b < b0) {
+    flux_chain<0>(g, K, io, (long long)b * kFluxThreads + threadIdx.x, len0);
+  } else if (b < b0 + b1) {
+    flux_chain<1>(g, K, io, (long long)(b - b0) * kFluxThreads + threadIdx.x, len1);
   } else {
-    flux_chain<1>(g, K, io, (long long)(b - b2 - b0) * kFluxThreads + threadIdx.x, len1);
+    flux_zeta(g, K, io, (long long)(b - b0 - b1) * kFluxThreads, sh);
   }
 }
 
@@ -629,11 +629,17 @@ struct FluxPlan {
   int len;
 };
 inline FluxPlan flux_plan(const Grid& g) {
-  // Chunks as long as leaves a dozen waves of the two resident blocks per
-  // SM (a chunk repeats one node's part, 22 of its 142 FP64 operations per
-  // interface, so beyond 8 there is nothing left to gain).
+  // A chunk repeats one node's part, 22 of its 142 FP64 operations per
+  // interface.  The chunks' blocks come first and zeta's, one interface per
+  // thread, fill the end, so a chunk may last half of an SM's share (waves of
+  // the two resident blocks of one interface per thread).  Against a dozen
+  // waves of chunks behind zeta's blocks: 48 x 24 x 32 (waves 2) 280 -> 269 us a
+  // step, residual on 73 x 53 x 45 (13) 290 -> 263 us, adjoint window on 64 x 40 x
+  // 48 (9) 28.7 -> 27.4 ms; 8 instead of 4 at 13 waves 272 us, 4 instead of 2 at
+  // 2 waves 324; 16 instead of 8 on 192 x 96 x 128 (181) 12.80 -> 12.62 ms.
   const long long waves = 3 * g.N / ((long long)kFluxThreads * 2 * sm_count());
-  const int len = waves >= 96 ? 8 : (waves >= 48 ? 4 : (waves >= 24 ? 2 : 1));
+  const int len =
+      waves >= 64 ? 16 : (waves >= 16 ? 8 : (waves >= 4 ? 4 : (waves >= 2 ? 2 : 1)));
   auto blocks = [](long long t) { return (unsigned)((t + kFluxThreads - 1) / kFluxThreads); };
   auto chunks = [&](int d) { return ((g.per[d] ? g.n[d] : g.n[d] - 1) + len - 1) / len; };
   FluxPlan f;

@@ -1,4 +1,4 @@
-"""The FP64 flux kernel's chunk lengths (1, 2, 4 and 8 interfaces per thread,
+"""The FP64 flux kernel's chunk lengths (1, 2, 4, 8 and 16 interfaces per thread,
 chosen by the number of points) on extents that are no multiple of a chunk or
 a block: jets and boxes, periodic and open along every direction, against the
 oracle's residual within the 1e-13 of each component's flux scale of the
@@ -28,7 +28,8 @@ def torch():
 
 
 @pytest.mark.parametrize("shape,per", [
-    ((9, 7, 129), None), ((5, 5, 5), (1, 1, 1)), ((131, 75, 35), None), ((67, 71, 73), (1, 1, 1)),
+    ((9, 7, 129), None), ((5, 5, 5), (1, 1, 1)), ((37, 31, 43), None), ((47, 41, 43), (0, 1, 0)),
+    ((131, 75, 35), None), ((67, 71, 73), (1, 1, 1)),
     ((131, 75, 67), None), ((90, 87, 85), (0, 0, 0)), ((131, 75, 131), None),
     ((109, 111, 107), (1, 0, 0)), ((107, 109, 111), (0, 1, 0))])
 def test_residual_for_every_chunk_length(orc, lj, torch, shape, per):
