@@ -31,23 +31,31 @@ struct JetBC {
   int forced;   // some forcing amplitude is non-zero
   double gamma, Mj, r_jet, theta_m, force_width;
   double gm1, igm1, ig;  // gamma - 1 and the reciprocals of it and of gamma
+  double rm, einf;       // -2/(gamma - 1) and (1/gamma)/(gamma - 1)
   double St[4];
   double amp[16];
 };
 
 // (The boundary nodes' chains of dependent FP64 operations are what their
-// launches take, and a division is ten of them: constants are multiplied by
-// their reciprocals, a node's density is inverted once, the sound speed and
-// its reciprocal come from one root, and Mach numbers are compared without
-// being formed.)
+// launches take, and a division is ten of them: what is divided by a constant
+// or by a node's density takes the reciprocal at hand, the sound speed and its
+// reciprocal come from one root, and Mach numbers are compared without being
+// formed.)
+// x/d from id, d's rounded reciprocal: the product corrected by its residual
+// (Markstein, 1990), so that the boundary states round as with divisions.
+__device__ __forceinline__ double div_by(double x, double d, double id) {
+  const double q = x * id;
+  return fma(fma(-q, d, x), id, q);
+}
+
 template <class Acc>
-__device__ __forceinline__ void store_prim(const Acc& Q, long long N, long long n, double igm1,
+__device__ __forceinline__ void store_prim(const Acc& Q, long long N, long long n, const JetBC& b,
                                            double rho, double u, double v, double w, double p) {
   Q.st(n, rho);
   Q.st(N + n, rho * u);
   Q.st(2 * N + n, rho * v);
   Q.st(3 * N + n, rho * w);
-  Q.st(4 * N + n, p * igm1 + 0.5 * rho * (u * u + v * v + w * w));
+  Q.st(4 * N + n, div_by(p, b.gm1, b.igm1) + 0.5 * rho * (u * u + v * v + w * w));
 }
 
 template <class Acc>
@@ -86,10 +94,11 @@ __device__ __forceinline__ double pow_entropy(double x, double e) {
 __device__ __forceinline__ bool far_field_state(const JetBC& b, double rho, double ir, double u,
                                                 double v, double w, double p, double nx, double ny,
                                                 double nz, double f[5]) {
-  const double T = b.gamma * p * ir, ra = rsqrt(T), ae = T * ra;
+  const double T = div_by(b.gamma * p, rho, ir), ra = rsqrt(T), a0 = T * ra;
+  const double ae = fma(fma(-a0, a0, T), 0.5 * ra, a0);  // sqrt(T), one Newton step on T ra
   const double qne = u * nx + v * ny + w * nz;
-  const double Rp = qne + 2.0 * ae * b.igm1;
-  const double Rm = -2.0 * b.igm1;
+  const double Rp = qne + div_by(2.0 * ae, b.gm1, b.igm1);
+  const double Rm = b.rm;
   const double qnf = 0.5 * (Rp + Rm);
   const double af = 0.25 * b.gm1 * (Rp - Rm);
   // q_n,e/a_e >= 1, >= 0, > -1
@@ -98,20 +107,20 @@ __device__ __forceinline__ bool far_field_state(const JetBC& b, double rho, doub
     // entropy of the interior node: rho_f = (rho_e^gamma a_f^2/(gamma p_e))^(1/(gamma-1))
     // = rho_e (a_f/a_e)^(2/(gamma-1)), one power instead of two
     const double dq = qnf - qne;
-    const double rf = rho * pow_entropy(af * ra, 2.0 * b.igm1);
+    const double rf = rho * pow_entropy(div_by(af, ae, ra), -b.rm);
     f[0] = rf;
     f[1] = u + dq * nx;
     f[2] = v + dq * ny;
     f[3] = w + dq * nz;
-    f[4] = rf * af * af * b.ig;
+    f[4] = div_by(rf * af * af, b.gamma, b.ig);
   } else if (qne > -ae) {
     // free-stream entropy (rho = 1, p = 1/gamma): rho_f = a_f^(2/(gamma-1))
-    const double rf = pow_entropy(af, 2.0 * b.igm1);
+    const double rf = pow_entropy(af, -b.rm);
     f[0] = rf;
     f[1] = qnf * nx;
     f[2] = qnf * ny;
     f[3] = qnf * nz;
-    f[4] = rf * af * af * b.ig;
+    f[4] = div_by(rf * af * af, b.gamma, b.ig);
   } else {
     f[0] = 1.0;
     f[1] = f[2] = f[3] = 0.0;
@@ -203,7 +212,7 @@ __device__ __forceinline__ void bc_inflow_part(const Grid& g, const JetBC& b,
 #pragma unroll
           for (int q = 0; q < 5; ++q) Q.st(q * N + n, Q.ld(q * N + ne));
         } else {
-          store_prim(Q, N, n, b.igm1, f[0], f[1], f[2], f[3], f[4]);
+          store_prim(Q, N, n, b, f[0], f[1], f[2], f[3], f[4]);
         }
       } else if (b.mode == LES_BC_JET_CHAR && b.Mj < 1.0) {
         const double gm1 = b.gm1;
@@ -212,9 +221,9 @@ __device__ __forceinline__ void bc_inflow_part(const Grid& g, const JetBC& b,
         const double Tt = 1.0 + 0.5 * gm1 * b.Mj * b.Mj;
         const double T = Tt / (1.0 + 0.5 * gm1 * (u * u + ve * ve + we * we));
         const double pf = pow(T, b.gamma / gm1) / b.gamma;
-        store_prim(Q, N, n, b.igm1, b.gamma * pf / T, u, ve, we, pf);
+        store_prim(Q, N, n, b, b.gamma * pf / T, u, ve, we, pf);
       } else {
-        store_prim(Q, N, n, b.igm1, 1.0, u, 0.0, 0.0, b.ig);
+        store_prim(Q, N, n, b, 1.0, u, 0.0, 0.0, b.ig);
       }
     }
     __syncthreads();  // the next 32 nodes' values replace these
@@ -251,7 +260,7 @@ __device__ __forceinline__ void bc_farfield_part(const Grid& g, const JetBC& b,
 #pragma unroll
       for (int q = 0; q < 5; ++q) Q.st(q * N + nf, Q.ld(q * N + ne));
     } else {
-      store_prim(Q, N, nf, b.igm1, f[0], f[1], f[2], f[3], f[4]);
+      store_prim(Q, N, nf, b, f[0], f[1], f[2], f[3], f[4]);
     }
   }
 }
@@ -350,7 +359,7 @@ __global__ void __launch_bounds__(kBcThreads)
       Q.st(N + nx_, rf * u);
       Q.st(2 * N + nx_, rf * v);
       Q.st(3 * N + nx_, rf * w);
-      Q.st(4 * N + nx_, b.ig * b.igm1 + 0.5 * rf * (u * u + v * v + w * w));
+      Q.st(4 * N + nx_, b.einf + 0.5 * rf * (u * u + v * v + w * w));
     }
   }
 }
@@ -443,6 +452,8 @@ static void bc_jet(const Grid& g, const les_params& p, Acc Q, const TM* M,
   b.gm1 = p.gamma - 1.0;
   b.igm1 = 1.0 / b.gm1;
   b.ig = 1.0 / p.gamma;
+  b.rm = -2.0 / b.gm1;
+  b.einf = b.ig / b.gm1;
   b.Mj = p.Mj;
   b.r_jet = p.r_jet;
   b.theta_m = p.theta_m;
