@@ -70,12 +70,6 @@ __device__ __forceinline__ void load_prim(const Acc& Q, long long N, long long n
   p = gm1 * (Q.ld(4 * N + n) - 0.5 * rho * (u * u + v * v + w * w));
 }
 
-// Riemann-invariant state of a far-field node from its interior neighbour's
-// primitives and the unit outward normal, the free stream at rest (rho = 1,
-// p = 1/gamma, a = 1): R+ = q_n,e + 2 a_e/(gamma-1), R- = -2/(gamma-1), four
-// branches by q_n,e/a_e.  Returns true for the supersonic exit (the caller
-// copies the neighbour's conserved values); otherwise the primitives of the
-// boundary state are in f = (rho, u, v, w, p).
 // x^(2/(gamma-1)).  When 2/(gamma-1) is an integer up to 8 (gamma = 1.4: 5;
 // gamma = 5/3: 3) the power is taken by repeated multiplication: it differs
 // from pow(x, 2/(gamma-1)) only by the rounding of the computed exponent
@@ -91,19 +85,38 @@ __device__ __forceinline__ double pow_entropy(double x, double e) {
   return pow(x, e);
 }
 
+// x > 0, finite and no subnormal (on the integer pipe).
+__device__ __forceinline__ bool is_ordinary(double x) {
+  return (unsigned)__double2hiint(x) - 0x00100000u < 0x7fe00000u;
+}
+
+// Riemann-invariant state of a far-field node from its interior neighbour's
+// primitives and the unit outward normal, the free stream at rest (rho = 1,
+// p = 1/gamma, a = 1): R+ = q_n,e + 2 a_e/(gamma-1), R- = -2/(gamma-1), four
+// branches by q_n,e/a_e.  Returns true for the supersonic exit (the caller
+// copies the neighbour's conserved values); otherwise the primitives of the
+// boundary state are in f = (rho, u, v, w, p).
+// (Where T = gamma p/rho has no ordinary root, a_e and the Mach number are
+// formed as written: a zero T makes it infinite, and with a NaN no comparison
+// holds, which leaves the free stream.)
 __device__ __forceinline__ bool far_field_state(const JetBC& b, double rho, double ir, double u,
                                                 double v, double w, double p, double nx, double ny,
                                                 double nz, double f[5]) {
   const double T = div_by(b.gamma * p, rho, ir), ra = rsqrt(T), a0 = T * ra;
-  const double ae = fma(fma(-a0, a0, T), 0.5 * ra, a0);  // sqrt(T), one Newton step on T ra
+  double ae = fma(fma(-a0, a0, T), 0.5 * ra, a0);  // sqrt(T), one Newton step on T ra
   const double qne = u * nx + v * ny + w * nz;
+  double Mn = qne, M1 = ae;  // q_n,e/a_e against 1 as q_n,e against a_e
+  if (!is_ordinary(T)) {
+    ae = sqrt(b.gamma * p / rho);
+    Mn = qne / ae;
+    M1 = 1.0;
+  }
   const double Rp = qne + div_by(2.0 * ae, b.gm1, b.igm1);
   const double Rm = b.rm;
   const double qnf = 0.5 * (Rp + Rm);
   const double af = 0.25 * b.gm1 * (Rp - Rm);
-  // q_n,e/a_e >= 1, >= 0, > -1
-  if (qne >= ae) return true;
-  if (qne >= 0.0) {
+  if (Mn >= M1) return true;
+  if (Mn >= 0.0) {
     // entropy of the interior node: rho_f = (rho_e^gamma a_f^2/(gamma p_e))^(1/(gamma-1))
     // = rho_e (a_f/a_e)^(2/(gamma-1)), one power instead of two
     const double dq = qnf - qne;
@@ -113,7 +126,7 @@ __device__ __forceinline__ bool far_field_state(const JetBC& b, double rho, doub
     f[2] = v + dq * ny;
     f[3] = w + dq * nz;
     f[4] = div_by(rf * af * af, b.gamma, b.ig);
-  } else if (qne > -ae) {
+  } else if (Mn > -M1) {
     // free-stream entropy (rho = 1, p = 1/gamma): rho_f = a_f^(2/(gamma-1))
     const double rf = pow_entropy(af, -b.rm);
     f[0] = rf;
