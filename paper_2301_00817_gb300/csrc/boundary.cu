@@ -361,8 +361,10 @@ __global__ void __launch_bounds__(kBcThreads)
     double rho, ir, u, v, w, p;
     load_prim(Q, N, ne, b.gm1, rho, ir, u, v, w, p);
     const double ae = sqrt(b.gamma * p * ir);
-    // q_n >= a_e, q_n = u . e/|e|
-    if (u * ex + v * ey + w * ez >= ae * gn) {
+    // q_n/a_e >= 1, q_n = u . e/|e| (as written where a_e is no ordinary value)
+    const double qg = u * ex + v * ey + w * ez, ag = ae * gn;
+    const bool ordinary = is_ordinary(ag);
+    if (ordinary ? qg >= ag : qg / ag >= 1.0) {
 #pragma unroll
       for (int q = 0; q < 5; ++q) Q.st(q * N + nx_, Q.ld(q * N + ne));
     } else {
@@ -372,7 +374,8 @@ __global__ void __launch_bounds__(kBcThreads)
       Q.st(N + nx_, rf * u);
       Q.st(2 * N + nx_, rf * v);
       Q.st(3 * N + nx_, rf * w);
-      Q.st(4 * N + nx_, b.einf + 0.5 * rf * (u * u + v * v + w * w));
+      const double q2 = u * u + v * v + w * w;
+      Q.st(4 * N + nx_, ordinary ? b.einf + 0.5 * rf * q2 : rf * (p / (b.gm1 * rho) + 0.5 * q2));
     }
   }
 }

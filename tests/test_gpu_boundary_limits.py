@@ -52,7 +52,7 @@ def _limits(flat, rng):
     return q
 
 
-@pytest.mark.parametrize("where", ["far_field", "entrance"])
+@pytest.mark.parametrize("where", ["far_field", "exit", "entrance"])
 def test_undefined_mach_numbers(orc, lj, torch, where):
     kw = dict(periodic=(0, 0, 1), bc=lj.BC_JET_CHAR if where == "entrance" else lj.BC_JET)
     xyz = lj.synth.jet_grid(*SHAPE)
