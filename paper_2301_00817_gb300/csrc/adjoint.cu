@@ -1066,7 +1066,7 @@ void launch_rhs_jvp(const Grid& g, const les_params& p, const Dual* Q, const dou
                    nullptr, nullptr, nullptr, 0.0);
   const FluxPlan f = flux_plan(g);
   launch_dependent(k_flux3<Dual, Dual, double>, f.b2 + f.b0 + f.b1, kFluxThreads, 0, L, g, K,
-                   FluxIO<Dual, Dual, double>{Q, M, node, mk, flux}, f.b0, f.b1, f.len, f.len);
+                   FluxIO<Dual, Dual, double>{Q, M, node, mk, flux}, f.b0, f.b1, f.len);
   launch_dependent(k_update<Dual, double, Dual, 0>, nb, 256, 0, L, g, flux, nullptr, M, nullptr,
                    0.0, R, nullptr, nullptr);
   *L.counter += 3;

@@ -61,7 +61,7 @@ void launch_flux64(const Grid& g, const les_params& p, const StageIO64& io, cons
   const FluxPlan f = flux_plan(g);
   const FluxIO<double, double, double> fio{io.Qin, io.M, io.node, io.mk, io.flux};
   launch_dependent(k_flux3<double, double, double>, f.b2 + f.b0 + f.b1, kFluxThreads, 0, L, g,
-                   make_consts<double>(p), fio, f.b0, f.b1, f.len, f.len);
+                   make_consts<double>(p), fio, f.b0, f.b1, f.len);
   ++*L.counter;
 }
 

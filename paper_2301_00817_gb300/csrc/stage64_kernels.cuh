@@ -155,11 +155,6 @@ __device__ __forceinline__ R node_diff(const Grid& g, const R* __restrict__ f, l
   if (c[d] == nd - 1) return R(3) * f[n] - R(4) * f[n - s] + f[n - 2 * s];
   return f[n + s] - f[n - s];
 }
-template <typename R>
-__device__ __forceinline__ R node_deriv(const Grid& g, const R* __restrict__ f, long long n,
-                                        const int c[3], int d) {
-  return R(0.5) * node_diff(g, f, n, c, d);
-}
 
 // mu_eff = (Mj/Re) T^1.5 (1+S)/(T+S) + mu_sgs; kappa_eff = mu_lam/((g-1)Pr)
 // + mu_sgs/((g-1)Pr_sgs).  Smagorinsky: rho (Cs Delta)^2 |S|; Vreman:
@@ -597,8 +592,8 @@ __device__ __forceinline__ void flux_zeta(const Grid& g, const Consts<R>& K,
 }
 
 // The interface fluxes of the three directions in one launch (2x their
-// value, F[D][5][N] at the interface's node a): blocks [0, b0) take xi in
-// chunks of len0, the next b1 eta in chunks of len1, the rest zeta.  Bound by
+// value, F[D][5][N] at the interface's node a): blocks [0, b0) take xi and the
+// next b1 eta in chunks of len interfaces, the rest zeta.  Bound by
 // the FP64 pipe, which issues one warp instruction per 64 cycles and
 // scheduler, so the shape is chosen for the fewest FP64 operations: about 157
 // per interface with chunks of 8 (205 before the node part was shared and
@@ -609,15 +604,14 @@ __device__ __forceinline__ void flux_zeta(const Grid& g, const Consts<R>& K,
 // launches fewer per residual) 0.50 -> 0.27 ms.
 template <typename R, typename TQ, typename TM>
 __global__ void __launch_bounds__(kFluxThreads, sizeof(R) == 8 ? 2 : 1)
-    k_flux3(Grid g, Consts<R> K, FluxIO<R, TQ, TM> io, unsigned b0, unsigned b1, int len0,
-            int len1) {
+    k_flux3(Grid g, Consts<R> K, FluxIO<R, TQ, TM> io, unsigned b0, unsigned b1, int len) {
   begin_dependent();
   __shared__ R sh[14][kFluxThreads];
   const unsigned b = blockIdx.x;
   if (b < b0) {
-    flux_chain<0>(g, K, io, (long long)b * kFluxThreads + threadIdx.x, len0);
+    flux_chain<0>(g, K, io, (long long)b * kFluxThreads + threadIdx.x, len);
   } else if (b < b0 + b1) {
-    flux_chain<1>(g, K, io, (long long)(b - b0) * kFluxThreads + threadIdx.x, len1);
+    flux_chain<1>(g, K, io, (long long)(b - b0) * kFluxThreads + threadIdx.x, len);
   } else {
     flux_zeta(g, K, io, (long long)(b - b0 - b1) * kFluxThreads, sh);
   }
