@@ -180,13 +180,18 @@ __device__ __forceinline__ double dev_max<double>(double a, double b) {
   return gt && ordered ? a : b;
 }
 
-// (double)x on the integer pipe (exact; zeros, denormals, infinities and NaN
-// take the conversion).
+// (double)x on the integer pipe (exact; infinities and NaN take the conversion,
+// subnormals that of their integer: a float conversion would flush them in the
+// translation units built so, and not in the others).
 __device__ __forceinline__ double widen(float x) {
   const unsigned b = __float_as_uint(x), mag = b & 0x7fffffffu;
+  const int sign = (int)(b & 0x80000000u);
   if (mag - 0x00800000u < 0x7f000000u)
-    return __hiloint2double((int)((b & 0x80000000u) | ((mag >> 3) + 0x38000000u)), (int)(b << 29));
-  return mag == 0u ? __hiloint2double((int)b, 0) : (double)x;
+    return __hiloint2double(sign | (int)((mag >> 3) + 0x38000000u), (int)(b << 29));
+  if (mag == 0u) return __hiloint2double(sign, 0);
+  if (mag > 0x007fffffu) return (double)x;
+  const double m = (double)(int)mag * 0x1p-149;
+  return __hiloint2double(sign | __double2hiint(m), __double2loint(m));
 }
 __device__ __forceinline__ double widen(double x) { return x; }
 
