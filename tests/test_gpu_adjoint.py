@@ -89,6 +89,60 @@ def test_residual_adjoint_dot_product(lj, torch, case):
     assert abs(_vdot(lamR, dR) - _vdot(lamMK, dMK)) <= 1e-12 * _vdot(lamR.abs(), dR.abs())
 
 
+CHUNK_GRIDS = [((37, 31, 43), None), ((47, 41, 43), (0, 1, 0)), ((131, 75, 35), None), ((67, 71, 73), (1, 1, 1)),
+               ((90, 87, 85), (0, 0, 0)), ((131, 75, 131), None), ((109, 111, 107), (1, 0, 0))]
+
+
+@pytest.mark.parametrize("shape,per", CHUNK_GRIDS)
+def test_residual_adjoint_for_every_chunk_length(lj, torch, shape, per):
+    """The tangent and the reverse on grids whose kernels walk chunks of 2, 4, 8
+    and 16 interfaces per thread (the other tests' grids take 1), none of them a
+    divisor of an extent.  The dot product as above; and the tangent against
+    central differences of the residual, node by node: they may miss it where a
+    sensor's |s| or the larger of two sensors switches within the step of 1e-6 x
+    1e-2 (pressure fluctuations of 1e-2 in the state: a share of some 1e-6 of the
+    sensors, each read by up to four nodes along its line), while an interface
+    value carried wrongly from one interface to the next would show at one node
+    in sixteen or more."""
+    if per is None:
+        ctx, xyz = _jet(lj, torch, shape, Re=300.0)
+        Q = torch.empty((5,) + shape, dtype=torch.float64, device="cuda")
+        ctx.les_init_jet(xyz, 3, 3e-2, Q)
+    else:
+        xyz_np, shift = lj.synth.box_grid(shape, (1.0, 1.3, 0.8), wave=0.25)
+        ctx = lj.Context(lj.make_params(periodic=per, bc=0, Re=300.0), shape, "cuda:0")
+        ctx.les_set_grid(torch.from_numpy(xyz_np).cuda(), shift)
+        import oracle
+        prim = lj.synth.smooth_periodic_prim(xyz_np, (1.0, 1.3, 0.8), amp=0.2, seed=4)
+        Q = torch.from_numpy(oracle.prim_to_cons(oracle.params(periodic=per, bc=0), prim)).cuda()
+    gen = torch.Generator(device="cuda").manual_seed(11)
+
+    def randn(*s):
+        return torch.randn(s + shape, dtype=torch.float64, device="cuda", generator=gen)
+
+    Q[4] += 1e-2 / 0.4 * randn()
+    dQ, lamR = 1e-2 * randn(5), randn(5)
+    eps = 1e-6
+    ends = [(Q + s * eps * dQ) for s in (1.0, -1.0)]
+    R2, MK2 = [torch.empty_like(Q) for _ in ends], [torch.empty_like(Q[:2]) for _ in ends]
+    for e, r, m in zip(ends, R2, MK2):
+        ctx.les_rhs(e, r)
+        ctx.les_mu_eff(e, m)
+    fd, dMK = (R2[0] - R2[1]) / (2 * eps), (MK2[0] - MK2[1]) / (2 * eps)
+    aw = ctx.adjoint_workspace()
+    R, dR, R_ref = torch.empty_like(Q), torch.empty_like(Q), torch.empty_like(Q)
+    ctx.les_rhs_jvp(Q, dQ, dMK, R, dR, aw)
+    ctx.les_rhs(Q, R_ref)
+    assert torch.equal(R, R_ref)
+    size = dR.abs().amax(dim=(1, 2, 3), keepdim=True)
+    off = ((fd - dR).abs() > 1e-6 * size).any(dim=0)
+    assert float(off.double().mean()) <= 1e-3
+    lamQ, lamMK = torch.empty_like(Q), torch.empty_like(dMK)
+    ctx.les_rhs_vjp(Q, lamR, lamQ, lamMK, aw)
+    lhs, rhs = _vdot(lamR, dR), _vdot(lamQ, dQ) + _vdot(lamMK, dMK)
+    assert abs(lhs - rhs) <= 1e-12 * _vdot(lamR.abs(), dR.abs()), (lhs, rhs)
+
+
 def _step_ctx(lj, torch, shape, amps):
     ctx, xyz = _jet(lj, torch, shape, Re=500.0, dt_mode=lj.DT_FIXED, dt_fixed=1.0e-3,
                     amp=tuple(amps))
