@@ -41,8 +41,11 @@ struct JetBC {
 // or by a node's density takes the reciprocal at hand, the sound speed and its
 // reciprocal come from one root, and Mach numbers are compared without being
 // formed.)
-// x/d from id, d's rounded reciprocal: the product corrected by its residual
-// (Markstein, 1990), so that the boundary states round as with divisions.
+// x/d from id, d's reciprocal: the product corrected by its residual (Markstein,
+// 1990).  With the rounded reciprocals of gamma, gamma - 1 and a density it
+// rounds as the division does; with a_e's (rsqrt) it may miss that by an ulp.
+// (Plain products remain, one rounding more than a division: velocities from
+// momenta, the exit's sound speed, unit normals from rsqrt.)
 __device__ __forceinline__ double div_by(double x, double d, double id) {
   const double q = x * id;
   return fma(fma(-q, d, x), id, q);
@@ -85,38 +88,33 @@ __device__ __forceinline__ double pow_entropy(double x, double e) {
   return pow(x, e);
 }
 
-// x > 0, finite and no subnormal (on the integer pipe).
-__device__ __forceinline__ bool is_ordinary(double x) {
-  return (unsigned)__double2hiint(x) - 0x00100000u < 0x7fe00000u;
-}
-
 // Riemann-invariant state of a far-field node from its interior neighbour's
 // primitives and the unit outward normal, the free stream at rest (rho = 1,
 // p = 1/gamma, a = 1): R+ = q_n,e + 2 a_e/(gamma-1), R- = -2/(gamma-1), four
 // branches by q_n,e/a_e.  Returns true for the supersonic exit (the caller
 // copies the neighbour's conserved values); otherwise the primitives of the
 // boundary state are in f = (rho, u, v, w, p).
-// (Where T = gamma p/rho has no ordinary root, a_e and the Mach number are
-// formed as written: a zero T makes it infinite, and with a NaN no comparison
-// holds, which leaves the free stream.)
+// (The comparisons of q_n,e select as those of q_n,e/a_e do beside a T = gamma
+// p/rho without a sound speed too: with T = 0 the quotient is infinite or, at
+// rest, a NaN, with a negative T or a NaN it is a NaN, which compares with
+// nothing and leaves the free stream.)
 __device__ __forceinline__ bool far_field_state(const JetBC& b, double rho, double ir, double u,
                                                 double v, double w, double p, double nx, double ny,
                                                 double nz, double f[5]) {
   const double T = div_by(b.gamma * p, rho, ir), ra = rsqrt(T), a0 = T * ra;
-  double ae = fma(fma(-a0, a0, T), 0.5 * ra, a0);  // sqrt(T), one Newton step on T ra
+  // sqrt(T): one Newton step on T ra, or T itself where it is 0 or infinite
+  const double T0 = b.gamma * p * ir;
+  const unsigned h0 = (unsigned)__double2hiint(T0);
+  const bool self = h0 == 0x7ff00000u || (h0 | (unsigned)__double2loint(T0)) == 0u;
+  const double ae = self ? T0 : fma(fma(-a0, a0, T), 0.5 * ra, a0);
   const double qne = u * nx + v * ny + w * nz;
-  double Mn = qne, M1 = ae;  // q_n,e/a_e against 1 as q_n,e against a_e
-  if (!is_ordinary(T)) {
-    ae = sqrt(b.gamma * p / rho);
-    Mn = qne / ae;
-    M1 = 1.0;
-  }
   const double Rp = qne + div_by(2.0 * ae, b.gm1, b.igm1);
   const double Rm = b.rm;
   const double qnf = 0.5 * (Rp + Rm);
   const double af = 0.25 * b.gm1 * (Rp - Rm);
-  if (Mn >= M1) return true;
-  if (Mn >= 0.0) {
+  // q_n,e/a_e >= 1, >= 0, > -1
+  if (qne >= ae && qne > 0.0) return true;
+  if (qne >= 0.0 && qne < ae) {
     // entropy of the interior node: rho_f = (rho_e^gamma a_f^2/(gamma p_e))^(1/(gamma-1))
     // = rho_e (a_f/a_e)^(2/(gamma-1)), one power instead of two
     const double dq = qnf - qne;
@@ -126,7 +124,7 @@ __device__ __forceinline__ bool far_field_state(const JetBC& b, double rho, doub
     f[2] = v + dq * ny;
     f[3] = w + dq * nz;
     f[4] = div_by(rf * af * af, b.gamma, b.ig);
-  } else if (Mn > -M1) {
+  } else if (qne < 0.0 && qne > -ae) {
     // free-stream entropy (rho = 1, p = 1/gamma): rho_f = a_f^(2/(gamma-1))
     const double rf = pow_entropy(af, -b.rm);
     f[0] = rf;
@@ -361,10 +359,9 @@ __global__ void __launch_bounds__(kBcThreads)
     double rho, ir, u, v, w, p;
     load_prim(Q, N, ne, b.gm1, rho, ir, u, v, w, p);
     const double ae = sqrt(b.gamma * p * ir);
-    // q_n/a_e >= 1, q_n = u . e/|e| (as written where a_e is no ordinary value)
-    const double qg = u * ex + v * ey + w * ez, ag = ae * gn;
-    const bool ordinary = is_ordinary(ag);
-    if (ordinary ? qg >= ag : qg / ag >= 1.0) {
+    // q_n/a_e >= 1, q_n = u . e/|e| (which a_e = 0 makes a NaN at rest)
+    const double qg = u * ex + v * ey + w * ez;
+    if (qg >= ae * gn && qg > 0.0) {
 #pragma unroll
       for (int q = 0; q < 5; ++q) Q.st(q * N + nx_, Q.ld(q * N + ne));
     } else {
@@ -374,8 +371,8 @@ __global__ void __launch_bounds__(kBcThreads)
       Q.st(N + nx_, rf * u);
       Q.st(2 * N + nx_, rf * v);
       Q.st(3 * N + nx_, rf * w);
-      const double q2 = u * u + v * v + w * w;
-      Q.st(4 * N + nx_, ordinary ? b.einf + 0.5 * rf * q2 : rf * (p / (b.gm1 * rho) + 0.5 * q2));
+      // (p - p is 0, and a NaN where rho_f e_int is one: p infinite)
+      Q.st(4 * N + nx_, (b.einf + (p - p)) + 0.5 * rf * (u * u + v * v + w * w));
     }
   }
 }
