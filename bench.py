@@ -68,16 +68,16 @@ NCU_SOURCES = {"stage_fused": ("paper_2301_00817_gb300/csrc/fused_kernel.cuh",
                           "paper_2301_00817_gb300/csrc/lesjet_dev.cuh")}
 NCU_COUNTS = {
     ("stage_fused", "bytes_per_point"):
-        (110.4, "f906b4f522285153b4758fb39878ed420391ea1df5375ee7ad8e4f483522b599"),
+        (110.4, "bcd3ef937c6ad9e4d935377e742e65b544502f2318244751bdc5ec3243c9a4df"),
     ("stage_fused", "fp32_flop_per_point"):
-        (901, "f906b4f522285153b4758fb39878ed420391ea1df5375ee7ad8e4f483522b599"),
+        (901, "bcd3ef937c6ad9e4d935377e742e65b544502f2318244751bdc5ec3243c9a4df"),
     # smsp__inst_executed.sum x 32 per point, mean of the five stages
     ("stage_fused", "inst_per_point"):
-        (1599, "f906b4f522285153b4758fb39878ed420391ea1df5375ee7ad8e4f483522b599"),
+        (1599, "bcd3ef937c6ad9e4d935377e742e65b544502f2318244751bdc5ec3243c9a4df"),
     # FP64 flop (dadd + 2 x dfma + dmul) per grid point of one residual's
     # k_flux3 on the 96 x 160 x 128 jet
     ("flux64", "fp64_flop_per_point"):
-        (658, "341666bbba272dd2dda07a3dca2e648d16974d38e599b531c3659f8a85118823"),
+        (658, "ee5d48a97e21075a39c8a977a2a7865eedf298c63e110bebfe4b662af026daf6"),
 }
 NCU_CAPTURE = {"stage_fused": "profiles/stage_fused_jet96x160x128.md",
                "flux64": "profiles/flux64_jet96x160x128.md"}

@@ -15,7 +15,9 @@
 //
 // Non-differentiable points follow the forward kernels' branch choices:
 // |x| has derivative -1 for x < 0 and +1 otherwise, max(a, b) passes the
-// cotangent to the operand the comparison selected.
+// cotangent to the operand the comparison selected.  (The boundary formulas
+// select by a Mach number that they round in their own way: within an ulp or two
+// of 1, 0 or -1 they may differentiate the branch beside the forward's.)
 //
 // Step adjoint (Eq. localdt with a fixed time step): with stage states S_l,
 // Q^(l) = Q^(0) - alpha_l dt J RHS(Q^(l-1)) on interior nodes and Q^(l) =
@@ -382,9 +384,9 @@ __device__ __forceinline__ void adj_zeta(const Grid& g, const Consts<double>& K,
 }
 
 // The three directions' records in one launch, split as k_flux3's.  Bound by
-// the FP64 pipe like the forward kernel: about 165 operations per interface
-// (some 420 when the gradient tensor was formed, the stress reversed term by
-// term and the centred flux reversed twice per node).
+// the FP64 pipe like the forward kernel: 206 operations per interface with
+// chunks of 16 (209 with 4, 222 without; 429 when the gradient tensor was formed,
+// the stress reversed term by term and the centred flux reversed twice per node).
 __global__ void __launch_bounds__(kFluxThreads, 2)
     k_adj_flux3(Grid g, Consts<double> K, AdjIO io, unsigned b0, unsigned b1, int len) {
   begin_dependent();
@@ -444,8 +446,8 @@ __global__ void __launch_bounds__(256) k_adj_sensor_terms(Grid g, const double* 
 // (g-1)(Q4 - rho|u|^2/2), T = g p/rho.  mu/kappa cotangents are added to
 // lamMK.  |grad d| comes from gn ([3][N], set-up).
 // A node reads about 240 values (its interfaces' records within two nodes
-// along each direction), few of them twice by one thread, and does about 400
-// FP64 operations, whose pipe bounds it; gathering straight into
+// along each direction), few of them twice by one thread, and does 373 FP64
+// operations, whose pipe bounds it; gathering straight into
 // the node's reverse saves the 18 accumulator fields of a pass of their own.
 __global__ void __launch_bounds__(128, 3)
     k_adj_node(Grid g, Consts<double> K, const double* __restrict__ Q,

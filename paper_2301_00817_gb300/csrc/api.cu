@@ -234,7 +234,7 @@ bool jet_bc(const les_ctx* c) { return c->p.bc == LES_BC_JET || c->p.bc == LES_B
 // conditions and totals read the FP32 metrics.
 bool has_m64(const les_ctx* c) { return c->p.precision != LES_PREC_MIXED_COMPACT; }
 
-// ---- FP64 form: node, viscosity, per-direction flux and update passes
+// ---- FP64 form: node, viscosity, flux and update passes
 lesjet::StageIO64 io64(les_ctx* c, const double* Qin) {
   lesjet::StageIO64 io;
   io.Qin = Qin;

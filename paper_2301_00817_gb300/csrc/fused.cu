@@ -17,7 +17,8 @@ namespace lesjet {
 // at most 2^28 units is exact in an int, whose float (rounded to nearest)
 // times the unit is lo.  Values that the bit form does not cover (the
 // neighbourhood of the float range's ends, infinities, NaN) take the
-// conversions.
+// conversions, which flush: below 2^-72 a lo, below 2^-126 a hi that would be
+// subnormal is a zero.
 __device__ __forceinline__ void split_value(double v, float& h, float& l) {
   const unsigned top = (unsigned)__double2hiint(v), low = (unsigned)__double2loint(v);
   const unsigned sign = top & 0x80000000u, mag = top & 0x7fffffffu, e = mag >> 20;

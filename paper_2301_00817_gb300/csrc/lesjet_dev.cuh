@@ -245,10 +245,12 @@ struct Launch {
 // more a step in series: the gap between two was a tenth of the 48 x 24 x 32
 // step (323 -> 285 us; the adjoint window on 64 x 40 x 48 30.8 -> 29.5 ms).
 // Letting the next kernel start before the last block of this one (an early
-// trigger) was slower everywhere, its waiting blocks taking SM places, and
-// the mixed step's graph, whose edges are cheap, gains nothing: its kernels
-// are launched plainly.  Every kernel that is launched so begins with
-// begin_dependent, so the end of one implies that of all before it.
+// trigger) was slower everywhere, its waiting blocks taking SM places.  The
+// mixed step's graph, whose edges are cheap, gains nothing: its prestep, axis
+// viscosity and stage kernels are launched plainly, while its boundary
+// conditions and dynamic procedure are launched so, as in the FP64 form (the
+// captured graph holds programmatic edges there).  Every kernel that is launched
+// so begins with begin_dependent, so the end of one implies that of all before it.
 template <typename... P, typename... A>
 inline void launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
                              const Launch& L, A&&... args) {

@@ -234,7 +234,7 @@ __global__ void __launch_bounds__(256) k_mu(Grid g, Consts<R> K, const TQ* __res
   }
 }
 
-// ------------------------------------------------------------------ k_flux
+// ----------------------------------------------------------------- k_flux3
 // Pressure sensor |p+ - 2p + p-| / (p+ + 2p + p-) from the three pressures
 // around a node; a face node of a non-periodic direction takes its inward
 // neighbour's value.  The second difference is that of the two first ones,
@@ -595,13 +595,14 @@ __device__ __forceinline__ void flux_zeta(const Grid& g, const Consts<R>& K,
 // value, F[D][5][N] at the interface's node a): blocks [0, b0) take xi and the
 // next b1 eta in chunks of len interfaces, the rest zeta.  Bound by
 // the FP64 pipe, which issues one warp instruction per 64 cycles and
-// scheduler, so the shape is chosen for the fewest FP64 operations: about 157
-// per interface with chunks of 8 (205 before the node part was shared and
-// the dissipation and viscous sums regrouped); 85 to 87 % of the pipe's rate.
+// scheduler, so the shape is chosen for the fewest FP64 operations: 160 per
+// interface with chunks of 16 (162 with 8, 165 with 4, 172 with 2, 185 without;
+// 218 with the sensor pass's share before the node part was shared and the
+// dissipation and viscous sums regrouped); 85 to 88 % of the pipe's rate.
 // Comparisons and absolute values are done on the integer pipe (dev_max,
 // dev_abs).  Against one launch per direction with a sensor pass ahead of
-// them: the 192 x 96 x 128 step 18.3 -> 13.1 ms, the 48 x 24 x 32 step (three
-// launches fewer per residual) 0.50 -> 0.27 ms.
+// them: the 192 x 96 x 128 step 18.3 -> 13.0 ms, the 48 x 24 x 32 step (three
+// launches fewer per residual) 0.50 -> 0.26 ms.
 template <typename R, typename TQ, typename TM>
 __global__ void __launch_bounds__(kFluxThreads, sizeof(R) == 8 ? 2 : 1)
     k_flux3(Grid g, Consts<R> K, FluxIO<R, TQ, TM> io, unsigned b0, unsigned b1, int len) {
@@ -623,7 +624,7 @@ struct FluxPlan {
   int len;
 };
 inline FluxPlan flux_plan(const Grid& g) {
-  // A chunk repeats one node's part, 22 of its 142 FP64 operations per
+  // A chunk repeats one node's part, 39 FP64 operations beside the 159 of each
   // interface.  The chunks' blocks come first and zeta's, one interface per
   // thread, fill the end, so a chunk may last half of an SM's share (waves of
   // the two resident blocks of one interface per thread).  Against a dozen

@@ -1,4 +1,4 @@
-"""The fused stage kernel's jet-grid instantiations on a grid that its 16 x 32
+"""The fused stage kernel's jet-grid instantiations on a grid that its 8 x 32
 (eta, zeta) tiles cover exactly (24 x 32 x 32): xi and eta bounded, zeta
 periodic, the shifted 16-byte staging and every thread owning a column are
 then fixed at compile time.  Every variant of the stage kernel runs 20 steps
@@ -7,9 +7,9 @@ in both mixed forms against the FP64 oracle's 20 steps (relative L2 within
 static SGS model, local steps (Eq. localdt), the characteristic entrance
 (Sec. "Entrance Boundary"), the dynamic model (Sec. "Dynamic Smagorinsky
 Model") and the centerline grid (Sec. "Centerline Boundary Condition").
-The other jet tests run on 48 x 24 x 32, whose eta extent the tiles do not
-cover, and so exercise the instantiations that decide the cover at run
-time."""
+(The tiles cover 48 x 24 x 32, which the other jet tests run on, as well; the
+instantiations that decide the cover at run time have the eta and zeta extents
+of test_gpu_tile_rows.)"""
 import numpy as np
 import pytest
 

@@ -1,6 +1,6 @@
 """The fused stage kernel on rows that its 16-byte staging cannot take: row
 lengths that are no multiple of four, shorter than a tile, one over a tile,
-and eta extents around the tile's 16 rows, on the jet grid and on boxes that
+and eta extents around the tiles' 8 and 16 rows, on the jet grid and on boxes that
 are periodic or open in every direction.  The residual against the oracle's,
 within the 2e-5 of each component's flux scale of the other mixed-form
 tests; then every variant of the stage on one such jet, five steps within
